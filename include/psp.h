@@ -110,15 +110,15 @@ typedef struct {
   int tc_min_dim;     /* complex64 path: fronts with s >= tc_min_dim and u >= tc_min_dim take the tensor
                          cores, the others CUDA cores; <= 0 selects the default (64) */
   int sweep_level_tasks; /* sweep schedule: tasks a tree level is split into at least (row / column
-                            blocks of 8..64); <= 0 selects the default (608) */
+                            blocks of 8..256); <= 0 selects the default (304) */
   int sweep_ctas_per_sm; /* sweep schedule: resident CTAs per SM of the persistent sweep (capped by
                             occupancy); <= 0 selects the default (8) */
   int setup_temp_mb;   /* cap, in MiB, on the per-front temporaries of one batch of fronts during setup
                           (a level whose fronts need more is factored in several batches); <= 0: up
                           to 80 % of the device memory left after the factors and update matrices */
-  int sweep_rhs_group; /* sweep schedule: most right-hand sides (1, 2, 4 or 8) one CTA carries through a
-                          pass over a factor block; <= 0: as many as the application has, at most 8 (the
-                          task's vector is staged through 64 KB of shared memory in chunks) */
+  int sweep_rhs_group; /* sweep schedule: most right-hand sides (1, 2, 4 or 8; complex128 factors: at most 4) one
+                          CTA carries through a pass over a factor block; <= 0: as many as the application has, at
+                          most 8 (the task's vector is staged through shared memory in chunks) */
   int solve_rhs_group; /* psp_solve: most right-hand sides per GMRES run; <= 0: as many as fit the free
                           device memory (single-problem handles) */
   int sweep_min_rows;   /* sweep schedule: fewest rows (up) / columns (down) of a front per task, 8 .. 64;

@@ -320,13 +320,17 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmTask<T>* __restrict__ ta
   }
 }
 
-// strict lower part of W -> strict lower part of F_TL (D stays on the diagonal)
+// strict lower part of W -> strict lower part of F_TL (D stays on the diagonal; without inversion L_TL stays
+// too), and the pivots' reciprocals for the sweep
 template <typename T>
 __global__ void __launch_bounds__(256) k_copy_linv(const FrontTask<T>* __restrict__ fronts,
                                                    const ColTask* __restrict__ tasks) {
   const ColTask tk = tasks[blockIdx.x];
   const FrontTask<T> ft = fronts[tk.front];
   const int ld = ft.s + ft.u;
+  for (int c = tk.c0 + threadIdx.x; c < tk.c1; c += blockDim.x)
+    ft.dinv[c] = cdiv(CplxTraits<T>::one(), ft.G[(int64_t)c * (ld + 1)]);
+  if (!ft.W) return;
   for (int c = tk.c0; c < tk.c1; ++c)
     for (int r = c + 1 + threadIdx.x; r < ft.s; r += blockDim.x)
       ft.G[(int64_t)c * ld + r] = ft.W[(int64_t)c * ft.s + r];

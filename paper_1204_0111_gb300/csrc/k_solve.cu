@@ -1,5 +1,5 @@
-// Multifrontal solve with selectively inverted fronts (§2.2), one tree level per launch, as the
-// T_i of Alg. 1.3 inside the sweep of Alg. 1.5.
+// Multifrontal solve with selectively inverted fronts (§2.2) as the T_i of Alg. 1.3 inside the sweep
+// of Alg. 1.5: the whole sweep in one persistent launch.
 //
 // Each front stores G = [inv(L_TL) (unit lower, D on the diagonal); M_BL = L_BL inv(L_TL)], so
 //   up the tree:   v_S = inv(L_TL) w_S,  x_S = D^{-1} v_S,  update_U = w_U - M_BL w_S
@@ -10,187 +10,285 @@
 // summation order is fixed.  Extension by zero over the pad, the plane coupling J_{i+1,i} of
 // the previous / next panel and the extraction of the panel's planes are fused into the
 // gathers and the final write.
+//
+// Work vectors (xf, xb, upd) are kept per right-hand-side group of RG columns, entry after entry
+// with the group's columns adjacent: a gathered entry is one contiguous read for the whole group.
 #include "cplx.cuh"
 #include "psp_internal.h"
 
 namespace psp {
 
+constexpr int kComputeThreads = 256;                    // product threads of a sweep CTA
+constexpr int kComputeWarps = kComputeThreads / 32;
+constexpr int kSweepThreads = kComputeThreads + 64;     // + the scheduling warp and the signalling warp
+constexpr int kGatherIdx = 256;   // index words (16 bytes) of front rows a slot holds; the rest are read from global memory
+constexpr int kOwnIdx = 256;      // index words of a task's own rows (sweep_max_rows at most)
+
+// named barriers: 1 among the product warps; per task slot, ready (scheduler -> product warps), done
+// (product warps -> signaller) and free (signaller -> scheduler)
+enum SweepBarrier { kBarCompute = 1, kBarReady = 2, kBarDone = 4, kBarFree = 6 };
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void compute_sync() { bar_sync(kBarCompute, kComputeThreads); }
+
+// one task as the product warps see it, filled by the scheduling warp.  The product warps read a field where they
+// need it (a broadcast from shared memory) rather than keep it in a register across their loops.
 template <typename T>
-__device__ __forceinline__ T input_value(const SolveCtx<T>& cx, int node, int q) {
-  const int nx = cx.sh.nx;
-  const int plane = nx * cx.sh.ny;
-  const int own = node - cx.lead * plane;                 // index within the panel's planes
-  if (own < 0) return CplxTraits<T>::zero();              // extension by zero over the pad (Alg. 1.3)
-  const int64_t g = (int64_t)own + (int64_t)plane * cx.z0;
-  const double2* uq = cx.u + (int64_t)q * cx.N;
-  double2 v;
-  if (cx.mode == 0) {
-    // u_i - J_{i,i-1} u_{i-1}: J's coupling entry is -s1 s2 / s3(z0 - 1/2) / h^2
-    v = __ldcg(uq + g);
-    if (cx.has_prev && own < plane) {
-      const int x = own % nx, y = own / nx;
-      const double2 a = cscale(cmul(cmul(cx.s1n[x], cx.s2n[y]), cx.s3h[cx.z0]), cx.inv_h2);
-      cfma(v, a, __ldcg(uq + g - plane));
+struct TaskSlot {
+  int ok;                 // 0: stop
+  int tr_log;             // up: 2^tr_log threads along the rows
+  int splits;             // down: warps that share a block of columns
+  int pad_;
+  const T* G;             // the front's block
+  const T* dinv;          // its reciprocal pivots
+  const int4* rows_g;     // its rows' index words in global memory
+  const int32_t* sel_g;   // its struct indices in global memory
+  T* xf;                  // the problem's work vectors and vector block
+  T* xb;
+  T* upd;                 // at the front's update vector: own_upd; children's entries are relative to upd
+  double2* u;
+  StepRec st;
+  QueueEntry e;
+  FrontRec fr;
+  int4 rows[kGatherIdx];  // up: index words of the S rows; down: struct indices (int32)
+  int4 own[kOwnIdx];      // up: index words of the task's rows r >= s
+};
+
+// shared-memory elements per vector entry: RG columns, padded by 16 bytes where the lanes of a quarter
+// warp reading consecutive entries with 128-bit loads would meet in the same banks
+template <typename T, int RG>
+__host__ __device__ constexpr int entry_stride() {
+  return RG * (int)sizeof(T) <= 16 ? RG : RG + 16 / (int)sizeof(T);
+}
+
+// RG adjacent entries from shared memory
+template <typename T, int RG>
+__device__ __forceinline__ void load_shared(const T* p, T (&v)[RG]) {
+  if constexpr (sizeof(T) == 8 && RG >= 2) {
+#pragma unroll
+    for (int q = 0; q < RG; q += 2) {
+      const float4 f = *reinterpret_cast<const float4*>(p + q);
+      v[q] = make_float2(f.x, f.y);
+      v[q + 1] = make_float2(f.z, f.w);
     }
   } else {
-    // J_{i+1,i}^T u_{i+1}: supported on the panel's last plane
-    v = make_double2(0.0, 0.0);
-    const int last = own - (cx.z1 - cx.z0 - 1) * plane;
-    if (cx.has_next && last >= 0) {
-      const int x = last % nx, y = last / nx;
-      const double2 a = cscale(cmul(cmul(cx.s1n[x], cx.s2n[y]), cx.s3h[cx.z1]), -cx.inv_h2);
-      v = cmul(a, __ldcg(uq + g + plane));
-    }
+#pragma unroll
+    for (int q = 0; q < RG; ++q) v[q] = p[q];
   }
-  return CplxTraits<T>::from(v);
 }
 
+// right-hand-side group g of the sweep: its columns [g RG, g RG + w); vec: the group is full and its vectors are
+// 16-byte aligned
+struct Group {
+  int g, w;
+  bool vec;
+};
+
+// the group's columns of one work-vector entry from global memory (L2: other SMs wrote them); base: group 0's
+// vector of ld entries
 template <typename T, int RG>
-__device__ __forceinline__ void pull_add(const SolveCtx<T>& cx, const int32_t* pl, int rhs0, T* out) {
+__device__ __forceinline__ void load_entry(const T* base, const int64_t ld, const int64_t entry, const Group gr, T (&v)[RG]) {
+  if constexpr (RG == 1) {
+    v[0] = __ldcg(base + gr.g * ld + entry);
+  } else {
+    const T* p = base + gr.g * RG * ld + entry * gr.w;
+    if (sizeof(T) == 8 && gr.vec) {
 #pragma unroll
-  for (int t = 0; t < 2; ++t) {
-    const int32_t o = pl[t];
-    if (o < 0) break;
+      for (int q = 0; q < RG; q += 2) {
+        const float4 f = __ldcg(reinterpret_cast<const float4*>(p + q));
+        v[q].x = f.x;
+        v[q].y = f.y;
+        v[q + 1].x = f.z;
+        v[q + 1].y = f.w;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < RG; ++q) v[q] = q < gr.w ? __ldcg(p + q) : CplxTraits<T>::zero();
+    }
+  }
+}
+template <typename T, int RG>
+__device__ __forceinline__ T* entry_ptr(T* base, const int64_t ld, const int64_t entry, const Group gr) {
+  if constexpr (RG == 1) return base + gr.g * ld + entry;
+  else return base + gr.g * RG * ld + entry * gr.w;
+}
+
+// children's update entries a and b (-1: none): both reads are issued before either is used
+template <typename T, int RG>
+__device__ __forceinline__ void pull_entries(const TaskSlot<T>& sl, const int64_t ld, const Group gr, const int a, const int b,
+                                             T (&v)[RG]) {
+  T t[RG];
+#pragma unroll
+  for (int q = 0; q < RG; ++q) v[q] = t[q] = CplxTraits<T>::zero();
+  if (a >= 0) load_entry<T, RG>(sl.upd, ld, a, gr, v);
+  if (b >= 0) load_entry<T, RG>(sl.upd, ld, b, gr, t);
+#pragma unroll
+  for (int q = 0; q < RG; ++q) v[q] = cadd(v[q], t[q]);
+}
+
+// The panel's input at a box node: forward u_i - J_{i,i-1} u_{i-1}, backward J_{i+1,i}^T u_{i+1} (supported on the
+// panel's last plane); zero over the pad (Alg. 1.3).  J's coupling entry is -s1 s2 / s3 / h^2.
+template <typename T, int RG>
+__device__ __forceinline__ void input_entry(const TaskSlot<T>& sl, const Group gr, const int node, T (&v)[RG]) {
+  const StepRec& st = sl.st;
+  const int own = node - st.lead * st.plane;   // index within the panel's planes
+  const int at = st.mode == 0 ? own : own - (st.z1 - st.z0 - 1) * st.plane;   // index within the coupled plane
+  const bool coupled = st.couple && own >= 0 && (st.mode == 0 ? own < st.plane : at >= 0);
+  double2 x[RG];
+#pragma unroll
+  for (int q = 0; q < RG; ++q) x[q] = make_double2(0.0, 0.0);
+  const double2* u = sl.u + gr.g * RG * st.N + ((int64_t)st.plane * st.z0 + own);
+  if (st.mode == 0 && own >= 0) {
 #pragma unroll
     for (int q = 0; q < RG; ++q)
-      if (rhs0 + q < cx.nrhs) out[q] = cadd(out[q], __ldcg(cx.upd + (int64_t)(rhs0 + q) * cx.upd_ld + o));
+      if (RG == 1 || q < gr.w) x[q] = __ldcg(u + q * st.N);
   }
+  if (coupled) {
+    u += st.mode == 0 ? -(int64_t)st.plane : (int64_t)st.plane;
+    const double2 a = cscale(cmul(cmul(__ldg(st.s1n + at % st.nx), __ldg(st.s2n + at / st.nx)), __ldg(st.s3c)), st.cz);
+#pragma unroll
+    for (int q = 0; q < RG; ++q)
+      if (RG == 1 || q < gr.w) cfma(x[q], a, __ldcg(u + q * st.N));
+  }
+#pragma unroll
+  for (int q = 0; q < RG; ++q) v[q] = CplxTraits<T>::from(x[q]);
 }
 
-// w_S entries [j0, j1) of front sn (zero-extended input + children's updates) for right-hand sides
-// [rhs0, rhs0 + RG) into w (right-hand side major, ld chunk).  Each thread first loads the node ids
-// and pull offsets of GU entries, then all of their values, so that a thread has GU independent
-// gathers in flight rather than one chain of dependent loads after another.
-template <typename T, int RG>
-__device__ __forceinline__ void gather_w(const SolveCtx<T>& cx, const int first, const int32_t* pull, const int j0,
-                                         const int j1, const int rhs0, T* w, const int chunk) {
-  constexpr int GU = RG >= 4 ? 1 : (RG == 2 ? 2 : 4);
-  for (int p0 = j0 + threadIdx.x; p0 < j1; p0 += GU * blockDim.x) {
-    int node[GU];
-    int32_t pa[GU], pb[GU];
+// Sums NV per-lane scalars over the warp with halving exchanges: after the exchange over `off` each lane keeps
+// half of its values, so NV values cost about NV + 5 shuffles instead of 5 NV.  Lane l ends with the totals of
+// indices base .. base + max(1, NV / 32) - 1; `lead` marks the one lane of each total that stores it.
+template <typename R, int NV>
+__device__ __forceinline__ void warp_sum(R (&v)[NV], const int lane, int& base, bool& lead) {
+  base = 0;
+  lead = true;
+  int off = 16;
 #pragma unroll
-    for (int t = 0; t < GU; ++t) {
-      const int p = p0 + t * blockDim.x;
-      const bool in = p < j1;
-      node[t] = in ? cx.sh.order[first + p] : 0;
-      pa[t] = in ? pull[2 * p] : -1;
-      pb[t] = in ? pull[2 * p + 1] : -1;
-    }
-    T v[GU][RG];
+  for (int n = NV; n > 1 && off > 0; n >>= 1, off >>= 1) {
+    const int half = n >> 1;
+    const bool up = lane & off;
 #pragma unroll
-    for (int t = 0; t < GU; ++t)
-#pragma unroll
-      for (int q = 0; q < RG; ++q) {
-        T x = CplxTraits<T>::zero();
-        if (p0 + t * blockDim.x < j1 && rhs0 + q < cx.nrhs) {
-          x = input_value(cx, node[t], rhs0 + q);
-          const T* uq = cx.upd + (int64_t)(rhs0 + q) * cx.upd_ld;
-          if (pa[t] >= 0) x = cadd(x, __ldcg(uq + pa[t]));
-          if (pb[t] >= 0) x = cadd(x, __ldcg(uq + pb[t]));
-        }
-        v[t][q] = x;
+    for (int k = 0; k < NV / 2; ++k)
+      if (k < half) {
+        const R send = up ? v[k] : v[k + half];
+        const R keep = up ? v[k + half] : v[k];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
       }
-#pragma unroll
-    for (int t = 0; t < GU; ++t) {
-      const int p = p0 + t * blockDim.x;
-      if (p < j1)
-#pragma unroll
-        for (int q = 0; q < RG; ++q) w[q * chunk + (p - j0)] = v[t][q];
-    }
+    if (up) base += half;
+  }
+  for (; off > 0; off >>= 1) {
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+    if (lane & off) lead = false;
   }
 }
 
-// up-the-tree task: rows [r0, r1) of front sn, right-hand sides [rhs0, rhs0 + RG).
+// factor entries in flight: columns per thread (up), blocks of `cols` columns times 32-row steps per warp (down)
+template <typename T, int RG>
+struct Tile {
+  static constexpr bool wide = sizeof(T) == 16;
+  static constexpr int up = wide ? (RG == 1 ? 2 : 4) : (RG == 1 ? 8 : 4);
+  static constexpr int cols = RG == 8 ? 2 : 4;
+  static constexpr int down = RG >= 2 ? 1 : (wide ? 1 : 2);
+};
+
+// up-the-tree task: rows [r0, r1) of one front, one right-hand-side group.
 // phase 0 gathers w_S (zero-extended input + children's updates) and, for rows r < s, writes
 // x_r = D^{-1} y_r with y_S = inv(L_TL) w_S (and y_r itself into xb when the second phase needs it);
 // for rows r >= s it writes the update w_U - M_BL w_S (extended selective inversion).
 // phase 1 (factors keeping L_BL) takes y_S from xb and writes the update w_U - L_BL y_S of rows r >= s.
-template <typename T, int RG>
-__device__ __forceinline__ void fwd_task(const SolveTask tk, const int rhs0, const SolveCtx<T>& cx, const int R,
-                                         unsigned char* smem_raw, const int phase, const int chunk) {
-  const int sn = tk.sn;
-  const int s = cx.sh.s[sn], u = cx.sh.u[sn], ld = s + u;
-  const int first = cx.sh.first[sn];
-  const T* G = cx.G + cx.sh.g_off[sn];
-  const int32_t* pull = cx.sh.pull + 2 * cx.sh.pull_ptr[sn];
-  // the vector w_S (or y_S) passes through shared memory in chunks of `chunk` entries (a multiple of
-  // 256), so a CTA carries RG right-hand sides over a factor block of any width and reads it once
-  T* w = reinterpret_cast<T*>(smem_raw);        // RG x chunk (right-hand side major: no bank conflicts
-                                                 // when a warp spans several columns, R < 32)
-  T* red = w + (int64_t)chunk * RG;              // blockDim x RG
-
-  const int i = threadIdx.x % R, grp = threadIdx.x / R, ngrp = blockDim.x / R;
-  const int r = tk.r0 + i;
-  const int jmax = r < tk.r1 ? (r < s ? r : s) : 0;   // strictly lower part of inv(L_TL), all of the bottom block
-  const int jend = min(tk.r1, s);                      // entries of w_S this task needs (w_r of its rows r < s too)
-  T acc[RG], wr[RG];
+//
+// Thread (i, grp) sums row r0 + i over the columns grp, grp + ngrp, ...
+template <typename T, int RG, int PHASE, bool EXT>
+__device__ __forceinline__ void fwd_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr, unsigned char* smem) {
+  constexpr int SP = entry_stride<T, RG>(), U = Tile<T, RG>::up;
+  const int tid = threadIdx.x;
+  T* own = reinterpret_cast<T*>(smem);            // the task's rows' own entries: w_r, r < s, or w_U
+  T* part = own + kComputeThreads * RG;           // partial sums, (group, row, right-hand side)
+  T* w = part + kComputeThreads * RG;             // chunk x SP: w_S (or y_S)
+  const int trl = sl.tr_log, ngrp = kComputeThreads >> trl, grp = tid >> trl;
+  const int s = sl.fr.s, r0 = sl.e.r0, jend = min(sl.e.r1, s);   // jend: entries of w_S this task needs
+  const int r = r0 + (tid & ((1 << trl) - 1));
+  for (int p = max(r0, s) + tid; p < sl.e.r1; p += kComputeThreads) {
+    const int4 ix = sl.own[p - r0];
+    T v[RG];
+    pull_entries<T, RG>(sl, a.upd_ld, gr, ix.y, ix.z, v);
 #pragma unroll
-  for (int q = 0; q < RG; ++q) acc[q] = wr[q] = CplxTraits<T>::zero();
-  const T* Gr = G + r;
-  const int64_t step = (int64_t)ngrp * ld;
-  for (int j0 = 0; j0 < jend; j0 += chunk) {
-    const int j1 = min(j0 + chunk, jend);
-    if (j0 > 0) __syncthreads();   // the previous chunk is consumed
-    if (phase == 0) {
-      gather_w<T, RG>(cx, first, pull, j0, j1, rhs0, w, chunk);   // w_S = zero-extended input + children's updates
-    } else {
-      for (int p = j0 + threadIdx.x; p < j1; p += blockDim.x)
+    for (int q = 0; q < RG; ++q) own[(p - r0) * RG + q] = v[q];
+  }
+  T acc[RG];
 #pragma unroll
-        for (int q = 0; q < RG; ++q)
-          w[q * chunk + (p - j0)] = (rhs0 + q < cx.nrhs) ? __ldcg(cx.xb + (int64_t)(rhs0 + q) * cx.n_loc + first + p)
-                                                      : CplxTraits<T>::zero();
+  for (int q = 0; q < RG; ++q) acc[q] = CplxTraits<T>::zero();
+  const int jmax = r < sl.e.r1 ? min(r, s) : 0;   // strictly lower part of inv(L_TL), all of the bottom block
+  for (int j0 = 0; j0 < jend; j0 += a.chunk) {
+    const int j1 = min(j0 + a.chunk, jend);
+    if (j0 > 0) compute_sync();   // the previous chunk is consumed
+    for (int p = j0 + tid; p < j1; p += kComputeThreads) {
+      T v[RG];
+      if constexpr (PHASE == 0) {
+        const int4 ix = p < kGatherIdx ? sl.rows[p] : __ldg(sl.rows_g + p);
+        T t[RG];
+        input_entry<T, RG>(sl, gr, ix.x, t);
+        pull_entries<T, RG>(sl, a.upd_ld, gr, ix.y, ix.z, v);
+#pragma unroll
+        for (int q = 0; q < RG; ++q) v[q] = cadd(v[q], t[q]);
+      } else {
+        load_entry<T, RG>(sl.xb, a.n_loc, sl.fr.first + p, gr, v);
+      }
+#pragma unroll
+      for (int q = 0; q < RG; ++q) w[(p - j0) * SP + q] = v[q];
+      if (p >= r0)
+#pragma unroll
+        for (int q = 0; q < RG; ++q) own[(p - r0) * RG + q] = v[q];
     }
-    __syncthreads();
-    if (r < tk.r1) {
-      if (r < s && r >= j0 && r < j1)
+    compute_sync();
+    const int jm = min(jmax, j1), ld = s + sl.fr.u;
+    int j = j0 + grp;
+    const T* Gp = sl.G + (int64_t)j * ld + r;
+    const T* wp = w + (j - j0) * SP;
+    for (; j < jm; j += U * ngrp, Gp += (int64_t)U * ngrp * ld, wp += U * ngrp * SP) {
+      T g[U];
 #pragma unroll
-        for (int q = 0; q < RG; ++q) wr[q] = w[q * chunk + (r - j0)];
-      // the same j sequence j = grp, grp + ngrp, ... in every chunking (j0 is a multiple of ngrp)
-      const int jm = min(jmax, j1);
-      int j = j0 + grp;
-      // eight independent factor loads in flight per thread
-      for (; j + 7 * ngrp < jm; j += 8 * ngrp) {
-        T gv[8];
+      for (int t = 0; t < U; ++t)
+        if (j + t * ngrp < jm) g[t] = __ldg(Gp + t * ngrp * ld);
 #pragma unroll
-        for (int t = 0; t < 8; ++t) gv[t] = __ldg(Gr + (int64_t)j * ld + t * step);
+      for (int t = 0; t < U; ++t)
+        if (j + t * ngrp < jm) {
+          T x[RG];
+          load_shared<T, RG>(wp + t * ngrp * SP, x);
 #pragma unroll
-        for (int t = 0; t < 8; ++t)
-#pragma unroll
-          for (int q = 0; q < RG; ++q) cfma(acc[q], gv[t], w[q * chunk + (j - j0 + t * ngrp)]);
-      }
-      for (; j < jm; j += ngrp) {
-        const T gv = __ldg(Gr + (int64_t)j * ld);
-#pragma unroll
-        for (int q = 0; q < RG; ++q) cfma(acc[q], gv, w[q * chunk + (j - j0)]);
-      }
+          for (int q = 0; q < RG; ++q) cfma(acc[q], g[t], x[q]);
+        }
     }
   }
+  // rows of a warp that several of its lanes share are summed over the lanes first
+  const int tr = 1 << trl;
+  if (tr < 32) {
 #pragma unroll
-  for (int q = 0; q < RG; ++q) red[threadIdx.x * RG + q] = acc[q];
-  __syncthreads();
-  if (grp == 0 && r < tk.r1) {
-    for (int g2 = 1; g2 < ngrp; ++g2)
+    for (int q = 0; q < RG; ++q)
+      for (int off = tr; off < 32; off <<= 1) {
+        acc[q].x += __shfl_xor_sync(0xffffffffu, acc[q].x, off);
+        acc[q].y += __shfl_xor_sync(0xffffffffu, acc[q].y, off);
+      }
+  }
+  if (tr >= 32 || (tid & 31) < tr) {
+    T* out = part + ((tr < 32 ? (tid >> 5) * tr + (tid & 31) : tid) * RG);
 #pragma unroll
-      for (int q = 0; q < RG; ++q) acc[q] = cadd(acc[q], red[(g2 * R + i) * RG + q]);
-    if (r < s) {
-      const T dinv = cdiv(CplxTraits<T>::one(), G[(int64_t)r * ld + r]);
-#pragma unroll
-      for (int q = 0; q < RG; ++q)
-        if (rhs0 + q < cx.nrhs) {
-          const T y = cadd(acc[q], wr[q]);
-          const int64_t o = (int64_t)(rhs0 + q) * cx.n_loc + first + r;
-          cx.xf[o] = cmul(y, dinv);
-          if (cx.si != PSP_SI_EXTENDED) cx.xb[o] = y;
-        }
+    for (int q = 0; q < RG; ++q) out[q] = acc[q];
+  }
+  const int nparts = tr < 32 ? kComputeWarps : ngrp;
+  compute_sync();
+  const int rows = sl.e.r1 - sl.e.r0;
+  for (int o = tid; o < rows * RG; o += kComputeThreads) {
+    const int ro = sl.e.r0 + o / RG, q = o % RG;
+    T sum = part[o];
+    for (int g2 = 1; g2 < nparts; ++g2) sum = cadd(sum, part[(g2 << trl) * RG + o]);
+    if (RG > 1 && q >= gr.w) continue;
+    if (ro < sl.fr.s) {
+      const T y = cadd(sum, own[o]);
+      const T d = __ldg(sl.dinv + ro);
+      entry_ptr<T, RG>(sl.xf, a.n_loc, sl.fr.first + ro, gr)[q] = cmul(y, d);
+      if (!EXT) entry_ptr<T, RG>(sl.xb, a.n_loc, sl.fr.first + ro, gr)[q] = y;
     } else {
-      T wu[RG];
-#pragma unroll
-      for (int q = 0; q < RG; ++q) wu[q] = CplxTraits<T>::zero();
-      pull_add<T, RG>(cx, pull + 2 * r, rhs0, wu);
-      const int64_t o = cx.sh.upd_off[sn] + (r - s);
-#pragma unroll
-      for (int q = 0; q < RG; ++q)
-        if (rhs0 + q < cx.nrhs) cx.upd[(int64_t)(rhs0 + q) * cx.upd_ld + o] = csub(wu[q], acc[q]);
+      entry_ptr<T, RG>(sl.upd, a.upd_ld, sl.fr.upd_off + (ro - sl.fr.s), gr)[q] = csub(own[o], sum);
     }
   }
 }
@@ -199,25 +297,21 @@ __device__ __forceinline__ void fwd_task(const SolveTask tk, const int rhs0, con
 // as above, then forward substitution y_S = L_TL^{-1} w_S in blocks of 32 columns (one warp solves
 // the diagonal block, all threads update the rows below it), x_S = D^{-1} y_S into xf, y_S into xb.
 template <typename T, int RG>
-__device__ __forceinline__ void fwd_tri_task(const SolveTask tk, const int rhs0, const SolveCtx<T>& cx,
-                                             unsigned char* smem_raw) {
-  const int sn = tk.sn;
-  const int s = cx.sh.s[sn], ld = s + cx.sh.u[sn];
-  const int first = cx.sh.first[sn];
-  const T* G = cx.G + cx.sh.g_off[sn];
-  const int32_t* pull = cx.sh.pull + 2 * cx.sh.pull_ptr[sn];
-  T* w = reinterpret_cast<T*>(smem_raw);        // RG x s (right-hand side major)
-  for (int p = threadIdx.x; p < s; p += blockDim.x) {
-    const int node = cx.sh.order[first + p];
-    T v[RG];
+__device__ __noinline__ void fwd_tri_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr, unsigned char* smem) {
+  const int s = sl.fr.s, ld = s + sl.fr.u;
+  const T* G = sl.G;
+  const int tid = threadIdx.x;
+  T* w = reinterpret_cast<T*>(smem);            // RG x s (right-hand side major)
+  for (int p = tid; p < s; p += kComputeThreads) {
+    const int4 ix = p < kGatherIdx ? sl.rows[p] : __ldg(sl.rows_g + p);
+    T v[RG], t[RG];
+    input_entry<T, RG>(sl, gr, ix.x, t);
+    pull_entries<T, RG>(sl, a.upd_ld, gr, ix.y, ix.z, v);
 #pragma unroll
-    for (int q = 0; q < RG; ++q) v[q] = (rhs0 + q < cx.nrhs) ? input_value(cx, node, rhs0 + q) : CplxTraits<T>::zero();
-    pull_add<T, RG>(cx, pull + 2 * p, rhs0, v);
-#pragma unroll
-    for (int q = 0; q < RG; ++q) w[q * s + p] = v[q];
+    for (int q = 0; q < RG; ++q) w[q * s + p] = cadd(v[q], t[q]);
   }
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  compute_sync();
+  const int lane = tid & 31, warp = tid >> 5;
   for (int b = 0; b < s; b += 32) {
     const int be = min(b + 32, s);
     if (warp == 0) {
@@ -232,9 +326,9 @@ __device__ __forceinline__ void fwd_tri_task(const SolveTask tk, const int rhs0,
         __syncwarp();
       }
     }
-    __syncthreads();
+    compute_sync();
     // rows below the block: w_i -= sum_{j in block} L[i, j] y_j
-    for (int i = be + threadIdx.x; i < s; i += blockDim.x) {
+    for (int i = be + tid; i < s; i += kComputeThreads) {
       T acc[RG];
 #pragma unroll
       for (int q = 0; q < RG; ++q) acc[q] = CplxTraits<T>::zero();
@@ -246,44 +340,39 @@ __device__ __forceinline__ void fwd_tri_task(const SolveTask tk, const int rhs0,
 #pragma unroll
       for (int q = 0; q < RG; ++q) w[q * s + i] = csub(w[q * s + i], acc[q]);
     }
-    __syncthreads();
+    compute_sync();
   }
-  for (int r = threadIdx.x; r < s; r += blockDim.x) {
-    const T dinv = cdiv(CplxTraits<T>::one(), G[(int64_t)r * ld + r]);
+  for (int r = tid; r < s; r += kComputeThreads) {
+    const T dinv = __ldg(sl.dinv + r);
 #pragma unroll
     for (int q = 0; q < RG; ++q)
-      if (rhs0 + q < cx.nrhs) {
-        const int64_t o = (int64_t)(rhs0 + q) * cx.n_loc + first + r;
-        cx.xb[o] = w[q * s + r];
-        cx.xf[o] = cmul(w[q * s + r], dinv);
+      if (q < gr.w) {
+        entry_ptr<T, RG>(sl.xb, a.n_loc, sl.fr.first + r, gr)[q] = w[q * s + r];
+        entry_ptr<T, RG>(sl.xf, a.n_loc, sl.fr.first + r, gr)[q] = cmul(w[q * s + r], dinv);
       }
   }
 }
 
-template <typename T, int RG>
-__global__ void __launch_bounds__(256) k_solve_fwd(const SolveTask* __restrict__ tasks, SolveCtx<T> cx, int R,
-                                                   int phase, int chunk) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (phase == 0 && cx.si == PSP_SI_NONE) fwd_tri_task<T, RG>(tasks[blockIdx.x], blockIdx.y * RG, cx, smem_raw);
-  else fwd_task<T, RG>(tasks[blockIdx.x], blockIdx.y * RG, cx, R, smem_raw, phase, chunk);
+// position of a box node in the problem's vector block, -1 over the pad (Alg. 1.3 extraction)
+__device__ __forceinline__ int64_t extracted(const StepRec& st, const int node) {
+  const int own = node - st.lead * st.plane;
+  return own < 0 ? -1 : (int64_t)st.plane * st.z0 + own;
 }
 
-// the final write of x_S column c of a front: xb (elimination order) and, for the panel's own
-// planes, the global vector (Alg. 1.3 extraction; assigned in the forward sweep, subtracted in the
-// backward sweep)
-template <typename T>
-__device__ __forceinline__ void write_solution(const SolveCtx<T>& cx, const int first, const int c, const int q,
-                                               const T out) {
-  cx.xb[(int64_t)q * cx.n_loc + first + c] = out;
-  const int node = cx.sh.order[first + c];
-  const int nx = cx.sh.nx, ny = cx.sh.ny;
-  const int k = node / (nx * ny);
-  if (k >= cx.lead) {
-    const int64_t g = (node % (nx * ny)) + (int64_t)nx * ny * (cx.z0 + k - cx.lead);
-    double2* uq = cx.u + (int64_t)q * cx.N + g;
+// the final write of column q of x_S entry c of a front: xb (elimination order) and, for the panel's own planes,
+// the global vector at g (assigned in the forward sweep, subtracted from `old` in the backward sweep)
+template <typename T, int RG>
+__device__ __forceinline__ void write_solution(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr, const int entry,
+                                               const int q, const int64_t g, const double2 old, const T out) {
+  entry_ptr<T, RG>(sl.xb, a.n_loc, entry, gr)[q] = out;
+  if (g >= 0) {
     const double2 o = to_c128(out);
-    *uq = (cx.mode == 0) ? o : csub(__ldcg(uq), o);
+    sl.u[(int64_t)(gr.g * RG + q) * sl.st.N + g] = sl.st.mode == 0 ? o : csub(old, o);
   }
+}
+template <typename T, int RG>
+__device__ __forceinline__ double2 old_solution(const TaskSlot<T>& sl, const Group gr, const int q, const int64_t g) {
+  return g >= 0 && sl.st.mode != 0 ? __ldcg(sl.u + (int64_t)(gr.g * RG + q) * sl.st.N + g) : make_double2(0.0, 0.0);
 }
 
 // down-the-tree task: columns [r0, r1) of S of front sn.
@@ -291,84 +380,129 @@ __device__ __forceinline__ void write_solution(const SolveCtx<T>& cx, const int 
 //     y = xf on S and -x_U on the struct rows; writes the solution.
 //   factors keeping L_BL, phase 0: t_c = xf_c - sum_{r >= s} L_BL[r, c] x_U[r] into xf.
 //   paper's factors, phase 1: x_c = t_c + sum_{c < r < s} inv(L_TL)[r, c] t_r; writes the solution.
-template <typename T, int RG>
-__device__ __forceinline__ void bwd_task(const SolveTask tk, const int rhs0, const SolveCtx<T>& cx,
-                                         unsigned char* smem_raw, const int phase, const int chunk) {
-  const int sn = tk.sn;
-  const int s = cx.sh.s[sn], u = cx.sh.u[sn], ld = s + u;
-  const int first = cx.sh.first[sn];
-  const T* G = cx.G + cx.sh.g_off[sn];
-  const int32_t* sel = cx.sh.struct_elim + cx.sh.struct_ptr[sn];
-  const int c0 = tk.r0;
-  const bool ext = cx.si == PSP_SI_EXTENDED;
-  // rows of the inner sums: [lo, hi), passed through shared memory in chunks of `chunk` rows
-  const int lo = (ext || phase == 1) ? c0 : s;
-  const int hi = (ext || phase == 0) ? ld : s;
-  // the columns the inner sums read: G's, or in the two-inverse form's second phase the second
-  // inverse of L_TL (s x s after G), which was built row by row for this direction
-  const bool second = phase == 1 && cx.si == PSP_SI_TWO;
-  const T* Gs = second ? G + second_inverse_offset(s, u) : G;
-  const int lds = second ? s : ld;
-  // right-hand side major (y[q * chunk + row]): the lanes of a warp read consecutive rows, so the
-  // loads are free of bank conflicts whatever RG is
-  T* y = reinterpret_cast<T*>(smem_raw);        // RG x chunk
-  T* sums = y + (int64_t)chunk * RG;            // (r1 - c0) x RG column sums (<= 256 columns)
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int e = threadIdx.x; e < (tk.r1 - c0) * RG; e += blockDim.x) sums[e] = CplxTraits<T>::zero();
-  for (int rb = lo; rb < hi; rb += chunk) {
-    const int re = min(rb + chunk, hi);
-    __syncthreads();   // sums initialised / the previous chunk consumed
-    for (int r = rb + threadIdx.x; r < re; r += blockDim.x) {
+//
+// A warp carries blocks of four adjacent columns, its lanes over the rows, so an entry of y serves four columns;
+// tasks of few columns split their rows over the warps instead.  Which rows a lane sums depends on the task alone
+// (quads of columns, steps of 32 rows), so every RG gives a column the same bits.
+template <typename T, int RG, int PHASE, bool EXT>
+__device__ __forceinline__ void bwd_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr, unsigned char* smem) {
+  using Real = typename CplxTraits<T>::real;
+  constexpr int SP = entry_stride<T, RG>(), CB = Tile<T, RG>::cols, U = Tile<T, RG>::down;
+  constexpr bool writes = EXT || PHASE == 1;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int s = sl.fr.s, c0 = sl.e.r0, nc = sl.e.r1 - c0;
+  // rows of the inner sums: [lo, hi), passed through shared memory in chunks of a.chunk rows
+  const int lo = writes ? c0 : s, hi = (EXT || PHASE == 0) ? s + sl.fr.u : s;
+  T* part = reinterpret_cast<T*>(smem);         // column sums, (split, column, right-hand side)
+  T* y = part + 2 * kComputeThreads * RG;       // chunk x SP
+  const int nb = (nc + CB - 1) / CB, splits = sl.splits;   // blocks of CB columns, warps that share a block's rows
+  // this thread's first output: its own entry and, where the solution is written, its place and (backward sweep) the
+  // old value there are read before the products
+  T own0 = CplxTraits<T>::zero();
+  int64_t g0 = -1;
+  double2 old0 = make_double2(0.0, 0.0);
+  if (tid < nc * RG && (RG == 1 || tid % RG < gr.w)) {
+    own0 = __ldcg(entry_ptr<T, RG>(sl.xf, a.n_loc, sl.fr.first + c0 + tid / RG, gr) + tid % RG);
+    if (writes) {
+      g0 = extracted(sl.st, __ldg(sl.rows_g + c0 + tid / RG).x);
+      old0 = old_solution<T, RG>(sl, gr, tid % RG, g0);
+    }
+  }
+  for (int rb = lo; rb < hi; rb += a.chunk) {
+    const int re = min(rb + a.chunk, hi);
+    if (rb > lo) compute_sync();   // the previous chunk is consumed
+    constexpr int GU = RG >= 2 ? 1 : 2;
+    for (int p0 = rb + tid; p0 < re; p0 += GU * kComputeThreads) {
+      T v[GU][RG];
 #pragma unroll
-      for (int q = 0; q < RG; ++q) {
-        T v = CplxTraits<T>::zero();
-        if (rhs0 + q < cx.nrhs) {
-          const int64_t base = (int64_t)(rhs0 + q) * cx.n_loc;
-          v = (r < s) ? __ldcg(cx.xf + base + first + r) : cneg(__ldcg(cx.xb + base + sel[r - s]));
+      for (int t = 0; t < GU; ++t) {
+        const int r = p0 + t * kComputeThreads;
+        if (r < re) {
+          const int k = r - s;
+          const int e = k < 0 ? sl.fr.first + r
+                              : (k < 4 * kGatherIdx ? reinterpret_cast<const int32_t*>(sl.rows)[k] : __ldg(sl.sel_g + k));
+          load_entry<T, RG>(k < 0 ? sl.xf : sl.xb, a.n_loc, e, gr, v[t]);
         }
-        y[q * chunk + (r - rb)] = v;
+      }
+#pragma unroll
+      for (int t = 0; t < GU; ++t) {
+        const int r = p0 + t * kComputeThreads;
+        if (r < re)
+#pragma unroll
+          for (int q = 0; q < RG; ++q) y[(r - rb) * SP + q] = r < s ? v[t][q] : cneg(v[t][q]);
       }
     }
-    __syncthreads();
-    for (int c = c0 + warp; c < tk.r1; c += nw) {
-      T acc[RG];
+    compute_sync();
+    // the columns the inner sums read: G's, or in the two-inverse form's second phase the second inverse of L_TL
+    // (s x s after G), which was built row by row for this direction
+    const bool second = PHASE == 1 && a.si == PSP_SI_TWO;
+    const T* Gs = second ? sl.G + second_inverse_offset(s, sl.fr.u) : sl.G;
+    const int lds = second ? s : s + sl.fr.u;
+    const int step = 32 * splits;
+    for (int wb = warp; wb < nb * splits; wb += kComputeWarps) {
+      const int b = splits > 1 ? wb % nb : wb, sp = splits > 1 ? wb / nb : 0;
+      const int c = c0 + b * CB, ncb = min(CB, c0 + nc - c);
+      Real acc[CB * RG * 2];
 #pragma unroll
-      for (int q = 0; q < RG; ++q) acc[q] = CplxTraits<T>::zero();
-      const T* Gc = Gs + (int64_t)c * lds;
-      int r = (rb > c + 1 ? rb : c + 1) + lane;
-      for (; r + 7 * 32 < re; r += 8 * 32) {   // eight independent factor loads in flight per lane
-        T gv[8];
+      for (int k = 0; k < CB * RG * 2; ++k) acc[k] = Real(0);
+      int r = max(rb, c0 + ((c - c0) & ~3) + 1) + sp * 32 + lane;
+      const T* Gp = Gs + (int64_t)c * lds + r;
+      const T* yp = y + (r - rb) * SP;
+      for (; r < re; r += U * step, Gp += U * step, yp += U * step * SP) {
+        T g[U][CB];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) gv[t] = __ldg(Gc + r + 32 * t);
+        for (int t = 0; t < U; ++t)
 #pragma unroll
-        for (int t = 0; t < 8; ++t)
+          for (int k = 0; k < CB; ++k)   // rows below each column's diagonal
+            if (k < ncb && r + step * t < re && r + step * t > c + k) g[t][k] = __ldg(Gp + k * lds + step * t);
 #pragma unroll
-          for (int q = 0; q < RG; ++q) cfma(acc[q], gv[t], y[q * chunk + (r + 32 * t - rb)]);
+        for (int t = 0; t < U; ++t)
+          if (r + step * t < re) {
+            T x[RG];
+            load_shared<T, RG>(yp + step * t * SP, x);
+#pragma unroll
+            for (int k = 0; k < CB; ++k)
+              if (k < ncb && r + step * t > c + k)
+#pragma unroll
+                for (int q = 0; q < RG; ++q) {
+                  T s2;
+                  s2.x = acc[(k * RG + q) * 2];
+                  s2.y = acc[(k * RG + q) * 2 + 1];
+                  cfma(s2, g[t][k], x[q]);
+                  acc[(k * RG + q) * 2] = s2.x;
+                  acc[(k * RG + q) * 2 + 1] = s2.y;
+                }
+          }
       }
-      for (; r < re; r += 32) {
-        const T gv = __ldg(Gc + r);
+      int base;
+      bool lead;
+      warp_sum<Real, CB * RG * 2>(acc, lane, base, lead);
+      if (lead) {
+        constexpr int per = CB * RG * 2 > 32 ? CB * RG * 2 / 32 : 1;
+        Real* out = reinterpret_cast<Real*>(part + (sp * nb * CB + b * CB) * RG);
 #pragma unroll
-        for (int q = 0; q < RG; ++q) cfma(acc[q], gv, y[q * chunk + (r - rb)]);
-      }
-#pragma unroll
-      for (int q = 0; q < RG; ++q) {
-        for (int off = 16; off > 0; off >>= 1) {
-          acc[q].x += __shfl_xor_sync(0xffffffffu, acc[q].x, off);
-          acc[q].y += __shfl_xor_sync(0xffffffffu, acc[q].y, off);
-        }
-        if (lane == 0) sums[(c - c0) * RG + q] = cadd(sums[(c - c0) * RG + q], acc[q]);
+        for (int k = 0; k < per; ++k) out[base + k] = rb == lo ? acc[k] : out[base + k] + acc[k];
       }
     }
   }
-  __syncthreads();
-  for (int c = c0 + threadIdx.x; c < tk.r1; c += blockDim.x) {
-#pragma unroll
-    for (int q = 0; q < RG; ++q) {
-      if (rhs0 + q >= cx.nrhs) continue;
-      const int64_t o = (int64_t)(rhs0 + q) * cx.n_loc + first + c;
-      const T v = cadd(sums[(c - c0) * RG + q], __ldcg(cx.xf + o));   // + xf_c (z_c, or t_c in phase 1)
-      if (!ext && phase == 0) cx.xf[o] = v;                           // t_c: this thread's column only
-      else write_solution(cx, first, c, rhs0 + q, v);
+  compute_sync();
+  for (int o = tid; o < nc * RG; o += kComputeThreads) {
+    const int c = o / RG, q = o % RG;
+    if (RG > 1 && q >= gr.w) continue;
+    const int entry = sl.fr.first + c0 + c;
+    T v = o == tid ? own0 : __ldcg(entry_ptr<T, RG>(sl.xf, a.n_loc, entry, gr) + q);
+    if (hi > lo)
+      for (int sp = 0; sp < splits; ++sp) v = cadd(v, part[sp * nb * CB * RG + o]);
+    if constexpr (!writes) {   // t_c
+      entry_ptr<T, RG>(sl.xf, a.n_loc, entry, gr)[q] = v;
+    } else {
+      int64_t g = g0;
+      double2 old = old0;
+      if (o != tid) {
+        g = extracted(sl.st, __ldg(sl.rows_g + c0 + c).x);
+        old = old_solution<T, RG>(sl, gr, q, g);
+      }
+      write_solution<T, RG>(sl, a, gr, entry, q, g, old, v);
     }
   }
 }
@@ -377,25 +511,24 @@ __device__ __forceinline__ void bwd_task(const SolveTask tk, const int rhs0, con
 // L_TL^T x_S = t (t in xf) in blocks of 32 columns from the last, each block first takes the
 // products with the solved rows below it (one warp per column), then one warp solves the block.
 template <typename T, int RG>
-__device__ __forceinline__ void bwd_tri_task(const SolveTask tk, const int rhs0, const SolveCtx<T>& cx,
-                                             unsigned char* smem_raw) {
-  const int sn = tk.sn;
-  const int s = cx.sh.s[sn], ld = s + cx.sh.u[sn];
-  const int first = cx.sh.first[sn];
-  const T* G = cx.G + cx.sh.g_off[sn];
-  T* x = reinterpret_cast<T*>(smem_raw);   // RG x s (right-hand side major): t, overwritten by x block by block
-  for (int r = threadIdx.x; r < s; r += blockDim.x)
+__device__ __noinline__ void bwd_tri_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr, unsigned char* smem) {
+  const int s = sl.fr.s, ld = s + sl.fr.u;
+  const T* G = sl.G;
+  const int tid = threadIdx.x;
+  T* x = reinterpret_cast<T*>(smem);   // RG x s (right-hand side major): t, overwritten by x block by block
+  for (int r = tid; r < s; r += kComputeThreads) {
+    T v[RG];
+    load_entry<T, RG>(sl.xf, a.n_loc, sl.fr.first + r, gr, v);
 #pragma unroll
-    for (int q = 0; q < RG; ++q)
-      x[q * s + r] = (rhs0 + q < cx.nrhs) ? __ldcg(cx.xf + (int64_t)(rhs0 + q) * cx.n_loc + first + r)
-                                           : CplxTraits<T>::zero();
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int q = 0; q < RG; ++q) x[q * s + r] = v[q];
+  }
+  compute_sync();
+  const int lane = tid & 31, warp = tid >> 5;
   const int nblk = (s + 31) / 32;
   for (int bi = nblk - 1; bi >= 0; --bi) {
     const int b = bi * 32, be = min(b + 32, s);
     // x_c -= sum_{r >= be} L[r, c] x_r for the block's columns
-    for (int c = b + warp; c < be; c += nw) {
+    for (int c = b + warp; c < be; c += kComputeWarps) {
       T acc[RG];
 #pragma unroll
       for (int q = 0; q < RG; ++q) acc[q] = CplxTraits<T>::zero();
@@ -413,7 +546,7 @@ __device__ __forceinline__ void bwd_tri_task(const SolveTask tk, const int rhs0,
         if (lane == 0) x[q * s + c] = csub(x[q * s + c], acc[q]);
       }
     }
-    __syncthreads();
+    compute_sync();
     if (warp == 0) {
       // the block, from its last column: x_c final, then x_k -= L[c, k] x_c for b <= k < c
       for (int c = be - 1; c >= b; --c) {
@@ -426,235 +559,266 @@ __device__ __forceinline__ void bwd_tri_task(const SolveTask tk, const int rhs0,
         __syncwarp();
       }
     }
-    __syncthreads();
+    compute_sync();
   }
-  for (int c = threadIdx.x; c < s; c += blockDim.x)
+  for (int c = tid; c < s; c += kComputeThreads) {
+    const int64_t g = extracted(sl.st, __ldg(sl.rows_g + c).x);
 #pragma unroll
     for (int q = 0; q < RG; ++q)
-      if (rhs0 + q < cx.nrhs) write_solution(cx, first, c, rhs0 + q, x[q * s + c]);
-}
-
-template <typename T, int RG>
-__global__ void __launch_bounds__(256) k_solve_bwd(const SolveTask* __restrict__ tasks, SolveCtx<T> cx, int phase,
-                                                   int chunk) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (phase == 1 && cx.si == PSP_SI_NONE) bwd_tri_task<T, RG>(tasks[blockIdx.x], blockIdx.y * RG, cx, smem_raw);
-  else bwd_task<T, RG>(tasks[blockIdx.x], blockIdx.y * RG, cx, smem_raw, phase, chunk);
-}
-
-// rhs group size so that the shared-memory footprint stays below ~200 KB
-template <typename T>
-static int pick_rg(int nrhs, size_t per_rhs_bytes) {
-  int rg = 8;
-  while (rg > 1 && (rg >= 2 * nrhs || per_rhs_bytes * rg > 200 * 1024)) rg >>= 1;
-  return rg;
+      if (q < gr.w) write_solution<T, RG>(sl, a, gr, sl.fr.first + c, q, g, old_solution<T, RG>(sl, gr, q, g), x[q * s + c]);
+  }
 }
 
 // ---------------------------------------------------------------------------
 // The whole sweep of Alg. 1.5 in one cooperative launch, as a dataflow over the elimination trees.
 // CTAs take tasks from one queue in topological order.  An up-the-tree task of a front waits until
 // every task of its children has finished (one counter per front, which its children's tasks
-// increment); a front without children waits for the previous panel solve of its problem's chain
-// (the chains of a batch of independent problems are interleaved in the queue and run side by
-// side), so every front does, through its descendants.  A down-the-tree task waits for its parent
-// (the root: for its own up-the-tree tasks).  A task only waits on tasks earlier in the queue.  A
-// CTA claims its tasks in queue order, one or two ahead of the task it runs; the earliest unfinished
+// increment); a front without children waits for the previous panel solve of its problem's chain: for the
+// same front's down tasks there when both boxes have the same tree (its input is read at its own (x, y) only,
+// and every work entry it overwrites has then been read), else for the whole solve.  (The chains of a batch of
+// independent problems are interleaved in the queue and run side by side.)  A down-the-tree task waits for its
+// parent (the root: for its own up-the-tree tasks).  A task only waits on tasks earlier in the queue.  A
+// CTA claims its tasks in queue order, a few ahead of the task it runs; the earliest unfinished
 // task is therefore the one some CTA runs (a CTA holding it only as a later task would be running an
 // earlier unfinished one), every task it waits for has finished, and since every CTA of a
 // cooperative launch is resident, the sweep progresses.  Each wait is bounded anyway: a CTA that
 // gives up sets status[2] and stops; the others then give up at their next wait.
+//
+// A CTA's warps have three roles, so that the latencies around a task's products overlap with the products of
+// the task before it.  A scheduling warp claims the next task, reads its records, copies the index words its
+// gathers need into shared memory, warms L2 with its factor block and waits for its dependency; eight product
+// warps gather, multiply and write; a signalling warp makes a finished task's writes visible and counts it.
+// Tasks alternate between two slots.
 // ---------------------------------------------------------------------------
 constexpr long long kWaitCycles = 4000000000LL;   // SM clock cycles: about two seconds at 2 GHz
 constexpr long long kWaitSpins = 400000000LL;     // and a hard cap on polls, whatever the clock does
 
+__device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 // a wait that gives up sets status[2] (cleared before every sweep) and the handle's sticky flag
 // (cleared only when the host reads it)
 __device__ __forceinline__ bool wait_count(const unsigned* p, unsigned target, int* status, int* sticky) {
+  if (load_acquire(p) >= target) return true;
   const long long t0 = clock64();
   long long it = 0;
-  while (*(volatile const unsigned*)p < target) {
-    if (*(volatile int*)(status + 2) != 0) return false;
-    if (++it > kWaitSpins || clock64() - t0 > kWaitCycles) {
-      atomicExch(status + 2, 1);
-      if (sticky) atomicExch(sticky, 1);
-      return false;
+  for (;;) {
+    if (load_acquire(p) >= target) return true;
+    if ((++it & 15) == 0) {
+      if (*(volatile int*)(status + 2) != 0) return false;
+      if (it > kWaitSpins || clock64() - t0 > kWaitCycles) {
+        atomicExch(status + 2, 1);
+        if (sticky) atomicExch(sticky, 1);
+        return false;
+      }
     }
-    __nanosleep(32);
+    __nanosleep(20);
   }
-  return true;
 }
 
 // Warm L2 with the factor lines a task will stream, while its dependencies are still being
 // waited for (the lines do not depend on them): up the tree rows [r0, r1) of the columns
-// j < min(r1, s), down the tree columns [c0, c1) from below their diagonal to the end.
+// j < min(r1, s), down the tree columns [c0, c1) from below their diagonal to the end.  One warp, at most
+// kPrefetchLines lines (the product reads the rest itself).
+constexpr int kPrefetchLines = 2048;
+
 template <typename T>
-__device__ __forceinline__ void prefetch_task(const SolveTask tk, const int dir, const SolveCtx<T>& cx) {
-  const int sn = tk.sn;
-  const int s = cx.sh.s[sn], ld = s + cx.sh.u[sn];
-  const char* G = reinterpret_cast<const char*>(cx.G + cx.sh.g_off[sn]);
+__device__ __forceinline__ void prefetch_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const int lane) {
+  const int s = sl.fr.s, u = sl.fr.u, ld = s + u, dir = sl.e.dir, r0 = sl.e.r0, r1 = sl.e.r1;
+  const char* G = reinterpret_cast<const char*>(sl.G);
   constexpr int kLine = 128;
   if (dir == 0 || dir == kDirUpB) {
-    const int ncol = min(tk.r1, s);
-    const int64_t seg = (int64_t)(tk.r1 - tk.r0) * sizeof(T);
-    const int lines = (int)((seg + kLine - 1) / kLine) + 1;   // the segment may straddle one more line
-    for (int w = threadIdx.x; w < ncol * lines; w += blockDim.x) {
-      const int j = w / lines, l = w % lines;
-      const char* col = G + ((int64_t)j * ld + tk.r0) * sizeof(T);
-      const char* a = col + (int64_t)l * kLine;
-      if (a < col + seg) asm volatile("prefetch.L2 [%0];" ::"l"(a));
+    const int ncol = min(r1, s);
+    const int seg = (r1 - r0) * (int)sizeof(T);
+    const int lines = (seg + kLine - 1) / kLine + 1;   // the segment may straddle one more line
+    const int total = min(ncol * lines, kPrefetchLines);
+    for (int w = lane; w < total; w += 32) {
+      const int j = w / lines, l = w - j * lines;
+      const char* col = G + ((int64_t)j * ld + r0) * sizeof(T);
+      if (l * kLine < seg) asm volatile("prefetch.global.L2 [%0];" ::"l"(col + (int64_t)l * kLine));
     }
   } else {
-    const bool second = dir == kDirDownB && cx.si == PSP_SI_TWO;   // the second inverse after G
-    const char* Gs = second ? G + second_inverse_offset(s, ld - s) * sizeof(T) : G;
+    const bool second = dir == kDirDownB && a.si == PSP_SI_TWO;   // the second inverse after G
+    const char* Gs = second ? G + second_inverse_offset(s, u) * sizeof(T) : G;
     const int lds = second ? s : ld;
-    for (int c = tk.r0; c < tk.r1; ++c) {
+    int left = kPrefetchLines;
+    for (int c = r0; c < r1 && left > 0; ++c) {
       const char* col = Gs + ((int64_t)c * lds + c + 1) * sizeof(T);
       const int64_t seg = (int64_t)(lds - c - 1) * sizeof(T);
-      for (int64_t off = (int64_t)threadIdx.x * kLine; off < seg; off += (int64_t)blockDim.x * kLine)
-        asm volatile("prefetch.L2 [%0];" ::"l"(col + off));
+      for (int64_t off = (int64_t)lane * kLine; off < seg; off += 32 * kLine)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(col + off));
+      left -= (int)(seg / kLine) + 1;
     }
   }
 }
 
-// tables cached in shared memory when they fit (a single problem: at most 3-4 shapes; batches
-// and very deep sweeps read them from global memory instead)
-constexpr int kMaxSweepShapes = 4, kMaxSweepSteps = 512, kMaxSweepPanels = 256;
-constexpr int kSweepThreads = 256;
-
-// one 16-byte asynchronous copy global -> shared (completed by cp_async_wait_all of the same thread)
+// asynchronous copies global -> shared (completed by cp_async_wait_all of the same thread)
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-template <typename T, int RG>
-__global__ void __launch_bounds__(kSweepThreads) k_sweep(SweepArgs<T> a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ __align__(16) QueueEntry s_q[2];   // the current task's queue entry and the next one's
-  __shared__ int s_idx, s_ok;
-  __shared__ SolveCtx<T> s_cx;      // this task's panel solve, filled by thread 0
-  __shared__ ShapeDev s_shape[kMaxSweepShapes];
-  __shared__ SweepStep s_step[kMaxSweepSteps];
-  __shared__ PanelSweep s_panel[kMaxSweepPanels];
-  // small per-sweep tables in shared memory when they fit; larger ones (batches of problems) are
-  // read from global memory by thread 0
-  const bool tab_smem = a.nshapes <= kMaxSweepShapes && a.nsteps <= kMaxSweepSteps && a.npanels <= kMaxSweepPanels;
-  if (tab_smem) {
-    for (int i = threadIdx.x; i < a.nshapes; i += blockDim.x) s_shape[i] = a.shapes[i];
-    for (int i = threadIdx.x; i < a.nsteps; i += blockDim.x) s_step[i] = a.steps[i];
-    for (int i = threadIdx.x; i < a.npanels; i += blockDim.x) s_panel[i] = a.panels[i];
-  }
-  unsigned* head = a.ctr;
-  unsigned* step_done = a.ctr + kSweepStepCounters;
-  const int nrg = (a.cx.nrhs + RG - 1) / RG;
-  // Thread 0 holds the index of this CTA's current task and of its next one, and the next one's queue
-  // entry is copied into the other shared-memory slot asynchronously, so that taking a task costs no
-  // dependent global load.  Claiming two ahead (claim_ahead 2), the task after the next one is claimed
-  // while the current one waits and runs, and the next one's entry is copied meanwhile; claiming one
-  // ahead, the next task is claimed as the current one starts waiting and its entry copied once the
-  // wait is over, so a CTA holds one task besides the one it runs, not two.
-  const bool two_ahead = a.claim_ahead > 1;
-  int cur = 0, nxt = 0, buf = 0;
-  if (threadIdx.x == 0) {
-    cur = (int)atomicAdd(head, 1u);
-    if (two_ahead) nxt = (int)atomicAdd(head, 1u);
-    if (cur < a.nqueue) s_q[0] = a.queue[cur];
-    s_cx = a.cx;   // fields common to every task; thread 0 sets the per-task ones below
-  }
-  for (;;) {
-    if (threadIdx.x == 0) {
-      s_idx = cur;
-      if (cur < a.nqueue) {
-        const QueueEntry& e = s_q[buf];
-        const SweepStep sp = tab_smem ? s_step[e.step] : a.steps[e.step];
-        const PanelSweep pi = tab_smem ? s_panel[sp.panel] : a.panels[sp.panel];
-        SolveCtx<T>& cx = s_cx;
-        cx.sh = tab_smem ? s_shape[pi.shape] : a.shapes[pi.shape];
-        cx.G = a.factor + pi.gbase;
-        cx.z0 = pi.z0;
-        cx.z1 = pi.z1;
-        cx.lead = pi.lead;
-        cx.has_prev = pi.has_prev;
-        cx.has_next = pi.has_next;
-        cx.mode = sp.mode;
-        if (a.nprobs > 1) {
-          // the problem's own vector block, coupling tables and work vectors
-          const ProblemSweep& pr = a.probs[sp.prob];
-          cx.u = a.cx.u + pr.off1 * a.cx.nrhs;
-          cx.N = pr.N;
-          cx.nz = pr.nz;
-          cx.s1n = pr.s1n;
-          cx.s2n = pr.s2n;
-          cx.s3h = pr.s3h;
-          cx.inv_h2 = pr.inv_h2;
-          cx.xf = a.cx.xf + (int64_t)sp.prob * a.cx.n_loc * a.cx.nrhs;
-          cx.xb = a.cx.xb + (int64_t)sp.prob * a.cx.n_loc * a.cx.nrhs;
-          cx.upd = a.cx.upd + (int64_t)sp.prob * a.cx.upd_ld * a.cx.nrhs;
-        }
-      }
+// the scheduling warp: task after task into alternating slots
+template <typename T>
+__device__ __forceinline__ void schedule(TaskSlot<T>* slots, const SweepArgs<T>& a, const int lane) {
+  constexpr int kEntryWords = sizeof(QueueEntry) / 4, kStepWords = sizeof(StepRec) / 4, kFrontWords = sizeof(FrontRec) / 4;
+  static_assert(kEntryWords <= 32 && kStepWords <= 32 && kFrontWords <= 32, "records are copied one word per lane");
+  const bool early = a.claim_ahead > 1;   // claim the next task before the slot it will use is free
+  auto claim = [&] {
+    int v = 0;
+    if (lane == 0) v = (int)atomicAdd(a.ctr, 1u);
+    return __shfl_sync(0xffffffffu, v, 0);
+  };
+  int next = early ? claim() : 0;
+  for (int n = 0;; ++n) {
+    TaskSlot<T>& sl = slots[n & 1];
+    int idx = next;
+    int ew = 0;
+    if (early && idx < a.nqueue && lane < kEntryWords) ew = __ldg(reinterpret_cast<const int*>(a.queue + idx) + lane);
+    if (n >= 2) bar_sync(kBarFree + (n & 1), 64);   // the slot's last task has been signalled
+    if (!early) {
+      idx = claim();
+      if (idx < a.nqueue && lane < kEntryWords) ew = __ldg(reinterpret_cast<const int*>(a.queue + idx) + lane);
     }
-    __syncthreads();
-    if (s_idx >= a.nqueue) break;
-    const QueueEntry& e = s_q[buf];
-    const SolveTask tk{e.sn, e.r0, e.r1};
-    const int dir = e.dir, R = e.R;
-    int after = 0;
-    if (threadIdx.x == 0) {
-      if (two_ahead) {
-        after = (int)atomicAdd(head, 1u);   // the task after the next one (its index is read at the end)
-        if (nxt < a.nqueue) {
-          const char* src = reinterpret_cast<const char*>(a.queue + nxt);
-          char* dst = reinterpret_cast<char*>(&s_q[buf ^ 1]);
-          cp_async16(dst, src);
-          cp_async16(dst + 16, src + 16);
-          cp_async16(dst + 32, src + 32);
-        }
-      } else {
-        nxt = (int)atomicAdd(head, 1u);   // the next task (its index is read after the wait)
+    bool ok = idx < a.nqueue;
+    if (ok) {
+      if (lane < kEntryWords) reinterpret_cast<int*>(&sl.e)[lane] = ew;
+      __syncwarp();
+      int sw = 0, fw = 0;
+      if (lane < kStepWords) sw = __ldg(reinterpret_cast<const int*>(a.steps + sl.e.step) + lane);
+      if (lane < kFrontWords) fw = __ldg(reinterpret_cast<const int*>(a.fronts + sl.e.front) + lane);
+      if (early) next = claim();
+      if (lane < kStepWords) reinterpret_cast<int*>(&sl.st)[lane] = sw;
+      if (lane < kFrontWords) reinterpret_cast<int*>(&sl.fr)[lane] = fw;
+      __syncwarp();
+      const int dir = sl.e.dir, r0 = sl.e.r0, r1 = sl.e.r1, s = sl.fr.s, u = sl.fr.u;
+      const int4* rows = sl.st.rows + sl.fr.row_off;
+      const int32_t* sel = sl.st.sel + sl.fr.sel_off;
+      if (lane == 0) {
+        int tl = 3;
+        while ((1 << tl) < r1 - r0 && (1 << tl) < kComputeThreads) ++tl;
+        sl.tr_log = tl;
+        int sp = 1;
+        while (2 * sp * ((r1 - r0 + 3) / 4) <= kComputeWarps) sp <<= 1;
+        sl.splits = sp;
+        sl.G = a.factor + sl.st.gbase + sl.fr.g_off;
+        sl.dinv = a.dinv + sl.st.dbase + sl.fr.first;
+        sl.rows_g = rows;
+        sl.sel_g = sel;
+        const int64_t box = (int64_t)sl.st.prob * a.n_loc * a.nrhs;
+        sl.xf = a.xf + box;
+        sl.xb = a.xb + box;
+        sl.upd = a.upd + (int64_t)sl.st.prob * a.upd_ld * a.nrhs;
+        sl.u = a.u + sl.st.off1 * a.nrhs;
       }
-    }
-    prefetch_task<T>(tk, dir, s_cx);
-    if (threadIdx.x == 0) {
-      const bool ok = e.wait < 0 || wait_count(a.ctr + e.wait, e.target, a.status, a.sticky);
-      if (!two_ahead && nxt < a.nqueue) {
-        const char* src = reinterpret_cast<const char*>(a.queue + nxt);
-        char* dst = reinterpret_cast<char*>(&s_q[buf ^ 1]);
-        cp_async16(dst, src);
-        cp_async16(dst + 16, src + 16);
-        cp_async16(dst + 32, src + 32);
+      __syncwarp();
+      const bool up = dir == 0 || dir == kDirUpB, tri = a.si == PSP_SI_NONE && (dir == 0 || dir == kDirDownB);
+      if (dir == 0) {
+        for (int p = lane; p < min(min(r1, s), kGatherIdx); p += 32) cp_async16(&sl.rows[p], rows + p);
+      } else if (dir == 1) {
+        int32_t* dst = reinterpret_cast<int32_t*>(sl.rows);
+        for (int p = lane; p < min(u, 4 * kGatherIdx); p += 32) cp_async4(dst + p, sel + p);
       }
+      if (up && !tri)
+        for (int p = max(r0, s) + lane; p < r1; p += 32) cp_async16(&sl.own[p - r0], rows + p);
+      prefetch_task<T>(sl, a, lane);
+      int got = 1;
+      if (lane == 0 && sl.e.wait >= 0) got = wait_count(a.ctr + sl.e.wait, sl.e.target, a.status, a.sticky);
+      ok = __shfl_sync(0xffffffffu, got, 0) != 0;
       __threadfence();
-      s_ok = ok;
+      cp_async_wait_all();
     }
-    __syncthreads();
-    if (!s_ok) break;
-    const bool tri = s_cx.si == PSP_SI_NONE;
-    for (int g = 0; g < nrg; ++g) {
-      if (dir == 0 && tri) fwd_tri_task<T, RG>(tk, g * RG, s_cx, smem_raw);
-      else if (dir == 0 || dir == kDirUpB) fwd_task<T, RG>(tk, g * RG, s_cx, R, smem_raw, dir == 0 ? 0 : 1, a.chunk);
-      else if (dir == kDirDownB && tri) bwd_tri_task<T, RG>(tk, g * RG, s_cx, smem_raw);
-      else bwd_task<T, RG>(tk, g * RG, s_cx, smem_raw, dir == 1 ? 0 : 1, a.chunk);
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-      // completion counters of this task's front (and of its parent's children, up the tree) and step
-      __threadfence();
-      atomicAdd(a.ctr + e.done, 1u);
-      if (e.kids >= 0) atomicAdd(a.ctr + e.kids, 1u);
-      atomicAdd(step_done + e.step, 1u);
-      cp_async_wait_all();   // the next task's entry has landed
-      cur = nxt;
-      if (two_ahead) nxt = after;
-    }
-    buf ^= 1;   // every thread: the next task's entry is in the other slot
+    if (lane == 0) sl.ok = ok;
+    __syncwarp();
+    bar_arrive(kBarReady + (n & 1), kComputeThreads + 32);
+    if (!ok) break;
   }
-  if (threadIdx.x == 0) cp_async_wait_all();
 }
 
+// the signalling warp: a finished task's completion counters
+template <typename T>
+__device__ __forceinline__ void signal_done(TaskSlot<T>* slots, const SweepArgs<T>& a, const int lane) {
+  for (int n = 0;; ++n) {
+    TaskSlot<T>& sl = slots[n & 1];
+    bar_sync(kBarDone + (n & 1), kComputeThreads + 32);
+    if (!sl.ok) break;
+    if (lane < 3) {
+      __threadfence();   // the product warps' writes, ordered before this by the barrier, become visible first
+      const int c = lane == 0 ? sl.e.done : (lane == 1 ? sl.e.kids : sl.e.step_done);
+      if (c >= 0) atomicAdd(a.ctr + c, 1u);
+    }
+    __syncwarp();
+    bar_arrive(kBarFree + (n & 1), 64);
+  }
+}
+
+// EXT: extended selective inversion (one task per front and direction); otherwise the forms that keep L_BL.
+// The registers are held to sweep_ctas CTAs per SM (65,536 / (320 threads x CTAs)).
 template <typename T, int RG>
+constexpr int sweep_ctas() { return 2; }
+
+template <typename T, int RG, bool EXT>
+__global__ void __launch_bounds__(kSweepThreads, (sweep_ctas<T, RG>())) k_sweep(const __grid_constant__ SweepArgs<T> a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(16) TaskSlot<T> slots[2];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp == kComputeWarps) {
+    schedule<T>(slots, a, lane);
+    return;
+  }
+  if (warp == kComputeWarps + 1) {
+    signal_done<T>(slots, a, lane);
+    return;
+  }
+  const int nrg = (a.nrhs + RG - 1) / RG;
+  for (int n = 0;; ++n) {
+    const TaskSlot<T>& sl = slots[n & 1];
+    bar_sync(kBarReady + (n & 1), kComputeThreads + 32);
+    const bool ok = sl.ok;
+    if (ok) {
+      for (int g = 0; g < nrg; ++g) {
+        Group gr{g, min(RG, a.nrhs - g * RG), false};
+        if (RG > 1)
+          gr.vec = gr.w == RG && ((reinterpret_cast<uintptr_t>(sl.xf + g * RG * a.n_loc) |
+                                   reinterpret_cast<uintptr_t>(sl.xb + g * RG * a.n_loc) |
+                                   reinterpret_cast<uintptr_t>(sl.upd + g * RG * a.upd_ld)) & 15) == 0;
+        if (g > 0) compute_sync();
+        const int dir = sl.e.dir;
+        if constexpr (EXT) {
+          if (dir == 0) fwd_task<T, RG, 0, true>(sl, a, gr, smem);
+          else bwd_task<T, RG, 0, true>(sl, a, gr, smem);
+        } else {
+          const bool tri = a.si == PSP_SI_NONE;
+          if (dir == 0) {
+            if (tri) fwd_tri_task<T, RG>(sl, a, gr, smem);
+            else fwd_task<T, RG, 0, false>(sl, a, gr, smem);
+          } else if (dir == kDirUpB) {
+            fwd_task<T, RG, 1, false>(sl, a, gr, smem);
+          } else if (dir == 1) {
+            bwd_task<T, RG, 0, false>(sl, a, gr, smem);
+          } else {
+            if (tri) bwd_tri_task<T, RG>(sl, a, gr, smem);
+            else bwd_task<T, RG, 1, false>(sl, a, gr, smem);
+          }
+        }
+      }
+    }
+    bar_arrive(kBarDone + (n & 1), kComputeThreads + 32);
+    if (!ok) break;
+  }
+}
+
+template <typename T, int RG, bool EXT>
 static int sweep_rg(const SweepArgs<T>& args, size_t smem, int max_per_sm, cudaStream_t st) {
-  if (cudaFuncSetAttribute(k_sweep<T, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+  if (cudaFuncSetAttribute(k_sweep<T, RG, EXT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
     cudaGetLastError();
     return -1;
   }
@@ -662,8 +826,7 @@ static int sweep_rg(const SweepArgs<T>& args, size_t smem, int max_per_sm, cudaS
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-  if (!coop) return -1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<T, RG>, kSweepThreads, smem) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<T, RG, EXT>, kSweepThreads, smem) != cudaSuccess ||
       per_sm < 1) {
     cudaGetLastError();
     return -1;
@@ -671,100 +834,69 @@ static int sweep_rg(const SweepArgs<T>& args, size_t smem, int max_per_sm, cudaS
   per_sm = per_sm > max_per_sm ? max_per_sm : per_sm;
   SweepArgs<T> a = args;
   void* kargs[] = {&a};
-  cudaError_t e =
-      cudaLaunchCooperativeKernel((const void*)k_sweep<T, RG>, dim3(sms * per_sm), dim3(kSweepThreads), kargs, smem, st);
+  cudaError_t e;
+  if (coop) {
+    e = cudaLaunchCooperativeKernel((const void*)k_sweep<T, RG, EXT>, dim3(sms * per_sm), dim3(kSweepThreads), kargs, smem, st);
+  } else {   // one CTA alone takes the queue in order and never waits
+    k_sweep<T, RG, EXT><<<1, kSweepThreads, smem, st>>>(a);
+    e = cudaGetLastError();
+  }
   return e == cudaSuccess ? 0 : (int)e;
 }
 
-// A CTA carries RG right-hand sides through each pass over a factor block (as many as nrhs, at most 8,
-// or rhs_group when > 0), and the vectors of a task pass through shared memory in chunks sized so
-// that a CTA keeps within kSweepSmem (several CTAs stay resident per SM: a CTA that waits on a
-// dependency leaves the SM to the others).  Substitution tasks (fronts keeping L_TL) hold a front's
+// A CTA carries RG right-hand sides through each pass over a factor block (as many as nrhs, at most 8 in complex64
+// and 4 in complex128, where the FP64 pipe and not the factor's bytes is the bound; or rhs_group when > 0), and the
+// vectors of a task pass through shared memory in chunks sized so that two CTAs stay resident per SM (a CTA that
+// waits on a dependency leaves the SM to the other).  Substitution tasks (fronts keeping L_TL) hold a front's
 // whole vector, so for them RG shrinks until that fits.
-constexpr size_t kSweepSmem = 64 * 1024;
+template <typename T, int RG>
+constexpr size_t sweep_smem() { return (sizeof(T) == 16 && RG == 4 ? 84 : 64) * 1024; }
 
-template <typename T>
-int launch_sweep(const SweepArgs<T>& args, int smax, int ldmax, int max_per_sm, int rhs_group, cudaStream_t st) {
-  const size_t es = sizeof(T);
-  int rg = 8;
-  while (rg > 1 && rg >= 2 * args.cx.nrhs) rg >>= 1;
-  if (rhs_group > 0)
-    while (rg > 1 && rg > rhs_group) rg >>= 1;
-  const int full = (ldmax > smax ? ldmax : smax);
-  int chunk;
-  if (args.cx.si == PSP_SI_NONE) {
-    chunk = full;
-    while (rg > 1 && ((size_t)chunk + 256) * rg * es > 200 * 1024) rg >>= 1;
-  } else {
-    chunk = (int)((kSweepSmem / (rg * es) - 256) / 256 * 256);
-    if (chunk < 256) chunk = 256;
-    if (chunk >= full) chunk = full;   // one chunk: every task's vector at once
-  }
+template <typename T, int RG>
+static int sweep_sized(const SweepArgs<T>& args, int smax, int ldmax, int max_per_sm, cudaStream_t st) {
+  constexpr size_t es = sizeof(T), entry = entry_stride<T, RG>() * es, fixed = 2 * (size_t)kComputeThreads * RG * es;
+  const int full = ldmax > smax ? ldmax : smax;
+  int chunk = (int)((sweep_smem<T, RG>() - fixed) / entry / 64 * 64);
+  if (chunk >= full) chunk = full > 0 ? full : 1;   // one chunk: every task's vector at once
   SweepArgs<T> a = args;
   a.chunk = chunk;
-  const size_t smem = ((size_t)chunk + 256) * rg * es;
-  switch (rg) {
-    case 8: return sweep_rg<T, 8>(a, smem, max_per_sm, st);
-    case 4: return sweep_rg<T, 4>(a, smem, max_per_sm, st);
-    case 2: return sweep_rg<T, 2>(a, smem, max_per_sm, st);
-    default: return sweep_rg<T, 1>(a, smem, max_per_sm, st);
-  }
-}
-
-template <typename T, int RG>
-static void fwd_rg(const SolveTask* tasks, int ntasks, const SolveCtx<T>& cx, int R, int smax, int phase, cudaStream_t st) {
-  const size_t smem = ((size_t)smax + 256) * RG * sizeof(T);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(k_solve_fwd<T, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    attr_set = true;
-  }
-  dim3 grid(ntasks, (cx.nrhs + RG - 1) / RG);
-  k_solve_fwd<T, RG><<<grid, 256, smem, st>>>(tasks, cx, R, phase, smax > 0 ? smax : 1);
-}
-
-template <typename T, int RG>
-static void bwd_rg(const SolveTask* tasks, int ntasks, const SolveCtx<T>& cx, int ldmax, int phase, cudaStream_t st) {
-  const size_t smem = ((size_t)ldmax + 256) * RG * sizeof(T);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(k_solve_bwd<T, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    attr_set = true;
-  }
-  dim3 grid(ntasks, (cx.nrhs + RG - 1) / RG);
-  k_solve_bwd<T, RG><<<grid, 256, smem, st>>>(tasks, cx, phase, ldmax > 0 ? ldmax : 1);
+  size_t smem = fixed + chunk * entry;
+  if (a.si == PSP_SI_NONE && smem < (size_t)smax * RG * es) smem = (size_t)smax * RG * es;
+  return a.si == PSP_SI_EXTENDED ? sweep_rg<T, RG, true>(a, smem, max_per_sm, st) : sweep_rg<T, RG, false>(a, smem, max_per_sm, st);
 }
 
 template <typename T>
-void launch_solve_fwd(const SolveTask* tasks, int ntasks, const SolveCtx<T>& cx, int R, int smax, int phase,
-                      cudaStream_t st) {
-  if (ntasks <= 0) return;
-  const int rg = pick_rg<T>(cx.nrhs, ((size_t)smax + 256) * sizeof(T));
+int launch_sweep(const SweepArgs<T>& a, int smax, int ldmax, int max_per_sm, int rhs_group, cudaStream_t st) {
+  int rg = sizeof(T) == 8 ? 8 : 4;
+  while (rg > 1 && rg >= 2 * a.nrhs) rg >>= 1;
+  if (rhs_group > 0)
+    while (rg > 1 && rg > rhs_group) rg >>= 1;
+  if (a.si == PSP_SI_NONE)
+    while (rg > 1 && (size_t)smax * rg * sizeof(T) > 180 * 1024) rg >>= 1;
   switch (rg) {
-    case 8: fwd_rg<T, 8>(tasks, ntasks, cx, R, smax, phase, st); break;
-    case 4: fwd_rg<T, 4>(tasks, ntasks, cx, R, smax, phase, st); break;
-    case 2: fwd_rg<T, 2>(tasks, ntasks, cx, R, smax, phase, st); break;
-    default: fwd_rg<T, 1>(tasks, ntasks, cx, R, smax, phase, st); break;
+    case 8:
+      if constexpr (sizeof(T) == 8) return sweep_sized<T, 8>(a, smax, ldmax, max_per_sm, st);
+    case 4: return sweep_sized<T, 4>(a, smax, ldmax, max_per_sm, st);
+    case 2: return sweep_sized<T, 2>(a, smax, ldmax, max_per_sm, st);
+    default: return sweep_sized<T, 1>(a, smax, ldmax, max_per_sm, st);
   }
 }
 
-template <typename T>
-void launch_solve_bwd(const SolveTask* tasks, int ntasks, const SolveCtx<T>& cx, int ldmax, int phase, cudaStream_t st) {
-  if (ntasks <= 0) return;
-  const int rg = pick_rg<T>(cx.nrhs, ((size_t)ldmax + 256) * sizeof(T));
-  switch (rg) {
-    case 8: bwd_rg<T, 8>(tasks, ntasks, cx, ldmax, phase, st); break;
-    case 4: bwd_rg<T, 4>(tasks, ntasks, cx, ldmax, phase, st); break;
-    case 2: bwd_rg<T, 2>(tasks, ntasks, cx, ldmax, phase, st); break;
-    default: bwd_rg<T, 1>(tasks, ntasks, cx, ldmax, phase, st); break;
-  }
-}
-
-template void launch_solve_fwd<double2>(const SolveTask*, int, const SolveCtx<double2>&, int, int, int, cudaStream_t);
-template void launch_solve_fwd<float2>(const SolveTask*, int, const SolveCtx<float2>&, int, int, int, cudaStream_t);
-template void launch_solve_bwd<double2>(const SolveTask*, int, const SolveCtx<double2>&, int, int, cudaStream_t);
-template void launch_solve_bwd<float2>(const SolveTask*, int, const SolveCtx<float2>&, int, int, cudaStream_t);
 template int launch_sweep<double2>(const SweepArgs<double2>&, int, int, int, int, cudaStream_t);
 template int launch_sweep<float2>(const SweepArgs<float2>&, int, int, int, int, cudaStream_t);
+
+// index words of a shape's front rows: row p of front f gets {its box node (p < s, else -1), the two update-vector
+// entries its children add to it, 0}, so that a gather reads one 16-byte word per row
+__global__ void __launch_bounds__(128) k_build_rows(ShapeDev sh, int4* rows) {
+  const int f = blockIdx.x;
+  const int s = sh.s[f], n = s + sh.u[f], first = sh.first[f];
+  const int64_t o = sh.pull_ptr[f];
+  for (int p = threadIdx.x; p < n; p += blockDim.x)
+    rows[o + p] = make_int4(p < s ? sh.order[first + p] : -1, sh.pull[2 * (o + p)], sh.pull[2 * (o + p) + 1], 0);
+}
+
+void launch_build_rows(const ShapeDev& sh, int4* rows, cudaStream_t st) {
+  if (sh.nsn > 0) k_build_rows<<<sh.nsn, 128, 0, st>>>(sh, rows);
+}
 
 }  // namespace psp

@@ -289,7 +289,7 @@ struct psp_ctx_s {
   // solve plan
   struct LevelPlan {
     int64_t fwd_off = 0;
-    int nfwd = 0, R = 64, smax = 0;
+    int nfwd = 0, smax = 0;
     int64_t bwd_off = 0;
     int nbwd = 0, ldmax = 0;
     // second phases of the fronts (factors that keep L_BL): up rows r >= s, down columns
@@ -299,17 +299,19 @@ struct psp_ctx_s {
     double vec = 0;       // vector entries gathered / written by one direction
   };
   std::vector<std::vector<LevelPlan>> splan;
-  DevBuf d_stasks;
   // persistent sweep plan
   struct SweepPlan {
     DevBuf steps, queue;
-    std::vector<SweepStep> hsteps;
     int nsteps = 0, nqueue = 0;
     int64_t nfront_steps = 0;                 // fronts summed over the steps
     double entries = 0, vec = 0;              // algorithmic factor entries / vector words per sweep
   };
   SweepPlan plans[3];              // 0: Alg. 1.5 over the handle's panels; 1: its forward part; 2: its backward part
-  DevBuf d_sweep_panels, d_sweep_sync;
+  DevBuf d_sweep_sync, d_front_recs;
+  std::vector<DevBuf> d_rows;      // per shape: index words of the fronts' rows
+  std::vector<int> front_base;     // per shape: its first record in d_front_recs
+  DevBuf d_dinv;                   // reciprocal pivots, per factored panel in elimination order
+  std::vector<int64_t> panel_dbase;
   size_t sweep_sync_words = 0;     // counters of the largest plan (one sweep runs at a time per handle)
   int sweep_smax = 0, sweep_ldmax = 0;   // the widest front's s and s + u (vector staging of the sweep)
   // block of panels [range_begin, range_end) this handle factors and sweeps (all of them unless the
@@ -342,7 +344,6 @@ struct psp_ctx_s {
   int gmres_basis = 0;   // 0 auto, 1 keep z_j, 2 V only
   int si_mode = 0;       // psp_si_mode: what the factor of each front keeps (selective inversion, §2.2)
   bool test_sweep_stall = false;
-  bool persistent_sweep = true;
   int64_t upd_arena_elems = 0;
   int64_t temp_budget_elems = 0;   // cap on setup temporaries per level group (0: what the device has free)
   // problems: one, or the independent problems of a batch (psp_setup_batch) with their panels
@@ -357,7 +358,7 @@ struct psp_ctx_s {
   std::vector<Prob> probs;
   std::vector<std::unique_ptr<psp_ctx_s>> subs;   // a batch's problems: their wave speeds and tables
   std::vector<BoxOp> h_boxops;                    // per panel, uploaded to d_boxops
-  DevBuf d_sweep_probs, d_cols;
+  DevBuf d_cols;
   int cols_nrhs = 0;
   Stats stats;
 };
@@ -653,6 +654,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       ft.G = fbase + X->panel_fbase[p] + sh.g_off[sn];
       ft.U = upd_ptr[ft.gfid];
       ft.ut = upd_tile[ft.gfid];
+      ft.dinv = X->d_dinv.as<T>() + X->panel_dbase[p] + sh.first[sn];
       ft.W = ft.Z = ft.ZD = ft.W2 = nullptr;
       ft.ldzd = ft.u;
       packs.push_back(nullptr);
@@ -871,15 +873,16 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         launches.push_back(lg);
       }
     }
-    // inv(L_TL) into F_TL's strict lower part (and the second inverse after G)
-    if (si != PSP_SI_NONE) {
+    // inv(L_TL) into F_TL's strict lower part (and the second inverse after G); the pivots' reciprocals
+    {
       const int64_t c0 = (int64_t)ctasks.size();
       for (int f = 0; f < nf; ++f) {
         const auto& ft = fronts[f0 + f];
         for (int c = 0; c < ft.s; c += 16) ctasks.push_back({f, c, std::min(c + 16, ft.s)});
       }
       Launch lc{COPY, f0, c0, (int)(ctasks.size() - c0), 0};
-      for (int f = 0; f < nf; ++f) lc.bytes += es * (double)fronts[f0 + f].s * (fronts[f0 + f].s - 1);
+      for (int f = 0; f < nf; ++f)
+        lc.bytes += es * (2.0 * fronts[f0 + f].s + (si != PSP_SI_NONE ? (double)fronts[f0 + f].s * (fronts[f0 + f].s - 1) : 0.0));
       launches.push_back(lc);
     }
     // Z = F_BL inv(L_TL)^T (= F_BL L^{-T}), then F_BR -= Z D^{-1} Z^T (lower) and M_BL = Z D^{-1} inv(L_TL).
@@ -1158,13 +1161,12 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
       const int rmin = std::max(8, std::min(64, X->sweep_min_rows));
       int R = X->sweep_max_rows;
       while (R > rmin && rows / R < X->sweep_level_tasks) R >>= 1;
-      P.R = R;
       int Cc = X->sweep_max_rows;
       while (Cc > rmin && cols / Cc < X->sweep_level_tasks) Cc >>= 1;
+      const bool two = X->si_mode != PSP_SI_EXTENDED, tri = X->si_mode == PSP_SI_NONE;
       // extended factors: one pass per front and direction over all s + u rows; factors keeping L_BL:
       // up, rows r < s (one whole-front substitution task without inversion) then rows r >= s; down,
       // columns for L_BL^T then columns for the triangle (one whole-front task without inversion)
-      const bool two = X->si_mode != PSP_SI_EXTENDED, tri = X->si_mode == PSP_SI_NONE;
       auto rows_of = [&](int sn, int a, int b, int step) {
         for (int r = a; r < b; r += step) tasks.push_back({sn, r, std::min(r + step, b)});
       };
@@ -1192,15 +1194,13 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
       P.nbwdB = (int)(tasks.size() - P.bwdB_off);
     }
   }
-  upload_async(X->d_stasks, tasks, side.s);
-
   // per shape: tasks per front, up and down
-  std::vector<int> front_base(X->shapes.size() + 1, 0), ntask_up, ntask_down, ntask_upA, ntask_downA;
+  const std::vector<int>& front_base = X->front_base;
+  std::vector<int> ntask_up, ntask_down, ntask_upA, ntask_downA;
   std::vector<double> shape_entries(X->shapes.size(), 0.0), shape_vec(X->shapes.size(), 0.0);
   std::vector<int> shape_tasks(X->shapes.size(), 0);
   for (size_t si = 0; si < X->shapes.size(); ++si) {
     const Shape& sh = X->shapes[si];
-    front_base[si] = (int)ntask_up.size();
     ntask_up.resize(ntask_up.size() + sh.nsn, 0);
     ntask_down.resize(ntask_down.size() + sh.nsn, 0);
     ntask_upA.resize(ntask_upA.size() + sh.nsn, 0);
@@ -1219,7 +1219,6 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
     ntask_up[f] += ntask_upA[f];
     ntask_down[f] += ntask_downA[f];
   }
-  front_base[X->shapes.size()] = (int)ntask_up.size();
   X->sweep_smax = 0;
   X->sweep_ldmax = 0;
   for (const auto& sp : X->splan)
@@ -1236,10 +1235,13 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
   size_t sync_words = 0;
   for (int pi = 0; pi < 3; ++pi) {
     psp_ctx_s::SweepPlan& SP = X->plans[pi];
-    std::vector<SweepStep> steps;
+    struct Step {
+      int panel, mode, prob;   // mode 0: forward sweep (assign), 1: backward sweep (subtract)
+    };
+    std::vector<Step> steps;
     std::vector<int> step_prev;
     const int np = (int)X->probs.size();
-    std::vector<std::vector<SweepStep>> chain(np);
+    std::vector<std::vector<Step>> chain(np);
     size_t longest = 0;
     for (int q = 0; q < np; ++q) {
       const auto& pr = X->probs[q];
@@ -1274,24 +1276,32 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
     const int64_t o_step = kSweepStepCounters, o_up = o_step + (int64_t)steps.size(), o_down = o_up + nfs,
                   o_kids = o_down + nfs, words = o_kids + nfs;
     if (words > INT_MAX) throw Error{PSP_ERR_ARG, "sweep plan too large"};
+    // steps some front of the next solve waits for as a whole
+    std::vector<char> step_waited(steps.size(), 0);
+    for (size_t k = 0; k < steps.size(); ++k)
+      if (step_prev[k] >= 0 && X->shape_of[steps[step_prev[k]].panel] != X->shape_of[steps[k].panel])
+        step_waited[step_prev[k]] = 1;
     std::vector<QueueEntry> queue;
     for (size_t k = 0; k < steps.size(); ++k) {
       const int si = X->shape_of[steps[k].panel];
       const Shape& sh = X->shapes[si];
       const int fb = front_base[si], sfb = step_front[k];
       const int prev = step_prev[k];
-      // a front without children waits for the previous panel solve of its chain (the tasks of a
-      // front with children wait for those, which waited for it)
-      const unsigned prev_target =
-          prev >= 0 ? (unsigned)step_tasks[prev] + (X->test_sweep_stall && prev == 0 ? 1u : 0u) : 0u;
-      auto entry = [&](const SolveTask& tk, int dir, int R) {
+      // A front without children waits for the previous panel solve of its chain (the tasks of a
+      // front with children wait for those, which waited for it).  Boxes of one shape have one tree, and a front
+      // reads the previous panel's solution at its own (x, y) only: then the same front's down tasks there are
+      // enough (they come after every down task of its ancestors, and every work entry that this solve's up tasks
+      // overwrite has been read once the fronts below it are done).
+      const bool same_tree = prev >= 0 && X->shape_of[steps[prev].panel] == si;
+      const unsigned stall = X->test_sweep_stall && prev == 0 ? 1u : 0u;
+      auto entry = [&](const SolveTask& tk, int dir) {
         QueueEntry e{};
         e.step = (int)k;
-        e.sn = tk.sn;
+        e.front = fb + tk.sn;
         e.r0 = tk.r0;
         e.r1 = tk.r1;
         e.dir = (short)dir;
-        e.R = (short)R;
+        e.step_done = step_waited[k] ? (int)(o_step + k) : -1;
         const int sn = tk.sn, par = sh.parent[sn];
         const bool up = dir == 0 || dir == kDirUpB;
         e.done = (int)((up ? o_up : o_down) + sfb + sn);
@@ -1303,9 +1313,12 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
           if (kids > 0) {
             e.wait = (int)(o_kids + sfb + sn);
             e.target = kids;
+          } else if (same_tree) {
+            e.wait = (int)(o_down + step_front[prev] + sn);
+            e.target = (unsigned)ntask_down[fb + sn] + stall;
           } else if (prev >= 0) {
             e.wait = (int)(o_step + prev);
-            e.target = prev_target;
+            e.target = (unsigned)step_tasks[prev] + stall;
           }
         } else if (dir == kDirUpB) {   // the front's own first phase up
           e.wait = (int)(o_up + sfb + sn);
@@ -1324,35 +1337,46 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
       };
       const auto& plan = X->splan[si];
       for (size_t lv = 0; lv < plan.size(); ++lv) {
-        for (int t = 0; t < plan[lv].nfwd; ++t) entry(tasks[plan[lv].fwd_off + t], 0, plan[lv].R);
-        for (int t = 0; t < plan[lv].nfwdB; ++t) entry(tasks[plan[lv].fwdB_off + t], kDirUpB, plan[lv].R);
+        for (int t = 0; t < plan[lv].nfwd; ++t) entry(tasks[plan[lv].fwd_off + t], 0);
+        for (int t = 0; t < plan[lv].nfwdB; ++t) entry(tasks[plan[lv].fwdB_off + t], kDirUpB);
       }
       for (int lv = (int)plan.size() - 1; lv >= 0; --lv) {
-        for (int t = 0; t < plan[lv].nbwd; ++t) entry(tasks[plan[lv].bwd_off + t], 1, 0);
-        for (int t = 0; t < plan[lv].nbwdB; ++t) entry(tasks[plan[lv].bwdB_off + t], kDirDownB, 0);
+        for (int t = 0; t < plan[lv].nbwd; ++t) entry(tasks[plan[lv].bwd_off + t], 1);
+        for (int t = 0; t < plan[lv].nbwdB; ++t) entry(tasks[plan[lv].bwdB_off + t], kDirDownB);
       }
     }
-    SP.hsteps = steps;
+    std::vector<StepRec> recs;
+    for (const Step& sp : steps) {
+      const auto& pr = X->probs[sp.prob];
+      const int i = sp.panel, si = X->shape_of[i];
+      StepRec r{};
+      r.gbase = X->panel_fbase[i];
+      r.dbase = X->panel_dbase[i];
+      r.off1 = pr.off1;
+      r.N = pr.N;
+      r.s1n = pr.s1n;
+      r.s2n = pr.s2n;
+      r.s3c = pr.s3hi + (sp.mode == 0 ? X->z0[i] : X->z1[i]);
+      r.cz = (sp.mode == 0 ? 1.0 : -1.0) / (pr.h * pr.h);
+      r.rows = X->d_rows[si].as<int4>();
+      r.sel = X->shdev[si].struct_elim;
+      r.z0 = X->z0[i];
+      r.z1 = X->z1[i];
+      r.lead = X->lead[i];
+      r.nx = X->shapes[si].nx;
+      r.plane = X->shapes[si].nx * X->shapes[si].ny;
+      r.mode = sp.mode;
+      r.couple = sp.mode == 0 ? i > pr.panel0 : i < pr.panel0 + pr.m - 1;
+      r.prob = sp.prob;
+      recs.push_back(r);
+    }
     SP.nsteps = (int)steps.size();
     SP.nqueue = (int)queue.size();
-    upload_async(SP.steps, steps, side.s);
+    upload_async(SP.steps, recs, side.s);
     upload_async(SP.queue, queue, side.s);
     SP.nfront_steps = nfs;
     sync_words = std::max(sync_words, (size_t)words);
   }
-  std::vector<ProblemSweep> pss;
-  for (const auto& pr : X->probs) {
-    ProblemSweep p{};
-    p.off1 = pr.off1;
-    p.N = pr.N;
-    p.s1n = pr.s1n;
-    p.s2n = pr.s2n;
-    p.s3h = pr.s3hi;
-    p.inv_h2 = 1.0 / (pr.h * pr.h);
-    p.nz = pr.nz;
-    pss.push_back(p);
-  }
-  upload_async(X->d_sweep_probs, pss, side.s);
   X->sweep_sync_words = sync_words;
   X->d_sweep_sync.alloc(X->sweep_sync_words * 4);
   side.join(st);
@@ -1378,105 +1402,44 @@ template <typename T>
 static void apply_core(psp_ctx_s* X, double2* u, int nrhs, T* xf, T* xb, T* upd, bool timed, cudaStream_t st,
                        int plan_index = 0) {
   const psp_ctx_s::SweepPlan& SP = X->plans[plan_index];
-  SolveCtx<T> cx{};
-  const int np = (int)X->probs.size();
-  // problem q's vectors and work vectors
-  auto set_problem = [&](int q) {
-    const auto& pr = X->probs[q];
-    cx.xf = xf + (int64_t)q * X->max_nloc * nrhs;
-    cx.xb = xb + (int64_t)q * X->max_nloc * nrhs;
-    cx.upd = upd + (int64_t)q * X->max_upd * nrhs;
-    cx.u = u + pr.off1 * nrhs;
-    cx.N = pr.N;
-    cx.nz = pr.nz;
-    cx.s1n = pr.s1n;
-    cx.s2n = pr.s2n;
-    cx.s3h = pr.s3hi;
-    cx.inv_h2 = 1.0 / (pr.h * pr.h);
-  };
-  cx.nrhs = nrhs;
-  cx.si = X->si_mode;
-  cx.upd_ld = X->max_upd;
-  cx.n_loc = X->max_nloc;
-  set_problem(0);
-  // the persistent sweep offsets problem q's pointers itself: hand it the bases
-  cx.xf = xf;
-  cx.xb = xb;
-  cx.upd = upd;
-  cx.u = u;
-  const SolveTask* tasks = X->d_stasks.as<SolveTask>();
+  if (SP.nsteps == 0) return;   // an empty part (the backward part of a block holding the last panel alone)
+  SweepArgs<T> sa{};
+  sa.xf = xf;
+  sa.xb = xb;
+  sa.upd = upd;
+  sa.u = u;
+  sa.n_loc = X->max_nloc;
+  sa.upd_ld = X->max_upd;
+  sa.nrhs = nrhs;
+  sa.si = X->si_mode;
+  sa.steps = SP.steps.as<StepRec>();
+  sa.fronts = X->d_front_recs.as<FrontRec>();
+  sa.factor = X->d_factor.as<T>();
+  sa.dinv = X->d_dinv.as<T>();
+  sa.queue = SP.queue.as<QueueEntry>();
+  sa.nqueue = SP.nqueue;
+  sa.claim_ahead = X->sweep_claim_ahead;
+  unsigned* sync = X->d_sweep_sync.as<unsigned>();
+  sa.ctr = sync;
+  sa.status = reinterpret_cast<int*>(sync + 1);
+  sa.sticky = X->d_status.as<int>() + 2;
+  const size_t words = kSweepStepCounters + (size_t)SP.nsteps + 3 * (size_t)SP.nfront_steps;
+  // queue head and completion counters start at zero; status[2] is cleared too
+  PSP_CK(cudaMemsetAsync(sync, 0, words * 4, st));
+  const double es = sizeof(T);
   const bool was_timing = X->stats.timing;
   if (!timed) X->stats.timing = false;
-  auto runT = [&](int q, int i, int mode) {
-    const auto& pr = X->probs[q];
-    set_problem(q);
-    const int si = X->shape_of[i];
-    cx.sh = X->shdev[si];
-    cx.G = X->d_factor.as<T>() + X->panel_fbase[i];
-    cx.z0 = X->z0[i];
-    cx.z1 = X->z1[i];
-    cx.lead = X->lead[i];
-    cx.mode = mode;
-    cx.has_prev = i > pr.panel0;
-    cx.has_next = i < pr.panel0 + pr.m - 1;
-    const auto& plan = X->splan[si];
-    const int nl = (int)plan.size();
-    const double es = sizeof(T);
-    for (int lv = 0; lv < nl; ++lv) {
-      const auto& P = plan[lv];
-      X->stats.run("k_solve_fwd", st, 1, 8.0 * P.entries * nrhs, P.entries * es + P.vec * es * nrhs, [&] {
-        launch_solve_fwd<T>(tasks + P.fwd_off, P.nfwd, cx, P.R, P.smax, 0, st);
-        launch_solve_fwd<T>(tasks + P.fwdB_off, P.nfwdB, cx, P.R, P.smax, 1, st);
-      });
-    }
-    for (int lv = nl - 1; lv >= 0; --lv) {
-      const auto& P = plan[lv];
-      X->stats.run("k_solve_bwd", st, 1, 8.0 * P.entries * nrhs, P.entries * es + P.vec * es * nrhs, [&] {
-        launch_solve_bwd<T>(tasks + P.bwd_off, P.nbwd, cx, P.ldmax, 0, st);
-        launch_solve_bwd<T>(tasks + P.bwdB_off, P.nbwdB, cx, P.ldmax, 1, st);
-      });
-    }
-  };
+  int rc = -1;
   try {
-    // one cooperative launch for the whole sweep when the device allows it
-    SweepArgs<T> sa{};
-    sa.cx = cx;
-    sa.nshapes = (int)X->shapes.size();
-    sa.nsteps = SP.nsteps;
-    sa.npanels = X->m;
-    sa.steps = SP.steps.as<SweepStep>();
-    sa.panels = X->d_sweep_panels.as<PanelSweep>();
-    sa.shapes = X->d_shapes.as<ShapeDev>();
-    sa.factor = X->d_factor.as<T>();
-    sa.queue = SP.queue.as<QueueEntry>();
-    sa.nqueue = SP.nqueue;
-    sa.claim_ahead = X->sweep_claim_ahead;
-    sa.nprobs = np;
-    sa.probs = X->d_sweep_probs.as<ProblemSweep>();
-    unsigned* sync = X->d_sweep_sync.as<unsigned>();
-    sa.ctr = sync;
-    sa.status = reinterpret_cast<int*>(sync + 1);
-    sa.sticky = X->d_status.as<int>() + 2;
-    const size_t words = kSweepStepCounters + (size_t)SP.nsteps + 3 * (size_t)SP.nfront_steps;
-    int rc = -1;
-    if (SP.nsteps == 0) rc = 0;   // an empty part (the backward part of a block holding the last panel alone)
-    else if (X->persistent_sweep) {
-      // queue head and completion counters start at zero; status[2] is cleared too
-      PSP_CK(cudaMemsetAsync(sync, 0, words * 4, st));
-      const double es = sizeof(T);
-      X->stats.run("k_sweep", st, 1, 8.0 * SP.entries * nrhs, SP.entries * es + SP.vec * es * nrhs,
-                   [&] { rc = launch_sweep<T>(sa, X->sweep_smax, X->sweep_ldmax, X->sweep_ctas_per_sm, X->sweep_rhs_group, st); });
-      if (rc > 0) throw Error{PSP_ERR_CUDA, std::string("sweep launch: ") + cudaGetErrorString((cudaError_t)rc)};
-    }
-    if (rc != 0) {
-      // one launch per tree level: mode 0 u_i := T_i (u_i - J_{i,i-1} u_{i-1}); mode 1 u_i -= T_i J_{i+1,i}^T u_{i+1}
-      for (const SweepStep& sp : SP.hsteps) runT(sp.prob, sp.panel, sp.mode);
-    }
+    X->stats.run("k_sweep", st, 1, 8.0 * SP.entries * nrhs, SP.entries * es + SP.vec * es * nrhs,
+                 [&] { rc = launch_sweep<T>(sa, X->sweep_smax, X->sweep_ldmax, X->sweep_ctas_per_sm, X->sweep_rhs_group, st); });
   } catch (...) {
     X->stats.timing = was_timing;
     throw;
   }
   X->stats.timing = was_timing;
+  if (rc > 0) throw Error{PSP_ERR_CUDA, std::string("sweep launch: ") + cudaGetErrorString((cudaError_t)rc)};
+  if (rc < 0) throw Error{PSP_ERR_CUDA, "the sweep does not fit the device's shared memory"};
   PSP_CK(cudaGetLastError());
 }
 
@@ -1853,13 +1816,41 @@ static void finish_setup(psp_ctx_s* X, cudaStream_t st) {
     X->shape_bufs.push_back(std::move(b));
   }
   upload(X->d_shapes, X->shdev);
+  // the sweep's records: per front, and per front row its index words
+  {
+    std::vector<FrontRec> recs;
+    X->front_base.clear();
+    X->d_rows.clear();
+    for (size_t si = 0; si < X->shapes.size(); ++si) {
+      const Shape& sh = X->shapes[si];
+      X->front_base.push_back((int)recs.size());
+      for (int f = 0; f < sh.nsn; ++f) {
+        FrontRec r{};
+        r.s = sh.s[f];
+        r.u = sh.u[f];
+        r.first = sh.first[f];
+        r.g_off = sh.g_off[f];
+        r.row_off = sh.pull_ptr[f];
+        r.sel_off = sh.struct_ptr[f];
+        r.upd_off = sh.upd_off[f];
+        recs.push_back(r);
+      }
+      DevBuf b;
+      b.alloc((size_t)sh.pull_ptr[sh.nsn] * sizeof(int4));
+      launch_build_rows(X->shdev[si], b.as<int4>(), st);
+      X->d_rows.push_back(std::move(b));
+    }
+    PSP_CK(cudaGetLastError());
+    upload(X->d_front_recs, recs);
+  }
   std::vector<int32_t> ps(X->shape_of.begin(), X->shape_of.end());
   upload(X->d_panel_shape, ps);
 
   // front ids and factor slabs
   X->sn_base.assign(X->m, 0);
   X->panel_fbase.assign(X->m, 0);
-  int64_t nf = 0, fe = 0;
+  X->panel_dbase.assign(X->m, 0);
+  int64_t nf = 0, fe = 0, de = 0;
   X->nfronts_factored = 0;
   X->distinct_panels = 0;
   for (int i = 0; i < X->m; ++i) {
@@ -1869,10 +1860,13 @@ static void finish_setup(psp_ctx_s* X, cudaStream_t st) {
     if (X->owner[i] == i) {
       X->panel_fbase[i] = fe;
       fe += sh.g_total;
+      X->panel_dbase[i] = de;
+      de += sh.first[sh.nsn];
       X->nfronts_factored += sh.nsn;
       X->distinct_panels += 1;
     } else if (X->owner[i] >= 0) {
       X->panel_fbase[i] = X->panel_fbase[X->owner[i]];   // the owner comes first
+      X->panel_dbase[i] = X->panel_dbase[X->owner[i]];
     } else {
       X->panel_fbase[i] = 0;                              // outside this handle's block: never read
     }
@@ -1880,23 +1874,10 @@ static void finish_setup(psp_ctx_s* X, cudaStream_t st) {
   X->nfronts = nf;
   X->factor_elems = fe;
   X->elem_bytes = X->prec == PSP_PREC_C64 ? 8 : 16;
-  {
-    std::vector<PanelSweep> ps(X->m);
-    for (const auto& pr : X->probs)
-      for (int i = pr.panel0; i < pr.panel0 + pr.m; ++i) {
-        ps[i].gbase = X->panel_fbase[i];
-        ps[i].shape = X->shape_of[i];
-        ps[i].z0 = X->z0[i];
-        ps[i].z1 = X->z1[i];
-        ps[i].lead = X->lead[i];
-        ps[i].has_prev = i > pr.panel0;
-        ps[i].has_next = i < pr.panel0 + pr.m - 1;
-      }
-    upload(X->d_sweep_panels, ps);
-  }
   X->stats.host("device_tables", ms_since(t_start));
   auto ta = std::chrono::steady_clock::now();
   X->d_factor.alloc((size_t)fe * X->elem_bytes);
+  X->d_dinv.alloc((size_t)de * X->elem_bytes);
   X->d_status.alloc(8 * sizeof(int));
   X->stats.host("alloc_factors", ms_since(ta));
   // the sweep's plan is host work the device does not need for the factorisation: it runs while
@@ -2221,8 +2202,8 @@ static void init_options(psp_ctx_s* X, const psp_options& o) {
   X->use_tc = o.tensor_cores != 0;
   X->diag_fp64 = o.c64_diag_fp64 != 0;
   X->tc_min_dim = o.tc_min_dim > 0 ? o.tc_min_dim : 64;
-  // measured on lens100: both precisions' sweeps are fastest at about 608 tasks per level
-  X->sweep_level_tasks = o.sweep_level_tasks > 0 ? o.sweep_level_tasks : 608;
+  // measured on lens100, 304 against 608 tasks per level: complex128 35.9 / 38.3 ms, complex64 11.7 / 14.4 ms
+  X->sweep_level_tasks = o.sweep_level_tasks > 0 ? o.sweep_level_tasks : 304;
   X->sweep_ctas_per_sm = o.sweep_ctas_per_sm > 0 ? o.sweep_ctas_per_sm : 8;
   X->sweep_rhs_group = o.sweep_rhs_group > 0 ? o.sweep_rhs_group : 0;
   X->sweep_min_rows = o.sweep_min_rows > 0 ? o.sweep_min_rows : 8;

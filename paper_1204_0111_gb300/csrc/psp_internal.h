@@ -150,6 +150,7 @@ struct FrontTask {
   T* Z;        // u x s work: F_BL L^{-T}
   T* ZD;       // u x s: Z D^{-1}, leading dimension ldzd (a work block for the extended selective
                // inversion of CUDA-core fronts, G's bottom block when L_BL itself is stored; else nullptr)
+  T* dinv;     // the front's reciprocal pivots (for the sweep)
   T* W2;       // s x s work: the second inverse of L_TL under construction (two-inverse form), else nullptr
   int s, u;
   int panel, sn;
@@ -218,104 +219,89 @@ void launch_copy_linv(const FrontTask<T>* fronts, const ColTask* tasks, int ntas
 template <typename T>
 void launch_scale_zd(const FrontTask<T>* fronts, const ColTask* tasks, int ntasks, cudaStream_t st);
 
-// ---- multifrontal solve of one panel (Alg. 1.3 inside Alg. 1.5) ----
-struct SolveTask {  // rows [r0, r1) of front sn (forward) or columns [r0, r1) of S (backward)
+// ---- the whole sweep (Alg. 1.5, each panel's multifrontal solve as in Alg. 1.3) in one cooperative launch ----
+struct SolveTask {  // rows [r0, r1) of front sn (up the tree) or columns [r0, r1) of S (down)
   int sn, r0, r1;
 };
 
-template <typename T>
-struct SolveCtx {
-  ShapeDev sh;
-  const T* G;              // this panel's factor slab
-  T* xf;                   // box vector after L^{-1} and D^{-1} (elimination order), ld = n_loc
-  T* xb;                   // box vector after L^{-T}
-  T* upd;                  // children's update vectors, ld = upd_ld
-  double2* u;              // global vector block, ld = N
-  int64_t N, n_loc, upd_ld;
-  int nrhs;
-  int z0, z1, lead, nz;    // panel planes, pad planes, global plane count
-  int mode;                // 0: forward sweep (u_i := T_i(u_i - J_{i,i-1} u_{i-1})); 1: backward (u_i -= T_i J^T u_{i+1})
-  int has_prev, has_next;
-  int si;                  // psp_si_mode of the factors (what G keeps)
-  const double2* s1n;      // global stretch tables for the plane coupling J_{i+1,i}
-  const double2* s2n;
-  const double2* s3h;
-  double inv_h2;
+// one front as a task reads it
+struct FrontRec {
+  int s, u, first, pad_;
+  int64_t g_off;      // its G block within the panel's factor slab (elements)
+  int64_t row_off;    // its rows' index words within the shape's
+  int64_t sel_off;    // its struct indices within the shape's
+  int64_t upd_off;    // its update vector within the panel's update vectors
+  int64_t pad2_[2];
 };
+static_assert(sizeof(FrontRec) == 64, "records are copied word by word");
 
-// phase 0: the single pass (extended factors) or first phase of a front; phase 1: its second phase
-template <typename T>
-void launch_solve_fwd(const SolveTask* tasks, int ntasks, const SolveCtx<T>& cx, int R, int smax, int phase,
-                      cudaStream_t st);
-template <typename T>
-void launch_solve_bwd(const SolveTask* tasks, int ntasks, const SolveCtx<T>& cx, int ldmax, int phase, cudaStream_t st);
-
-// ---- the whole sweep in one cooperative launch ----
-struct SweepStep {      // one panel solve of Alg. 1.5, in order
-  int panel, mode;      // mode 0: forward sweep (assign), 1: backward sweep (subtract)
-  int prob;             // problem of a batch (0 for a single problem)
-};
-// per problem of a batch: where its vectors sit and its coupling tables
-struct ProblemSweep {
-  int64_t off1;         // offset of the problem's block in a batched vector, per right-hand side
-  int64_t N;            // points of the problem
-  const double2* s1n;
+// one panel solve of Alg. 1.5: its panel, its problem's vectors and coupling tables
+struct StepRec {
+  int64_t gbase;         // factor slab offset (elements)
+  int64_t dbase;         // offset of the panel's reciprocal pivots
+  int64_t off1;          // offset of the problem's block in a batched vector, per right-hand side
+  int64_t N;             // points of the problem
+  const double2* s1n;    // global stretch tables for the plane coupling J_{i+1,i}: s1 s2 (1 / s3 at the plane boundary)
   const double2* s2n;
-  const double2* s3h;
-  double inv_h2;
-  int nz, pad_;
+  const double2* s3c;
+  double cz;             // +- 1 / h^2
+  const int4* rows;      // the shape's index words per front row: {node, child update entry, child update entry, 0}
+  const int32_t* sel;    // the shape's struct indices (elimination order)
+  int z0, z1, lead;      // panel planes, pad planes
+  int nx, plane;         // nx, nx * ny
+  int mode;              // 0: forward sweep (u_i := T_i(u_i - J_{i,i-1} u_{i-1})); 1: backward (u_i -= T_i J^T u_{i+1})
+  int couple;            // there is a previous (mode 0) / next (mode 1) panel
+  int prob;              // problem of a batch (0 for a single problem)
+  int pad_[4];
 };
-struct PanelSweep {
-  int64_t gbase;        // factor slab offset (elements)
-  int shape, z0, z1, lead, has_prev, has_next;
-};
-struct LevelSweep {
-  int64_t fwd_off, bwd_off;
-  int nfwd, nbwd, R, pad_;
-};
-// one entry of the sweep's task queue (topological order: panel solves in Alg. 1.5 order; inside
+static_assert(sizeof(StepRec) == 128, "records are copied word by word");
+
+// one task of the sweep's queue (topological order: panel solves in Alg. 1.5 order; inside
 // one, the up-the-tree tasks level by level, then the down-the-tree tasks from the root).  An entry
-// carries its one dependency and the counters it signals, so that a CTA takes a task with a single
-// 48-byte read.  Counters are words of the sweep's counter array (zeroed before every sweep):
+// carries its one dependency and the counters it signals.  Counters are words of the sweep's counter array
+// (zeroed before every sweep):
 //   [0] dequeue head, [1, 5) status, then per step the tasks completed, then per step and front the
 //   up tasks completed, the down tasks completed and the up tasks of the front's children completed.
 struct QueueEntry {
-  int step;                     // panel solve index
-  int sn, r0, r1;               // the task: rows (up) or columns (down) [r0, r1) of front sn
+  int step, front;              // panel solve index, front record
+  int r0, r1;                   // rows (up) or columns (down) [r0, r1) of the front
   int wait;                     // counter the task waits for (-1: none) ...
   unsigned target;              // ... until it reaches this count
   int done;                     // counter of the front's own completed tasks (this direction)
   int kids;                     // counter of the parent's children's completed up tasks (-1: none)
+  int step_done;                // counter of the step's completed tasks (-1: nothing waits for it)
   short dir;                    // 0 up the tree, 1 down the tree; 2 / 3 the second phase up / down of a front
                                 // whose factor keeps L_BL (the first phase is then 0 / 1)
-  short R;                      // rows per up-the-tree task
-  int pad_[3];
+  short pad0_;
+  int pad_[2];
 };
-static_assert(sizeof(QueueEntry) == 48, "queue entries are copied as three 16-byte words");
+static_assert(sizeof(QueueEntry) == 48, "queue entries are copied word by word");
 // second phases of a front (factors that keep L_BL rather than L_BL inv(L_TL))
 constexpr int kDirUpB = 2, kDirDownB = 3;
 constexpr int kSweepStepCounters = 5;   // first word of the per-step counters
 template <typename T>
 struct SweepArgs {
-  SolveCtx<T> cx;               // fields common to every panel (vectors, sizes, coupling tables); for a batch
-                                // (nprobs > 1) the vector and work-vector bases, offset per problem
-  int nshapes, nsteps, npanels; // sizes of the three tables below (kept in shared memory)
-  const SweepStep* steps;
-  const PanelSweep* panels;
-  const ShapeDev* shapes;
+  T* xf;                        // box vectors after L^{-1} and D^{-1} (elimination order), n_loc x nrhs per problem
+  T* xb;                        // box vectors after L^{-T}
+  T* upd;                       // fronts' update vectors, upd_ld x nrhs per problem
+  double2* u;                   // global vector block
+  int64_t n_loc, upd_ld;
+  int nrhs;
+  int si;                       // psp_si_mode of the factors (what G keeps)
+  const StepRec* steps;
+  const FrontRec* fronts;
   const T* factor;
+  const T* dinv;                // reciprocal pivots, per panel in elimination order
   const QueueEntry* queue;
   int nqueue;
   unsigned* ctr;                // counter array (layout above)
   int* status;                  // status[2] set when a wait gave up (= ctr + 1)
   int* sticky;                  // also set then; kept until the host reads it (psp_check_status)
-  // batches of independent problems (nprobs > 1): each problem's steps form their own chain
-  int nprobs;
-  const ProblemSweep* probs;    // per problem; cx's vectors and work vectors are offset per problem
   int chunk;                    // vector entries a task stages in shared memory at a time (set by launch_sweep)
   int claim_ahead;              // 2: a CTA holds the two tasks after the one it runs; 1: the next one only
 };
-// returns 0 on success, -1 when a cooperative launch is not possible, else a cudaError_t; smax / ldmax:
+void launch_build_rows(const ShapeDev& sh, int4* rows, cudaStream_t st);
+// returns 0 on success, -1 when the kernel does not fit the device, else a cudaError_t; smax / ldmax:
 // the widest front's s and s + u
 template <typename T>
 int launch_sweep(const SweepArgs<T>& args, int smax, int ldmax, int max_per_sm, int rhs_group, cudaStream_t st);
