@@ -393,6 +393,8 @@ static double ms_since(std::chrono::steady_clock::time_point t0) {
   return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
 }
 
+constexpr int kOzMinDim = 16;   // complex128: fewest s and u of a front on the tensor cores
+
 // `while_device_runs` is host work done after the last launch is enqueued, before waiting for them.
 template <typename T>
 static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()>& while_device_runs) {
@@ -428,6 +430,25 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   const bool tc_ok = std::is_same<T, float2>::value && X->use_tc && si != PSP_SI_NONE;
   auto use_tc = [&](int64_t s_, int64_t u_) { return tc_ok && s_ >= X->tc_min_dim && u_ >= X->tc_min_dim; };
   const int64_t TBLK = tc_block_bytes() / (int64_t)sizeof(T);   // packed block in T elements
+  // complex128: fronts of at least kOzMinDim rows each way run the same products on the tensor cores from exact digit
+  // products; below that the tiles are mostly padding (128 x 32 outputs, k in 16s), and there is next to no work
+  const OzShape oz = oz_shape();
+  bool oz_ok = std::is_same<T, double2>::value && X->use_tc && si != PSP_SI_NONE;
+  auto use_oz = [&](int64_t s_, int64_t u_) { return oz_ok && s_ >= kOzMinDim && u_ >= kOzMinDim; };
+  auto cdiv_i = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
+  // bytes of a packed operand of R rows and K columns and of its row exponents (A: 128-row blocks, B: 32-row blocks)
+  auto oz_bytes = [&](int64_t R, int64_t K, bool b) {
+    return cdiv_i(R, b ? oz.tile_n : oz.tile_m) * cdiv_i(K, oz.k) * (b ? oz.b_block : oz.a_block);
+  };
+  auto oz_exps = [&](int64_t R, int64_t K, bool b) {
+    return (int64_t)sizeof(int) * cdiv_i(R, b ? oz.tile_n : oz.tile_m) * cdiv_i(K, oz.kc) * (b ? oz.tile_n : oz.tile_m);
+  };
+  // F_BL and, once Z is made, Z D^-1 in its place (A operands); inv(L); Z; inv(L)^T (extended form)
+  auto oz_elems = [&](int64_t s_, int64_t u_) {
+    int64_t b = oz_bytes(u_, s_, false) + oz_exps(u_, s_, false) + oz_bytes(u_, s_, true) + oz_exps(u_, s_, true) +
+                oz_bytes(s_, s_, true) + oz_exps(s_, s_, true);
+    return pad16(cdiv_i(b, (int64_t)sizeof(T)) + 64);
+  };
   auto nrb = [](int64_t r) { return (r + 127) / 128; };
   auto nkb16 = [](int64_t k) { return (k + 15) / 16; };
   auto packed_elems = [&](int64_t s_, int64_t u_) {   // F_BL, Z D^-1, Z (u x s) and two inv(L) (s x s)
@@ -436,24 +457,39 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   auto front_temp = [&](int64_t s_, int64_t u_) {     // W (s x s), Z (u x s), Z D^-1 or packed operands,
     if (si == PSP_SI_NONE) return (int64_t)0;         // the second inverse under construction (s x s)
     return pad16(s_ * s_) + pad16(u_ * s_) + (si == PSP_SI_TWO ? pad16(s_ * s_) : 0) +
-           (use_tc(s_, u_) ? packed_elems(s_, u_) : si == PSP_SI_EXTENDED ? pad16(u_ * s_) : 0);
+           (use_tc(s_, u_) ? packed_elems(s_, u_)
+            : use_oz(s_, u_) ? oz_elems(s_, u_)
+                             : si == PSP_SI_EXTENDED ? pad16(u_ * s_) : 0);
   };
   int64_t arena[2] = {0, 0}, temp_level_max = 0, temp_front_max = 16;
-  for (int lv = 0; lv < L; ++lv) {
-    int64_t slab = 0, tsum = 0;
-    for (auto [p, sn] : lev_fronts[lv]) {
-      const Shape& sh = X->shapes[X->shape_of[p]];
-      const int64_t s = sh.s[sn], u = sh.u[sn];
-      if (u > 0) {
-        uoff[X->sn_base[p] + sn] = slab;
-        slab += pad16(upd_packed_elems((int)u, use_tc(s, u) ? 128 : 64));
+  auto plan_memory = [&] {
+    arena[0] = arena[1] = temp_level_max = 0;
+    temp_front_max = 16;
+    for (int lv = 0; lv < L; ++lv) {
+      int64_t slab = 0, tsum = 0;
+      for (auto [p, sn] : lev_fronts[lv]) {
+        const Shape& sh = X->shapes[X->shape_of[p]];
+        const int64_t s = sh.s[sn], u = sh.u[sn];
+        if (u > 0) {
+          uoff[X->sn_base[p] + sn] = slab;
+          slab += pad16(upd_packed_elems((int)u, use_tc(s, u) || use_oz(s, u) ? 128 : 64));
+        }
+        const int64_t t = front_temp(s, u);
+        tsum += t;
+        temp_front_max = std::max(temp_front_max, t);
       }
-      const int64_t t = front_temp(s, u);
-      tsum += t;
-      temp_front_max = std::max(temp_front_max, t);
+      arena[lv & 1] = std::max(arena[lv & 1], slab);
+      temp_level_max = std::max(temp_level_max, tsum);
     }
-    arena[lv & 1] = std::max(arena[lv & 1], slab);
-    temp_level_max = std::max(temp_level_max, tsum);
+  };
+  plan_memory();
+  if (oz_ok) {   // where the device has no room for the widest front's packed operands, every product stays on FP64 units
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
+        (double)(arena[0] + arena[1] + temp_front_max) * sizeof(T) > 0.8 * ((double)free_b - 2.0e9)) {
+      oz_ok = false;
+      plan_memory();
+    }
   }
   X->upd_arena_elems = arena[0] + arena[1];
   X->stats.host("plan_memory", ms_since(tp));
@@ -509,7 +545,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   for (int p = 0; p < X->m; ++p) {
     const Shape& sh = X->shapes[X->shape_of[p]];
     for (int sn = 0; sn < sh.nsn; ++sn)
-      if (use_tc(sh.s[sn], sh.u[sn])) upd_tile[X->sn_base[p] + sn] = 128;
+      if (use_tc(sh.s[sn], sh.u[sn]) || use_oz(sh.s[sn], sh.u[sn])) upd_tile[X->sn_base[p] + sn] = 128;
   }
   DevBuf d_upd_ptr, d_upd_tile;
   upload(d_upd_ptr, upd_ptr);
@@ -523,7 +559,9 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   std::vector<unsigned char*> packs;     // per front: base of its packed operands (tensor-core fronts)
   std::vector<TcPackTask> ptasks;
   std::vector<TcGemmTask> ttasks;
-  enum Kind { ASSEMBLE, DIAG, PRIGHT, PLEFT, GEMM, COPY, TCGEMM, TCPACK, SCALE, RSOLVE };
+  std::vector<OzPackTask> optasks;
+  std::vector<OzGemmTask> otasks;
+  enum Kind { ASSEMBLE, DIAG, PRIGHT, PLEFT, GEMM, COPY, TCGEMM, TCPACK, SCALE, RSOLVE, OZPACK, OZGEMM };
   struct Launch {
     Kind kind;
     int64_t front_off;
@@ -559,7 +597,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   // [4..5] ~bits of the smallest |pivot| (0: none yet)
   PSP_CK(cudaMemsetAsync(status, 0, 8 * sizeof(int), st));
   static const char* names[] = {"k_assemble", "k_diag_ldlt", "k_panel_right", "k_panel_left", "k_gemm", "k_copy_linv",
-                                "k_tc_gemm", "k_tc_pack", "k_scale_zd", "k_panel_rsolve"};
+                                "k_tc_gemm", "k_tc_pack", "k_scale_zd", "k_panel_rsolve", "k_oz_pack", "k_oz_gemm"};
   // task arrays go up on a side stream, so that the next group's planning overlaps the device's work
   SideStream up;
   std::vector<void*> chunks;
@@ -594,16 +632,18 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
     }
     return d;
   };
-  size_t up_f = 0, up_c = 0, up_d = 0, up_g = 0, up_p = 0, up_t = 0;
+  size_t up_f = 0, up_c = 0, up_d = 0, up_g = 0, up_p = 0, up_t = 0, up_op = 0, up_o = 0;
   double plan_ms = 0, enqueue_ms = 0;
   auto enqueue_group = [&](size_t lb) {
-    const size_t f0 = up_f, c0 = up_c, d0 = up_d, g0 = up_g, p0 = up_p, t0 = up_t;
+    const size_t f0 = up_f, c0 = up_c, d0 = up_d, g0 = up_g, p0 = up_p, t0 = up_t, op0 = up_op, o0 = up_o;
     const FrontTask<T>* F = upload_tail(fronts, up_f);
     const ColTask* CT = upload_tail(ctasks, up_c);
     const int* DL = upload_tail(dlist, up_d);
     const GemmTask<T>* GT = upload_tail(gtasks, up_g);
     const TcPackTask* PT = upload_tail(ptasks, up_p);
     const TcGemmTask* TT = upload_tail(ttasks, up_t);
+    const OzPackTask* OP = upload_tail(optasks, up_op);
+    const OzGemmTask* OT = upload_tail(otasks, up_o);
     up.join(st);   // the group's kernels after its task arrays
     up_f = fronts.size();
     up_c = ctasks.size();
@@ -611,6 +651,8 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
     up_g = gtasks.size();
     up_p = ptasks.size();
     up_t = ttasks.size();
+    up_op = optasks.size();
+    up_o = otasks.size();
     for (size_t li = lb; li < launches.size(); ++li) {
       const Launch& l = launches[li];
       if (l.count <= 0) continue;
@@ -629,6 +671,8 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
           case GEMM: launch_gemm<T>(GT + (l.off - (int64_t)g0), l.count, st); break;
           case COPY: launch_copy_linv<T>(Fl, CT + (l.off - (int64_t)c0), l.count, st); break;
           case TCGEMM: launch_tc_gemm(TT + (l.off - (int64_t)t0), l.count, status, st); break;
+          case OZPACK: launch_oz_pack(OP + (l.off - (int64_t)op0), l.count, st); break;
+          case OZGEMM: launch_oz_gemm(OT + (l.off - (int64_t)o0), l.count, status, st); break;
           case TCPACK: launch_tc_pack(PT + (l.off - (int64_t)p0), l.count, st); break;
           case SCALE: launch_scale_zd<T>(Fl, CT + (l.off - (int64_t)c0), l.count, st); break;
           case RSOLVE: launch_panel_rsolve<T>(Fl, CT + (l.off - (int64_t)c0), l.count, l.kb, wide, st); break;
@@ -666,6 +710,9 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         if (use_tc(ft.s, ft.u)) {
           packs.back() = reinterpret_cast<unsigned char*>(tbase + toff);
           toff += packed_elems(ft.s, ft.u);
+        } else if (use_oz(ft.s, ft.u)) {
+          packs.back() = reinterpret_cast<unsigned char*>(tbase + toff);
+          toff += oz_elems(ft.s, ft.u);
         } else if (si == PSP_SI_EXTENDED) {
           ft.ZD = tbase + toff;
           toff += pad16((int64_t)ft.u * ft.s);
@@ -1022,7 +1069,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       double tflops = 0, tflops_si = 0;
       for (int f : ord) {
         const auto& ft = fronts[f0 + f];
-        if (ft.u == 0 || !packs[f0 + f]) continue;
+        if (std::is_same<T, double2>::value || ft.u == 0 || !packs[f0 + f]) continue;
         const int ld = ft.s + ft.u;
         const Packed P = packed_of(f);
         const int64_t bb = tc_block_bytes();
@@ -1086,6 +1133,97 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
               tflops_si += 8.0 * gemm_cmacs(sh);   // M_BL: selective inversion
             }
         }
+      }
+      if constexpr (std::is_same<T, double2>::value) {
+        // complex128 fronts on the tensor cores.  Phase 0: F_BL (A) and inv(L) (B), Z = F_BL inv(L)^T.  Phase 1: Z D^-1 in
+        // F_BL's place and Z (B), the Schur update; then (extended form) inv(L)^T in inv(L)'s place and M_BL.
+        auto oz_pack = [&](const T* src, const T* dinv, unsigned char* dst, int64_t ld_, int64_t R, int64_t K, int mode, bool b) {
+          const int64_t nkb = cdiv_i(K, oz.k), nkc = cdiv_i(K, oz.kc), rows = b ? oz.tile_n : oz.tile_m;
+          int* exps = reinterpret_cast<int*>(dst + oz_bytes(R, K, b));
+          for (int64_t r0 = 0; r0 < R; r0 += oz.tile_m)
+            for (int64_t kc = 0; kc < nkc; ++kc) {
+              OzPackTask t{};
+              t.src = src;
+              t.dinv = dinv;
+              t.dst = dst + (r0 / rows * nkb + kc * (oz.kc / oz.k)) * (b ? oz.b_block : oz.a_block);
+              t.exps = exps + (r0 / rows * nkc + kc) * rows;
+              t.sub_stride = nkb * oz.b_block;
+              t.exp_stride = nkc * oz.tile_n;
+              t.ld = (int)ld_;
+              t.r0 = (int)r0;
+              t.k0 = (int)(kc * oz.kc);
+              t.R = (int)R;
+              t.K = (int)K;
+              t.mode = mode;
+              t.rows_b = b;
+              optasks.push_back(t);
+            }
+          const double e = (double)R * K;
+          return e * (16.0 + (double)(b ? oz.b_block / (oz.tile_n * oz.k) : oz.a_block / (oz.tile_m * oz.k)));
+        };
+        // tiles of C (R x N) = +-A B^T with k in [klo(col), khi(col))
+        auto oz_tile = [&](unsigned char* A, int64_t RA, unsigned char* B, int64_t RB, int64_t K, int ti, int tj, T* C, int ldc,
+                           int64_t k0, int64_t k1, int doff, int flags) {
+          const int64_t nkb = cdiv_i(K, oz.k), nkc = cdiv_i(K, oz.kc);
+          OzGemmTask t{};
+          t.A = A + ti / oz.tile_m * nkb * oz.a_block;
+          t.B = B + tj / oz.tile_n * nkb * oz.b_block;
+          t.ea = reinterpret_cast<const int*>(A + oz_bytes(RA, K, false)) + ti / oz.tile_m * nkc * oz.tile_m;
+          t.eb = reinterpret_cast<const int*>(B + oz_bytes(RB, K, true)) + tj / oz.tile_n * nkc * oz.tile_n;
+          t.C = C;
+          t.ldc = ldc;
+          t.m = (int)std::min<int64_t>(oz.tile_m, RA - ti);
+          t.n = (int)std::min<int64_t>(oz.tile_n, RB - tj);
+          t.kb0 = (int)(k0 / oz.k);
+          t.nkb = (int)(cdiv_i(k1, oz.k) - k0 / oz.k);
+          t.doff = doff;
+          t.flags = flags;
+          otasks.push_back(t);
+        };
+        constexpr int kAll = 1 << 30;   // no triangle mask
+        for (int step = 0; step < (phase == 0 ? 1 : si == PSP_SI_EXTENDED ? 2 : 1); ++step) {
+          const int64_t op0 = (int64_t)optasks.size(), o0 = (int64_t)otasks.size();
+          Launch lp{OZPACK, f0, op0, 0, -1}, lt{OZGEMM, f0, o0, 0, -1};
+          for (int f : ord) {
+            const auto& ft = fronts[f0 + f];
+            if (ft.u == 0 || !packs[f0 + f]) continue;
+            const int ld = ft.s + ft.u;
+            const int64_t s_ = ft.s, u_ = ft.u;
+            unsigned char* PA = packs[f0 + f];
+            unsigned char* PB = PA + (oz_bytes(u_, s_, false) + oz_exps(u_, s_, false));
+            unsigned char* PL = PB + (oz_bytes(u_, s_, true) + oz_exps(u_, s_, true));
+            if (phase == 0) {
+              lp.bytes += oz_pack(ft.G + ft.s, nullptr, PA, ld, u_, s_, TC_PACK_PLAIN, false);
+              lp.bytes += oz_pack(ft.G, nullptr, PL, ld, s_, s_, TC_PACK_UNIT_LOWER, true);
+              for (int tj = 0; tj < ft.s; tj += oz.tile_n)
+                for (int ti = 0; ti < ft.u; ti += oz.tile_m)
+                  oz_tile(PA, u_, PL, s_, s_, ti, tj, ft.Z + (int64_t)tj * ft.u + ti, ft.u, 0,
+                          std::min<int64_t>(tj + oz.tile_n, s_), kAll, GF_BETA0);
+              lt.flops += 8.0 * u_ * s_ * (s_ + 1.0) / 2;
+            } else if (step == 0) {
+              lp.bytes += oz_pack(ft.Z, ft.dinv, PA, u_, u_, s_, TC_PACK_PLAIN, false);
+              lp.bytes += oz_pack(ft.Z, nullptr, PB, u_, u_, s_, TC_PACK_PLAIN, true);
+              for (int tj = 0; tj < ft.u; tj += oz.tile_n)
+                for (int ti = tj / oz.tile_m * oz.tile_m; ti < ft.u; ti += oz.tile_m)
+                  oz_tile(PA, u_, PB, u_, s_, ti, tj, ft.U + upd_index(std::max(ti, tj), tj, ft.u, 128) - std::max(0, tj - ti),
+                          128, 0, s_, ti > tj ? kAll : ti - tj, GF_NEG);
+              lt.flops += 8.0 * s_ * u_ * (u_ + 1.0) / 2;
+            } else {
+              lp.bytes += oz_pack(ft.G, nullptr, PL, ld, s_, s_, TC_PACK_UNIT_LOWER_T, true);
+              for (int tj = 0; tj < ft.s; tj += oz.tile_n)
+                for (int ti = 0; ti < ft.u; ti += oz.tile_m)
+                  oz_tile(PA, u_, PL, s_, s_, ti, tj, ft.G + (int64_t)tj * ld + ft.s + ti, ld, tj, s_, kAll, GF_BETA0);
+              lt.extra += 8.0 * u_ * s_ * (s_ + 1.0) / 2;   // M_BL: selective inversion
+            }
+          }
+          lp.count = (int)(optasks.size() - op0);
+          lt.count = (int)(otasks.size() - o0);
+          for (size_t i = o0; i < otasks.size(); ++i)
+            lt.bytes += (double)otasks[i].nkb * (oz.a_block + oz.b_block) + 32.0 * otasks[i].m * otasks[i].n;
+          launches.push_back(lp);
+          launches.push_back(lt);
+        }
+        continue;
       }
       if ((int64_t)ptasks.size() > p0) {
         Launch lp{TCPACK, f0, p0, (int)(ptasks.size() - p0), -1};

@@ -211,6 +211,35 @@ struct TcGemmTask {        // one 128 x 128 tile of C (+)= +-A B^T from packed b
 };
 void launch_tc_pack(const TcPackTask* tasks, int ntasks, cudaStream_t st);
 void launch_tc_gemm(const TcGemmTask* tasks, int ntasks, int* status, cudaStream_t st);
+// tensor-core path of complex128 fronts: operands written once as eight base-256 digits, then 128 x 32 tiles
+struct OzShape { int tile_m, tile_n, k, kc; int64_t a_block, b_block; };   // tile, k per block and per row scale, bytes per block
+OzShape oz_shape();
+struct OzPackTask {        // 128 rows x 128 k of an operand
+  const double2* src;      // column-major source, ld
+  const double2* dinv;     // PLAIN only: column k times dinv[k] (nullptr: no scaling)
+  unsigned char* dst;      // first block (16 k) of these rows; the following ones adjacent
+  int* exps;               // row exponents of this block of k
+  int64_t sub_stride;      // B operands: bytes between the blocks of 32 rows ...
+  int64_t exp_stride;      // ... and entries between their exponents
+  int ld, r0, k0, R, K;    // first row / k, source extents (outside -> 0)
+  int mode;                // TcPackMode
+  int rows_b;              // 0: A operand (128-row blocks), 1: B operand (32-row blocks)
+  int pad_;
+};
+struct OzGemmTask {        // one 128 x 32 tile of C (+)= +-A B^T
+  const unsigned char* A;  // block of 16 k number 0 of its 128 rows
+  const unsigned char* B;  // block of 16 k number 0 of its 32 rows
+  const int* ea;           // row exponents, 128 per 128 k
+  const int* eb;           // 32 per 128 k
+  double2* C;
+  int ldc, m, n;
+  int kb0, nkb;            // blocks of 16 k [kb0, kb0 + nkb)
+  int doff;                // entries with row + doff < column are not written
+  int flags;               // GF_NEG, GF_BETA0
+  int pad_;
+};
+void launch_oz_pack(const OzPackTask* tasks, int ntasks, cudaStream_t st);
+void launch_oz_gemm(const OzGemmTask* tasks, int ntasks, int* status, cudaStream_t st);
 int tc_block_k();
 int64_t tc_block_bytes();
 int tc_gemm_tile();
