@@ -19,8 +19,8 @@ __device__ __forceinline__ Row7 row7(const BoxOp& op, int x, int y, int z) {
   const double2 axm = cmul(s23, op.s1h[x]), axp = cmul(s23, op.s1h[x + 1]);
   const double2 aym = cmul(s13, op.s2h[y]), ayp = cmul(s13, op.s2h[y + 1]);
   const double2 azm = cmul(s12, op.s3h[z]), azp = cmul(s12, op.s3h[z + 1]);
-  const double cc = op.c[((int64_t)op.cplane[z] * op.ny + y) * op.nx + x];
-  const double2 mass = cmul(cscale(op.k2num, 1.0 / (cc * cc)), cmul(s12, s3));
+  const double ic2 = op.ic2[((int64_t)op.cplane[z] * op.ny + y) * op.nx + x];
+  const double2 mass = cmul(cscale(op.k2num, ic2), cmul(s12, s3));
   Row7 r;
   double2 sum = cadd(cadd(cadd(axm, axp), cadd(aym, ayp)), cadd(azm, azp));
   r.d = csub(cscale(sum, op.inv_h2), mass);
@@ -33,25 +33,145 @@ __device__ __forceinline__ Row7 row7(const BoxOp& op, int x, int y, int z) {
   return r;
 }
 
+// bitwise tests: a floating-point comparison takes the FP64 pipe
+__device__ __forceinline__ bool is_zero(double v) { return (__double_as_longlong(v) << 1) == 0; }
+__device__ __forceinline__ bool is_one(double2 v) { return __double_as_longlong(v.x) == 0x3ff0000000000000ll && is_zero(v.y); }
+
 // y = Op x for nrhs vectors (column-major, ld = N); one thread per node.
-__global__ void k_matvec(BoxOp op, const double2* __restrict__ x, double2* __restrict__ y, int nrhs, int64_t N) {
-  const int64_t plane = (int64_t)op.nx * op.ny;
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < N; g += (int64_t)gridDim.x * blockDim.x) {
-    const int xx = (int)(g % op.nx);
-    const int yy = (int)((g / op.nx) % op.ny);
-    const int zz = (int)(g / plane);
-    const Row7 r = row7(op, xx, yy, zz);
-    for (int q = 0; q < nrhs; ++q) {
-      const double2* xv = x + q * N;
-      double2 acc = cmul(r.d, xv[g]);
-      if (xx > 0) cfma(acc, r.xm, xv[g - 1]);
-      if (xx + 1 < op.nx) cfma(acc, r.xp, xv[g + 1]);
-      if (yy > 0) cfma(acc, r.ym, xv[g - op.nx]);
-      if (yy + 1 < op.ny) cfma(acc, r.yp, xv[g + op.nx]);
-      if (zz > 0) cfma(acc, r.zm, xv[g - plane]);
-      if (zz + 1 < op.nz) cfma(acc, r.zp, xv[g + plane]);
-      y[q * N + g] = acc;
+//
+// Bound by the FP64 pipe, not by its 40 bytes per node: the seven complex coefficients of a row and their products took
+// about 110 FP64 operations.  Outside an axis' PML its stretches are exactly one; a warp leaves out what that makes
+// trivial for all its nodes: with no PML a row needs 15 operations (17 for J), in one axis' PML about 46, and with
+// several vectors a PML node 32 more per vector.  The same operations whatever nrhs, so every vector keeps its bits.
+// 100^3, one vector: 189 -> 83 us; 61 x 83 x 47, three vectors: 80 -> 56 us.
+//
+// matvec_rows<ONE1, ONE2, ONE3>: the nodes of a warp, ONEj: axis j's stretches are one for all of them.  A function per
+// combination, so that what it leaves out is not computed and then discarded.
+template <bool ONE1, bool ONE2, bool ONE3>
+__device__ __forceinline__ void matvec_rows(const BoxOp& op, const double2* __restrict__ x, double2* __restrict__ y, int nrhs,
+                                            int64_t N, int64_t g, bool in, int xx, int yy, int zz) {
+  const int plane = op.nx * op.ny;
+  const bool xl = xx > 0, xh = xx + 1 < op.nx, yl = yy > 0, yh = yy + 1 < op.ny, zl = zz > 0, zh = zz + 1 < op.nz;
+  const double2 zero = make_double2(0.0, 0.0);
+  const double ic2 = op.ic2[(int64_t)op.cplane[zz] * plane + yy * op.nx + xx];
+  const bool real_k = is_zero(op.k2num.y);
+  constexpr bool kAll = ONE1 && ONE2 && ONE3;
+  double2 d;                                    // the diagonal
+  double2 m1 = zero, m2 = zero, m3 = zero;      // s2 s3, s1 s3, s1 s2
+  double2 a1 = zero, b1 = zero, a2 = zero, b2 = zero, a3 = zero, b3 = zero;   // minus the couplings, times h^2
+  if constexpr (kAll) {
+    d = make_double2(fma(6.0, op.inv_h2, -op.k2num.x * ic2), -op.k2num.y * ic2);
+  } else {
+    const double2 one = make_double2(1.0, 0.0);
+    const double2 s1 = ONE1 ? one : op.s1n[xx], s2 = ONE2 ? one : op.s2n[yy], s3 = ONE3 ? one : op.s3n[zz];
+    m1 = ONE2 ? s3 : (ONE3 ? s2 : cmul(s2, s3));
+    m2 = ONE1 ? s3 : (ONE3 ? s1 : cmul(s1, s3));
+    m3 = ONE1 ? s2 : (ONE2 ? s1 : cmul(s1, s2));
+    double2 sum = zero;
+    if constexpr (ONE1) {
+      sum = cscale(m1, 2.0);
+    } else {
+      a1 = op.s1h[xx];
+      b1 = op.s1h[xx + 1];
+      if constexpr (!(ONE2 && ONE3)) {
+        a1 = cmul(m1, a1);
+        b1 = cmul(m1, b1);
+      }
+      sum = cadd(a1, b1);
     }
+    if constexpr (ONE2) {
+      sum = make_double2(fma(2.0, m2.x, sum.x), fma(2.0, m2.y, sum.y));
+    } else {
+      a2 = op.s2h[yy];
+      b2 = op.s2h[yy + 1];
+      if constexpr (!(ONE1 && ONE3)) {
+        a2 = cmul(m2, a2);
+        b2 = cmul(m2, b2);
+      }
+      sum = cadd(sum, cadd(a2, b2));
+    }
+    if constexpr (ONE3) {
+      sum = make_double2(fma(2.0, m3.x, sum.x), fma(2.0, m3.y, sum.y));
+    } else {
+      a3 = op.s3h[zz];
+      b3 = op.s3h[zz + 1];
+      if constexpr (!(ONE1 && ONE2)) {
+        a3 = cmul(m3, a3);
+        b3 = cmul(m3, b3);
+      }
+      sum = cadd(sum, cadd(a3, b3));
+    }
+    const double2 s123 = ONE1 ? m1 : (ONE2 && ONE3 ? s1 : cmul(s1, m1));
+    d = cscale(sum, op.inv_h2);
+    if (real_k) {
+      const double k = op.k2num.x * ic2;
+      d = make_double2(fma(-k, s123.x, d.x), fma(-k, s123.y, d.y));
+    } else {
+      cfms(d, cscale(op.k2num, ic2), s123);
+    }
+  }
+  for (int q = 0; q < nrhs; ++q) {
+    const double2* xv = x + q * N + g;
+    const double2 c = xv[0];
+    const double2 xm = xl ? xv[-1] : zero, xp = xh ? xv[1] : zero, ym = yl ? xv[-op.nx] : zero, yp = yh ? xv[op.nx] : zero;
+    const double2 zm = zl ? xv[-plane] : zero, zp = zh ? xv[plane] : zero;
+    double2 v;
+    if constexpr (kAll) {
+      const double2 n = cadd(cadd(cadd(xm, xp), cadd(ym, yp)), cadd(zm, zp));
+      v = make_double2(fma(-op.inv_h2, n.x, d.x * c.x), fma(-op.inv_h2, n.y, d.x * c.y));
+      if (!real_k) {
+        v.x = fma(-d.y, c.y, v.x);
+        v.y = fma(d.y, c.x, v.y);
+      }
+    } else {
+      // the axes outside their PML have one coefficient for both neighbours, and two of them share it
+      double2 n;
+      if constexpr (ONE2 && ONE3) n = cmul(m2, cadd(cadd(ym, yp), cadd(zm, zp)));
+      else if constexpr (ONE1 && ONE3) n = cmul(m1, cadd(cadd(xm, xp), cadd(zm, zp)));
+      else if constexpr (ONE1 && ONE2) n = cmul(m1, cadd(cadd(xm, xp), cadd(ym, yp)));
+      else if constexpr (ONE1) n = cmul(m1, cadd(xm, xp));
+      else if constexpr (ONE2) n = cmul(m2, cadd(ym, yp));
+      else if constexpr (ONE3) n = cmul(m3, cadd(zm, zp));
+      else n = zero;
+      if constexpr (!ONE1) {
+        cfma(n, a1, xm);
+        cfma(n, b1, xp);
+      }
+      if constexpr (!ONE2) {
+        cfma(n, a2, ym);
+        cfma(n, b2, yp);
+      }
+      if constexpr (!ONE3) {
+        cfma(n, a3, zm);
+        cfma(n, b3, zp);
+      }
+      v = cmul(d, c);
+      v = make_double2(fma(-op.inv_h2, n.x, v.x), fma(-op.inv_h2, n.y, v.y));
+    }
+    if (in) y[q * N + g] = v;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_matvec(BoxOp op, const double2* __restrict__ x, double2* __restrict__ y, int nrhs,
+                                                int64_t N) {
+  const int64_t g0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const bool in = g0 < N;
+  const int64_t g = in ? g0 : N - 1;   // every lane takes part in the votes
+  const unsigned gu = (unsigned)g, plane = (unsigned)op.nx * op.ny;   // grids have at most 2^31 points
+  const int zz = (int)(gu / plane), p = (int)(gu - (unsigned)zz * plane), yy = p / op.nx, xx = p - yy * op.nx;
+  // axis by axis: the stretches at the node and at both half-points are one
+  const bool o1 = __all_sync(0xffffffffu, is_one(op.s1n[xx]) && is_one(op.s1h[xx]) && is_one(op.s1h[xx + 1]));
+  const bool o2 = __all_sync(0xffffffffu, is_one(op.s2n[yy]) && is_one(op.s2h[yy]) && is_one(op.s2h[yy + 1]));
+  const bool o3 = __all_sync(0xffffffffu, is_one(op.s3n[zz]) && is_one(op.s3h[zz]) && is_one(op.s3h[zz + 1]));
+  switch ((o1 ? 1 : 0) | (o2 ? 2 : 0) | (o3 ? 4 : 0)) {
+    case 7: matvec_rows<true, true, true>(op, x, y, nrhs, N, g, in, xx, yy, zz); break;
+    case 6: matvec_rows<false, true, true>(op, x, y, nrhs, N, g, in, xx, yy, zz); break;
+    case 5: matvec_rows<true, false, true>(op, x, y, nrhs, N, g, in, xx, yy, zz); break;
+    case 3: matvec_rows<true, true, false>(op, x, y, nrhs, N, g, in, xx, yy, zz); break;
+    case 4: matvec_rows<false, false, true>(op, x, y, nrhs, N, g, in, xx, yy, zz); break;
+    case 2: matvec_rows<false, true, false>(op, x, y, nrhs, N, g, in, xx, yy, zz); break;
+    case 1: matvec_rows<true, false, false>(op, x, y, nrhs, N, g, in, xx, yy, zz); break;
+    default: matvec_rows<false, false, false>(op, x, y, nrhs, N, g, in, xx, yy, zz);
   }
 }
 
@@ -74,7 +194,16 @@ static int grid_for(int64_t n, int threads) {
 }
 
 void launch_matvec(const BoxOp& op, const double2* x, double2* y, int nrhs, int64_t N, cudaStream_t st) {
-  k_matvec<<<grid_for(N, 256), 256, 0, st>>>(op, x, y, nrhs, N);
+  k_matvec<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(op, x, y, nrhs, N);
+}
+
+// 1 / c^2 once per handle: every row of every operator divides by c^2
+__global__ void k_inverse_square(double* c, int64_t N) {
+  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < N; g += (int64_t)gridDim.x * blockDim.x)
+    c[g] = 1.0 / (c[g] * c[g]);
+}
+void launch_inverse_square(double* c, int64_t N, cudaStream_t st) {
+  k_inverse_square<<<grid_for(N, 256), 256, 0, st>>>(c, N);
 }
 void launch_scale_rhs(const BoxOp& op, const double2* f, double2* b, int nrhs, int64_t N, cudaStream_t st) {
   k_scale_rhs<<<grid_for(N, 256), 256, 0, st>>>(op, f, b, nrhs, N);

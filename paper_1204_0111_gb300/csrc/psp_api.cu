@@ -278,7 +278,7 @@ struct psp_ctx_s {
   std::vector<DevBuf> shape_bufs;
   DevBuf d_shapes, d_panel_shape;
   // operators
-  DevBuf d_c, d_gtab, d_ptab, d_boxops;
+  DevBuf d_ic2, d_gtab, d_ptab, d_boxops;
   BoxOp opA{}, opJ{};
   const double2 *s1n = nullptr, *s2n = nullptr, *s3hi = nullptr;
   // factors
@@ -1686,8 +1686,10 @@ static void build_problem(psp_ctx_s* X, const double* c, cudaStream_t st) {
   const int nx = X->nx, ny = X->ny, nz = X->nz;
   X->N = (int64_t)nx * ny * nz;
   // wave speed (host or device input)
-  X->d_c.alloc(X->N * sizeof(double));
-  PSP_CK(cudaMemcpyAsync(X->d_c.p, c, X->N * sizeof(double), cudaMemcpyDefault, st));
+  X->d_ic2.alloc(X->N * sizeof(double));
+  PSP_CK(cudaMemcpyAsync(X->d_ic2.p, c, X->N * sizeof(double), cudaMemcpyDefault, st));
+  launch_inverse_square(X->d_ic2.as<double>(), X->N, st);
+  PSP_CK(cudaGetLastError());
 
   // global stretch tables: s1n, 1/s1h, s2n, 1/s2h, s3n, 1/s3h
   const bool f[6] = {bool(X->faces & 1), bool(X->faces & 2), bool(X->faces & 4),
@@ -1851,7 +1853,7 @@ static void build_problem(psp_ctx_s* X, const double* c, cudaStream_t st) {
     op.nx = nx; op.ny = ny; op.nz = bz;
     op.inv_h2 = 1.0 / (X->h * X->h);
     op.k2num = k2num;
-    op.c = X->d_c.as<double>();
+    op.ic2 = X->d_ic2.as<double>();
     op.cplane = cpl;
     op.s1n = G + goff[0]; op.s1h = G + goff[1];
     op.s2n = G + goff[2]; op.s2h = G + goff[3];

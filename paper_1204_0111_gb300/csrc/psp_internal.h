@@ -82,7 +82,7 @@ struct BoxOp {
   int nx, ny, nz;
   double inv_h2;
   double2 k2num;            // omega^2 (A) or (omega + i alpha)^2 (J)
-  const double* c;          // global wave speed, nx*ny*nz_global
+  const double* ic2;        // 1 / c^2 of the global wave speed, nx*ny*nz_global
   const int32_t* cplane;    // box plane -> global plane whose c is used
   const double2* s1n;
   const double2* s1h;
@@ -172,6 +172,7 @@ struct ColTask {   // a chunk of columns / rows of one front
 // Launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------
 void launch_matvec(const BoxOp& op, const double2* x, double2* y, int nrhs, int64_t N, cudaStream_t st);
+void launch_inverse_square(double* c, int64_t N, cudaStream_t st);   // c := 1 / c^2
 void launch_scale_rhs(const BoxOp& op, const double2* f, double2* b, int nrhs, int64_t N, cudaStream_t st);
 
 template <typename T>
