@@ -122,8 +122,8 @@ typedef struct {
                           most 8 (the task's vector is staged through shared memory in chunks) */
   int solve_rhs_group; /* psp_solve: most right-hand sides per GMRES run; <= 0: as many as fit the free
                           device memory (single-problem handles) */
-  int sweep_min_rows;   /* sweep schedule: fewest rows (up) / columns (down) of a front per task, 8 .. 64;
-                           <= 0 selects the default (8).  Each task gathers its front's vector for every
+  int sweep_min_rows;   /* sweep schedule: fewest rows (up) / columns (down) of a front per task, 2 .. 64;
+                           <= 0 selects the default (4).  Each task gathers its front's vector for every
                            right-hand side, so with many right-hand sides wider tasks gather less */
   int test_sweep_stall; /* tests only: 1 makes one dependency of the persistent sweep impossible to
                            meet, so its bounded wait (about 2 s) gives up; psp_solve then returns
@@ -359,7 +359,7 @@ psp_status psp_stats(psp_handle h, psp_kernel_stat* out, int capacity, int* coun
  * times psp_apply with nrhs right-hand sides (per problem of a batch) under candidate schedules
  * and keeps the fastest: the tasks a tree level is split into (152 .. 2432), the resident CTAs per
  * SM (2, 3, 4, 6, 8), the cap on rows / columns per task (64 .. 256), the floor on rows per task
- * (8 .. 64), the queue tasks a CTA holds ahead (1, 2) and, for nrhs > 1, the right-hand sides per
+ * (4 .. 64), the queue tasks a CTA holds ahead (1, 2) and, for nrhs > 1, the right-hand sides per
  * CTA pass (1 .. 8).  It searches one
  * coordinate at a time, starting from the handle's current schedule, timing `reps` applications
  * (CUDA events on `stream`) per candidate after one untimed one.  Results do not change beyond

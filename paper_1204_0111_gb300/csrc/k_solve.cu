@@ -703,7 +703,7 @@ __device__ __forceinline__ void schedule(TaskSlot<T>* slots, const SweepArgs<T>&
       const int4* rows = sl.st.rows + sl.fr.row_off;
       const int32_t* sel = sl.st.sel + sl.fr.sel_off;
       if (lane == 0) {
-        int tl = 3;
+        int tl = 1;
         while ((1 << tl) < r1 - r0 && (1 << tl) < kComputeThreads) ++tl;
         sl.tr_log = tl;
         int sp = 1;

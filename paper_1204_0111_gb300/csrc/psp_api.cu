@@ -338,7 +338,7 @@ struct psp_ctx_s {
   bool use_tc = true;
   bool diag_fp64 = false;   // complex64: diagonal blocks factored and applied in complex128
   int tc_min_dim = 64;
-  int sweep_level_tasks = 608, sweep_ctas_per_sm = 8, sweep_rhs_group = 0, solve_rhs_group = 0, sweep_min_rows = 8;
+  int sweep_level_tasks = 304, sweep_ctas_per_sm = 8, sweep_rhs_group = 0, solve_rhs_group = 0, sweep_min_rows = 4;
   int sweep_max_rows = 256;
   int sweep_claim_ahead = 1;   // tasks a sweep CTA holds besides the one it runs
   int gmres_basis = 0;   // 0 auto, 1 keep z_j, 2 V only
@@ -1296,7 +1296,7 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
       // its front's vector for every right-hand side, so narrow tasks over wide fronts gather much and
       // stream little, and at the bottom of the tree, where tasks far outnumber CTAs, one task per
       // front gathers once)
-      const int rmin = std::max(8, std::min(64, X->sweep_min_rows));
+      const int rmin = std::max(2, std::min(64, X->sweep_min_rows));
       int R = X->sweep_max_rows;
       while (R > rmin && rows / R < X->sweep_level_tasks) R >>= 1;
       int Cc = X->sweep_max_rows;
@@ -2346,7 +2346,9 @@ static void init_options(psp_ctx_s* X, const psp_options& o) {
   X->sweep_level_tasks = o.sweep_level_tasks > 0 ? o.sweep_level_tasks : 304;
   X->sweep_ctas_per_sm = o.sweep_ctas_per_sm > 0 ? o.sweep_ctas_per_sm : 8;
   X->sweep_rhs_group = o.sweep_rhs_group > 0 ? o.sweep_rhs_group : 0;
-  X->sweep_min_rows = o.sweep_min_rows > 0 ? o.sweep_min_rows : 8;
+  // 4 against 8 rows: top levels of one or two fronts still have a task for every SM (100^3 lens complex128 33.9 / 35.7 ms,
+  // complex64 11.5 / 11.7 ms, the waveguide's 48^3 solve with four columns 193 / 213 ms; 2 rows: 35.0, 12.0, 185)
+  X->sweep_min_rows = o.sweep_min_rows > 0 ? o.sweep_min_rows : 4;
   X->sweep_max_rows = o.sweep_max_rows > 0 ? std::min(256, std::max(64, o.sweep_max_rows)) : 256;
   X->sweep_claim_ahead = o.sweep_claim_ahead > 0 ? o.sweep_claim_ahead : 1;
   X->solve_rhs_group = o.solve_rhs_group > 0 ? o.solve_rhs_group : 0;
@@ -2801,7 +2803,7 @@ psp_status psp_tune_sweep(psp_handle X, int nrhs, int reps, void* stream, psp_sw
     if (nrhs > 1)
       for (int rg : {1, 2, 4, 8})
         if (rg <= nrhs && rg != best.rg) consider({best.lt, best.cps, rg, best.mr, best.xr, best.ca});
-    for (int mr : {8, 16, 32, 64})
+    for (int mr : {4, 8, 16, 32, 64})
       if (mr != best.mr) consider({best.lt, best.cps, best.rg, mr, best.xr, best.ca});
     for (int ca : {1, 2})
       if (ca != best.ca) consider({best.lt, best.cps, best.rg, best.mr, best.xr, ca});

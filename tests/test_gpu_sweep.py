@@ -70,3 +70,19 @@ def test_consecutive_panels_of_different_depths(nz):
     out = P.apply(torch.from_numpy(r).cuda(), torch.empty((3, case.c.size), dtype=torch.complex128, device="cuda"))
     ref = O.apply(r)
     assert np.linalg.norm(out.cpu().numpy() - ref) < 1e-10 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("precision", ["c128", "c64"])
+@pytest.mark.parametrize("si", ["extended", "paper", "two"])
+@pytest.mark.parametrize("min_rows", [2, 4, 8, 64])
+def test_narrowest_tasks(min_rows, si, precision):
+    # tasks of 2 rows or columns: several lanes share a row, all warps share a block of columns
+    import torch
+    from oracle import sweep as osw
+    case = box(19, 14, 13)
+    O = osw.SweepingPreconditioner(case.oracle_problem(), case.depth, case.pad, case.leaf)
+    r = wl.random_vector(case.c.size, 3, seed=min_rows)
+    P = handle(case, precision=precision, selective_inversion=si, sweep_min_rows=min_rows, sweep_level_tasks=2432)
+    out = P.apply(torch.from_numpy(r).cuda(), torch.empty((3, case.c.size), dtype=torch.complex128, device="cuda"))
+    ref = O.apply(r)
+    assert np.linalg.norm(out.cpu().numpy() - ref) < (1e-10 if precision == "c128" else 1e-4) * np.linalg.norm(ref)
