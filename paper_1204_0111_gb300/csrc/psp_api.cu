@@ -8,10 +8,12 @@
 #include <cmath>
 #include <cstring>
 #include <functional>
+#include <future>
 #include <map>
 #include <memory>
 #include <new>
 #include <stdexcept>
+#include <system_error>
 #include <thread>
 #include <tuple>
 #include <type_traits>
@@ -551,16 +553,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   upload(d_upd_ptr, upd_ptr);
   upload(d_upd_tile, upd_tile);
 
-  // --- task lists ---
-  std::vector<FrontTask<T>> fronts;
-  std::vector<ColTask> ctasks;
-  std::vector<int> dlist;
-  std::vector<GemmTask<T>> gtasks;
-  std::vector<unsigned char*> packs;     // per front: base of its packed operands (tensor-core fronts)
-  std::vector<TcPackTask> ptasks;
-  std::vector<TcGemmTask> ttasks;
-  std::vector<OzPackTask> optasks;
-  std::vector<OzGemmTask> otasks;
+  // --- task lists, one set per group of fronts ---
   enum Kind { ASSEMBLE, DIAG, PRIGHT, PLEFT, GEMM, COPY, TCGEMM, TCPACK, SCALE, RSOLVE, OZPACK, OZGEMM };
   struct Launch {
     Kind kind;
@@ -571,27 +564,34 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
     double flops = 0, bytes = 0;
     double extra = 0;   // selective-inversion flops (not part of the algorithmic count)
   };
-  std::vector<Launch> launches;
-  const double es = sizeof(T);
-  // work of the gemm tasks [g0, end): algorithmic flops, selective-inversion flops, bytes
-  auto gemm_work = [&](int64_t g0, double& fl, double& ex, double& by) {
-    fl = 0;
-    ex = 0;
-    by = 0;
-    for (size_t i = g0; i < gtasks.size(); ++i) {
-      (gtasks[i].flags & GF_SI ? ex : fl) += 8.0 * gemm_cmacs(gtasks[i]);
-      by += es * ((double)gtasks[i].m * gtasks[i].k + (double)gtasks[i].n * gtasks[i].k + 2.0 * gtasks[i].m * gtasks[i].n);
+  struct Tasks {
+    std::vector<FrontTask<T>> fronts;
+    std::vector<ColTask> ctasks;
+    std::vector<int> dlist;
+    std::vector<GemmTask<T>> gtasks;
+    std::vector<unsigned char*> packs;   // per front: base of its packed operands (tensor-core fronts)
+    std::vector<TcPackTask> ptasks;
+    std::vector<TcGemmTask> ttasks;
+    std::vector<OzPackTask> optasks;
+    std::vector<OzGemmTask> otasks;
+    std::vector<Launch> launches;
+    void clear() {
+      fronts.clear();
+      ctasks.clear();
+      dlist.clear();
+      gtasks.clear();
+      packs.clear();
+      ptasks.clear();
+      ttasks.clear();
+      optasks.clear();
+      otasks.clear();
+      launches.clear();
     }
   };
-
-  auto tiles_lower = [&](T* C, int ldc, int M, auto&& emit) {
-    for (int tj = 0; tj < M; tj += 64)
-      for (int ti = tj; ti < M; ti += 64) emit(C, ldc, ti, tj, std::min(64, M - ti), std::min(64, M - tj));
-  };
-
-  // Each group's tasks are uploaded and its launches enqueued as soon as the group is planned, so
-  // the host plans the next group while the device factors this one.  Task arrays go to
-  // stream-ordered device chunks, one per group and array, freed after the final synchronisation.
+  const double es = sizeof(T);
+  // A worker thread plans the next group's tasks while this thread uploads the planned one's and enqueues its launches, and the
+  // device factors the ones before.  Task arrays go to stream-ordered device chunks, one per group and array, freed
+  // after the final synchronisation.
   int* status = X->d_status.as<int>();
   // status: [0] 1 + front of a zero pivot, [1] tensor-core wait gave up, [2] sweep wait gave up (sticky),
   // [4..5] ~bits of the smallest |pivot| (0: none yet)
@@ -618,73 +618,85 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       }
     }
   } chunk_guard{chunks, st, up.s, chunk_alloc};
-  // copies v[done, size) to a new device chunk (the copy from pageable memory is staged before the
-  // call returns, so the vector may grow afterwards); returns the chunk and advances done
-  auto upload_tail = [&](const auto& v, size_t& done) {
+  // copies v to a new device chunk (the copy from pageable memory is staged before the call returns)
+  auto upload_list = [&](const auto& v) {
     using E = typename std::decay_t<decltype(v)>::value_type;
-    const size_t n = v.size() - done;
     E* d = nullptr;
-    if (n > 0) {
-      if (chunk_alloc) d = static_cast<E*>(dev_alloc(n * sizeof(E), chunk_alloc));
-      else PSP_CK(cudaMallocAsync(reinterpret_cast<void**>(&d), n * sizeof(E), up.s));
+    if (!v.empty()) {
+      if (chunk_alloc) d = static_cast<E*>(dev_alloc(v.size() * sizeof(E), chunk_alloc));
+      else PSP_CK(cudaMallocAsync(reinterpret_cast<void**>(&d), v.size() * sizeof(E), up.s));
       chunks.push_back(d);
-      PSP_CK(cudaMemcpyAsync(d, v.data() + done, n * sizeof(E), cudaMemcpyHostToDevice, up.s));
+      PSP_CK(cudaMemcpyAsync(d, v.data(), v.size() * sizeof(E), cudaMemcpyHostToDevice, up.s));
     }
     return d;
   };
-  size_t up_f = 0, up_c = 0, up_d = 0, up_g = 0, up_p = 0, up_t = 0, up_op = 0, up_o = 0;
-  double plan_ms = 0, enqueue_ms = 0;
-  auto enqueue_group = [&](size_t lb) {
-    const size_t f0 = up_f, c0 = up_c, d0 = up_d, g0 = up_g, p0 = up_p, t0 = up_t, op0 = up_op, o0 = up_o;
-    const FrontTask<T>* F = upload_tail(fronts, up_f);
-    const ColTask* CT = upload_tail(ctasks, up_c);
-    const int* DL = upload_tail(dlist, up_d);
-    const GemmTask<T>* GT = upload_tail(gtasks, up_g);
-    const TcPackTask* PT = upload_tail(ptasks, up_p);
-    const TcGemmTask* TT = upload_tail(ttasks, up_t);
-    const OzPackTask* OP = upload_tail(optasks, up_op);
-    const OzGemmTask* OT = upload_tail(otasks, up_o);
+  double enqueue_ms = 0, waited_ms = 0;
+  auto enqueue_group = [&](const Tasks& tk) {
+    const FrontTask<T>* F = upload_list(tk.fronts);
+    const ColTask* CT = upload_list(tk.ctasks);
+    const int* DL = upload_list(tk.dlist);
+    const GemmTask<T>* GT = upload_list(tk.gtasks);
+    const TcPackTask* PT = upload_list(tk.ptasks);
+    const TcGemmTask* TT = upload_list(tk.ttasks);
+    const OzPackTask* OP = upload_list(tk.optasks);
+    const OzGemmTask* OT = upload_list(tk.otasks);
     up.join(st);   // the group's kernels after its task arrays
-    up_f = fronts.size();
-    up_c = ctasks.size();
-    up_d = dlist.size();
-    up_g = gtasks.size();
-    up_p = ptasks.size();
-    up_t = ttasks.size();
-    up_op = optasks.size();
-    up_o = otasks.size();
-    for (size_t li = lb; li < launches.size(); ++li) {
-      const Launch& l = launches[li];
+    for (const Launch& l : tk.launches) {
       if (l.count <= 0) continue;
       const bool wide = X->prec == PSP_PREC_C64 && X->diag_fp64;
-      const FrontTask<T>* Fl = F + (l.front_off - (int64_t)f0);
+      const FrontTask<T>* Fl = F + l.front_off;
       X->stats.run(names[l.kind], st, 1, l.flops, l.bytes, [&] {
         switch (l.kind) {
           case ASSEMBLE:
-            launch_assemble_impl<T>(Fl, CT + (l.off - (int64_t)c0), l.count, X->d_shapes.as<ShapeDev>(),
+            launch_assemble_impl<T>(Fl, CT + l.off, l.count, X->d_shapes.as<ShapeDev>(),
                                     X->d_boxops.as<BoxOp>(), d_upd_ptr.as<T*>(), d_upd_tile.as<int32_t>(),
                                     X->d_panel_shape.as<int32_t>(), st);
             break;
-          case DIAG: launch_diag_ldlt<T>(Fl, DL + (l.off - (int64_t)d0), l.count, l.kb, tiny, status, wide, st); break;
-          case PRIGHT: launch_panel_right<T>(Fl, CT + (l.off - (int64_t)c0), l.count, l.kb, wide, st); break;
-          case PLEFT: launch_panel_left<T>(Fl, CT + (l.off - (int64_t)c0), l.count, l.kb, wide, st); break;
-          case GEMM: launch_gemm<T>(GT + (l.off - (int64_t)g0), l.count, st); break;
-          case COPY: launch_copy_linv<T>(Fl, CT + (l.off - (int64_t)c0), l.count, st); break;
-          case TCGEMM: launch_tc_gemm(TT + (l.off - (int64_t)t0), l.count, status, st); break;
-          case OZPACK: launch_oz_pack(OP + (l.off - (int64_t)op0), l.count, st); break;
-          case OZGEMM: launch_oz_gemm(OT + (l.off - (int64_t)o0), l.count, status, st); break;
-          case TCPACK: launch_tc_pack(PT + (l.off - (int64_t)p0), l.count, st); break;
-          case SCALE: launch_scale_zd<T>(Fl, CT + (l.off - (int64_t)c0), l.count, st); break;
-          case RSOLVE: launch_panel_rsolve<T>(Fl, CT + (l.off - (int64_t)c0), l.count, l.kb, wide, st); break;
+          case DIAG: launch_diag_ldlt<T>(Fl, DL + l.off, l.count, l.kb, tiny, status, wide, st); break;
+          case PRIGHT: launch_panel_right<T>(Fl, CT + l.off, l.count, l.kb, wide, st); break;
+          case PLEFT: launch_panel_left<T>(Fl, CT + l.off, l.count, l.kb, wide, st); break;
+          case GEMM: launch_gemm<T>(GT + l.off, l.count, st); break;
+          case COPY: launch_copy_linv<T>(Fl, CT + l.off, l.count, st); break;
+          case TCGEMM: launch_tc_gemm(TT + l.off, l.count, status, st); break;
+          case OZPACK: launch_oz_pack(OP + l.off, l.count, st); break;
+          case OZGEMM: launch_oz_gemm(OT + l.off, l.count, status, st); break;
+          case TCPACK: launch_tc_pack(PT + l.off, l.count, st); break;
+          case SCALE: launch_scale_zd<T>(Fl, CT + l.off, l.count, st); break;
+          case RSOLVE: launch_panel_rsolve<T>(Fl, CT + l.off, l.count, l.kb, wide, st); break;
         }
       }, true, l.extra);
     }
     PSP_CK(cudaGetLastError());
   };
 
-  for (const auto& grp : groups) {
-    const size_t lb = launches.size();
-    const int64_t f0 = (int64_t)fronts.size();
+  auto plan_group = [&](const std::vector<std::pair<int, int>>& grp, Tasks& tk) {
+    tk.clear();
+    auto& fronts = tk.fronts;
+    auto& ctasks = tk.ctasks;
+    auto& dlist = tk.dlist;
+    auto& gtasks = tk.gtasks;
+    auto& packs = tk.packs;
+    auto& ptasks = tk.ptasks;
+    auto& ttasks = tk.ttasks;
+    auto& optasks = tk.optasks;
+    auto& otasks = tk.otasks;
+    auto& launches = tk.launches;
+    // work of the gemm tasks [g0, end): algorithmic flops, selective-inversion flops, bytes
+    auto gemm_work = [&](int64_t g0, double& fl, double& ex, double& by) {
+      fl = 0;
+      ex = 0;
+      by = 0;
+      for (size_t i = g0; i < gtasks.size(); ++i) {
+        (gtasks[i].flags & GF_SI ? ex : fl) += 8.0 * gemm_cmacs(gtasks[i]);
+        by += es * ((double)gtasks[i].m * gtasks[i].k + (double)gtasks[i].n * gtasks[i].k + 2.0 * gtasks[i].m * gtasks[i].n);
+      }
+    };
+
+    auto tiles_lower = [&](T* C, int ldc, int M, auto&& emit) {
+      for (int tj = 0; tj < M; tj += 64)
+        for (int ti = tj; ti < M; ti += 64) emit(C, ldc, ti, tj, std::min(64, M - ti), std::min(64, M - tj));
+    };
+    const int64_t f0 = 0;
     int smax = 0;
     int64_t toff = 0;
     for (auto [p, sn] : grp) {
@@ -1237,14 +1249,38 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         launches.push_back(lt);
       }
     }
-    plan_ms += ms_since(tp);
-    tp = std::chrono::steady_clock::now();
-    enqueue_group(lb);
-    enqueue_ms += ms_since(tp);
-    tp = std::chrono::steady_clock::now();
+  };
+  {
+    Tasks lists[2];
+    std::future<void> planned;
+    auto start = [&](size_t i) {
+      auto plan = [&, i] { plan_group(groups[i], lists[i & 1]); };
+      try {
+        planned = std::async(std::launch::async, plan);
+      } catch (const std::system_error&) {   // no thread to be had: planned when it is asked for
+        planned = std::async(std::launch::deferred, plan);
+      }
+    };
+    // declared after the lists: on an error the worker ends (the future's destructor waits) before they go
+    struct Wait {
+      std::future<void>& f;
+      ~Wait() {
+        if (f.valid()) f.wait();
+      }
+    } wait{planned};
+    if (!groups.empty()) start(0);
+    for (size_t i = 0; i < groups.size(); ++i) {
+      tp = std::chrono::steady_clock::now();
+      planned.get();
+      if (i + 1 < groups.size()) start(i + 1);
+      waited_ms += ms_since(tp);
+      tp = std::chrono::steady_clock::now();
+      enqueue_group(lists[i & 1]);
+      enqueue_ms += ms_since(tp);
+    }
   }
 
-  X->stats.host("plan_tasks", plan_ms);
+  X->stats.host("wait_plan_tasks", waited_ms);
   X->stats.host("enqueue_setup", enqueue_ms);
   while_device_runs();
   tp = std::chrono::steady_clock::now();
