@@ -121,9 +121,11 @@ __global__ void __launch_bounds__(256) k_oz_pack(const OzPackTask* __restrict__ 
     if (rg < tk.R && k < tk.K) {
       if (tk.mode == TC_PACK_PLAIN) {
         v = tk.src[(int64_t)k * tk.ld + rg];
-        if (tk.dinv) v = cmul(v, tk.dinv[k]);
+        if (tk.scale) v = cmul(v, tk.scale[(int64_t)k * tk.lds]);
       } else if (tk.mode == TC_PACK_UNIT_LOWER) {   // T[rg, k], unit lower
         v = k == rg ? make_double2(1.0, 0.0) : (k < rg ? tk.src[(int64_t)k * tk.ld + rg] : v);
+      } else if (tk.mode == TC_PACK_TRANSPOSED) {   // X[k, rg]
+        v = tk.src[(int64_t)rg * tk.ld + k];
       } else {                                      // T[k, rg], unit lower (transposed read)
         v = k == rg ? make_double2(1.0, 0.0) : (k > rg ? tk.src[(int64_t)rg * tk.ld + k] : v);
       }

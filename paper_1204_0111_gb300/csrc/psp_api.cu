@@ -396,6 +396,11 @@ static double ms_since(std::chrono::steady_clock::time_point t0) {
 }
 
 constexpr int kOzMinDim = 16;   // complex128: fewest s and u of a front on the tensor cores
+// complex128: fronts of at least this many rows S factor F_TL and build inv(L_TL) in blocks of 128 columns: inside a block by
+// steps of 32 on the FP64 units, the rest of F_TL and of W once per block, with k = 128, on the tensor cores (80^3 lens
+// setup: k_gemm 75.7 -> 32.7 ms, the tensor-core products and their operands 93.8 -> 98.8 ms; half of k_gemm's work was the
+// root of each panel, 960 rows).  Below two blocks there is no second one to update
+constexpr int kOzBlock = 128, kOzBlockMin = 256;
 
 // `while_device_runs` is host work done after the last launch is enqueued, before waiting for them.
 template <typename T>
@@ -451,6 +456,13 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
                 oz_bytes(s_, s_, true) + oz_exps(s_, s_, true);
     return pad16(cdiv_i(b, (int64_t)sizeof(T)) + 64);
   };
+  auto in_blocks = [&](int64_t s_) { return oz_ok && s_ >= kOzBlockMin; };
+  // packed operands of one block of 128 columns: L D and L of the rows below (A), L again and W's block row (B)
+  auto block_elems = [&](int64_t s_) {
+    const int64_t b = 2 * (oz_bytes(s_, kOzBlock, false) + oz_exps(s_, kOzBlock, false)) +
+                      2 * (oz_bytes(s_, kOzBlock, true) + oz_exps(s_, kOzBlock, true));
+    return pad16(cdiv_i(b, (int64_t)sizeof(T)) + 64);
+  };
   auto nrb = [](int64_t r) { return (r + 127) / 128; };
   auto nkb16 = [](int64_t k) { return (k + 15) / 16; };
   auto packed_elems = [&](int64_t s_, int64_t u_) {   // F_BL, Z D^-1, Z (u x s) and two inv(L) (s x s)
@@ -458,7 +470,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   };
   auto front_temp = [&](int64_t s_, int64_t u_) {     // W (s x s), Z (u x s), Z D^-1 or packed operands,
     if (si == PSP_SI_NONE) return (int64_t)0;         // the second inverse under construction (s x s)
-    return pad16(s_ * s_) + pad16(u_ * s_) + (si == PSP_SI_TWO ? pad16(s_ * s_) : 0) +
+    return pad16(s_ * s_) + pad16(u_ * s_) + (si == PSP_SI_TWO ? pad16(s_ * s_) : 0) + (in_blocks(s_) ? block_elems(s_) : 0) +
            (use_tc(s_, u_) ? packed_elems(s_, u_)
             : use_oz(s_, u_) ? oz_elems(s_, u_)
                              : si == PSP_SI_EXTENDED ? pad16(u_ * s_) : 0);
@@ -570,6 +582,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
     std::vector<int> dlist;
     std::vector<GemmTask<T>> gtasks;
     std::vector<unsigned char*> packs;   // per front: base of its packed operands (tensor-core fronts)
+    std::vector<unsigned char*> blocks;  // per front: base of a block's packed operands (fronts factored in blocks of 128)
     std::vector<TcPackTask> ptasks;
     std::vector<TcGemmTask> ttasks;
     std::vector<OzPackTask> optasks;
@@ -581,6 +594,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       dlist.clear();
       gtasks.clear();
       packs.clear();
+      blocks.clear();
       ptasks.clear();
       ttasks.clear();
       optasks.clear();
@@ -676,6 +690,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
     auto& dlist = tk.dlist;
     auto& gtasks = tk.gtasks;
     auto& packs = tk.packs;
+    auto& blocks = tk.blocks;
     auto& ptasks = tk.ptasks;
     auto& ttasks = tk.ttasks;
     auto& optasks = tk.optasks;
@@ -714,6 +729,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       ft.W = ft.Z = ft.ZD = ft.W2 = nullptr;
       ft.ldzd = ft.u;
       packs.push_back(nullptr);
+      blocks.push_back(nullptr);
       if (si != PSP_SI_NONE) {
         ft.W = tbase + toff;
         toff += pad16((int64_t)ft.s * ft.s);
@@ -736,6 +752,10 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         if (si == PSP_SI_TWO) {
           ft.W2 = tbase + toff;
           toff += pad16((int64_t)ft.s * ft.s);
+        }
+        if (in_blocks(ft.s)) {
+          blocks.back() = reinterpret_cast<unsigned char*>(tbase + toff);
+          toff += block_elems(ft.s);
         }
       }
       fronts.push_back(ft);
@@ -772,6 +792,52 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       }
       launches.push_back(la);
     }
+    // packs an operand (R rows, K columns; columns times scale[k lds_]) of the complex128 tensor-core products; returns its bytes
+    auto oz_pack = [&](const T* src, const T* scale, int64_t lds_, unsigned char* dst, int64_t ld_, int64_t R, int64_t K, int mode, bool b) {
+      const int64_t nkb = cdiv_i(K, oz.k), nkc = cdiv_i(K, oz.kc), rows = b ? oz.tile_n : oz.tile_m;
+      int* exps = reinterpret_cast<int*>(dst + oz_bytes(R, K, b));
+      for (int64_t r0 = 0; r0 < R; r0 += oz.tile_m)
+        for (int64_t kc = 0; kc < nkc; ++kc) {
+          OzPackTask t{};
+          t.src = reinterpret_cast<const double2*>(src);
+          t.scale = reinterpret_cast<const double2*>(scale);
+          t.lds = (int)lds_;
+          t.dst = dst + (r0 / rows * nkb + kc * (oz.kc / oz.k)) * (b ? oz.b_block : oz.a_block);
+          t.exps = exps + (r0 / rows * nkc + kc) * rows;
+          t.sub_stride = nkb * oz.b_block;
+          t.exp_stride = nkc * oz.tile_n;
+          t.ld = (int)ld_;
+          t.r0 = (int)r0;
+          t.k0 = (int)(kc * oz.kc);
+          t.R = (int)R;
+          t.K = (int)K;
+          t.mode = mode;
+          t.rows_b = b;
+          optasks.push_back(t);
+        }
+      const double e = (double)R * K;
+      return e * (16.0 + (double)(b ? oz.b_block / (oz.tile_n * oz.k) : oz.a_block / (oz.tile_m * oz.k)));
+    };
+    // tiles of C (R x N) = +-A B^T with k in [klo(col), khi(col))
+    auto oz_tile = [&](unsigned char* A, int64_t RA, unsigned char* B, int64_t RB, int64_t K, int ti, int tj, T* C, int ldc,
+                       int64_t k0, int64_t k1, int doff, int flags) {
+      const int64_t nkb = cdiv_i(K, oz.k), nkc = cdiv_i(K, oz.kc);
+      OzGemmTask t{};
+      t.A = A + ti / oz.tile_m * nkb * oz.a_block;
+      t.B = B + tj / oz.tile_n * nkb * oz.b_block;
+      t.ea = reinterpret_cast<const int*>(A + oz_bytes(RA, K, false)) + ti / oz.tile_m * nkc * oz.tile_m;
+      t.eb = reinterpret_cast<const int*>(B + oz_bytes(RB, K, true)) + tj / oz.tile_n * nkc * oz.tile_n;
+      t.C = reinterpret_cast<double2*>(C);
+      t.ldc = ldc;
+      t.m = (int)std::min<int64_t>(oz.tile_m, RA - ti);
+      t.n = (int)std::min<int64_t>(oz.tile_n, RB - tj);
+      t.kb0 = (int)(k0 / oz.k);
+      t.nkb = (int)(cdiv_i(k1, oz.k) - k0 / oz.k);
+      t.doff = doff;
+      t.flags = flags;
+      otasks.push_back(t);
+    };
+    constexpr int kAll = 1 << 30;   // no triangle mask
     // blocked LDL^T of F_TL with the inverse of L_TL built alongside in W; without selective
     // inversion the blocked factorisation runs over all s + u rows, so F_BL becomes L_BL directly
     const int nblk = (smax + nb - 1) / nb;
@@ -825,8 +891,12 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         const int ld = ft.s + ft.u;
         const int bs = std::min(nb, ft.s - o);
         const int t0 = o + nb;  // first row/col of the trailing block
+        // fronts factored in blocks of 128: only the block's own columns of F_TL and rows of W now
+        const int cmax = blocks[f0 + f] ? std::min(ft.s, (o / kOzBlock + 1) * kOzBlock) : ft.s;
         // F_TL trailing update: F(r, c) -= L(r, kb) D_kb L(c, kb)^T, lower
         tiles_lower(ft.G, ld, ft.s - t0, [&](T*, int, int ti, int tj, int mm, int nn) {
+          if (t0 + tj >= cmax) return;
+          nn = std::min(nn, cmax - t0 - tj);
           GemmTask<T> g{};
           g.C = ft.G + (int64_t)(t0 + tj) * ld + (t0 + ti);
           g.ldc = ld;
@@ -864,7 +934,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         // W(r, c) -= L(r, kb) W(kb, c) for rows below the block, columns up to its end
         const int cend = o + bs;
         for (int tj = 0; tj < cend; tj += 64)
-          for (int ti = t0; ti < ft.s; ti += 64) {
+          for (int ti = t0; ti < cmax; ti += 64) {
             GemmTask<T> g{};
             g.C = ft.W + (int64_t)tj * ft.s + ti;
             g.ldc = ft.s;
@@ -872,7 +942,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
             g.lda = ld;
             g.B = ft.W + (int64_t)tj * ft.s + o;  // B(n, k) = W[o + k, tj + n]
             g.ldb = ft.s;
-            g.m = std::min(64, ft.s - ti);
+            g.m = std::min(64, cmax - ti);
             g.n = std::min(64, cend - tj);
             g.k = bs;
             g.kg0 = o;              // W is unit lower: B(n, k) = W[o + k, tj + n] vanishes for o + k < tj + n
@@ -884,6 +954,43 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       Launch lg{GEMM, f0, g0, (int)(gtasks.size() - g0), kb};
       gemm_work(g0, lg.flops, lg.extra, lg.bytes);
       launches.push_back(lg);
+      // the end of a block of 128 columns [b0, b1): F_TL(r, c) -= L(r, blk) D L(c, blk)^T for r >= c >= b1, and
+      // W(r, c) -= L(r, blk) W(blk, c) for r >= b1 > c
+      if ((o + nb) % kOzBlock == 0) {
+        const int b0 = o + nb - kOzBlock, b1 = o + nb;
+        Launch lp{OZPACK, f0, (int64_t)optasks.size(), 0, kb}, lt{OZGEMM, f0, (int64_t)otasks.size(), 0, kb};
+        for (int f : ord) {
+          const auto& ft = fronts[f0 + f];
+          if (!blocks[f0 + f] || ft.s <= b1) continue;
+          const int64_t ld = ft.s + ft.u, R = ft.s - b1;
+          unsigned char* LD = blocks[f0 + f];
+          unsigned char* LA = LD + oz_bytes(R, kOzBlock, false) + oz_exps(R, kOzBlock, false);
+          unsigned char* LB = LA + oz_bytes(R, kOzBlock, false) + oz_exps(R, kOzBlock, false);
+          unsigned char* WB = LB + oz_bytes(R, kOzBlock, true) + oz_exps(R, kOzBlock, true);
+          T* blk = ft.G + b0 * ld;
+          lp.bytes += oz_pack(blk + b1, blk + b0, ld + 1, LD, ld, R, kOzBlock, TC_PACK_PLAIN, false);
+          lp.bytes += oz_pack(blk + b1, nullptr, 0, LA, ld, R, kOzBlock, TC_PACK_PLAIN, false);
+          lp.bytes += oz_pack(blk + b1, nullptr, 0, LB, ld, R, kOzBlock, TC_PACK_PLAIN, true);
+          lp.bytes += oz_pack(ft.W + b0, nullptr, 0, WB, ft.s, b1, kOzBlock, TC_PACK_TRANSPOSED, true);
+          for (int tj = 0; tj < R; tj += oz.tile_n)
+            for (int ti = tj / oz.tile_m * oz.tile_m; ti < R; ti += oz.tile_m)
+              oz_tile(LD, R, LB, R, kOzBlock, ti, tj, ft.G + (b1 + tj) * ld + b1 + ti, (int)ld, 0, kOzBlock,
+                      ti > tj ? kAll : ti - tj, GF_NEG);
+          for (int tj = 0; tj < b1; tj += oz.tile_n)
+            for (int ti = 0; ti < R; ti += oz.tile_m)
+              oz_tile(LA, R, WB, b1, kOzBlock, ti, tj, ft.W + (int64_t)tj * ft.s + b1 + ti, ft.s, 0, kOzBlock, kAll, GF_NEG);
+          lt.flops += 8.0 * kOzBlock * R * (R + 1.0) / 2;
+          lt.extra += 8.0 * R * ((double)kOzBlock * b0 + kOzBlock * (kOzBlock + 1.0) / 2);
+        }
+        lp.count = (int)(optasks.size() - lp.off);
+        lt.count = (int)(otasks.size() - lt.off);
+        for (size_t i = lt.off; i < otasks.size(); ++i)
+          lt.bytes += (double)otasks[i].nkb * (oz.a_block + oz.b_block) + 32.0 * otasks[i].m * otasks[i].n;
+        if (lt.count > 0) {
+          launches.push_back(lp);
+          launches.push_back(lt);
+        }
+      }
     }
     // The two-inverse form: the second inverse X of L_TL row by row, X L_TL = I, by block columns from
     // the last: X(:, kb) := X(:, kb) L_kk^{-1}, then X(:, j) -= X(:, kb) L(kb, j) for the blocks j < kb
@@ -1149,50 +1256,6 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       if constexpr (std::is_same<T, double2>::value) {
         // complex128 fronts on the tensor cores.  Phase 0: F_BL (A) and inv(L) (B), Z = F_BL inv(L)^T.  Phase 1: Z D^-1 in
         // F_BL's place and Z (B), the Schur update; then (extended form) inv(L)^T in inv(L)'s place and M_BL.
-        auto oz_pack = [&](const T* src, const T* dinv, unsigned char* dst, int64_t ld_, int64_t R, int64_t K, int mode, bool b) {
-          const int64_t nkb = cdiv_i(K, oz.k), nkc = cdiv_i(K, oz.kc), rows = b ? oz.tile_n : oz.tile_m;
-          int* exps = reinterpret_cast<int*>(dst + oz_bytes(R, K, b));
-          for (int64_t r0 = 0; r0 < R; r0 += oz.tile_m)
-            for (int64_t kc = 0; kc < nkc; ++kc) {
-              OzPackTask t{};
-              t.src = src;
-              t.dinv = dinv;
-              t.dst = dst + (r0 / rows * nkb + kc * (oz.kc / oz.k)) * (b ? oz.b_block : oz.a_block);
-              t.exps = exps + (r0 / rows * nkc + kc) * rows;
-              t.sub_stride = nkb * oz.b_block;
-              t.exp_stride = nkc * oz.tile_n;
-              t.ld = (int)ld_;
-              t.r0 = (int)r0;
-              t.k0 = (int)(kc * oz.kc);
-              t.R = (int)R;
-              t.K = (int)K;
-              t.mode = mode;
-              t.rows_b = b;
-              optasks.push_back(t);
-            }
-          const double e = (double)R * K;
-          return e * (16.0 + (double)(b ? oz.b_block / (oz.tile_n * oz.k) : oz.a_block / (oz.tile_m * oz.k)));
-        };
-        // tiles of C (R x N) = +-A B^T with k in [klo(col), khi(col))
-        auto oz_tile = [&](unsigned char* A, int64_t RA, unsigned char* B, int64_t RB, int64_t K, int ti, int tj, T* C, int ldc,
-                           int64_t k0, int64_t k1, int doff, int flags) {
-          const int64_t nkb = cdiv_i(K, oz.k), nkc = cdiv_i(K, oz.kc);
-          OzGemmTask t{};
-          t.A = A + ti / oz.tile_m * nkb * oz.a_block;
-          t.B = B + tj / oz.tile_n * nkb * oz.b_block;
-          t.ea = reinterpret_cast<const int*>(A + oz_bytes(RA, K, false)) + ti / oz.tile_m * nkc * oz.tile_m;
-          t.eb = reinterpret_cast<const int*>(B + oz_bytes(RB, K, true)) + tj / oz.tile_n * nkc * oz.tile_n;
-          t.C = C;
-          t.ldc = ldc;
-          t.m = (int)std::min<int64_t>(oz.tile_m, RA - ti);
-          t.n = (int)std::min<int64_t>(oz.tile_n, RB - tj);
-          t.kb0 = (int)(k0 / oz.k);
-          t.nkb = (int)(cdiv_i(k1, oz.k) - k0 / oz.k);
-          t.doff = doff;
-          t.flags = flags;
-          otasks.push_back(t);
-        };
-        constexpr int kAll = 1 << 30;   // no triangle mask
         for (int step = 0; step < (phase == 0 ? 1 : si == PSP_SI_EXTENDED ? 2 : 1); ++step) {
           const int64_t op0 = (int64_t)optasks.size(), o0 = (int64_t)otasks.size();
           Launch lp{OZPACK, f0, op0, 0, -1}, lt{OZGEMM, f0, o0, 0, -1};
@@ -1205,23 +1268,23 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
             unsigned char* PB = PA + (oz_bytes(u_, s_, false) + oz_exps(u_, s_, false));
             unsigned char* PL = PB + (oz_bytes(u_, s_, true) + oz_exps(u_, s_, true));
             if (phase == 0) {
-              lp.bytes += oz_pack(ft.G + ft.s, nullptr, PA, ld, u_, s_, TC_PACK_PLAIN, false);
-              lp.bytes += oz_pack(ft.G, nullptr, PL, ld, s_, s_, TC_PACK_UNIT_LOWER, true);
+              lp.bytes += oz_pack(ft.G + ft.s, nullptr, 0, PA, ld, u_, s_, TC_PACK_PLAIN, false);
+              lp.bytes += oz_pack(ft.G, nullptr, 0, PL, ld, s_, s_, TC_PACK_UNIT_LOWER, true);
               for (int tj = 0; tj < ft.s; tj += oz.tile_n)
                 for (int ti = 0; ti < ft.u; ti += oz.tile_m)
                   oz_tile(PA, u_, PL, s_, s_, ti, tj, ft.Z + (int64_t)tj * ft.u + ti, ft.u, 0,
                           std::min<int64_t>(tj + oz.tile_n, s_), kAll, GF_BETA0);
               lt.flops += 8.0 * u_ * s_ * (s_ + 1.0) / 2;
             } else if (step == 0) {
-              lp.bytes += oz_pack(ft.Z, ft.dinv, PA, u_, u_, s_, TC_PACK_PLAIN, false);
-              lp.bytes += oz_pack(ft.Z, nullptr, PB, u_, u_, s_, TC_PACK_PLAIN, true);
+              lp.bytes += oz_pack(ft.Z, ft.dinv, 1, PA, u_, u_, s_, TC_PACK_PLAIN, false);
+              lp.bytes += oz_pack(ft.Z, nullptr, 0, PB, u_, u_, s_, TC_PACK_PLAIN, true);
               for (int tj = 0; tj < ft.u; tj += oz.tile_n)
                 for (int ti = tj / oz.tile_m * oz.tile_m; ti < ft.u; ti += oz.tile_m)
                   oz_tile(PA, u_, PB, u_, s_, ti, tj, ft.U + upd_index(std::max(ti, tj), tj, ft.u, 128) - std::max(0, tj - ti),
                           128, 0, s_, ti > tj ? kAll : ti - tj, GF_NEG);
               lt.flops += 8.0 * s_ * u_ * (u_ + 1.0) / 2;
             } else {
-              lp.bytes += oz_pack(ft.G, nullptr, PL, ld, s_, s_, TC_PACK_UNIT_LOWER_T, true);
+              lp.bytes += oz_pack(ft.G, nullptr, 0, PL, ld, s_, s_, TC_PACK_UNIT_LOWER_T, true);
               for (int tj = 0; tj < ft.s; tj += oz.tile_n)
                 for (int ti = 0; ti < ft.u; ti += oz.tile_m)
                   oz_tile(PA, u_, PL, s_, s_, ti, tj, ft.G + (int64_t)tj * ld + ft.s + ti, ld, tj, s_, kAll, GF_BETA0);

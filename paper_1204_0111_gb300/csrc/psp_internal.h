@@ -191,7 +191,7 @@ void launch_panel_rsolve(const FrontTask<T>* fronts, const ColTask* tasks, int n
 template <typename T>
 void launch_gemm(const GemmTask<T>* tasks, int ntasks, cudaStream_t st);
 // tensor-core path (complex64): operands packed once per front into TF32 planes, then tiles
-enum TcPackMode { TC_PACK_PLAIN = 0, TC_PACK_UNIT_LOWER = 1, TC_PACK_UNIT_LOWER_T = 2 };
+enum TcPackMode { TC_PACK_PLAIN = 0, TC_PACK_UNIT_LOWER = 1, TC_PACK_UNIT_LOWER_T = 2, TC_PACK_TRANSPOSED = 3 };
 struct TcPackTask {        // one 128-row x 16-k block of a packed operand
   const float2* src;       // column-major source, ld
   const float2* d;         // PLAIN only: divide column k by d[k * ldd] (nullptr: no scaling)
@@ -217,15 +217,14 @@ struct OzShape { int tile_m, tile_n, k, kc; int64_t a_block, b_block; };   // ti
 OzShape oz_shape();
 struct OzPackTask {        // 128 rows x 128 k of an operand
   const double2* src;      // column-major source, ld
-  const double2* dinv;     // PLAIN only: column k times dinv[k] (nullptr: no scaling)
+  const double2* scale;    // PLAIN only: column k times scale[k * lds] (nullptr: no scaling)
   unsigned char* dst;      // first block (16 k) of these rows; the following ones adjacent
   int* exps;               // row exponents of this block of k
   int64_t sub_stride;      // B operands: bytes between the blocks of 32 rows ...
   int64_t exp_stride;      // ... and entries between their exponents
-  int ld, r0, k0, R, K;    // first row / k, source extents (outside -> 0)
-  int mode;                // TcPackMode
+  int ld, lds, r0, k0, R, K;   // first row / k, source extents (outside -> 0)
+  int mode;                // TcPackMode (TRANSPOSED: X[k, r])
   int rows_b;              // 0: A operand (128-row blocks), 1: B operand (32-row blocks)
-  int pad_;
 };
 struct OzGemmTask {        // one 128 x 32 tile of C (+)= +-A B^T
   const unsigned char* A;  // block of 16 k number 0 of its 128 rows

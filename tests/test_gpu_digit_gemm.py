@@ -28,7 +28,7 @@ def box(nx, ny, D, high=1.0, leaf=64):
 
 # separators of nx D and ny D rows and structs of up to 2 (nx + ny) D: s and u just below, at and above 16, 32, 128 and 144
 @pytest.mark.parametrize("nx,ny,D,leaf", [(7, 5, 3, 16), (16, 16, 2, 16), (17, 15, 8, 64), (18, 16, 8, 64), (33, 32, 4, 64),
-                                          (43, 41, 3, 64), (36, 36, 4, 64), (19, 17, 16, 64)])
+                                          (43, 41, 3, 64), (36, 36, 4, 64), (19, 17, 16, 64), (30, 26, 16, 64)])
 @pytest.mark.parametrize("si", ["extended", "paper", "two"])
 def test_fronts_match_the_oracle_as_closely_as_fp64_products(nx, ny, D, leaf, si):
     from oracle import sweep as osw
