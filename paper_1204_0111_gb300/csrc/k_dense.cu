@@ -203,8 +203,11 @@ __global__ void __launch_bounds__(64) k_panel_rsolve(const FrontTask<T>* __restr
 // Complex products use three real multiplications (Gauss): with the pre-sums ar + ai and
 // br + bi staged in shared memory, t1 += ar br, t2 += ai bi, t3 += (ar + ai)(br + bi), and at the
 // end re = t1 - t2, im = t3 - t1 - t2.  Three FMAs per complex MAC instead of four.
+// The next chunk of k is read into registers while this one's products run, since two CTAs per SM at most hide
+// little of a read, and single precision takes 16 k per chunk (100^3 layered complex64 setup: 46.9 -> 41.2 ms; the
+// complex128 products are bound by the FP64 pipe, 32.7 -> 32.3 ms on the 80^3 lens).
 // ---------------------------------------------------------------------------
-constexpr int GT = 64, GK = 8;
+constexpr int GT = 64;
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_gemm(const GemmTask<T>* __restrict__ tasks) {
@@ -213,6 +216,7 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmTask<T>* __restrict__ ta
   // or columns with one 128-bit load); double precision: 65 (no bank conflicts in the staging)
   constexpr bool kSingle = sizeof(R) == 4;
   constexpr int GP = kSingle ? GT + 4 : GT + 1;
+  constexpr int GK = kSingle ? 16 : 8, PER = GT * GK / 256;   // k per chunk, operand entries per thread and chunk
   __shared__ __align__(16) R Ar[GK][GP], Ai[GK][GP], As[GK][GP];
   __shared__ __align__(16) R Br[GK][GP], Bi[GK][GP], Bs[GK][GP];
   const GemmTask<T> tk = tasks[blockIdx.x];
@@ -225,10 +229,23 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmTask<T>* __restrict__ ta
     for (int b = 0; b < 4; ++b) t1[a][b] = t2[a][b] = t3[a][b] = R(0);
 
   const bool bnn = tk.flags & GF_B_NN, lower = tk.flags & GF_C_LOWER;
-  for (int k0 = 0; k0 < tk.k; k0 += GK) {
-    // A chunk: 64 rows x GK k
-    for (int e = threadIdx.x; e < GT * GK; e += 256) {
-      const int i = e % GT, kk = e / GT;
+  // the chunk's entries of this thread: A 64 rows x GK k, B 64 n x GK k; the next chunk's are read while this one's
+  // products run
+  T va[PER], vb[PER];
+  auto b_at = [&](int p, int& j, int& kk) {
+    const int e = threadIdx.x + 256 * p;
+    if (bnn) {
+      kk = e % GK;
+      j = e / GK;
+    } else {
+      j = e % GT;
+      kk = e / GT;
+    }
+  };
+  auto load_chunk = [&](int k0) {
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int e = threadIdx.x + 256 * p, i = e % GT, kk = e / GT;
       T v = zero;
       if (i < tk.m && k0 + kk < tk.k) {
         v = tk.A[(int64_t)(k0 + kk) * tk.lda + i];
@@ -237,14 +254,12 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmTask<T>* __restrict__ ta
           v = (tk.flags & GF_D_MUL) ? cmul(v, dd) : cdiv(v, dd);
         }
       }
-      Ar[kk][i] = v.x;
-      Ai[kk][i] = v.y;
-      As[kk][i] = v.x + v.y;
+      va[p] = v;
     }
-    // B chunk: 64 n x GK k
-    for (int e = threadIdx.x; e < GT * GK; e += 256) {
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
       int j, kk;
-      if (bnn) { kk = e % GK; j = e / GK; } else { j = e % GT; kk = e / GT; }
+      b_at(p, j, kk);
       T v = zero;
       if (j < tk.n && k0 + kk < tk.k) {
         v = bnn ? tk.B[(int64_t)j * tk.ldb + (k0 + kk)] : tk.B[(int64_t)(k0 + kk) * tk.ldb + j];
@@ -254,11 +269,25 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmTask<T>* __restrict__ ta
           else if ((tk.flags & GF_B_UNIT_LOWER_NT) ? (kg > ng) : (kg < ng)) v = zero;
         }
       }
-      Br[kk][j] = v.x;
-      Bi[kk][j] = v.y;
-      Bs[kk][j] = v.x + v.y;
+      vb[p] = v;
+    }
+  };
+  load_chunk(0);
+  for (int k0 = 0; k0 < tk.k; k0 += GK) {
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int e = threadIdx.x + 256 * p, i = e % GT, kk = e / GT;
+      Ar[kk][i] = va[p].x;
+      Ai[kk][i] = va[p].y;
+      As[kk][i] = va[p].x + va[p].y;
+      int j, kb;
+      b_at(p, j, kb);
+      Br[kb][j] = vb[p].x;
+      Bi[kb][j] = vb[p].y;
+      Bs[kb][j] = vb[p].x + vb[p].y;
     }
     __syncthreads();
+    if (k0 + GK < tk.k) load_chunk(k0 + GK);
     if constexpr (kSingle) {
       // single precision: the FP32 pipe is fast enough that issue slots, not FMAs, bound the
       // loop, so all 16 blocks run; thread (tx, ty) owns rows 4 ty .. 4 ty + 3 and columns
