@@ -16,7 +16,8 @@
 // each (48 by their shared-memory reads of 6 KB; 70 before their descriptors were unrolled to constants), and the
 // blocks' way from L2 (88 KB per 16 k) is next: with a sixth of the MMAs the time falls to 0.57.  One CTA per SM over
 // many tiles, so copies and MMAs of the next tile overlap this one's additions (one tile per CTA: 107 against 92 ms
-// then).  The front products of an 80^3 lens setup: 860 ms with FP64 FMAs, 71 ms here plus 22 ms to write the digits.
+// then).  The front products of an 80^3 lens setup: 860 ms with FP64 FMAs, 71 ms here plus 22 ms to write the digits
+// (75 plus 24 with the wide fronts' F_TL and inverse, psp_api.cu kOzBlock).
 #include <cstdint>
 
 #include "cplx.cuh"

@@ -181,11 +181,13 @@ __device__ __forceinline__ void warp_sum(R (&v)[NV], const int lane, int& base, 
   }
 }
 
-// factor entries in flight: columns per thread (up), blocks of `cols` columns times 32-row steps per warp (down)
+// factor entries in flight: columns per thread (up), blocks of `cols` columns times 32-row steps per warp (down).
+// Bounded by the 96 registers of a thread with two CTAs per SM: one more step spills.  Complex64 groups with eight
+// columns in flight instead of four: salt body 128^3 x 8 46.6 -> 44.8 ms, 88^3 x 8 18.3 -> 18.2 ms.
 template <typename T, int RG>
 struct Tile {
   static constexpr bool wide = sizeof(T) == 16;
-  static constexpr int up = wide ? (RG == 1 ? 2 : 4) : (RG == 1 ? 8 : 4);
+  static constexpr int up = wide ? (RG == 1 ? 2 : 4) : 8;
   static constexpr int cols = RG == 8 ? 2 : 4;
   static constexpr int down = RG >= 2 ? 1 : (wide ? 1 : 2);
 };
@@ -589,6 +591,14 @@ __device__ __noinline__ void bwd_tri_task(const TaskSlot<T>& sl, const SweepArgs
 // gathers need into shared memory, warms L2 with its factor block and waits for its dependency; eight product
 // warps gather, multiply and write; a signalling warp makes a finished task's writes visible and counts it.
 // Tasks alternate between two slots.
+//
+// What bounds it: in complex128 the FP64 pipe (2 FMAs per clock and SM, 4 per factor entry and column) together with
+// the chain of levels; in complex64 the chain, about 3 us of gather and reduction per task around its products, and
+// with many columns the shared-memory reads of the gathered vector.  With all of a CTA's warps doing every role in
+// turn a task took about 8 us for 2.6 us of products.  Two CTAs of 320 threads per SM (96 registers); three with
+// 64 registers spill.  One application, all roles in turn -> as it is: 100^3 lens complex128 51.6 -> 33.9 ms (25.4 ms
+// of FP64), complex64 15.2 -> 11.5 ms (4.1 ms of HBM), 88^3 complex64 x 8 40.3 -> 18.2 ms, salt body 128^3 x 8
+// 65.7 -> 44.8 ms, 20^3 complex128 1.07 -> 0.70 ms.
 // ---------------------------------------------------------------------------
 constexpr long long kWaitCycles = 4000000000LL;   // SM clock cycles: about two seconds at 2 GHz
 constexpr long long kWaitSpins = 400000000LL;     // and a hard cap on polls, whatever the clock does
