@@ -49,6 +49,7 @@ FP32_DERIVED_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12   # FP32 lanes x FMA x max S
 TF32_PER_BF16 = 1.1 / 2.25                            # nominal dense TF32 / bf16 tensor rates
 TC_EXECUTED_PER_USEFUL = 18.0 / 8.0                   # 3M x (hi.hi + hi.lo + lo.hi) TF32 products per complex MAC
 GEMM_3M_EXECUTED_PER_USEFUL = 6.0 / 8.0               # CUDA-core complex GEMM: 3 real FMAs per complex MAC (8 flops)
+OZ_EXECUTED_PER_USEFUL = 36 * 8.0 / 8.0               # complex128 on tensor cores: 36 digit products x 4 real FMAs per complex MAC
 
 GRID_N = 100
 
@@ -261,8 +262,8 @@ def traffic_from_profiles(kernel):
 
 
 SETUP_KERNELS = ("k_assemble", "k_diag_ldlt", "k_panel_right", "k_panel_left", "k_gemm", "k_copy_linv", "k_tc_gemm",
-                 "k_tc_pack", "k_scale_zd")
-SWEEP_KERNELS = ("k_sweep", "k_solve_fwd", "k_solve_bwd")
+                 "k_tc_pack", "k_scale_zd", "k_oz_gemm", "k_oz_pack")
+SWEEP_KERNELS = ("k_sweep",)
 
 
 def max_over_ranks(x, device=None):
@@ -363,6 +364,7 @@ def summarize(stats_timed, stats_full, infos, factor_bytes, steps, fp64_peak=FP6
         tk, tv = top_name, agg[top_name]
     else:
         tk, tv = max(agg.items(), key=lambda kv: kv[1]["total_ms"])
+    share = full.get(tk, {"total_ms": 0.0})["total_ms"] / tot_all
     sec = max(tv["total_ms"] * 1e-3, 1e-12)
     achieved = tv["flops"] / sec / 1e12
     # the complex products are 3M (3 real FMAs = 6 executed flops per 8 counted), so in counted complex
@@ -377,11 +379,14 @@ def summarize(stats_timed, stats_full, infos, factor_bytes, steps, fp64_peak=FP6
                                "flops per 8 counted, so 8/6 of the FP64 rate is the ceiling in counted flops; "
                                "fp64_pipe_frac = executed FP64 flops (algorithmic + selective inversion) over the "
                                "FP64 peak",
-                "kernel_share": full.get(tk, {"total_ms": 0.0})["total_ms"] / tot_all,
+                "kernel_share": share,
                 "work": "algorithmic flops of the plain multifrontal factorisation (8 per complex MAC); "
                         "achieved_incl_si adds the selective-inversion flops the kernel also executes",
                 "timing": "achieved from CUDA events around every launch of this kernel inside the timed region; "
                           "share from one fully instrumented step after it"}
+    if tk == "k_oz_gemm":
+        roofline = roofline_generic(tk, tv, share, "CUDA events around every launch of this kernel inside the timed region; "
+                                                   "share from one fully instrumented step after it")
     setup_ms = sum(v["total_ms"] for k, v in agg.items() if k in SETUP_KERNELS) / steps
     setup_flops = sum(v["flops"] for k, v in agg.items() if k in SETUP_KERNELS)
     sweep = [v for k, v in full.items() if k in SWEEP_KERNELS]
@@ -420,7 +425,17 @@ def roofline_generic(name, v, share, timing, alu_peaks=None):
                 "peak_source": f"TF32 dense from the {src} bf16 peak x 1.1/2.25 (of {src}); achieved counts the "
                                "algorithmic complex flops (8 per complex MAC), executed the split-TF32 3M products "
                                "(18 real TF32 flops per useful complex MAC)"}
-    if name in ("k_sweep", "k_assemble", "k_tc_pack", "k_matvec", "k_multiaxpy", "k_solve_fwd", "k_solve_bwd"):
+    if name == "k_oz_gemm":
+        peak = pk["bf16_tflops"]
+        useful_all = v["flops"] + v.get("extra_flops", 0.0)
+        exe = useful_all * OZ_EXECUTED_PER_USEFUL / ms / 1e9
+        return {"kernel": name, "bound": "tensor", "achieved": v["flops"] / ms / 1e9, "peak": peak / OZ_EXECUTED_PER_USEFUL,
+                "unit": "TFLOP/s", "frac": v["flops"] / ms / 1e9 * OZ_EXECUTED_PER_USEFUL / peak, "traffic": None,
+                "kernel_share": share, "timing": timing, "achieved_incl_si": useful_all / ms / 1e9, "executed": exe,
+                "executed_frac": exe / peak,
+                "peak_source": f"fp16 dense = the {src} bf16 peak (of {src}) over 36: a complex128 multiply-add (8 counted "
+                               "flops) is 36 exact fp16 digit products of 4 real FMAs"}
+    if name in ("k_sweep", "k_assemble", "k_tc_pack", "k_oz_pack", "k_matvec", "k_multiaxpy"):
         peak = pk["hbm_gbs"]
         ach = v["bytes"] / ms / 1e6
         return {"kernel": name, "bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",
@@ -452,6 +467,11 @@ def rooflines(full128, full64, alu):
                         "achieved_incl_si": (g["flops"] + g["extra_flops"]) / sec / 1e12,
                         "fp64_executed": exe, "fp64_pipe_frac": exe / fp64, "kernel_share": g["total_ms"] / tot,
                         "peak_source": "FP64 peak x 8/6 (3M products): " + alu.get("fp64_source", "derived")})
+        z = full128.get("k_oz_gemm")
+        if z and z["total_ms"] > 0:
+            r = roofline_generic("k_oz_gemm", z, z["total_ms"] / tot, "instrumented step", alu)
+            r["path"] = "c128"
+            out.append(r)
         s = full128.get("k_sweep")
         if s and s["total_ms"] > 0:
             sec = s["total_ms"] * 1e-3
