@@ -776,7 +776,8 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       const int64_t c0 = (int64_t)ctasks.size();
       for (int f = 0; f < nf; ++f) {
         const auto& ft = fronts[f0 + f];
-        for (int c = 0; c < ft.s + ft.u; c += 32) ctasks.push_back({f, c, std::min(c + 32, ft.s + ft.u)});
+        for (int c = 0; c < ft.s + ft.u; c += kAssembleCols)
+          ctasks.push_back({f, c, std::min(c + kAssembleCols, ft.s + ft.u)});
       }
       Launch la{ASSEMBLE, f0, c0, (int)(ctasks.size() - c0), 0};
       for (int f = 0; f < nf; ++f) {

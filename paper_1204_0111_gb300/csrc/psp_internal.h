@@ -136,6 +136,20 @@ __host__ __device__ __forceinline__ int64_t upd_index(int r, int c, int u, int u
   const int nt = (u + ut - 1) >> sh;
   return upd_tile_offset(r >> sh, c >> sh, nt, ut) + ((int64_t)(c & (ut - 1)) << sh) + (r & (ut - 1));
 }
+// column c of that matrix, for many r
+struct UpdColumn {
+  int64_t tile0, within;   // tiles before tile row 0 of the column's tiles; the column's start in a tile
+  int sh;
+  __host__ __device__ __forceinline__ UpdColumn(int c, int u, int ut) {
+    sh = ut == 128 ? 7 : 6;
+    const int64_t nt = (u + ut - 1) >> sh, J = c >> sh;
+    tile0 = J * nt - J * (J - 1) / 2 - J;
+    within = (int64_t)(c & (ut - 1)) << sh;
+  }
+  __host__ __device__ __forceinline__ int64_t at(int r) const {
+    return ((tile0 + (r >> sh)) << (2 * sh)) + within + (r & ((1 << sh) - 1));
+  }
+};
 __host__ __device__ __forceinline__ int64_t upd_packed_elems(int u, int ut) {
   const int64_t nt = (u + ut - 1) / ut;
   return nt * (nt + 1) / 2 * (int64_t)ut * ut;
@@ -162,6 +176,8 @@ struct FrontTask {
 __host__ __device__ __forceinline__ int64_t second_inverse_offset(int64_t s, int64_t u) {
   return ((s + u) * s + 15) / 16 * 16;
 }
+
+constexpr int kAssembleCols = 32;   // columns of a front per assembly CTA
 
 struct ColTask {   // a chunk of columns / rows of one front
   int front;       // index into the level's FrontTask array
