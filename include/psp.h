@@ -127,6 +127,8 @@ typedef struct {
                            right-hand side, so with many right-hand sides wider tasks gather less */
   int test_sweep_stall; /* tests only: 1 makes one dependency of the persistent sweep impossible to
                            meet, so its bounded wait (about 2 s) gives up; psp_solve then returns
+                           PSP_ERR_TIMEOUT and the device stays usable.  2 leaves out an operand block of the
+                           setup's first tensor-core product, whose waits then give up: psp_setup returns
                            PSP_ERR_TIMEOUT and the device stays usable.  0 (default): off */
   int gmres_basis;      /* psp_solve: 1 keeps z_j = M^{-1} v_j for every Krylov vector (2k + 1 vectors per
                            right-hand side); 2 keeps V only and forms x += M^{-1}(V y) with one more

@@ -192,7 +192,9 @@ __global__ void __launch_bounds__(256) k_oz_pack(const OzPackTask* __restrict__ 
 // run while this one's sums are added to C (tiles of a small front spend more on that than on their MMAs).  Warp 8 copies the operands' blocks of 16 k into two stages, warp 9
 // issues the MMAs (Re += Ar Br - Ai Bi and Im += Ar Bi + Ai Br as two N = 64 MMAs per digit pair: B's rows are stored as
 // [-Im | Re | Im], so [Re | Im] and [-Im | Re] are windows of it), warps 0 - 7 combine the sums after every 128 k.
-// Every wait is bounded; one that gives up records an error in status[1].
+// Every wait is bounded; one that gives up records an error in status[1] and raises the CTA's abort flag.  The additions'
+// tensor-memory reads are warp-wide instructions, so whether a warp goes on is one decision of the whole warp; after an
+// abort the CTA's copies and MMAs in flight are waited for (bounded too) before its shared and tensor memory go back.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const OzGemmTask* __restrict__ tasks, int ntasks, int* status) {
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -201,7 +203,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const OzGemmTask* __rest
   uint64_t* empty = full + NSTAGE;
   uint64_t* sums = empty + NSTAGE;       // the sums of 128 k are complete
   uint64_t* drained = sums + 1;          // ... and have been read
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drained + 1);
+  uint64_t* quiet = drained + 1;         // after an abort: the MMAs issued have ended
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(quiet + 1);
   volatile int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
 
   if (tid == 0) {
@@ -211,6 +214,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const OzGemmTask* __rest
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(sums)) : "memory");
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(drained)), "r"(EPI_THREADS) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(quiet)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *abort_flag = 0;
   }
@@ -230,9 +234,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const OzGemmTask* __rest
     atomicCAS(status + 1, 0, 1);
   };
 
+  int i = 0;   // warps 8 and 9: blocks of 16 k copied, consumed
   if (warp == 8) {
     if (lane == 0) {
-      int i = 0;   // blocks of 16 k copied
       for (int t = blockIdx.x; t < ntasks && !*abort_flag; t += gridDim.x) {
         const OzGemmTask& tk = tasks[t];
         const unsigned char *A = tk.A, *B = tk.B;
@@ -246,17 +250,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const OzGemmTask* __rest
           const uint32_t fb = smem_u32(&full[s]);
           const uint32_t dst = smem_u32(smem + s * STAGE);
           expect_tx(fb, STAGE);
+          if (kb == tk.kb0 && (tk.flags & GF_TEST_STALL)) continue;   // announced, never copied
           bulk_copy(dst, A + (int64_t)kb * A_BLOCK, A_BLOCK, fb);
           bulk_copy(dst + A_BLOCK, B + (int64_t)kb * B_BLOCK, B_BLOCK, fb);
         }
       }
-      // after a give-up, the copies in flight end before the CTA does
-      if (*abort_flag)
-        for (int j = i > NSTAGE ? i - NSTAGE : 0; j < i; ++j) mbar_wait(smem_u32(&full[j & 1]), (uint32_t)((j >> 1) & 1));
     }
   } else if (warp == 9) {
     if (lane == 0) {
-      int i = 0, chunk = 0;   // blocks of 16 k consumed, accumulations made
+      int chunk = 0;   // accumulations made
       for (int t = blockIdx.x; t < ntasks && !*abort_flag; t += gridDim.x) {
         const int kb0 = tasks[t].kb0, kb1 = kb0 + tasks[t].nkb;
         for (int kb = kb0; kb < kb1; ++kb, ++i) {
@@ -294,7 +296,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const OzGemmTask* __rest
     const int row = 32 * q + lane, col0 = half * (ON / 2);
     constexpr int W = ON / 4;   // columns a thread combines at a time (two turns)
     int chunk = 0;
-    for (int tile = blockIdx.x; tile < ntasks && !*abort_flag; tile += gridDim.x) {
+    for (int tile = blockIdx.x; tile < ntasks; tile += gridDim.x) {
+      if (__any_sync(0xffffffffu, *abort_flag)) break;
       const OzGemmTask tk = tasks[tile];
       const bool neg = tk.flags & GF_NEG, beta0 = tk.flags & GF_BETA0;
       const int kb1 = tk.kb0 + tk.nkb;
@@ -314,10 +317,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const OzGemmTask* __rest
                        ? cp[(int64_t)c * tk.ldc]
                        : make_double2(0.0, 0.0);
           if (turn == 0) {
-            ready = mbar_wait(smem_u32(sums), (uint32_t)(chunk & 1));
+            ready = __all_sync(0xffffffffu, mbar_wait(smem_u32(sums), (uint32_t)(chunk & 1)));
             if (!ready) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           }
+          __syncwarp();
           const uint32_t base = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0;
           int64_t hr[W], hi[W];
           uint32_t rem[W];   // what d = 5 .. 7 leave below a unit: 14 bits each, real | imaginary
@@ -371,6 +375,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const OzGemmTask* __rest
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  if (*abort_flag) {   // nothing writes it any more
+    if (warp == 8 && lane == 0) {
+      for (int j = i > NSTAGE ? i - NSTAGE : 0; j < i; ++j) mbar_wait(smem_u32(&full[j & 1]), (uint32_t)((j >> 1) & 1));
+    } else if (warp == 9 && lane == 0) {
+      mma_commit(smem_u32(quiet));
+      mbar_wait(smem_u32(quiet), 0u);
+    }
+    __syncthreads();
+  }
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");

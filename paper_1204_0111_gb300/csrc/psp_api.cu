@@ -345,7 +345,7 @@ struct psp_ctx_s {
   int sweep_claim_ahead = 1;   // tasks a sweep CTA holds besides the one it runs
   int gmres_basis = 0;   // 0 auto, 1 keep z_j, 2 V only
   int si_mode = 0;       // psp_si_mode: what the factor of each front keeps (selective inversion, §2.2)
-  bool test_sweep_stall = false;
+  bool test_sweep_stall = false, test_product_stall = false;
   int64_t upd_arena_elems = 0;
   int64_t temp_budget_elems = 0;   // cap on setup temporaries per level group (0: what the device has free)
   // problems: one, or the independent problems of a batch (psp_setup_batch) with their panels
@@ -683,6 +683,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
     PSP_CK(cudaGetLastError());
   };
 
+  bool stall_next = X->test_product_stall;   // the first tensor-core product stalls (groups are planned one at a time)
   auto plan_group = [&](const std::vector<std::pair<int, int>>& grp, Tasks& tk) {
     tk.clear();
     auto& fronts = tk.fronts;
@@ -1296,6 +1297,10 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
           lt.count = (int)(otasks.size() - o0);
           for (size_t i = o0; i < otasks.size(); ++i)
             lt.bytes += (double)otasks[i].nkb * (oz.a_block + oz.b_block) + 32.0 * otasks[i].m * otasks[i].n;
+          if (stall_next && o0 < (int64_t)otasks.size()) {
+            otasks[o0].flags |= GF_TEST_STALL;
+            stall_next = false;
+          }
           launches.push_back(lp);
           launches.push_back(lt);
         }
@@ -2458,6 +2463,7 @@ static void init_options(psp_ctx_s* X, const psp_options& o) {
   X->range_begin = o.panel_begin;
   X->range_count = o.panel_count;
   X->test_sweep_stall = o.test_sweep_stall == 1;
+  X->test_product_stall = o.test_sweep_stall == 2;
   X->temp_budget_elems = o.setup_temp_mb > 0 ? ((int64_t)o.setup_temp_mb << 20) / (o.precision == PSP_PREC_C64 ? 8 : 16) : 0;
 }
 

@@ -6,7 +6,9 @@
 
 namespace psp {
 
-constexpr long long WAIT_LIMIT = 1ll << 24;   // polls of one mbarrier before a wait gives up
+// A wait on one mbarrier gives up after about two seconds of SM clocks, or after this many polls whatever the clock does.
+// (A count of polls alone is no limit in time: each poll may suspend the thread for as long as the hardware chooses.)
+constexpr long long kMbarWaitClocks = 4000000000ll, kMbarWaitPolls = 1ll << 24;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -30,8 +32,12 @@ __device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
 
 // bounded wait; false when it gave up
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
-  for (long long i = 0; i < WAIT_LIMIT; ++i)
+  if (mbar_try(mbar, parity)) return true;
+  const long long t0 = clock64();
+  for (long long i = 0; i < kMbarWaitPolls; ++i) {
     if (mbar_try(mbar, parity)) return true;
+    if (clock64() - t0 > kMbarWaitClocks) return false;
+  }
   return false;
 }
 
