@@ -150,6 +150,7 @@ __global__ void __launch_bounds__(256, 1) k_tc_gemm(const TcGemmTask* __restrict
   const uint32_t tmem = *tmem_slot;
   const int nkb = tk.nkb;
 
+  int copied = 0;   // thread 0: k-blocks announced
   if (tid == 0) {
     // producer: stage i & 1 holds k-block i; refill a stage once its MMAs have completed
     for (int i = 0; i < nkb; ++i) {
@@ -162,6 +163,8 @@ __global__ void __launch_bounds__(256, 1) k_tc_gemm(const TcGemmTask* __restrict
       const uint32_t fb = smem_u32(&full[s]);
       const uint32_t dst = smem_u32(smem + s * STAGE_BYTES);
       expect_tx(fb, STAGE_BYTES);
+      ++copied;
+      if (i == 0 && (tk.flags & GF_TEST_STALL)) continue;   // announced, never copied
       bulk_copy(dst, tk.A + (int64_t)(tk.kb0 + i) * BLOCK_BYTES, BLOCK_BYTES, fb);
       bulk_copy(dst + BLOCK_BYTES, tk.B + (int64_t)(tk.kb0 + i) * BLOCK_BYTES, BLOCK_BYTES, fb);
     }
@@ -237,6 +240,14 @@ __global__ void __launch_bounds__(256, 1) k_tc_gemm(const TcGemmTask* __restrict
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  if (*abort_flag) {   // the copies and MMAs in flight end (bounded waits) before shared and tensor memory go back
+    if (tid == 0)
+      for (int j = copied > NSTAGE ? copied - NSTAGE : 0; j < copied; ++j)
+        mbar_wait(smem_u32(&full[j & 1]), (uint32_t)((j >> 1) & 1));
+    else if (tid == 32 && nkb > 0)
+      mbar_wait(smem_u32(done), 0u);
+    __syncthreads();
+  }
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");

@@ -1311,6 +1311,10 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         lp.bytes = (double)(ptasks.size() - p0) * (tc_block_bytes() + 128.0 * 16 * sizeof(T));
         launches.push_back(lp);
         Launch lt{TCGEMM, f0, t0, (int)(ttasks.size() - t0), -1};
+        if (stall_next) {
+          ttasks[t0].flags |= GF_TEST_STALL;
+          stall_next = false;
+        }
         double fl_unused = 0;
         tc_work(fl_unused, lt.bytes, t0);
         lt.flops = tflops;

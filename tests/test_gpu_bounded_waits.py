@@ -12,7 +12,7 @@ from _cases import Case, random_velocity
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("precision", ["c128"])
+@pytest.mark.parametrize("precision", ["c128", "c64"])
 def test_a_stalled_product_is_reported_and_the_device_stays_usable(precision):
     import torch
     from oracle import sweep as osw
