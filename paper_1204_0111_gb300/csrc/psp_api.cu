@@ -108,8 +108,6 @@ static void upload(DevBuf& d, const std::vector<U>& h) {
   d.alloc(std::max<size_t>(h.size() * sizeof(U), 16));
   if (!h.empty()) PSP_CK(cudaMemcpy(d.p, h.data(), h.size() * sizeof(U), cudaMemcpyHostToDevice));
 }
-// Stream-ordered upload: the copy from pageable memory is staged before the call returns, and it
-// does not wait for work already queued on the stream.
 // A stream for host-to-device uploads of tables built on the host: a copy from pageable memory may
 // wait for the work already on the stream it is issued on, so uploads issued on the compute stream
 // would hold the host until the device caught up; join() makes the compute stream wait for them.
@@ -132,10 +130,16 @@ struct SideStream {
   }
 };
 
+// upload on a side stream, which carries nothing but uploads: h may go once this returns (a copy from pageable memory may
+// still be reading it when cudaMemcpyAsync returns)
 template <typename U>
-static void upload_async(DevBuf& d, const std::vector<U>& h, cudaStream_t st) {
+static void upload_aside(DevBuf& d, const std::vector<U>& h, const SideStream& side) {
   d.alloc(std::max<size_t>(h.size() * sizeof(U), 16));
-  if (!h.empty()) PSP_CK(cudaMemcpyAsync(d.p, h.data(), h.size() * sizeof(U), cudaMemcpyHostToDevice, st));
+  if (h.empty()) return;
+  const cudaError_t e = cudaMemcpyAsync(d.p, h.data(), h.size() * sizeof(U), cudaMemcpyHostToDevice, side.s);
+  const cudaError_t w = cudaStreamSynchronize(side.s);
+  PSP_CK(e);
+  PSP_CK(w);
 }
 
 // true for device (or managed) memory, false for host memory; device memory of a device other than
@@ -632,7 +636,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       }
     }
   } chunk_guard{chunks, st, up.s, chunk_alloc};
-  // copies v to a new device chunk (the copy from pageable memory is staged before the call returns)
+  // copies v to a new device chunk; the copy may read v until the side stream has passed it
   auto upload_list = [&](const auto& v) {
     using E = typename std::decay_t<decltype(v)>::value_type;
     E* d = nullptr;
@@ -1325,6 +1329,13 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   };
   {
     Tasks lists[2];
+    struct Event {   // passed once the copies of a list's tasks have ended
+      cudaEvent_t e = nullptr;
+      Event() { PSP_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming)); }
+      Event(const Event&) = delete;
+      Event& operator=(const Event&) = delete;
+      ~Event() { cudaEventDestroy(e); }
+    } copied[2];
     std::future<void> planned;
     auto start = [&](size_t i) {
       auto plan = [&, i] { plan_group(groups[i], lists[i & 1]); };
@@ -1334,21 +1345,27 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         planned = std::async(std::launch::deferred, plan);
       }
     };
-    // declared after the lists: on an error the worker ends (the future's destructor waits) before they go
+    // declared after the lists: the worker and the copies that read them end before they go, on an error too
     struct Wait {
       std::future<void>& f;
+      cudaStream_t up;
       ~Wait() {
         if (f.valid()) f.wait();
+        cudaStreamSynchronize(up);
       }
-    } wait{planned};
+    } wait{planned, up.s};
     if (!groups.empty()) start(0);
     for (size_t i = 0; i < groups.size(); ++i) {
       tp = std::chrono::steady_clock::now();
       planned.get();
-      if (i + 1 < groups.size()) start(i + 1);
+      if (i + 1 < groups.size()) {
+        if (i > 0) PSP_CK(cudaEventSynchronize(copied[(i + 1) & 1].e));   // group i - 1's copies from these lists
+        start(i + 1);
+      }
       waited_ms += ms_since(tp);
       tp = std::chrono::steady_clock::now();
       enqueue_group(lists[i & 1]);
+      PSP_CK(cudaEventRecord(copied[i & 1].e, up.s));
       enqueue_ms += ms_since(tp);
     }
   }
@@ -1619,8 +1636,8 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
     }
     SP.nsteps = (int)steps.size();
     SP.nqueue = (int)queue.size();
-    upload_async(SP.steps, recs, side.s);
-    upload_async(SP.queue, queue, side.s);
+    upload_aside(SP.steps, recs, side);
+    upload_aside(SP.queue, queue, side);
     SP.nfront_steps = nfs;
     sync_words = std::max(sync_words, (size_t)words);
   }
