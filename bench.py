@@ -262,7 +262,7 @@ def traffic_from_profiles(kernel):
 
 
 SETUP_KERNELS = ("k_assemble", "k_diag_ldlt", "k_panel_right", "k_panel_left", "k_gemm", "k_copy_linv", "k_tc_gemm",
-                 "k_tc_pack", "k_scale_zd", "k_oz_gemm", "k_oz_pack")
+                 "k_tc_pack", "k_scale_zd", "k_oz_gemm", "k_oz_pack", "k_oz_colmax")
 SWEEP_KERNELS = ("k_sweep",)
 
 
@@ -435,7 +435,7 @@ def roofline_generic(name, v, share, timing, alu_peaks=None):
                 "executed_frac": exe / peak,
                 "peak_source": f"fp16 dense = the {src} bf16 peak (of {src}) over 36: a complex128 multiply-add (8 counted "
                                "flops) is 36 exact fp16 digit products of 4 real FMAs"}
-    if name in ("k_sweep", "k_assemble", "k_tc_pack", "k_oz_pack", "k_matvec", "k_multiaxpy"):
+    if name in ("k_sweep", "k_assemble", "k_tc_pack", "k_oz_pack", "k_oz_colmax", "k_matvec", "k_multiaxpy"):
         peak = pk["hbm_gbs"]
         ach = v["bytes"] / ms / 1e6
         return {"kernel": name, "bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s",

@@ -106,8 +106,9 @@ typedef struct {
   int collect_stats;  /* CUDA-event timing of launches (psp_stats): 0 none (default), 1 every kernel,
                          2 the setup kernels only (a few hundred launches per setup) */
   int tensor_cores;   /* 1 (default) runs the Schur update and the selective-inversion multiplies on tcgen05 tensor
-                         cores (complex64: split TF32 products; complex128: exact digit products, in 64-bit
-                         accuracy), 0 keeps them on CUDA cores */
+                         cores (complex64: split TF32 products; complex128: exact digit products, whose entries'
+                         errors are at the level of 64-bit products relative to the largest entries of their
+                         row and column of |A| |B|), 0 keeps them on CUDA cores */
   int tc_min_dim;     /* complex64 path: fronts with s >= tc_min_dim and u >= tc_min_dim take the tensor
                          cores, the others CUDA cores; <= 0 selects the default (64) */
   int sweep_level_tasks; /* sweep schedule: tasks a tree level is split into at least (row / column

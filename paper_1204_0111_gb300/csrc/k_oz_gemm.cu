@@ -8,16 +8,25 @@
 // exact in fp16).  The digit products a_i b_j of i + j = d share a weight; for each d = 0 .. 7 they are accumulated in
 // FP32 in tensor memory, exactly: over 128 k a sum of d = 3 stays below 4 x 2 x 128 x 2^14 = 2^24, and the lower
 // d (4 .. 7), which may pass it, weigh 2^-32 and less.  The eight sums are then combined in 64-bit integers, rounded
-// once to 53 bits or at 2^-63 of the row scales' product, and added to C in FP64.  Products of i + j >= 8 are dropped
-// (2^-68).  On fronts of a lens model the error against 80-bit products is 0.2 - 0.6 of the FP64 product's in norm.
+// once to 53 bits or at 2^-63 of the row scales' product, and added to C in FP64.
+//
+// Accuracy.  Products of i + j >= 8 are dropped: one real product loses up to 2^-59 of the row scales' product, the 256
+// of an accumulation 2^-51 at worst and about 2^-59 on entries with random digits.  That is relative to the largest
+// entries of two rows, so it is as good as 64-bit arithmetic only if those meet: before the rows are scaled, column k of A
+// is multiplied and column k of B divided by a power of two that makes their largest entries equal (k_oz_colmax; the sum
+// over k does not change).  Then C_ij's error is below 2^-51 sqrt(max_j' P_ij' max_i' P_i'j), P = |A| |B|^T, whatever
+// the entries' sizes.  Measured against 80-bit products as the largest entry's error over that square root: on lens
+// fronts 1e-16 (FP64 products: 2e-15), with PML amplitudes of 4e4 .. 4e6 or frequencies of 1e-4, whose pivots differ by
+// many orders, 2e-16 (FP64: 2e-15; without the balance up to 5e-10).
 //
 // What bounds it: FP64 units do 2 DFMA per clock and SM, and the CUDA-core product (k_gemm) already ran them at 0.9 of
 // their measured rate.  The 36 digit products are 72 fp16 MMAs of 128 x 64 x 16 per 16 k of a tile, at about 42 clocks
 // each (48 by their shared-memory reads of 6 KB; 70 before their descriptors were unrolled to constants), and the
 // blocks' way from L2 (88 KB per 16 k) is next: with a sixth of the MMAs the time falls to 0.57.  One CTA per SM over
 // many tiles, so copies and MMAs of the next tile overlap this one's additions (one tile per CTA: 107 against 92 ms
-// then).  The front products of an 80^3 lens setup: 860 ms with FP64 FMAs, 71 ms here plus 22 ms to write the digits
-// (75 plus 24 with the wide fronts' F_TL and inverse, psp_api.cu kOzBlock).
+// then).  The front products of an 80^3 lens setup: 860 ms with FP64 FMAs, 76 ms here plus 29 ms to write the digits
+// and 3 ms for the columns' balance (the wide fronts' F_TL and inverse among them, psp_api.cu kOzBlock).  Without the
+// balance, which gives Z D^-1 different digits in the Schur update and in M_BL, the digits took 24 ms.
 #include <cstdint>
 
 #include "cplx.cuh"
@@ -41,8 +50,9 @@ constexpr int SMEM = NSTAGE * STAGE + 1024;    // + barriers and the TMEM slot
 constexpr uint32_t LBO = 128, SBO = 256;       // next core matrix (8 rows x 16 bytes) along k, next 8 rows
 constexpr uint32_t TMEM_COLS = 512;            // ND sums x (32 real + 32 imaginary columns)
 constexpr int EPI_THREADS = 256, THREADS = EPI_THREADS + 64;   // + the copying warp and the MMA warp
-constexpr int kEmptyRow = -4096;               // exponent of a row of zeros
+constexpr int kEmptyRow = -(1 << 16);          // exponent of a row of zeros
 constexpr int kBadRow = 1 << 20;               // exponent of a row with an infinity or a NaN
+constexpr int kFar = 1 << 12;                  // balance of a column whose partner is zero: past every exponent
 
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
   uint64_t d = 0;
@@ -64,18 +74,22 @@ __device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t adesc, uint64_t
       "l"(adesc), "l"(bdesc), "r"(kInstr), "r"(acc));
 }
 
+// biased exponent of |x|: 0 for zero, 1 for denormals too, 2047 for infinities and NaN
+__device__ __forceinline__ int exponent(double x) {
+  const int hi = __double2hiint(x) & 0x7fffffff;
+  return (hi | __double2loint(x)) == 0 ? 0 : max(hi >> 20, 1);
+}
+__device__ __forceinline__ int exponent(double2 v) { return max(exponent(v.x), exponent(v.y)); }
+
 // x as the 62-bit integer x 2^(62 - e), rounded, every base-256 digit biased by 128; emax = biased exponent of the
-// row's largest entry (e = emax - 1022)
+// row's largest entry (e = emax - 1022) in units of x
 __device__ __forceinline__ unsigned long long biased_digits(double x, int emax) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
   const int e = (int)(bits >> 52) & 0x7ff;
-  unsigned long long m = 0;
-  if (e > 0) {
-    m = (bits & 0xfffffffffffffull) | 0x10000000000000ull;
-    const int sh = emax - e - 9;
-    if (sh <= 0) m <<= -sh;
-    else m = sh < 56 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
-  }
+  unsigned long long m = (bits & 0xfffffffffffffull) | (e > 0 ? 0x10000000000000ull : 0ull);
+  const int sh = emax - max(e, 1) - 9;
+  if (sh <= 0) m <<= -sh;
+  else m = sh < 56 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
   if (bits >> 63) m = 0ull - m;
   return m + 0x8080808080808080ull;
 }
@@ -93,53 +107,101 @@ __device__ __forceinline__ uint32_t digit_pair(unsigned long long x, unsigned lo
 }
 
 // acc +-= (h + rem 2^-14) 2^(e - 54), rounded to 53 bits or at 2^(e - 63), whichever is coarser: sums below 2^53 units take nine of
-// the bits below a unit along.  A row with an infinity or a NaN gives NaN, a product below the normal range zero.
+// the bits below a unit along.  A row with an infinity or a NaN gives NaN
 __device__ __forceinline__ void add_scaled(double& acc, int64_t h, uint32_t rem, int e, bool neg) {
   const bool fine = (uint64_t)(h + (1ll << 53)) < (1ull << 54);
-  const int64_t x = fine ? (h << 9) + (rem >> 5) : h;
-  const int ex = min(max(e + (fine ? 1023 - 63 : 1023 - 54), 0), 2046);
+  double x = (double)(fine ? (h << 9) + (rem >> 5) : h);
+  int ex = e + (fine ? 1023 - 63 : 1023 - 54);
+  if ((unsigned)(ex - 1) >= 2046u) {   // a scale that is not a normal number: part of it goes to x first, exactly
+    const int over = ex < 1 ? max(ex - 1, -1022) : min(ex - 2046, 900);
+    x *= __hiloint2double((1023 + over) << 20, 0);
+    ex = ex < 1 ? (ex - over < 1 ? 0 : 1) : 2046;
+  }
   const int hi = e > kBadRow / 2 ? 0x7ff80000 : ex << 20;
-  acc = fma((double)x, __hiloint2double(neg ? hi | (int)0x80000000 : hi, 0), acc);
+  acc = fma(x, __hiloint2double(neg ? hi | (int)0x80000000 : hi, 0), acc);
 }
 
 __device__ __forceinline__ int64_t rounded_sum(const float v) { return (int64_t)__float2int_rn(v); }
 
 }  // namespace
 
+// entry (r, k) of an operand before its scale: r < R, k < K
+template <typename Task>
+__device__ __forceinline__ double2 operand_entry(const Task& tk, int r, int k) {
+  if (tk.mode == TC_PACK_PLAIN) return tk.src[(int64_t)k * tk.ld + r];
+  if (tk.mode == TC_PACK_TRANSPOSED) return tk.src[(int64_t)r * tk.ld + k];   // X[k, r]
+  if (k == r) return make_double2(1.0, 0.0);
+  if (tk.mode == TC_PACK_UNIT_LOWER) return k < r ? tk.src[(int64_t)k * tk.ld + r] : make_double2(0.0, 0.0);   // T[r, k]
+  return k > r ? tk.src[(int64_t)r * tk.ld + k] : make_double2(0.0, 0.0);     // T[k, r], unit lower (transposed read)
+}
+
+// ---------------------------------------------------------------------------
+// k_oz_colmax: exponent of the largest entry of 32 columns k of an operand, over its R rows.  Reads the operand once,
+// 16 bytes an entry, contiguous over rows (a warp per column) or, for transposed operands, over k (a lane per column).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_oz_colmax(const OzColTask* __restrict__ tasks) {
+  __shared__ int part[8][32];
+  const OzColTask tk = tasks[blockIdx.x];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (tk.mode == TC_PACK_PLAIN || tk.mode == TC_PACK_UNIT_LOWER) {
+    for (int k = tk.k0 + warp; k < min(tk.k0 + 32, tk.K); k += 8) {
+      int em = 0;
+#pragma unroll 4
+      for (int r = (tk.mode == TC_PACK_PLAIN ? 0 : k) + lane; r < tk.R; r += 32) em = max(em, exponent(operand_entry(tk, r, k)));
+      em = __reduce_max_sync(0xffffffffu, em);
+      if (lane == 0) tk.out[k] = em;
+    }
+  } else {
+    const int k = tk.k0 + lane, rend = tk.mode == TC_PACK_TRANSPOSED ? tk.R : min(tk.R, k + 1);
+    int em = 0;
+    if (k < tk.K)
+#pragma unroll 4
+      for (int r = warp; r < rend; r += 8) em = max(em, exponent(operand_entry(tk, r, k)));
+    part[warp][lane] = em;
+    __syncthreads();
+    if (warp == 0 && k < tk.K) {
+      for (int w = 1; w < 8; ++w) em = max(em, part[w][lane]);
+      tk.out[k] = em;
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // k_oz_pack: digits of 128 rows x 128 k of an operand (rows r0.., k from k0) per CTA, laid out as the MMAs read
 // them from shared memory (K-major, 8-row x 16-byte core matrices).  Thread (row, half): k in [8 half, 8 half + 8) of
-// every 16.  Two passes over the source (the second from L2): row exponents, then digits.  HBM-bound: 16 bytes
-// read and 32 (A) or 48 (B) written per entry.
+// every 16.  Two passes over the source (the second from L2): row exponents, then digits.  The balance 2^s(k) of a
+// column is added to its entries' exponents.  HBM-bound: 16 bytes read and 32 (A) or 48 (B) written per entry.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_oz_pack(const OzPackTask* __restrict__ tasks) {
-  __shared__ int emax_s[2][OM];
+  __shared__ int emax_s[2][OM], bal[OKC];
   const OzPackTask tk = tasks[blockIdx.x];
   const int row = threadIdx.x & (OM - 1), half = threadIdx.x >> 7;
   const int rg = tk.r0 + row;
+  if (threadIdx.x < OKC) {
+    const int k = tk.k0 + threadIdx.x;
+    int s = 0;
+    if (k < tk.K && (tk.ka || tk.kd)) {
+      const int ea = tk.ka ? tk.ka[k] : 1, eb = tk.ka ? tk.kb[k] : 1, ed = tk.kd ? exponent(tk.kd[(int64_t)k * tk.ldk]) - 1023 : 0;
+      s = ea == 0 ? kFar : eb == 0 ? -kFar : (eb - ea - ed) >> 1;
+    }
+    bal[threadIdx.x] = tk.rows_b ? -s : s;
+  }
+  __syncthreads();
   auto load = [&](int k) {
     double2 v = make_double2(0.0, 0.0);
     if (rg < tk.R && k < tk.K) {
-      if (tk.mode == TC_PACK_PLAIN) {
-        v = tk.src[(int64_t)k * tk.ld + rg];
-        if (tk.scale) v = cmul(v, tk.scale[(int64_t)k * tk.lds]);
-      } else if (tk.mode == TC_PACK_UNIT_LOWER) {   // T[rg, k], unit lower
-        v = k == rg ? make_double2(1.0, 0.0) : (k < rg ? tk.src[(int64_t)k * tk.ld + rg] : v);
-      } else if (tk.mode == TC_PACK_TRANSPOSED) {   // X[k, rg]
-        v = tk.src[(int64_t)rg * tk.ld + k];
-      } else {                                      // T[k, rg], unit lower (transposed read)
-        v = k == rg ? make_double2(1.0, 0.0) : (k > rg ? tk.src[(int64_t)rg * tk.ld + k] : v);
-      }
+      v = operand_entry(tk, rg, k);
+      if (tk.scale) v = cmul(v, tk.scale[(int64_t)k * tk.lds]);
     }
     return v;
   };
   const int nkb = min((tk.K - tk.k0 + OK - 1) / OK, OKC / OK);
-  int em = 0;
+  int em = 2 * kEmptyRow;
   for (int kb = 0; kb < nkb; ++kb)
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const double2 v = load(tk.k0 + kb * OK + half * 8 + q);
-      em = max(em, max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff));
+      const int kk = kb * OK + half * 8 + q, e = exponent(load(tk.k0 + kk));
+      if (e > 0) em = max(em, e == 0x7ff ? kBadRow : e + bal[kk]);
     }
   emax_s[half][row] = em;
   __syncthreads();
@@ -148,15 +210,17 @@ __global__ void __launch_bounds__(256) k_oz_pack(const OzPackTask* __restrict__ 
   const bool live = !tk.rows_b || tk.r0 + sub * ON < tk.R;
   if (half == 0 && live)
     tk.exps[tk.rows_b ? (int64_t)sub * tk.exp_stride + (row & 31) : row] =
-        em == 0x7ff ? kBadRow : (em == 0 ? kEmptyRow : em - 1022);
+        em == kBadRow ? kBadRow : (em < kEmptyRow ? kEmptyRow : em - 1022);
   if (!live) return;
+  if (em < kEmptyRow) em = kBadRow;   // every digit zero
   for (int kb = 0; kb < nkb; ++kb) {
     unsigned long long re[8], im[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const double2 v = load(tk.k0 + kb * OK + half * 8 + q);
-      re[q] = biased_digits(v.x, em);
-      im[q] = biased_digits(v.y, em);
+      const int kk = kb * OK + half * 8 + q;
+      const double2 v = load(tk.k0 + kk);
+      re[q] = biased_digits(v.x, em - bal[kk]);
+      im[q] = biased_digits(v.y, em - bal[kk]);
     }
     unsigned char* dst = tk.dst + (int64_t)kb * (tk.rows_b ? B_BLOCK : A_BLOCK);
     if (tk.rows_b) dst += (int64_t)sub * tk.sub_stride;
@@ -388,6 +452,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const OzGemmTask* __rest
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
   }
+}
+
+void launch_oz_colmax(const OzColTask* tasks, int ntasks, cudaStream_t st) {
+  if (ntasks > 0) k_oz_colmax<<<ntasks, 256, 0, st>>>(tasks);
 }
 
 void launch_oz_pack(const OzPackTask* tasks, int ntasks, cudaStream_t st) {

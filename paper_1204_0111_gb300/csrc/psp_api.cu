@@ -454,6 +454,8 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   auto oz_exps = [&](int64_t R, int64_t K, bool b) {
     return (int64_t)sizeof(int) * cdiv_i(R, b ? oz.tile_n : oz.tile_m) * cdiv_i(K, oz.kc) * (b ? oz.tile_n : oz.tile_m);
   };
+  // exponents of the columns of four operands (the products' balance): 4 ints = one element per row of S
+  auto kx_elems = [&](int64_t s_) { return pad16(s_); };
   // F_BL and, once Z is made, Z D^-1 in its place (A operands); inv(L); Z; inv(L)^T (extended form)
   auto oz_elems = [&](int64_t s_, int64_t u_) {
     int64_t b = oz_bytes(u_, s_, false) + oz_exps(u_, s_, false) + oz_bytes(u_, s_, true) + oz_exps(u_, s_, true) +
@@ -475,6 +477,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   auto front_temp = [&](int64_t s_, int64_t u_) {     // W (s x s), Z (u x s), Z D^-1 or packed operands,
     if (si == PSP_SI_NONE) return (int64_t)0;         // the second inverse under construction (s x s)
     return pad16(s_ * s_) + pad16(u_ * s_) + (si == PSP_SI_TWO ? pad16(s_ * s_) : 0) + (in_blocks(s_) ? block_elems(s_) : 0) +
+           (use_oz(s_, u_) || in_blocks(s_) ? kx_elems(s_) : 0) +
            (use_tc(s_, u_) ? packed_elems(s_, u_)
             : use_oz(s_, u_) ? oz_elems(s_, u_)
                              : si == PSP_SI_EXTENDED ? pad16(u_ * s_) : 0);
@@ -570,7 +573,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   upload(d_upd_tile, upd_tile);
 
   // --- task lists, one set per group of fronts ---
-  enum Kind { ASSEMBLE, DIAG, PRIGHT, PLEFT, GEMM, COPY, TCGEMM, TCPACK, SCALE, RSOLVE, OZPACK, OZGEMM };
+  enum Kind { ASSEMBLE, DIAG, PRIGHT, PLEFT, GEMM, COPY, TCGEMM, TCPACK, SCALE, RSOLVE, OZPACK, OZGEMM, OZCOL };
   struct Launch {
     Kind kind;
     int64_t front_off;
@@ -587,10 +590,12 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
     std::vector<GemmTask<T>> gtasks;
     std::vector<unsigned char*> packs;   // per front: base of its packed operands (tensor-core fronts)
     std::vector<unsigned char*> blocks;  // per front: base of a block's packed operands (fronts factored in blocks of 128)
+    std::vector<int*> kx;                // per front: column exponents of its digit products' operands
     std::vector<TcPackTask> ptasks;
     std::vector<TcGemmTask> ttasks;
     std::vector<OzPackTask> optasks;
     std::vector<OzGemmTask> otasks;
+    std::vector<OzColTask> octasks;
     std::vector<Launch> launches;
     void clear() {
       fronts.clear();
@@ -599,10 +604,12 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       gtasks.clear();
       packs.clear();
       blocks.clear();
+      kx.clear();
       ptasks.clear();
       ttasks.clear();
       optasks.clear();
       otasks.clear();
+      octasks.clear();
       launches.clear();
     }
   };
@@ -615,7 +622,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   // [4..5] ~bits of the smallest |pivot| (0: none yet)
   PSP_CK(cudaMemsetAsync(status, 0, 8 * sizeof(int), st));
   static const char* names[] = {"k_assemble", "k_diag_ldlt", "k_panel_right", "k_panel_left", "k_gemm", "k_copy_linv",
-                                "k_tc_gemm", "k_tc_pack", "k_scale_zd", "k_panel_rsolve", "k_oz_pack", "k_oz_gemm"};
+                                "k_tc_gemm", "k_tc_pack", "k_scale_zd", "k_panel_rsolve", "k_oz_pack", "k_oz_gemm", "k_oz_colmax"};
   // task arrays go up on a side stream, so that the next group's planning overlaps the device's work
   SideStream up;
   std::vector<void*> chunks;
@@ -658,6 +665,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
     const TcGemmTask* TT = upload_list(tk.ttasks);
     const OzPackTask* OP = upload_list(tk.optasks);
     const OzGemmTask* OT = upload_list(tk.otasks);
+    const OzColTask* OC = upload_list(tk.octasks);
     up.join(st);   // the group's kernels after its task arrays
     for (const Launch& l : tk.launches) {
       if (l.count <= 0) continue;
@@ -676,6 +684,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
           case GEMM: launch_gemm<T>(GT + l.off, l.count, st); break;
           case COPY: launch_copy_linv<T>(Fl, CT + l.off, l.count, st); break;
           case TCGEMM: launch_tc_gemm(TT + l.off, l.count, status, st); break;
+          case OZCOL: launch_oz_colmax(OC + l.off, l.count, st); break;
           case OZPACK: launch_oz_pack(OP + l.off, l.count, st); break;
           case OZGEMM: launch_oz_gemm(OT + l.off, l.count, status, st); break;
           case TCPACK: launch_tc_pack(PT + l.off, l.count, st); break;
@@ -696,6 +705,8 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
     auto& gtasks = tk.gtasks;
     auto& packs = tk.packs;
     auto& blocks = tk.blocks;
+    auto& kx = tk.kx;
+    auto& octasks = tk.octasks;
     auto& ptasks = tk.ptasks;
     auto& ttasks = tk.ttasks;
     auto& optasks = tk.optasks;
@@ -735,6 +746,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       ft.ldzd = ft.u;
       packs.push_back(nullptr);
       blocks.push_back(nullptr);
+      kx.push_back(nullptr);
       if (si != PSP_SI_NONE) {
         ft.W = tbase + toff;
         toff += pad16((int64_t)ft.s * ft.s);
@@ -761,6 +773,10 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         if (in_blocks(ft.s)) {
           blocks.back() = reinterpret_cast<unsigned char*>(tbase + toff);
           toff += block_elems(ft.s);
+        }
+        if (use_oz(ft.s, ft.u) || in_blocks(ft.s)) {
+          kx.back() = reinterpret_cast<int*>(tbase + toff);
+          toff += kx_elems(ft.s);
         }
       }
       fronts.push_back(ft);
@@ -798,8 +814,29 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       }
       launches.push_back(la);
     }
+    // exponents of the columns of an operand (R rows, K columns); returns its bytes
+    auto oz_colmax = [&](const T* src, int64_t ld_, int64_t R, int64_t K, int mode, int* out) {
+      for (int64_t k0 = 0; k0 < K; k0 += 32) {
+        OzColTask t{};
+        t.src = reinterpret_cast<const double2*>(src);
+        t.out = out;
+        t.ld = (int)ld_;
+        t.k0 = (int)k0;
+        t.R = (int)R;
+        t.K = (int)K;
+        t.mode = mode;
+        octasks.push_back(t);
+      }
+      return es * (double)R * K * (mode == TC_PACK_UNIT_LOWER || mode == TC_PACK_UNIT_LOWER_T ? 0.5 : 1.0);
+    };
+    struct Balance {   // of a product's columns k (k_oz_pack): both operands are packed with the same one
+      const int *ka = nullptr, *kb = nullptr;
+      const T* kd = nullptr;
+      int64_t ldk = 0;
+    };
     // packs an operand (R rows, K columns; columns times scale[k lds_]) of the complex128 tensor-core products; returns its bytes
-    auto oz_pack = [&](const T* src, const T* scale, int64_t lds_, unsigned char* dst, int64_t ld_, int64_t R, int64_t K, int mode, bool b) {
+    auto oz_pack = [&](const T* src, const T* scale, int64_t lds_, unsigned char* dst, int64_t ld_, int64_t R, int64_t K, int mode, bool b,
+                       const Balance& bal) {
       const int64_t nkb = cdiv_i(K, oz.k), nkc = cdiv_i(K, oz.kc), rows = b ? oz.tile_n : oz.tile_m;
       int* exps = reinterpret_cast<int*>(dst + oz_bytes(R, K, b));
       for (int64_t r0 = 0; r0 < R; r0 += oz.tile_m)
@@ -819,6 +856,10 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
           t.K = (int)K;
           t.mode = mode;
           t.rows_b = b;
+          t.ka = bal.ka;
+          t.kb = bal.kb;
+          t.kd = reinterpret_cast<const double2*>(bal.kd);
+          t.ldk = (int)bal.ldk;
           optasks.push_back(t);
         }
       const double e = (double)R * K;
@@ -964,7 +1005,8 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       // W(r, c) -= L(r, blk) W(blk, c) for r >= b1 > c
       if ((o + nb) % kOzBlock == 0) {
         const int b0 = o + nb - kOzBlock, b1 = o + nb;
-        Launch lp{OZPACK, f0, (int64_t)optasks.size(), 0, kb}, lt{OZGEMM, f0, (int64_t)otasks.size(), 0, kb};
+        Launch lx{OZCOL, f0, (int64_t)octasks.size(), 0, kb}, lp{OZPACK, f0, (int64_t)optasks.size(), 0, kb},
+            lt{OZGEMM, f0, (int64_t)otasks.size(), 0, kb};
         for (int f : ord) {
           const auto& ft = fronts[f0 + f];
           if (!blocks[f0 + f] || ft.s <= b1) continue;
@@ -974,10 +1016,13 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
           unsigned char* LB = LA + oz_bytes(R, kOzBlock, false) + oz_exps(R, kOzBlock, false);
           unsigned char* WB = LB + oz_bytes(R, kOzBlock, true) + oz_exps(R, kOzBlock, true);
           T* blk = ft.G + b0 * ld;
-          lp.bytes += oz_pack(blk + b1, blk + b0, ld + 1, LD, ld, R, kOzBlock, TC_PACK_PLAIN, false);
-          lp.bytes += oz_pack(blk + b1, nullptr, 0, LA, ld, R, kOzBlock, TC_PACK_PLAIN, false);
-          lp.bytes += oz_pack(blk + b1, nullptr, 0, LB, ld, R, kOzBlock, TC_PACK_PLAIN, true);
-          lp.bytes += oz_pack(ft.W + b0, nullptr, 0, WB, ft.s, b1, kOzBlock, TC_PACK_TRANSPOSED, true);
+          const Balance with_d{nullptr, nullptr, blk + b0, ld + 1}, with_w{kx[f0 + f], kx[f0 + f] + kOzBlock, nullptr, 0};
+          lx.bytes += oz_colmax(blk + b1, ld, R, kOzBlock, TC_PACK_PLAIN, kx[f0 + f]);
+          lx.bytes += oz_colmax(ft.W + b0, ft.s, b1, kOzBlock, TC_PACK_TRANSPOSED, kx[f0 + f] + kOzBlock);
+          lp.bytes += oz_pack(blk + b1, blk + b0, ld + 1, LD, ld, R, kOzBlock, TC_PACK_PLAIN, false, with_d);
+          lp.bytes += oz_pack(blk + b1, nullptr, 0, LA, ld, R, kOzBlock, TC_PACK_PLAIN, false, with_w);
+          lp.bytes += oz_pack(blk + b1, nullptr, 0, LB, ld, R, kOzBlock, TC_PACK_PLAIN, true, with_d);
+          lp.bytes += oz_pack(ft.W + b0, nullptr, 0, WB, ft.s, b1, kOzBlock, TC_PACK_TRANSPOSED, true, with_w);
           for (int tj = 0; tj < R; tj += oz.tile_n)
             for (int ti = tj / oz.tile_m * oz.tile_m; ti < R; ti += oz.tile_m)
               oz_tile(LD, R, LB, R, kOzBlock, ti, tj, ft.G + (b1 + tj) * ld + b1 + ti, (int)ld, 0, kOzBlock,
@@ -988,11 +1033,13 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
           lt.flops += 8.0 * kOzBlock * R * (R + 1.0) / 2;
           lt.extra += 8.0 * R * ((double)kOzBlock * b0 + kOzBlock * (kOzBlock + 1.0) / 2);
         }
+        lx.count = (int)(octasks.size() - lx.off);
         lp.count = (int)(optasks.size() - lp.off);
         lt.count = (int)(otasks.size() - lt.off);
         for (size_t i = lt.off; i < otasks.size(); ++i)
           lt.bytes += (double)otasks[i].nkb * (oz.a_block + oz.b_block) + 32.0 * otasks[i].m * otasks[i].n;
         if (lt.count > 0) {
+          launches.push_back(lx);
           launches.push_back(lp);
           launches.push_back(lt);
         }
@@ -1261,10 +1308,11 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       }
       if constexpr (std::is_same<T, double2>::value) {
         // complex128 fronts on the tensor cores.  Phase 0: F_BL (A) and inv(L) (B), Z = F_BL inv(L)^T.  Phase 1: Z D^-1 in
-        // F_BL's place and Z (B), the Schur update; then (extended form) inv(L)^T in inv(L)'s place and M_BL.
+        // F_BL's place and Z (B), the Schur update; then (extended form) Z D^-1 again, balanced against inv(L)^T, and
+        // inv(L)^T in inv(L)'s place, M_BL.  The Schur update's operands are balanced by their pivots alone.
         for (int step = 0; step < (phase == 0 ? 1 : si == PSP_SI_EXTENDED ? 2 : 1); ++step) {
-          const int64_t op0 = (int64_t)optasks.size(), o0 = (int64_t)otasks.size();
-          Launch lp{OZPACK, f0, op0, 0, -1}, lt{OZGEMM, f0, o0, 0, -1};
+          const int64_t op0 = (int64_t)optasks.size(), o0 = (int64_t)otasks.size(), oc0 = (int64_t)octasks.size();
+          Launch lx{OZCOL, f0, oc0, 0, -1}, lp{OZPACK, f0, op0, 0, -1}, lt{OZGEMM, f0, o0, 0, -1};
           for (int f : ord) {
             const auto& ft = fronts[f0 + f];
             if (ft.u == 0 || !packs[f0 + f]) continue;
@@ -1273,30 +1321,40 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
             unsigned char* PA = packs[f0 + f];
             unsigned char* PB = PA + (oz_bytes(u_, s_, false) + oz_exps(u_, s_, false));
             unsigned char* PL = PB + (oz_bytes(u_, s_, true) + oz_exps(u_, s_, true));
+            int* const kx0 = kx[f0 + f];
             if (phase == 0) {
-              lp.bytes += oz_pack(ft.G + ft.s, nullptr, 0, PA, ld, u_, s_, TC_PACK_PLAIN, false);
-              lp.bytes += oz_pack(ft.G, nullptr, 0, PL, ld, s_, s_, TC_PACK_UNIT_LOWER, true);
+              const Balance bal{kx0, kx0 + s_, nullptr, 0};
+              lx.bytes += oz_colmax(ft.G + ft.s, ld, u_, s_, TC_PACK_PLAIN, kx0);
+              lx.bytes += oz_colmax(ft.G, ld, s_, s_, TC_PACK_UNIT_LOWER, kx0 + s_);
+              lp.bytes += oz_pack(ft.G + ft.s, nullptr, 0, PA, ld, u_, s_, TC_PACK_PLAIN, false, bal);
+              lp.bytes += oz_pack(ft.G, nullptr, 0, PL, ld, s_, s_, TC_PACK_UNIT_LOWER, true, bal);
               for (int tj = 0; tj < ft.s; tj += oz.tile_n)
                 for (int ti = 0; ti < ft.u; ti += oz.tile_m)
                   oz_tile(PA, u_, PL, s_, s_, ti, tj, ft.Z + (int64_t)tj * ft.u + ti, ft.u, 0,
                           std::min<int64_t>(tj + oz.tile_n, s_), kAll, GF_BETA0);
               lt.flops += 8.0 * u_ * s_ * (s_ + 1.0) / 2;
             } else if (step == 0) {
-              lp.bytes += oz_pack(ft.Z, ft.dinv, 1, PA, u_, u_, s_, TC_PACK_PLAIN, false);
-              lp.bytes += oz_pack(ft.Z, nullptr, 0, PB, u_, u_, s_, TC_PACK_PLAIN, true);
+              const Balance bal{nullptr, nullptr, ft.dinv, 1};
+              lp.bytes += oz_pack(ft.Z, ft.dinv, 1, PA, u_, u_, s_, TC_PACK_PLAIN, false, bal);
+              lp.bytes += oz_pack(ft.Z, nullptr, 0, PB, u_, u_, s_, TC_PACK_PLAIN, true, bal);
               for (int tj = 0; tj < ft.u; tj += oz.tile_n)
                 for (int ti = tj / oz.tile_m * oz.tile_m; ti < ft.u; ti += oz.tile_m)
                   oz_tile(PA, u_, PB, u_, s_, ti, tj, ft.U + upd_index(std::max(ti, tj), tj, ft.u, 128) - std::max(0, tj - ti),
                           128, 0, s_, ti > tj ? kAll : ti - tj, GF_NEG);
               lt.flops += 8.0 * s_ * u_ * (u_ + 1.0) / 2;
             } else {
-              lp.bytes += oz_pack(ft.G, nullptr, 0, PL, ld, s_, s_, TC_PACK_UNIT_LOWER_T, true);
+              const Balance bal{kx0 + 2 * s_, kx0 + 3 * s_, ft.dinv, 1};
+              lx.bytes += oz_colmax(ft.Z, u_, u_, s_, TC_PACK_PLAIN, kx0 + 2 * s_);
+              lx.bytes += oz_colmax(ft.G, ld, s_, s_, TC_PACK_UNIT_LOWER_T, kx0 + 3 * s_);
+              lp.bytes += oz_pack(ft.Z, ft.dinv, 1, PA, u_, u_, s_, TC_PACK_PLAIN, false, bal);
+              lp.bytes += oz_pack(ft.G, nullptr, 0, PL, ld, s_, s_, TC_PACK_UNIT_LOWER_T, true, bal);
               for (int tj = 0; tj < ft.s; tj += oz.tile_n)
                 for (int ti = 0; ti < ft.u; ti += oz.tile_m)
                   oz_tile(PA, u_, PL, s_, s_, ti, tj, ft.G + (int64_t)tj * ld + ft.s + ti, ld, tj, s_, kAll, GF_BETA0);
               lt.extra += 8.0 * u_ * s_ * (s_ + 1.0) / 2;   // M_BL: selective inversion
             }
           }
+          lx.count = (int)(octasks.size() - oc0);
           lp.count = (int)(optasks.size() - op0);
           lt.count = (int)(otasks.size() - o0);
           for (size_t i = o0; i < otasks.size(); ++i)
@@ -1305,6 +1363,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
             otasks[o0].flags |= GF_TEST_STALL;
             stall_next = false;
           }
+          launches.push_back(lx);
           launches.push_back(lp);
           launches.push_back(lt);
         }

@@ -242,6 +242,16 @@ struct OzPackTask {        // 128 rows x 128 k of an operand
   int ld, lds, r0, k0, R, K;   // first row / k, source extents (outside -> 0)
   int mode;                // TcPackMode (TRANSPOSED: X[k, r])
   int rows_b;              // 0: A operand (128-row blocks), 1: B operand (32-row blocks)
+  const int* ka;           // balance of the product's columns k (k_oz_pack): exponents of A's columns before its scale ...
+  const int* kb;           // ... and of B's (both nullptr: taken as equal)
+  const double2* kd;       // A's scale, stride ldk (nullptr: none)
+  int ldk, pad_;
+};
+struct OzColTask {         // 32 columns k of an operand: exponents of their largest entries
+  const double2* src;
+  int* out;                // out[k]
+  int ld, k0, R, K, mode;  // as in OzPackTask
+  int pad_;
 };
 struct OzGemmTask {        // one 128 x 32 tile of C (+)= +-A B^T
   const unsigned char* A;  // block of 16 k number 0 of its 128 rows
@@ -255,6 +265,7 @@ struct OzGemmTask {        // one 128 x 32 tile of C (+)= +-A B^T
   int flags;               // GF_NEG, GF_BETA0
   int pad_;
 };
+void launch_oz_colmax(const OzColTask* tasks, int ntasks, cudaStream_t st);
 void launch_oz_pack(const OzPackTask* tasks, int ntasks, cudaStream_t st);
 void launch_oz_gemm(const OzGemmTask* tasks, int ntasks, int* status, cudaStream_t st);
 int tc_block_k();
