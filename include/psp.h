@@ -116,8 +116,13 @@ typedef struct {
   int sweep_ctas_per_sm; /* sweep schedule: resident CTAs per SM of the persistent sweep (capped by
                             occupancy); <= 0 selects the default (8) */
   int setup_temp_mb;   /* cap, in MiB, on the per-front temporaries of one batch of fronts during setup
-                          (a level whose fronts need more is factored in several batches); <= 0: up
-                          to 80 % of the device memory left after the factors and update matrices */
+                          (a level whose fronts need more is factored in several batches, and a complex128
+                          front whose tensor-core operands need more takes its products in pieces; neither
+                          changes a result.  A front that needs more on CUDA cores takes that; one that has
+                          room for no piece stays on CUDA cores); <= 0: up to 80 % of the device memory
+                          left after the factors and update matrices.  Where an allocation is refused, setup
+                          tries again with less, last with complex128 products on CUDA cores.  psp_stats gives
+                          the bytes taken (host:alloc_work) and the tensor-core launches (k_oz_gemm) */
   int sweep_rhs_group; /* sweep schedule: most right-hand sides (1, 2, 4 or 8; complex128 factors: at most 4) one
                           CTA carries through a pass over a factor block; <= 0: as many as the application has, at
                           most 8 (the task's vector is staged through shared memory in chunks) */

@@ -406,9 +406,18 @@ constexpr int kOzMinDim = 16;   // complex128: fewest s and u of a front on the 
 // root of each panel, 960 rows).  Below two blocks there is no second one to update
 constexpr int kOzBlock = 128, kOzBlockMin = 256;
 
-// `while_device_runs` is host work done after the last launch is enqueued, before waiting for them.
+// How a factorisation used its temporaries, for the next attempt when device memory ran out
+struct TempUse {
+  int64_t budget = 0;      // elements taken for them (0: memory ran out before)
+  int64_t front_max = 16;  // what the widest front needs on CUDA cores
+  bool digits = false;     // some front took the complex128 tensor-core products
+};
+
+// `while_device_runs` is host work done after the last launch is enqueued, before waiting for them; the temporaries take at most
+// temp_limit elements (but what the widest front needs on CUDA cores), `digits`: complex128 fronts may take the tensor cores.
 template <typename T>
-static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()>& while_device_runs) {
+static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<void()>& while_device_runs, int64_t temp_limit,
+                           bool digits, TempUse& use) {
   auto tp = std::chrono::steady_clock::now();
   const int nb = 32;
   const double tiny = sizeof(T) == 16 ? 1e-300 : 1e-30;
@@ -444,8 +453,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   // complex128: fronts of at least kOzMinDim rows each way run the same products on the tensor cores from exact digit
   // products; below that the tiles are mostly padding (128 x 32 outputs, k in 16s), and there is next to no work
   const OzShape oz = oz_shape();
-  bool oz_ok = std::is_same<T, double2>::value && X->use_tc && si != PSP_SI_NONE;
-  auto use_oz = [&](int64_t s_, int64_t u_) { return oz_ok && s_ >= kOzMinDim && u_ >= kOzMinDim; };
+  const bool oz_ok = std::is_same<T, double2>::value && X->use_tc && si != PSP_SI_NONE && digits;
   auto cdiv_i = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
   // bytes of a packed operand of R rows and K columns and of its row exponents (A: 128-row blocks, B: 32-row blocks)
   auto oz_bytes = [&](int64_t R, int64_t K, bool b) {
@@ -454,34 +462,65 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   auto oz_exps = [&](int64_t R, int64_t K, bool b) {
     return (int64_t)sizeof(int) * cdiv_i(R, b ? oz.tile_n : oz.tile_m) * cdiv_i(K, oz.kc) * (b ? oz.tile_n : oz.tile_m);
   };
-  // exponents of the columns of four operands (the products' balance): 4 ints = one element per row of S
-  auto kx_elems = [&](int64_t s_) { return pad16(s_); };
-  // F_BL and, once Z is made, Z D^-1 in its place (A operands); inv(L); Z; inv(L)^T (extended form)
-  auto oz_elems = [&](int64_t s_, int64_t u_) {
-    int64_t b = oz_bytes(u_, s_, false) + oz_exps(u_, s_, false) + oz_bytes(u_, s_, true) + oz_exps(u_, s_, true) +
-                oz_bytes(s_, s_, true) + oz_exps(s_, s_, true);
-    return pad16(cdiv_i(b, (int64_t)sizeof(T)) + 64);
-  };
-  auto in_blocks = [&](int64_t s_) { return oz_ok && s_ >= kOzBlockMin; };
-  // packed operands of one block of 128 columns: L D and L of the rows below (A), L again and W's block row (B)
-  auto block_elems = [&](int64_t s_) {
-    const int64_t b = 2 * (oz_bytes(s_, kOzBlock, false) + oz_exps(s_, kOzBlock, false)) +
-                      2 * (oz_bytes(s_, kOzBlock, true) + oz_exps(s_, kOzBlock, true));
-    return pad16(cdiv_i(b, (int64_t)sizeof(T)) + 64);
-  };
+  // bytes of an operand with its row exponents
+  auto oz_size = [&](int64_t R, int64_t K, bool b) { return oz_bytes(R, K, b) + oz_exps(R, K, b); };
   auto nrb = [](int64_t r) { return (r + 127) / 128; };
   auto nkb16 = [](int64_t k) { return (k + 15) / 16; };
   auto packed_elems = [&](int64_t s_, int64_t u_) {   // F_BL, Z D^-1, Z (u x s) and two inv(L) (s x s)
     return TBLK * (3 * nrb(u_) * nkb16(s_) + 2 * nrb(s_) * nkb16(s_));
   };
-  auto front_temp = [&](int64_t s_, int64_t u_) {     // W (s x s), Z (u x s), Z D^-1 or packed operands,
-    if (si == PSP_SI_NONE) return (int64_t)0;         // the second inverse under construction (s x s)
-    return pad16(s_ * s_) + pad16(u_ * s_) + (si == PSP_SI_TWO ? pad16(s_ * s_) : 0) + (in_blocks(s_) ? block_elems(s_) : 0) +
-           (use_oz(s_, u_) || in_blocks(s_) ? kx_elems(s_) : 0) +
-           (use_tc(s_, u_) ? packed_elems(s_, u_)
-            : use_oz(s_, u_) ? oz_elems(s_, u_)
-                             : si == PSP_SI_EXTENDED ? pad16(u_ * s_) : 0);
+  // A front's temporaries, in elements: W and the second inverse under construction (s x s each), Z (u x s) and Z D^-1 or
+  // packed operands.  Operands of the complex128 products lie where nothing else is alive: while F_TL is factored beyond W
+  // and the second inverse, in Z's place too, and once these are copied into the factor in their place, up to Z.  Such a
+  // front may take `allowed` elements: the limit, or what it needs on CUDA cores if that is more.  Within that its products
+  // run in one piece or in several (oz_product), with the same sums; a front that has no room for the smallest pieces
+  // stays on CUDA cores.
+  struct FrontTemp {
+    int64_t total;            // elements
+    bool oz, blocks;          // complex128: front products, F_TL's blocks of 128 columns on the tensor cores
+    int64_t w, tail, kx;      // W and the second inverse at the start; Z (and Z D^-1) and the column exponents at the end
   };
+  int64_t limit = X->temp_budget_elems > 0 ? std::min(temp_limit, X->temp_budget_elems) : temp_limit;
+  auto cuda_core_temp = [&](int64_t s_, int64_t u_) {
+    return pad16(s_ * s_) * (si == PSP_SI_TWO ? 2 : 1) + pad16(u_ * s_) * (si == PSP_SI_EXTENDED ? 2 : 1);
+  };
+  auto front_temp = [&](int64_t s_, int64_t u_) {
+    FrontTemp t{};
+    if (si == PSP_SI_NONE) return t;
+    t.w = pad16(s_ * s_) * (si == PSP_SI_TWO ? 2 : 1);
+    const int64_t z = pad16(u_ * s_);
+    if (use_tc(s_, u_)) {
+      t.tail = z + packed_elems(s_, u_);
+      t.total = t.w + t.tail;
+      return t;
+    }
+    t.total = cuda_core_temp(s_, u_);
+    t.tail = t.total - t.w;
+    const bool oz_dims = oz_ok && s_ >= kOzMinDim && u_ >= kOzMinDim, block_dims = oz_ok && s_ >= kOzBlockMin;
+    if (!oz_dims && !block_dims) return t;
+    const int64_t allowed = std::max(limit, t.total), kx = pad16(s_), tail = oz_dims ? z : t.tail;
+    auto elems = [&](int64_t bytes) { return pad16(cdiv_i(bytes, (int64_t)sizeof(T))); };
+    const int64_t A = oz.tile_m, B = oz.tile_n, K = std::min<int64_t>(s_, oz.kc), kb = kOzBlock;
+    int64_t in_f_tl = 0, in_f_tl_min = 0, in_front = 0, in_front_min = 0;
+    if (block_dims) {   // L D and L again, L and W's block row
+      in_f_tl = elems(2 * oz_size(s_ - kb, kb, false) + oz_size(s_, kb, true));
+      in_f_tl_min = elems(oz_size(A, kb, false) + oz_size(B, kb, true));
+    }
+    if (oz_dims) {      // F_BL or Z D^-1, and inv(L), Z or inv(L)^T
+      in_front = elems(oz_size(u_, s_, false) + std::max(oz_size(u_, s_, true), oz_size(s_, s_, true)));
+      in_front_min = elems(oz_size(A, K, false) + oz_size(B, K, true));
+    }
+    const int64_t full = kx + std::max(t.w + std::max(tail, in_f_tl), in_front + tail);
+    const int64_t least = kx + std::max(t.w + std::max(tail, in_f_tl_min), in_front_min + tail);
+    if (least > allowed) return t;
+    t.oz = oz_dims;
+    t.blocks = block_dims;
+    t.tail = tail;
+    t.kx = kx;
+    t.total = std::min(full, allowed / 16 * 16);
+    return t;
+  };
+  auto use_oz = [&](int64_t s_, int64_t u_) { return oz_ok && front_temp(s_, u_).oz; };
   int64_t arena[2] = {0, 0}, temp_level_max = 0, temp_front_max = 16;
   auto plan_memory = [&] {
     arena[0] = arena[1] = temp_level_max = 0;
@@ -495,7 +534,10 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
           uoff[X->sn_base[p] + sn] = slab;
           slab += pad16(upd_packed_elems((int)u, use_tc(s, u) || use_oz(s, u) ? 128 : 64));
         }
-        const int64_t t = front_temp(s, u);
+        const FrontTemp ft = front_temp(s, u);
+        const int64_t t = ft.total;
+        use.digits = use.digits || ft.oz || ft.blocks;
+        if (si != PSP_SI_NONE) use.front_max = std::max(use.front_max, use_tc(s, u) ? t : cuda_core_temp(s, u));
         tsum += t;
         temp_front_max = std::max(temp_front_max, t);
       }
@@ -504,12 +546,18 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
     }
   };
   plan_memory();
-  if (oz_ok) {   // where the device has no room for the widest front's packed operands, every product stays on FP64 units
+  // where the device has no room for the widest front's packed operands, its products take smaller pieces.  What a caller's
+  // allocator holds is not in these figures: it is asked, and factor_all takes less when it refuses
+  if (use.digits && !(g_alloc && g_alloc->alloc)) {
     size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
-        (double)(arena[0] + arena[1] + temp_front_max) * sizeof(T) > 0.8 * ((double)free_b - 2.0e9)) {
-      oz_ok = false;
-      plan_memory();
+    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
+      const double room = 0.8 * ((double)free_b - 2.0e9) / sizeof(T) - (double)(arena[0] + arena[1]);
+      if ((double)temp_front_max > room) {
+        limit = std::min(limit, (int64_t)std::max(0.0, room));
+        plan_memory();
+      }
+    } else {
+      cudaGetLastError();
     }
   }
   X->upd_arena_elems = arena[0] + arena[1];
@@ -519,19 +567,20 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   d_upd.alloc((size_t)std::max<int64_t>(X->upd_arena_elems, 16) * sizeof(T));
   // per-front temporaries of one group of a level; a level whose temporaries exceed what the device
   // has left is processed in several groups
-  int64_t temp_budget = temp_level_max;
+  int64_t temp_budget = std::max(temp_front_max, std::min(temp_level_max, limit));
   {
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
       const double avail = 0.8 * ((double)free_b - 2.0e9);
       const int64_t cap = (int64_t)std::max(0.0, avail / (double)sizeof(T));
-      if (X->temp_budget_elems > 0) temp_budget = std::min(temp_budget, X->temp_budget_elems);
       temp_budget = std::max(temp_front_max, std::min(temp_budget, cap));
     } else {
       cudaGetLastError();
     }
   }
+  use.budget = temp_budget;
   d_temp.alloc((size_t)std::max<int64_t>(temp_budget, 16) * sizeof(T));
+  X->stats.k["host:alloc_work"].bytes = (double)d_temp.bytes;
   X->stats.host("alloc_work", ms_since(tp));
   tp = std::chrono::steady_clock::now();
   std::vector<std::vector<std::pair<int, int>>> groups;   // (panel, sn) lists, in level order
@@ -540,7 +589,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
     bool fresh = true;   // every level starts a new group
     for (auto [p, sn] : lev_fronts[lv]) {
       const Shape& sh = X->shapes[X->shape_of[p]];
-      const int64_t t = front_temp(sh.s[sn], sh.u[sn]);
+      const int64_t t = front_temp(sh.s[sn], sh.u[sn]).total;
       if (fresh || run + t > temp_budget) {
         groups.emplace_back();
         run = 0;
@@ -583,13 +632,17 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
     double flops = 0, bytes = 0;
     double extra = 0;   // selective-inversion flops (not part of the algorithmic count)
   };
+  struct Region {
+    unsigned char* p = nullptr;
+    int64_t bytes = 0;
+  };
   struct Tasks {
     std::vector<FrontTask<T>> fronts;
     std::vector<ColTask> ctasks;
     std::vector<int> dlist;
     std::vector<GemmTask<T>> gtasks;
-    std::vector<unsigned char*> packs;   // per front: base of its packed operands (tensor-core fronts)
-    std::vector<unsigned char*> blocks;  // per front: base of a block's packed operands (fronts factored in blocks of 128)
+    std::vector<Region> packs;           // per front: place of its packed operands (tensor-core fronts)
+    std::vector<Region> blocks;          // per front: place of a block's packed operands (fronts factored in blocks of 128)
     std::vector<int*> kx;                // per front: column exponents of its digit products' operands
     std::vector<TcPackTask> ptasks;
     std::vector<TcGemmTask> ttasks;
@@ -744,40 +797,28 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       ft.dinv = X->d_dinv.as<T>() + X->panel_dbase[p] + sh.first[sn];
       ft.W = ft.Z = ft.ZD = ft.W2 = nullptr;
       ft.ldzd = ft.u;
-      packs.push_back(nullptr);
-      blocks.push_back(nullptr);
+      packs.push_back({});
+      blocks.push_back({});
       kx.push_back(nullptr);
       if (si != PSP_SI_NONE) {
-        ft.W = tbase + toff;
-        toff += pad16((int64_t)ft.s * ft.s);
-        ft.Z = tbase + toff;
-        toff += pad16((int64_t)ft.u * ft.s);
-        if (use_tc(ft.s, ft.u)) {
-          packs.back() = reinterpret_cast<unsigned char*>(tbase + toff);
-          toff += packed_elems(ft.s, ft.u);
-        } else if (use_oz(ft.s, ft.u)) {
-          packs.back() = reinterpret_cast<unsigned char*>(tbase + toff);
-          toff += oz_elems(ft.s, ft.u);
-        } else if (si == PSP_SI_EXTENDED) {
-          ft.ZD = tbase + toff;
-          toff += pad16((int64_t)ft.u * ft.s);
-        }
+        const FrontTemp tp_ = front_temp(ft.s, ft.u);
+        T* const base = tbase + toff;
+        toff += tp_.total;
+        T* const tail = base + tp_.total - tp_.kx - tp_.tail;
+        auto region = [&](T* from, T* to) { return Region{reinterpret_cast<unsigned char*>(from), (to - from) * (int64_t)sizeof(T)}; };
+        ft.W = base;
+        if (si == PSP_SI_TWO) ft.W2 = base + pad16((int64_t)ft.s * ft.s);
+        ft.Z = tail;
+        T* const rest = tail + pad16((int64_t)ft.u * ft.s);
+        if (use_tc(ft.s, ft.u)) packs.back() = region(rest, tail + tp_.tail);
+        else if (tp_.oz) packs.back() = region(base, tail);
+        else if (si == PSP_SI_EXTENDED) ft.ZD = rest;
         if (si == PSP_SI_PAPER || si == PSP_SI_TWO) {   // L_BL = Z D^{-1} is the factor's bottom block
           ft.ZD = ft.G + ft.s;
           ft.ldzd = ft.s + ft.u;
         }
-        if (si == PSP_SI_TWO) {
-          ft.W2 = tbase + toff;
-          toff += pad16((int64_t)ft.s * ft.s);
-        }
-        if (in_blocks(ft.s)) {
-          blocks.back() = reinterpret_cast<unsigned char*>(tbase + toff);
-          toff += block_elems(ft.s);
-        }
-        if (use_oz(ft.s, ft.u) || in_blocks(ft.s)) {
-          kx.back() = reinterpret_cast<int*>(tbase + toff);
-          toff += kx_elems(ft.s);
-        }
+        if (tp_.kx > 0) kx.back() = reinterpret_cast<int*>(base + tp_.total - tp_.kx);
+        if (tp_.blocks) blocks.back() = region(base + tp_.w, base + tp_.total - tp_.kx);
       }
       fronts.push_back(ft);
       smax = std::max(smax, ft.s);
@@ -834,55 +875,155 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       const T* kd = nullptr;
       int64_t ldk = 0;
     };
-    // packs an operand (R rows, K columns; columns times scale[k lds_]) of the complex128 tensor-core products; returns its bytes
-    auto oz_pack = [&](const T* src, const T* scale, int64_t lds_, unsigned char* dst, int64_t ld_, int64_t R, int64_t K, int mode, bool b,
-                       const Balance& bal) {
-      const int64_t nkb = cdiv_i(K, oz.k), nkc = cdiv_i(K, oz.kc), rows = b ? oz.tile_n : oz.tile_m;
-      int* exps = reinterpret_cast<int*>(dst + oz_bytes(R, K, b));
-      for (int64_t r0 = 0; r0 < R; r0 += oz.tile_m)
-        for (int64_t kc = 0; kc < nkc; ++kc) {
-          OzPackTask t{};
-          t.src = reinterpret_cast<const double2*>(src);
-          t.scale = reinterpret_cast<const double2*>(scale);
-          t.lds = (int)lds_;
-          t.dst = dst + (r0 / rows * nkb + kc * (oz.kc / oz.k)) * (b ? oz.b_block : oz.a_block);
-          t.exps = exps + (r0 / rows * nkc + kc) * rows;
-          t.sub_stride = nkb * oz.b_block;
-          t.exp_stride = nkc * oz.tile_n;
-          t.ld = (int)ld_;
-          t.r0 = (int)r0;
-          t.k0 = (int)(kc * oz.kc);
-          t.R = (int)R;
-          t.K = (int)K;
-          t.mode = mode;
-          t.rows_b = b;
-          t.ka = bal.ka;
-          t.kb = bal.kb;
-          t.kd = reinterpret_cast<const double2*>(bal.kd);
-          t.ldk = (int)bal.ldk;
-          optasks.push_back(t);
-        }
-      const double e = (double)R * K;
-      return e * (16.0 + (double)(b ? oz.b_block / (oz.tile_n * oz.k) : oz.a_block / (oz.tile_m * oz.k)));
+    // The complex128 tensor-core products of one step: C = +-A B^T, A of RA rows (src, ld, its columns k times
+    // scale[k lds]) and B of RB rows, over K columns.  tile(ti, tj, t) says whether a tile exists and gives its place
+    // in C, the columns [k0, k1) it sums and its flags.
+    struct OzOperand {
+      const T* src;
+      int64_t ld, R;
+      int mode;
+      const T* scale = nullptr;
+      int64_t lds = 0;
     };
-    // tiles of C (R x N) = +-A B^T with k in [klo(col), khi(col))
-    auto oz_tile = [&](unsigned char* A, int64_t RA, unsigned char* B, int64_t RB, int64_t K, int ti, int tj, T* C, int ldc,
-                       int64_t k0, int64_t k1, int doff, int flags) {
-      const int64_t nkb = cdiv_i(K, oz.k), nkc = cdiv_i(K, oz.kc);
-      OzGemmTask t{};
-      t.A = A + ti / oz.tile_m * nkb * oz.a_block;
-      t.B = B + tj / oz.tile_n * nkb * oz.b_block;
-      t.ea = reinterpret_cast<const int*>(A + oz_bytes(RA, K, false)) + ti / oz.tile_m * nkc * oz.tile_m;
-      t.eb = reinterpret_cast<const int*>(B + oz_bytes(RB, K, true)) + tj / oz.tile_n * nkc * oz.tile_n;
-      t.C = reinterpret_cast<double2*>(C);
-      t.ldc = ldc;
-      t.m = (int)std::min<int64_t>(oz.tile_m, RA - ti);
-      t.n = (int)std::min<int64_t>(oz.tile_n, RB - tj);
-      t.kb0 = (int)(k0 / oz.k);
-      t.nkb = (int)(cdiv_i(k1, oz.k) - k0 / oz.k);
-      t.doff = doff;
-      t.flags = flags;
-      otasks.push_back(t);
+    struct OzTile {
+      T* C;
+      int64_t ldc, k0, k1;
+      int doff, flags;
+    };
+    // Passes of a step beyond the first (whose tasks go straight to the lists): a front whose operands do not fit their
+    // place at once takes a pass for each piece, packed where the piece before it was
+    struct OzPass {
+      std::vector<OzPackTask> packs;
+      std::vector<OzGemmTask> tiles;
+    };
+    std::vector<OzPass> more;
+    struct OzPlace {   // where a front packs in a step: the pass and what that pass has taken of the region
+      Region rg;
+      size_t pass = 0;
+      int64_t off = 0;
+    };
+    auto oz_piece = [&](const OzOperand& A, const OzOperand& B, int64_t K, const Balance& bal, auto&& tile, OzPlace& at, int64_t ra,
+                        int64_t rb, int64_t ca, int64_t cb, int64_t ka, int64_t kb_) {
+      if (at.pass > more.size()) more.resize(at.pass);
+      std::vector<OzPackTask>& op = at.pass == 0 ? optasks : more[at.pass - 1].packs;
+      std::vector<OzGemmTask>& ot = at.pass == 0 ? otasks : more[at.pass - 1].tiles;
+      const int64_t nkb = cdiv_i(kb_ - ka, oz.k), nkc = cdiv_i(kb_ - ka, oz.kc);
+      unsigned char* const PA = at.rg.p + at.off;
+      unsigned char* const PB = PA + oz_size(rb - ra, kb_ - ka, false);
+      int* const EA = reinterpret_cast<int*>(PA + oz_bytes(rb - ra, kb_ - ka, false));
+      int* const EB = reinterpret_cast<int*>(PB + oz_bytes(cb - ca, kb_ - ka, true));
+      const size_t first = ot.size();
+      for (int64_t tj = ca; tj < cb; tj += oz.tile_n)
+        for (int64_t ti = ra; ti < rb; ti += oz.tile_m) {
+          OzTile w{};
+          if (!tile(ti, tj, w)) continue;
+          const int64_t k0 = std::max(w.k0, ka), k1 = std::min(w.k1, kb_);
+          if (k0 >= k1) continue;
+          OzGemmTask t{};
+          t.A = PA + (ti - ra) / oz.tile_m * nkb * oz.a_block;
+          t.B = PB + (tj - ca) / oz.tile_n * nkb * oz.b_block;
+          t.ea = EA + (ti - ra) / oz.tile_m * nkc * oz.tile_m;
+          t.eb = EB + (tj - ca) / oz.tile_n * nkc * oz.tile_n;
+          t.C = reinterpret_cast<double2*>(w.C);
+          t.ldc = (int)w.ldc;
+          t.m = (int)std::min<int64_t>(oz.tile_m, A.R - ti);
+          t.n = (int)std::min<int64_t>(oz.tile_n, B.R - tj);
+          t.kb0 = (int)((k0 - ka) / oz.k);
+          t.nkb = (int)(cdiv_i(k1 - ka, oz.k) - t.kb0);
+          t.doff = w.doff;
+          t.flags = k0 > w.k0 ? w.flags & ~GF_BETA0 : w.flags;   // a later piece adds to the ones before it
+          ot.push_back(t);
+        }
+      if (ot.size() == first) return false;
+      auto pack = [&](const OzOperand& X_, bool b, unsigned char* dst, int* exps, int64_t r_first, int64_t r_end) {
+        const int64_t rows = b ? oz.tile_n : oz.tile_m, block = b ? oz.b_block : oz.a_block;
+        for (int64_t r0 = r_first; r0 < r_end; r0 += oz.tile_m)
+          for (int64_t k0 = ka; k0 < kb_; k0 += oz.kc) {
+            OzPackTask t{};
+            t.src = reinterpret_cast<const double2*>(X_.src);
+            t.scale = reinterpret_cast<const double2*>(X_.scale);
+            t.lds = (int)X_.lds;
+            t.dst = dst + ((r0 - r_first) / rows * nkb + (k0 - ka) / oz.k) * block;
+            t.exps = exps + ((r0 - r_first) / rows * nkc + (k0 - ka) / oz.kc) * rows;
+            t.sub_stride = nkb * oz.b_block;
+            t.exp_stride = nkc * oz.tile_n;
+            t.ld = (int)X_.ld;
+            t.r0 = (int)r0;
+            t.k0 = (int)k0;
+            t.R = (int)r_end;
+            t.K = (int)K;
+            t.mode = X_.mode;
+            t.rows_b = b;
+            t.ka = bal.ka;
+            t.kb = bal.kb;
+            t.kd = reinterpret_cast<const double2*>(bal.kd);
+            t.ldk = (int)bal.ldk;
+            op.push_back(t);
+          }
+      };
+      pack(A, false, PA, EA, ra, rb);
+      pack(B, true, PB, EB, ca, cb);
+      return true;
+    };
+    // the whole product, in one piece where its operands fit beside what the pass has already taken, else in the next
+    // pass; where they fit no pass, first in pieces of fewer columns (nothing is packed twice), then of fewer rows too.
+    // A tile's sums run over the same 128 columns in the same order either way.  Returns the bytes of packing it once
+    auto oz_product = [&](const OzOperand& A, const OzOperand& B, int64_t K, const Balance& bal, auto&& tile, OzPlace& at) {
+      const int64_t need = oz_size(A.R, K, false) + oz_size(B.R, K, true);
+      if (at.off > 0 && at.off + need > at.rg.bytes) {
+        ++at.pass;
+        at.off = 0;
+      }
+      if (need <= at.rg.bytes) {
+        oz_piece(A, B, K, bal, tile, at, 0, A.R, 0, B.R, 0, K);
+        at.off += need;
+      } else {
+        const int64_t k1 = std::min<int64_t>(K, oz.kc), rowA = oz_size(oz.tile_m, k1, false), rowB = oz_size(oz.tile_n, k1, true);
+        const int64_t nA = cdiv_i(A.R, oz.tile_m), nB = cdiv_i(B.R, oz.tile_n), room = at.rg.bytes;
+        int64_t q = 1, a = nA, b = nB;   // 128s of columns, 128s of A's rows and 32s of B's per piece
+        if (nA * rowA + nB * rowB <= room) {
+          q = room / (nA * rowA + nB * rowB);
+        } else {
+          a = std::min(nA, std::max<int64_t>(1, (room - std::min(nB * rowB, room / 2)) / rowA));
+          b = std::min(nB, std::max<int64_t>(1, (room - a * rowA) / rowB));
+        }
+        for (int64_t ka = 0; ka < K; ka += q * oz.kc)
+          for (int64_t ra = 0; ra < A.R; ra += a * oz.tile_m)
+            for (int64_t ca = 0; ca < B.R; ca += b * oz.tile_n)
+              if (oz_piece(A, B, K, bal, tile, at, ra, std::min(A.R, ra + a * oz.tile_m), ca, std::min(B.R, ca + b * oz.tile_n), ka,
+                           std::min(K, ka + q * oz.kc)))
+                ++at.pass;
+      }
+      return (double)K * (A.R * (16.0 + oz.a_block / (oz.tile_m * oz.k)) + B.R * (16.0 + oz.b_block / (oz.tile_n * oz.k)));
+    };
+    // the launches of a step: its columns' exponents, then operands and tiles pass by pass
+    auto oz_launches = [&](Launch lx, Launch lp, Launch lt) {
+      lx.count = (int)(octasks.size() - lx.off);
+      lp.count = (int)(optasks.size() - lp.off);
+      lt.count = (int)(otasks.size() - lt.off);
+      if (lt.count == 0) return;
+      auto tile_bytes = [&](Launch& l) {
+        for (int64_t i = l.off; i < l.off + l.count; ++i)
+          l.bytes += (double)otasks[i].nkb * (oz.a_block + oz.b_block) + 32.0 * otasks[i].m * otasks[i].n;
+      };
+      if (stall_next) {
+        otasks[lt.off].flags |= GF_TEST_STALL;
+        stall_next = false;
+      }
+      tile_bytes(lt);
+      launches.push_back(lx);
+      launches.push_back(lp);
+      launches.push_back(lt);
+      for (const OzPass& m : more) {
+        Launch mp{OZPACK, lp.front_off, (int64_t)optasks.size(), (int)m.packs.size(), lp.kb};
+        Launch mt{OZGEMM, lt.front_off, (int64_t)otasks.size(), (int)m.tiles.size(), lt.kb};
+        optasks.insert(optasks.end(), m.packs.begin(), m.packs.end());
+        otasks.insert(otasks.end(), m.tiles.begin(), m.tiles.end());
+        tile_bytes(mt);
+        launches.push_back(mp);
+        launches.push_back(mt);
+      }
+      more.clear();
     };
     constexpr int kAll = 1 << 30;   // no triangle mask
     // blocked LDL^T of F_TL with the inverse of L_TL built alongside in W; without selective
@@ -939,7 +1080,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         const int bs = std::min(nb, ft.s - o);
         const int t0 = o + nb;  // first row/col of the trailing block
         // fronts factored in blocks of 128: only the block's own columns of F_TL and rows of W now
-        const int cmax = blocks[f0 + f] ? std::min(ft.s, (o / kOzBlock + 1) * kOzBlock) : ft.s;
+        const int cmax = blocks[f0 + f].p ? std::min(ft.s, (o / kOzBlock + 1) * kOzBlock) : ft.s;
         // F_TL trailing update: F(r, c) -= L(r, kb) D_kb L(c, kb)^T, lower
         tiles_lower(ft.G, ld, ft.s - t0, [&](T*, int, int ti, int tj, int mm, int nn) {
           if (t0 + tj >= cmax) return;
@@ -1009,40 +1150,33 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
             lt{OZGEMM, f0, (int64_t)otasks.size(), 0, kb};
         for (int f : ord) {
           const auto& ft = fronts[f0 + f];
-          if (!blocks[f0 + f] || ft.s <= b1) continue;
+          if (!blocks[f0 + f].p || ft.s <= b1) continue;
           const int64_t ld = ft.s + ft.u, R = ft.s - b1;
-          unsigned char* LD = blocks[f0 + f];
-          unsigned char* LA = LD + oz_bytes(R, kOzBlock, false) + oz_exps(R, kOzBlock, false);
-          unsigned char* LB = LA + oz_bytes(R, kOzBlock, false) + oz_exps(R, kOzBlock, false);
-          unsigned char* WB = LB + oz_bytes(R, kOzBlock, true) + oz_exps(R, kOzBlock, true);
           T* blk = ft.G + b0 * ld;
-          const Balance with_d{nullptr, nullptr, blk + b0, ld + 1}, with_w{kx[f0 + f], kx[f0 + f] + kOzBlock, nullptr, 0};
-          lx.bytes += oz_colmax(blk + b1, ld, R, kOzBlock, TC_PACK_PLAIN, kx[f0 + f]);
-          lx.bytes += oz_colmax(ft.W + b0, ft.s, b1, kOzBlock, TC_PACK_TRANSPOSED, kx[f0 + f] + kOzBlock);
-          lp.bytes += oz_pack(blk + b1, blk + b0, ld + 1, LD, ld, R, kOzBlock, TC_PACK_PLAIN, false, with_d);
-          lp.bytes += oz_pack(blk + b1, nullptr, 0, LA, ld, R, kOzBlock, TC_PACK_PLAIN, false, with_w);
-          lp.bytes += oz_pack(blk + b1, nullptr, 0, LB, ld, R, kOzBlock, TC_PACK_PLAIN, true, with_d);
-          lp.bytes += oz_pack(ft.W + b0, nullptr, 0, WB, ft.s, b1, kOzBlock, TC_PACK_TRANSPOSED, true, with_w);
-          for (int tj = 0; tj < R; tj += oz.tile_n)
-            for (int ti = tj / oz.tile_m * oz.tile_m; ti < R; ti += oz.tile_m)
-              oz_tile(LD, R, LB, R, kOzBlock, ti, tj, ft.G + (b1 + tj) * ld + b1 + ti, (int)ld, 0, kOzBlock,
-                      ti > tj ? kAll : ti - tj, GF_NEG);
-          for (int tj = 0; tj < b1; tj += oz.tile_n)
-            for (int ti = 0; ti < R; ti += oz.tile_m)
-              oz_tile(LA, R, WB, b1, kOzBlock, ti, tj, ft.W + (int64_t)tj * ft.s + b1 + ti, ft.s, 0, kOzBlock, kAll, GF_NEG);
+          int* const kx0 = kx[f0 + f];
+          lx.bytes += oz_colmax(blk + b1, ld, R, kOzBlock, TC_PACK_PLAIN, kx0);
+          lx.bytes += oz_colmax(ft.W + b0, ft.s, b1, kOzBlock, TC_PACK_TRANSPOSED, kx0 + kOzBlock);
+          OzPlace at{blocks[f0 + f]};
+          lp.bytes += oz_product(
+              OzOperand{blk + b1, ld, R, TC_PACK_PLAIN, blk + b0, ld + 1}, OzOperand{blk + b1, ld, R, TC_PACK_PLAIN}, kOzBlock,
+              Balance{nullptr, nullptr, blk + b0, ld + 1},
+              [&](int64_t ti, int64_t tj, OzTile& t) {
+                t = {ft.G + (b1 + tj) * ld + b1 + ti, ld, 0, kOzBlock, ti > tj ? kAll : (int)(ti - tj), GF_NEG};
+                return ti >= tj / oz.tile_m * oz.tile_m;
+              },
+              at);
+          lp.bytes += oz_product(
+              OzOperand{blk + b1, ld, R, TC_PACK_PLAIN}, OzOperand{ft.W + b0, ft.s, b1, TC_PACK_TRANSPOSED}, kOzBlock,
+              Balance{kx0, kx0 + kOzBlock, nullptr, 0},
+              [&](int64_t ti, int64_t tj, OzTile& t) {
+                t = {ft.W + tj * ft.s + b1 + ti, ft.s, 0, kOzBlock, kAll, GF_NEG};
+                return true;
+              },
+              at);
           lt.flops += 8.0 * kOzBlock * R * (R + 1.0) / 2;
           lt.extra += 8.0 * R * ((double)kOzBlock * b0 + kOzBlock * (kOzBlock + 1.0) / 2);
         }
-        lx.count = (int)(octasks.size() - lx.off);
-        lp.count = (int)(optasks.size() - lp.off);
-        lt.count = (int)(otasks.size() - lt.off);
-        for (size_t i = lt.off; i < otasks.size(); ++i)
-          lt.bytes += (double)otasks[i].nkb * (oz.a_block + oz.b_block) + 32.0 * otasks[i].m * otasks[i].n;
-        if (lt.count > 0) {
-          launches.push_back(lx);
-          launches.push_back(lp);
-          launches.push_back(lt);
-        }
+        oz_launches(lx, lp, lt);
       }
     }
     // The two-inverse form: the second inverse X of L_TL row by row, X L_TL = I, by block columns from
@@ -1180,7 +1314,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       const auto& ft = fronts[f0 + f];
       const int64_t bb = tc_block_bytes();
       const int64_t uu = nrb(ft.u) * nkb16(ft.s) * bb, ss = nrb(ft.s) * nkb16(ft.s) * bb;
-      unsigned char* b = packs[f0 + f];
+      unsigned char* b = packs[f0 + f].p;
       return Packed{b, b + uu, b + 2 * uu, b + 3 * uu, b + 3 * uu + ss, nkb16(ft.s)};
     };
     auto pack = [&](const T* src, const T* d, unsigned char* dst, int ld_, int ldd_, int R, int K, int mode) {
@@ -1214,7 +1348,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         Launch ls{SCALE, f0, c0, 0, 0};
         for (int f : ord) {
           const auto& ft = fronts[f0 + f];
-          if (ft.u == 0 || (packs[f0 + f] && si == PSP_SI_EXTENDED)) continue;
+          if (ft.u == 0 || (packs[f0 + f].p && si == PSP_SI_EXTENDED)) continue;
           for (int c = 0; c < ft.s; c += 16) ctasks.push_back({f, c, std::min(c + 16, ft.s)});
           ls.bytes += 2.0 * es * ft.u * ft.s;
         }
@@ -1226,7 +1360,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         const int64_t g0 = (int64_t)gtasks.size();
         for (int f : ord) {
           const auto& ft = fronts[f0 + f];
-          if (ft.u == 0 || packs[f0 + f]) continue;
+          if (ft.u == 0 || packs[f0 + f].p) continue;
           if (phase == 0) emit_z(ft);
           else emit_schur_m(ft);
         }
@@ -1241,7 +1375,7 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
       double tflops = 0, tflops_si = 0;
       for (int f : ord) {
         const auto& ft = fronts[f0 + f];
-        if (std::is_same<T, double2>::value || ft.u == 0 || !packs[f0 + f]) continue;
+        if (std::is_same<T, double2>::value || ft.u == 0 || !packs[f0 + f].p) continue;
         const int ld = ft.s + ft.u;
         const Packed P = packed_of(f);
         const int64_t bb = tc_block_bytes();
@@ -1307,65 +1441,57 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
         }
       }
       if constexpr (std::is_same<T, double2>::value) {
-        // complex128 fronts on the tensor cores.  Phase 0: F_BL (A) and inv(L) (B), Z = F_BL inv(L)^T.  Phase 1: Z D^-1 in
-        // F_BL's place and Z (B), the Schur update; then (extended form) Z D^-1 again, balanced against inv(L)^T, and
-        // inv(L)^T in inv(L)'s place, M_BL.  The Schur update's operands are balanced by their pivots alone.
+        // complex128 fronts on the tensor cores.  Phase 0: Z = F_BL inv(L)^T.  Phase 1: the Schur update (Z D^-1) Z^T; then
+        // (extended form) M_BL = (Z D^-1) inv(L), for which Z D^-1 is packed again, balanced against inv(L).  The
+        // Schur update's operands are balanced by their pivots alone.
         for (int step = 0; step < (phase == 0 ? 1 : si == PSP_SI_EXTENDED ? 2 : 1); ++step) {
-          const int64_t op0 = (int64_t)optasks.size(), o0 = (int64_t)otasks.size(), oc0 = (int64_t)octasks.size();
-          Launch lx{OZCOL, f0, oc0, 0, -1}, lp{OZPACK, f0, op0, 0, -1}, lt{OZGEMM, f0, o0, 0, -1};
+          Launch lx{OZCOL, f0, (int64_t)octasks.size(), 0, -1}, lp{OZPACK, f0, (int64_t)optasks.size(), 0, -1},
+              lt{OZGEMM, f0, (int64_t)otasks.size(), 0, -1};
           for (int f : ord) {
             const auto& ft = fronts[f0 + f];
-            if (ft.u == 0 || !packs[f0 + f]) continue;
-            const int ld = ft.s + ft.u;
-            const int64_t s_ = ft.s, u_ = ft.u;
-            unsigned char* PA = packs[f0 + f];
-            unsigned char* PB = PA + (oz_bytes(u_, s_, false) + oz_exps(u_, s_, false));
-            unsigned char* PL = PB + (oz_bytes(u_, s_, true) + oz_exps(u_, s_, true));
+            if (ft.u == 0 || !packs[f0 + f].p) continue;
+            const int64_t s_ = ft.s, u_ = ft.u, ld = s_ + u_;
             int* const kx0 = kx[f0 + f];
+            OzPlace at{packs[f0 + f]};
             if (phase == 0) {
-              const Balance bal{kx0, kx0 + s_, nullptr, 0};
-              lx.bytes += oz_colmax(ft.G + ft.s, ld, u_, s_, TC_PACK_PLAIN, kx0);
+              lx.bytes += oz_colmax(ft.G + s_, ld, u_, s_, TC_PACK_PLAIN, kx0);
               lx.bytes += oz_colmax(ft.G, ld, s_, s_, TC_PACK_UNIT_LOWER, kx0 + s_);
-              lp.bytes += oz_pack(ft.G + ft.s, nullptr, 0, PA, ld, u_, s_, TC_PACK_PLAIN, false, bal);
-              lp.bytes += oz_pack(ft.G, nullptr, 0, PL, ld, s_, s_, TC_PACK_UNIT_LOWER, true, bal);
-              for (int tj = 0; tj < ft.s; tj += oz.tile_n)
-                for (int ti = 0; ti < ft.u; ti += oz.tile_m)
-                  oz_tile(PA, u_, PL, s_, s_, ti, tj, ft.Z + (int64_t)tj * ft.u + ti, ft.u, 0,
-                          std::min<int64_t>(tj + oz.tile_n, s_), kAll, GF_BETA0);
+              lp.bytes += oz_product(
+                  OzOperand{ft.G + s_, ld, u_, TC_PACK_PLAIN}, OzOperand{ft.G, ld, s_, TC_PACK_UNIT_LOWER}, s_,
+                  Balance{kx0, kx0 + s_, nullptr, 0},
+                  [&](int64_t ti, int64_t tj, OzTile& t) {
+                    t = {ft.Z + tj * u_ + ti, u_, 0, std::min<int64_t>(tj + oz.tile_n, s_), kAll, GF_BETA0};
+                    return true;
+                  },
+                  at);
               lt.flops += 8.0 * u_ * s_ * (s_ + 1.0) / 2;
             } else if (step == 0) {
-              const Balance bal{nullptr, nullptr, ft.dinv, 1};
-              lp.bytes += oz_pack(ft.Z, ft.dinv, 1, PA, u_, u_, s_, TC_PACK_PLAIN, false, bal);
-              lp.bytes += oz_pack(ft.Z, nullptr, 0, PB, u_, u_, s_, TC_PACK_PLAIN, true, bal);
-              for (int tj = 0; tj < ft.u; tj += oz.tile_n)
-                for (int ti = tj / oz.tile_m * oz.tile_m; ti < ft.u; ti += oz.tile_m)
-                  oz_tile(PA, u_, PB, u_, s_, ti, tj, ft.U + upd_index(std::max(ti, tj), tj, ft.u, 128) - std::max(0, tj - ti),
-                          128, 0, s_, ti > tj ? kAll : ti - tj, GF_NEG);
+              lp.bytes += oz_product(
+                  OzOperand{ft.Z, u_, u_, TC_PACK_PLAIN, ft.dinv, 1}, OzOperand{ft.Z, u_, u_, TC_PACK_PLAIN}, s_,
+                  Balance{nullptr, nullptr, ft.dinv, 1},
+                  [&](int64_t ti, int64_t tj, OzTile& t) {
+                    if (ti < tj / oz.tile_m * oz.tile_m) return false;
+                    t = {ft.U + upd_index((int)std::max(ti, tj), (int)tj, ft.u, 128) - std::max<int64_t>(0, tj - ti), 128, 0, s_,
+                         ti > tj ? kAll : (int)(ti - tj), GF_NEG};
+                    return true;
+                  },
+                  at);
               lt.flops += 8.0 * s_ * u_ * (u_ + 1.0) / 2;
             } else {
-              const Balance bal{kx0 + 2 * s_, kx0 + 3 * s_, ft.dinv, 1};
               lx.bytes += oz_colmax(ft.Z, u_, u_, s_, TC_PACK_PLAIN, kx0 + 2 * s_);
               lx.bytes += oz_colmax(ft.G, ld, s_, s_, TC_PACK_UNIT_LOWER_T, kx0 + 3 * s_);
-              lp.bytes += oz_pack(ft.Z, ft.dinv, 1, PA, u_, u_, s_, TC_PACK_PLAIN, false, bal);
-              lp.bytes += oz_pack(ft.G, nullptr, 0, PL, ld, s_, s_, TC_PACK_UNIT_LOWER_T, true, bal);
-              for (int tj = 0; tj < ft.s; tj += oz.tile_n)
-                for (int ti = 0; ti < ft.u; ti += oz.tile_m)
-                  oz_tile(PA, u_, PL, s_, s_, ti, tj, ft.G + (int64_t)tj * ld + ft.s + ti, ld, tj, s_, kAll, GF_BETA0);
+              lp.bytes += oz_product(
+                  OzOperand{ft.Z, u_, u_, TC_PACK_PLAIN, ft.dinv, 1}, OzOperand{ft.G, ld, s_, TC_PACK_UNIT_LOWER_T}, s_,
+                  Balance{kx0 + 2 * s_, kx0 + 3 * s_, ft.dinv, 1},
+                  [&](int64_t ti, int64_t tj, OzTile& t) {
+                    t = {ft.G + tj * ld + s_ + ti, ld, tj, s_, kAll, GF_BETA0};
+                    return true;
+                  },
+                  at);
               lt.extra += 8.0 * u_ * s_ * (s_ + 1.0) / 2;   // M_BL: selective inversion
             }
           }
-          lx.count = (int)(octasks.size() - oc0);
-          lp.count = (int)(optasks.size() - op0);
-          lt.count = (int)(otasks.size() - o0);
-          for (size_t i = o0; i < otasks.size(); ++i)
-            lt.bytes += (double)otasks[i].nkb * (oz.a_block + oz.b_block) + 32.0 * otasks[i].m * otasks[i].n;
-          if (stall_next && o0 < (int64_t)otasks.size()) {
-            otasks[o0].flags |= GF_TEST_STALL;
-            stall_next = false;
-          }
-          launches.push_back(lx);
-          launches.push_back(lp);
-          launches.push_back(lt);
+          oz_launches(lx, lp, lt);
         }
         continue;
       }
@@ -1449,6 +1575,33 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
   if (hs[0] != 0) {
     X->zero_pivot_front = hs[0] - 1;
     throw Error{PSP_ERR_ZERO_PIVOT, "zero pivot in front " + std::to_string(hs[0] - 1)};
+  }
+}
+
+// The factorisation with as much room for temporaries as the device (or the caller's allocator) gives: where an allocation
+// is refused it is made again with half of them, down to what the widest front needs on CUDA cores, and last with
+// complex128 products on CUDA cores, whose update matrices take smaller tiles.
+template <typename T>
+static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()>& while_device_runs) {
+  int64_t limit = INT64_MAX;
+  bool digits = true;
+  for (;;) {
+    TempUse use;
+    try {
+      factor_attempt<T>(X, st, while_device_runs, limit, digits, use);
+      return;
+    } catch (const Error& e) {
+      if (e.st != PSP_ERR_OOM) throw;
+      cudaGetLastError();   // the refused allocation's error
+      if (use.budget > use.front_max) {
+        limit = std::max(use.front_max, use.budget / 2);
+      } else if (use.digits) {
+        digits = false;
+        limit = INT64_MAX;
+      } else {
+        throw;
+      }
+    }
   }
 }
 
