@@ -298,12 +298,13 @@ __device__ __forceinline__ void fwd_task(const TaskSlot<T>& sl, const SweepArgs<
 // Without inversion (G keeps L_TL): the first phase up the tree of front sn by one CTA: w_S gathered
 // as above, then forward substitution y_S = L_TL^{-1} w_S in blocks of 32 columns (one warp solves
 // the diagonal block, all threads update the rows below it), x_S = D^{-1} y_S into xf, y_S into xb.
+// w: room for RG x s entries (right-hand side major), in shared memory or, for a front too wide for it, the front's
+// own entries of xb, which no other task reads or writes before this one is done.
 template <typename T, int RG>
-__device__ __noinline__ void fwd_tri_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr, unsigned char* smem) {
+__device__ __noinline__ void fwd_tri_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr, T* w) {
   const int s = sl.fr.s, ld = s + sl.fr.u;
   const T* G = sl.G;
   const int tid = threadIdx.x;
-  T* w = reinterpret_cast<T*>(smem);            // RG x s (right-hand side major)
   for (int p = tid; p < s; p += kComputeThreads) {
     const int4 ix = p < kGatherIdx ? sl.rows[p] : __ldg(sl.rows_g + p);
     T v[RG], t[RG];
@@ -512,12 +513,12 @@ __device__ __forceinline__ void bwd_task(const TaskSlot<T>& sl, const SweepArgs<
 // Without inversion: the second phase down the tree of front sn by one CTA: back substitution
 // L_TL^T x_S = t (t in xf) in blocks of 32 columns from the last, each block first takes the
 // products with the solved rows below it (one warp per column), then one warp solves the block.
+// x: RG x s entries (right-hand side major) as fwd_tri_task's w: t, overwritten by x block by block.
 template <typename T, int RG>
-__device__ __noinline__ void bwd_tri_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr, unsigned char* smem) {
+__device__ __noinline__ void bwd_tri_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr, T* x) {
   const int s = sl.fr.s, ld = s + sl.fr.u;
   const T* G = sl.G;
   const int tid = threadIdx.x;
-  T* x = reinterpret_cast<T*>(smem);   // RG x s (right-hand side major): t, overwritten by x block by block
   for (int r = tid; r < s; r += kComputeThreads) {
     T v[RG];
     load_entry<T, RG>(sl.xf, a.n_loc, sl.fr.first + r, gr, v);
@@ -807,15 +808,16 @@ __global__ void __launch_bounds__(kSweepThreads, (sweep_ctas<T, RG>())) k_sweep(
           else bwd_task<T, RG, 0, true>(sl, a, gr, smem);
         } else {
           const bool tri = a.si == PSP_SI_NONE;
+          T* const whole = a.tri_global ? entry_ptr<T, RG>(sl.xb, a.n_loc, sl.fr.first, gr) : reinterpret_cast<T*>(smem);
           if (dir == 0) {
-            if (tri) fwd_tri_task<T, RG>(sl, a, gr, smem);
+            if (tri) fwd_tri_task<T, RG>(sl, a, gr, whole);
             else fwd_task<T, RG, 0, false>(sl, a, gr, smem);
           } else if (dir == kDirUpB) {
             fwd_task<T, RG, 1, false>(sl, a, gr, smem);
           } else if (dir == 1) {
             bwd_task<T, RG, 0, false>(sl, a, gr, smem);
           } else {
-            if (tri) bwd_tri_task<T, RG>(sl, a, gr, smem);
+            if (tri) bwd_tri_task<T, RG>(sl, a, gr, whole);
             else bwd_task<T, RG, 1, false>(sl, a, gr, smem);
           }
         }
@@ -858,7 +860,8 @@ static int sweep_rg(const SweepArgs<T>& args, size_t smem, int max_per_sm, cudaS
 // and 4 in complex128, where the FP64 pipe and not the factor's bytes is the bound; or rhs_group when > 0), and the
 // vectors of a task pass through shared memory in chunks sized so that two CTAs stay resident per SM (a CTA that
 // waits on a dependency leaves the SM to the other).  Substitution tasks (fronts keeping L_TL) hold a front's
-// whole vector, so for them RG shrinks until that fits.
+// whole vector, so for them RG shrinks until that fits; one column of a front wider than shared memory (13,400 rows in
+// complex128) stays in its work vector.
 template <typename T, int RG>
 constexpr size_t sweep_smem() { return (sizeof(T) == 16 && RG == 4 ? 84 : 64) * 1024; }
 
@@ -871,7 +874,11 @@ static int sweep_sized(const SweepArgs<T>& args, int smax, int ldmax, int max_pe
   SweepArgs<T> a = args;
   a.chunk = chunk;
   size_t smem = fixed + chunk * entry;
-  if (a.si == PSP_SI_NONE && smem < (size_t)smax * RG * es) smem = (size_t)smax * RG * es;
+  if (a.si == PSP_SI_NONE) {
+    const size_t whole = (size_t)smax * RG * es;
+    a.tri_global = RG == 1 && whole + 2 * sizeof(TaskSlot<T>) > 226 * 1024;
+    if (!a.tri_global && smem < whole) smem = whole;
+  }
   return a.si == PSP_SI_EXTENDED ? sweep_rg<T, RG, true>(a, smem, max_per_sm, st) : sweep_rg<T, RG, false>(a, smem, max_per_sm, st);
 }
 

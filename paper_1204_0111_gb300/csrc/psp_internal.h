@@ -355,6 +355,7 @@ struct SweepArgs {
   int* status;                  // status[2] set when a wait gave up (= ctr + 1)
   int* sticky;                  // also set then; kept until the host reads it (psp_check_status)
   int chunk;                    // vector entries a task stages in shared memory at a time (set by launch_sweep)
+  int tri_global;               // substitution tasks keep their vector in xb: too wide for shared memory (set by launch_sweep)
   int claim_ahead;              // 2: a CTA holds the two tasks after the one it runs; 1: the next one only
 };
 void launch_build_rows(const ShapeDev& sh, int4* rows, cudaStream_t st);
