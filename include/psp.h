@@ -114,7 +114,7 @@ typedef struct {
   int sweep_level_tasks; /* sweep schedule: tasks a tree level is split into at least (row / column
                             blocks of 8..256); <= 0 selects the default (304) */
   int sweep_ctas_per_sm; /* sweep schedule: resident CTAs per SM of the persistent sweep (capped by
-                            occupancy); <= 0 selects the default (8) */
+                            occupancy: the kernel is built for two); <= 0 selects the default (as many as fit) */
   int setup_temp_mb;   /* cap, in MiB, on the per-front temporaries of one batch of fronts during setup
                           (a level whose fronts need more is factored in several batches, and a complex128
                           front whose tensor-core operands need more takes its products in pieces; neither
@@ -368,7 +368,8 @@ psp_status psp_stats(psp_handle h, psp_kernel_stat* out, int capacity, int* coun
  * and keeps the fastest: the tasks a tree level is split into (152 .. 2432), the resident CTAs per
  * SM (2, 3, 4, 6, 8), the cap on rows / columns per task (64 .. 256), the floor on rows per task
  * (4 .. 64), the queue tasks a CTA holds ahead (1, 2) and, for nrhs > 1, the right-hand sides per
- * CTA pass (1 .. 8).  It searches one
+ * CTA pass (1 .. 8; complex128 factors 1 .. 4).  Schedules that come to the same tasks and the
+ * same launch are timed once.  It searches one
  * coordinate at a time, starting from the handle's current schedule, timing `reps` applications
  * (CUDA events on `stream`) per candidate after one untimed one.  Results do not change beyond
  * rounding (the schedule only regroups the same sums).  The work vectors are the handle's own; the

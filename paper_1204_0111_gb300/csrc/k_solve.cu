@@ -829,7 +829,7 @@ __global__ void __launch_bounds__(kSweepThreads, (sweep_ctas<T, RG>())) k_sweep(
 }
 
 template <typename T, int RG, bool EXT>
-static int sweep_rg(const SweepArgs<T>& args, size_t smem, int max_per_sm, cudaStream_t st) {
+static int sweep_rg(const SweepArgs<T>& args, size_t smem, int max_per_sm, SweepFit* fit, cudaStream_t st) {
   if (cudaFuncSetAttribute(k_sweep<T, RG, EXT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
     cudaGetLastError();
     return -1;
@@ -844,6 +844,10 @@ static int sweep_rg(const SweepArgs<T>& args, size_t smem, int max_per_sm, cudaS
     return -1;
   }
   per_sm = per_sm > max_per_sm ? max_per_sm : per_sm;
+  if (fit) {
+    *fit = SweepFit{RG, per_sm};
+    return 0;
+  }
   SweepArgs<T> a = args;
   void* kargs[] = {&a};
   cudaError_t e;
@@ -866,7 +870,7 @@ template <typename T, int RG>
 constexpr size_t sweep_smem() { return (sizeof(T) == 16 && RG == 4 ? 84 : 64) * 1024; }
 
 template <typename T, int RG>
-static int sweep_sized(const SweepArgs<T>& args, int smax, int ldmax, int max_per_sm, cudaStream_t st) {
+static int sweep_sized(const SweepArgs<T>& args, int smax, int ldmax, int max_per_sm, SweepFit* fit, cudaStream_t st) {
   constexpr size_t es = sizeof(T), entry = entry_stride<T, RG>() * es, fixed = 2 * (size_t)kComputeThreads * RG * es;
   const int full = ldmax > smax ? ldmax : smax;
   int chunk = (int)((sweep_smem<T, RG>() - fixed) / entry / 64 * 64);
@@ -879,11 +883,12 @@ static int sweep_sized(const SweepArgs<T>& args, int smax, int ldmax, int max_pe
     a.tri_global = RG == 1 && whole + 2 * sizeof(TaskSlot<T>) > 226 * 1024;
     if (!a.tri_global && smem < whole) smem = whole;
   }
-  return a.si == PSP_SI_EXTENDED ? sweep_rg<T, RG, true>(a, smem, max_per_sm, st) : sweep_rg<T, RG, false>(a, smem, max_per_sm, st);
+  return a.si == PSP_SI_EXTENDED ? sweep_rg<T, RG, true>(a, smem, max_per_sm, fit, st)
+                                 : sweep_rg<T, RG, false>(a, smem, max_per_sm, fit, st);
 }
 
 template <typename T>
-int launch_sweep(const SweepArgs<T>& a, int smax, int ldmax, int max_per_sm, int rhs_group, cudaStream_t st) {
+static int sweep(const SweepArgs<T>& a, int smax, int ldmax, int max_per_sm, int rhs_group, SweepFit* fit, cudaStream_t st) {
   int rg = sizeof(T) == 8 ? 8 : 4;
   while (rg > 1 && rg >= 2 * a.nrhs) rg >>= 1;
   if (rhs_group > 0)
@@ -892,15 +897,31 @@ int launch_sweep(const SweepArgs<T>& a, int smax, int ldmax, int max_per_sm, int
     while (rg > 1 && (size_t)smax * rg * sizeof(T) > 180 * 1024) rg >>= 1;
   switch (rg) {
     case 8:
-      if constexpr (sizeof(T) == 8) return sweep_sized<T, 8>(a, smax, ldmax, max_per_sm, st);
-    case 4: return sweep_sized<T, 4>(a, smax, ldmax, max_per_sm, st);
-    case 2: return sweep_sized<T, 2>(a, smax, ldmax, max_per_sm, st);
-    default: return sweep_sized<T, 1>(a, smax, ldmax, max_per_sm, st);
+      if constexpr (sizeof(T) == 8) return sweep_sized<T, 8>(a, smax, ldmax, max_per_sm, fit, st);
+    case 4: return sweep_sized<T, 4>(a, smax, ldmax, max_per_sm, fit, st);
+    case 2: return sweep_sized<T, 2>(a, smax, ldmax, max_per_sm, fit, st);
+    default: return sweep_sized<T, 1>(a, smax, ldmax, max_per_sm, fit, st);
   }
+}
+
+template <typename T>
+int launch_sweep(const SweepArgs<T>& a, int smax, int ldmax, int max_per_sm, int rhs_group, cudaStream_t st) {
+  return sweep<T>(a, smax, ldmax, max_per_sm, rhs_group, nullptr, st);
+}
+template <typename T>
+SweepFit sweep_fit(int nrhs, int si, int smax, int ldmax, int max_per_sm, int rhs_group) {
+  SweepArgs<T> a{};
+  a.nrhs = nrhs;
+  a.si = si;
+  SweepFit f;
+  sweep<T>(a, smax, ldmax, max_per_sm, rhs_group, &f, nullptr);
+  return f;
 }
 
 template int launch_sweep<double2>(const SweepArgs<double2>&, int, int, int, int, cudaStream_t);
 template int launch_sweep<float2>(const SweepArgs<float2>&, int, int, int, int, cudaStream_t);
+template SweepFit sweep_fit<double2>(int, int, int, int, int, int);
+template SweepFit sweep_fit<float2>(int, int, int, int, int, int);
 
 // index words of a shape's front rows: row p of front f gets {its box node (p < s, else -1), the two update-vector
 // entries its children add to it, 0}, so that a gather reads one 16-byte word per row

@@ -11,6 +11,7 @@
 #include <future>
 #include <map>
 #include <memory>
+#include <set>
 #include <new>
 #include <stdexcept>
 #include <system_error>
@@ -3124,9 +3125,19 @@ psp_status psp_tune_sweep(psp_handle X, int nrhs, int reps, void* stream, psp_sw
   Sched best{X->sweep_level_tasks, X->sweep_ctas_per_sm, X->sweep_rhs_group, X->sweep_min_rows, X->sweep_max_rows,
              X->sweep_claim_ahead};
   double best_ms = 0, initial_ms = 0;
+  // schedules that come to the same tasks and the same launch are timed once
+  std::set<std::tuple<int, int, int, int, int, int>> seen;
+  auto fresh = [&](const Sched& c) {
+    const SweepFit f = X->prec == PSP_PREC_C64
+                           ? sweep_fit<float2>(nrhs, X->si_mode, X->sweep_smax, X->sweep_ldmax, c.cps, c.rg)
+                           : sweep_fit<double2>(nrhs, X->si_mode, X->sweep_smax, X->sweep_ldmax, c.cps, c.rg);
+    return seen.insert({c.lt, f.per_sm, f.rg, c.mr, c.xr, c.ca}).second;
+  };
   try {
+    fresh(best);
     best_ms = initial_ms = time_one(best);
     auto consider = [&](Sched c) {
+      if (!fresh(c)) return;
       const double ms = time_one(c);
       if (ms < best_ms) {
         best_ms = ms;
@@ -3134,18 +3145,18 @@ psp_status psp_tune_sweep(psp_handle X, int nrhs, int reps, void* stream, psp_sw
       }
     };
     for (int xr : {64, 128, 256})
-      if (xr != best.xr) consider({best.lt, best.cps, best.rg, best.mr, xr, best.ca});
+      consider({best.lt, best.cps, best.rg, best.mr, xr, best.ca});
     for (int lt : {152, 304, 608, 1216, 2432})
-      if (lt != best.lt) consider({lt, best.cps, best.rg, best.mr, best.xr, best.ca});
+      consider({lt, best.cps, best.rg, best.mr, best.xr, best.ca});
     for (int cps : {2, 3, 4, 6, 8})
-      if (cps != best.cps) consider({best.lt, cps, best.rg, best.mr, best.xr, best.ca});
+      consider({best.lt, cps, best.rg, best.mr, best.xr, best.ca});
     if (nrhs > 1)
       for (int rg : {1, 2, 4, 8})
-        if (rg <= nrhs && rg != best.rg) consider({best.lt, best.cps, rg, best.mr, best.xr, best.ca});
+        consider({best.lt, best.cps, rg, best.mr, best.xr, best.ca});
     for (int mr : {4, 8, 16, 32, 64})
-      if (mr != best.mr) consider({best.lt, best.cps, best.rg, mr, best.xr, best.ca});
+      consider({best.lt, best.cps, best.rg, mr, best.xr, best.ca});
     for (int ca : {1, 2})
-      if (ca != best.ca) consider({best.lt, best.cps, best.rg, best.mr, best.xr, ca});
+      consider({best.lt, best.cps, best.rg, best.mr, best.xr, ca});
   } catch (...) {
     X->stats.timing = was_timing;
     cudaEventDestroy(e0);

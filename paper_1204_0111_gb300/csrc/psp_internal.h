@@ -363,6 +363,10 @@ void launch_build_rows(const ShapeDev& sh, int4* rows, cudaStream_t st);
 // the widest front's s and s + u
 template <typename T>
 int launch_sweep(const SweepArgs<T>& args, int smax, int ldmax, int max_per_sm, int rhs_group, cudaStream_t st);
+// what that launch would take: columns a CTA carries through a pass, resident CTAs per SM
+struct SweepFit { int rg = 0, per_sm = 0; };
+template <typename T>
+SweepFit sweep_fit(int nrhs, int si, int smax, int ldmax, int max_per_sm, int rhs_group);
 
 // ---- GMRES helpers (complex128) ----
 // A block of vectors holds ncol columns (right-hand sides, and problems of a batch); column c of
