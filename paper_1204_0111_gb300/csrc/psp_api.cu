@@ -2267,9 +2267,6 @@ static void finish_setup(psp_ctx_s* X, cudaStream_t st) {
     size_t o_rel = put(sh.rel.data(), sh.rel.size() * 4);
     size_t o_pp = put(sh.pull_ptr.data(), sh.pull_ptr.size() * 8);
     size_t o_pl = put(sh.pull.data(), sh.pull.size() * 4);
-    size_t o_go = put(sh.g_off.data(), sh.g_off.size() * 8);
-    size_t o_uo = put(sh.upd_off.data(), sh.upd_off.size() * 8);
-    size_t o_par = put(sh.parent.data(), sh.parent.size() * 4);
     DevBuf b;
     b.alloc(blob.size());
     PSP_CK(cudaMemcpy(b.p, blob.data(), blob.size(), cudaMemcpyHostToDevice));
@@ -2288,9 +2285,6 @@ static void finish_setup(psp_ctx_s* X, cudaStream_t st) {
     d.rel = (const int32_t*)(base + o_rel);
     d.pull_ptr = (const int64_t*)(base + o_pp);
     d.pull = (const int32_t*)(base + o_pl);
-    d.g_off = (const int64_t*)(base + o_go);
-    d.upd_off = (const int64_t*)(base + o_uo);
-    d.parent = (const int32_t*)(base + o_par);
     X->shdev.push_back(d);
     X->shape_bufs.push_back(std::move(b));
   }

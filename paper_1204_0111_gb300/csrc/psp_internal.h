@@ -71,9 +71,6 @@ struct ShapeDev {
   const int32_t* rel;
   const int64_t* pull_ptr;
   const int32_t* pull;
-  const int64_t* g_off;
-  const int64_t* upd_off;
-  const int32_t* parent;
 };
 
 // 7-point operator on a box: -sum_j d_j(a_j d_j u) - k2num / c^2 * s1 s2 s3 u (Eq. (1.1)/(1.5),
@@ -90,13 +87,6 @@ struct BoxOp {
   const double2* s2h;
   const double2* s3n;
   const double2* s3h;
-};
-
-// One panel's auxiliary problem (Alg. 1.4) as seen by the apply kernels.
-struct PanelDev {
-  int z0, z1, lead;         // global planes [z0, z1); lead pad (or exact-mode) planes before them
-  int shape;
-  int64_t sn_base;          // global front id of supernode 0
 };
 
 enum GemmFlags : int {
