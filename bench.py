@@ -577,6 +577,43 @@ def extra_workload(name, w, precision, dev, sched=None, maxit=400, desc="", tune
 
 
 # ---------------------------------------------------------------------------------------------
+# the printed line
+# ---------------------------------------------------------------------------------------------
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks")
+BRIEF_KEYS = {"roofline": ("kernel", "bound", "achieved", "peak", "unit", "frac", "traffic", "kernel_share"),
+              "cpu_baseline": ("value", "unit", "cores", "kind"),
+              "detail": ("gmres_iters", "relres", "apply_ms", "setup_kernel_ms", "sweep_gbs"),
+              "mixed": ("value", "ms_per_step", "gmres_iters", "apply_ms", "apply_rel_err_vs_c128"),
+              "salt256": ("ms_per_step", "gmres_iters", "apply_ms", "relres_max"),
+              "layered200": ("ms_per_step", "gmres_iters", "apply_ms", "relres_max"),
+              "batch16": ("ms_per_step", "gmres_iters", "relres")}
+
+
+def brief(line):
+    """The benchmark's line without its tables: every key of the contract whole, the rest in a few figures each.  With the
+    tables the line passes 25 kB, and readers that keep the end of a log lose its beginning."""
+    def short(v):
+        if isinstance(v, float):
+            return float(f"{v:.7g}")
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items()}
+        return [short(x) for x in v] if isinstance(v, list) else v
+
+    out = {k: line[k] for k in LINE_KEYS if k in line}
+    for key, keep in BRIEF_KEYS.items():
+        if line.get(key):
+            out[key] = {k: short(line[key][k]) for k in keep if k in line[key]}
+    return out
+
+
+def report(line):
+    """One JSON line on stdout; the same with every table on stderr."""
+    print(json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(brief(line)), flush=True)
+
+
+# ---------------------------------------------------------------------------------------------
 # GPU arm
 # ---------------------------------------------------------------------------------------------
 def gpu_main(a):
@@ -803,7 +840,7 @@ def gpu_main(a):
                 "si_forms": si_forms,
                 "mixed": mixed}
         line.update(extras)
-        print(json.dumps(line))
+        report(line)
     if world > 1:
         dist.destroy_process_group()
 
