@@ -66,7 +66,7 @@ typedef struct {
 } psp_grid;
 
 typedef enum {
-  PSP_PREC_C128 = 0,  /* fronts and sweeps in complex128 (FP64 CUDA cores) */
+  PSP_PREC_C128 = 0,  /* fronts and sweeps in complex128 (FP64 CUDA cores; front products: tensor_cores) */
   PSP_PREC_C64 = 1    /* fronts and sweeps in complex64; GMRES and matvec stay complex128 */
 } psp_precision;
 
@@ -112,7 +112,7 @@ typedef struct {
   int tc_min_dim;     /* complex64 path: fronts with s >= tc_min_dim and u >= tc_min_dim take the tensor
                          cores, the others CUDA cores; <= 0 selects the default (64) */
   int sweep_level_tasks; /* sweep schedule: tasks a tree level is split into at least (row / column
-                            blocks of 8..256); <= 0 selects the default (304) */
+                            blocks of sweep_min_rows to sweep_max_rows); <= 0 selects the default (304) */
   int sweep_ctas_per_sm; /* sweep schedule: resident CTAs per SM of the persistent sweep (capped by
                             occupancy: the kernel is built for two); <= 0 selects the default (as many as fit) */
   int setup_temp_mb;   /* cap, in MiB, on the per-front temporaries of one batch of fronts during setup

@@ -253,8 +253,8 @@ __global__ void __launch_bounds__(256) k_oz_pack(const OzPackTask* __restrict__ 
 
 // ---------------------------------------------------------------------------
 // k_oz_gemm: 128 x 32 output tiles, one CTA per SM over every gridDim.x-th tile, so that the next tile's copies and MMAs
-// run while this one's sums are added to C (tiles of a small front spend more on that than on their MMAs).  Warp 8 copies the operands' blocks of 16 k into two stages, warp 9
-// issues the MMAs (Re += Ar Br - Ai Bi and Im += Ar Bi + Ai Br as two N = 64 MMAs per digit pair: B's rows are stored as
+// run while this one's sums are added to C (tiles of a small front spend more on that than on their MMAs).  Warp 8
+// copies the operands' blocks of 16 k into two stages, warp 9 issues the MMAs (Re += Ar Br - Ai Bi and Im += Ar Bi + Ai Br as two N = 64 MMAs per digit pair: B's rows are stored as
 // [-Im | Re | Im], so [Re | Im] and [-Im | Re] are windows of it), warps 0 - 7 combine the sums after every 128 k.
 // Every wait is bounded; one that gives up records an error in status[1] and raises the CTA's abort flag.  The additions'
 // tensor-memory reads are warp-wide instructions, so whether a warp goes on is one decision of the whole warp; after an

@@ -386,7 +386,9 @@ __device__ __forceinline__ double2 old_solution(const TaskSlot<T>& sl, const Gro
 //
 // A warp carries blocks of four adjacent columns, its lanes over the rows, so an entry of y serves four columns;
 // tasks of few columns split their rows over the warps instead.  Which rows a lane sums depends on the task alone
-// (quads of columns, steps of 32 rows), so every RG gives a column the same bits.
+// (quads of columns, steps of 32 rows) where a front's vector is staged in one chunk, and then every RG gives a column the
+// same bits, as up the tree.  A front wider than a chunk (384 entries at eight complex64 columns, 7,680 at one) is summed
+// chunk by chunk, so there the groups differ by the rounding of another order.
 template <typename T, int RG, int PHASE, bool EXT>
 __device__ __forceinline__ void bwd_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr, unsigned char* smem) {
   using Real = typename CplxTraits<T>::real;

@@ -400,7 +400,9 @@ static double ms_since(std::chrono::steady_clock::time_point t0) {
   return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
 }
 
-constexpr int kOzMinDim = 16;   // complex128: fewest s and u of a front on the tensor cores
+// complex128: fewest s and u of a front on the tensor cores.  16 / 32 / 64, lens setups: 24^3 12.1 / 12.6 / 14.4 ms, 48^3
+// 48.5 / 51.0 / 71.8, 80^3 216 / 226 / 315; below 16 a tile of k = 16 is mostly padding
+constexpr int kOzMinDim = 16;
 // complex128: fronts of at least this many rows S factor F_TL and build inv(L_TL) in blocks of 128 columns: inside a block by
 // steps of 32 on the FP64 units, the rest of F_TL and of W once per block, with k = 128, on the tensor cores (80^3 lens
 // setup: k_gemm 75.7 -> 32.7 ms, the tensor-core products and their operands 93.8 -> 98.8 ms; half of k_gemm's work was the
@@ -1240,8 +1242,8 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
       launches.push_back(lc);
     }
     // Z = F_BL inv(L_TL)^T (= F_BL L^{-T}), then F_BR -= Z D^{-1} Z^T (lower) and M_BL = Z D^{-1} inv(L_TL).
-    // Fronts with s, u >= 96 (complex64) run them on tcgen05 tiles of 128 x 128 from packed operands;
-    // the others on 64 x 64 CUDA-core tiles.
+    // Fronts with s, u >= tc_min_dim (complex64; 64 by default) run them on tcgen05 tiles of 128 x 128 from packed
+    // operands, complex128 fronts of kOzMinDim and more on 128 x 32 tiles, the others on 64 x 64 CUDA-core tiles.
     auto emit_z = [&](const FrontTask<T>& ft) {
       const int ld = ft.s + ft.u;
       for (int tj = 0; tj < ft.s; tj += 64)
@@ -2675,7 +2677,9 @@ static void init_options(psp_ctx_s* X, const psp_options& o) {
   X->use_tc = o.tensor_cores != 0;
   X->diag_fp64 = o.c64_diag_fp64 != 0;
   X->tc_min_dim = o.tc_min_dim > 0 ? o.tc_min_dim : 64;
-  // measured on lens100, 304 against 608 tasks per level: complex128 35.9 / 38.3 ms, complex64 11.7 / 14.4 ms
+  // 304 = two CTAs on each of 152 SMs.  152 / 228 / 304 / 456 / 608 tasks per level: lens100 complex128 41.1 / 37.0 / 33.9 /
+  // 34.3 / 36.4 ms, complex64 13.1 / 12.1 / 11.6 / 13.3 / 15.0; 88^3 x 8 complex64 19.8 / 18.9 / 18.2 / 20.4 / 22.6; salt body
+  // 128^3 x 8 51.0 / 45.8 / 45.3 / 45.5 / 46.5; on 32^3 and 48^3 fewer gain up to 5 % (1.72 / 1.72 / 1.76 / 1.80 / 2.06)
   X->sweep_level_tasks = o.sweep_level_tasks > 0 ? o.sweep_level_tasks : 304;
   X->sweep_ctas_per_sm = o.sweep_ctas_per_sm > 0 ? o.sweep_ctas_per_sm : 8;
   X->sweep_rhs_group = o.sweep_rhs_group > 0 ? o.sweep_rhs_group : 0;
