@@ -45,6 +45,8 @@ constexpr int B_PLANE = 3 * ON * OK * 2;       // 3 KB: rows [-Im | Re | Im] of 
 constexpr int A_BLOCK = ND * 2 * A_PLANE;      // 64 KB per 16 k
 constexpr int B_BLOCK = ND * B_PLANE;          // 24 KB per 16 k
 constexpr int STAGE = A_BLOCK + B_BLOCK;       // 88 KB
+static_assert(OM == kOz.tile_m && ON == kOz.tile_n && OK == kOz.k && OKC == kOz.kc && A_BLOCK == kOz.a_block && B_BLOCK == kOz.b_block,
+              "the planner's figures");
 constexpr int NSTAGE = 2;
 constexpr int SMEM = NSTAGE * STAGE + 1024;    // + barriers and the TMEM slot
 constexpr uint32_t LBO = 128, SBO = 256;       // next core matrix (8 rows x 16 bytes) along k, next 8 rows
@@ -470,7 +472,5 @@ void launch_oz_gemm(const OzGemmTask* tasks, int ntasks, int* status, cudaStream
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   k_oz_gemm<<<ntasks < sms ? ntasks : sms, THREADS, SMEM, st>>>(tasks, ntasks, status);
 }
-
-OzShape oz_shape() { return OzShape{OM, ON, OK, OKC, A_BLOCK, B_BLOCK}; }
 
 }  // namespace psp

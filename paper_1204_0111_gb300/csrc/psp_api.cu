@@ -455,15 +455,14 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
   const int64_t TBLK = tc_block_bytes() / (int64_t)sizeof(T);   // packed block in T elements
   // complex128: fronts of at least kOzMinDim rows each way run the same products on the tensor cores from exact digit
   // products; below that the tiles are mostly padding (128 x 32 outputs, k in 16s), and there is next to no work
-  const OzShape oz = oz_shape();
   const bool oz_ok = std::is_same<T, double2>::value && X->use_tc && si != PSP_SI_NONE && digits;
   auto cdiv_i = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
   // bytes of a packed operand of R rows and K columns and of its row exponents (A: 128-row blocks, B: 32-row blocks)
   auto oz_bytes = [&](int64_t R, int64_t K, bool b) {
-    return cdiv_i(R, b ? oz.tile_n : oz.tile_m) * cdiv_i(K, oz.k) * (b ? oz.b_block : oz.a_block);
+    return cdiv_i(R, b ? kOz.tile_n : kOz.tile_m) * cdiv_i(K, kOz.k) * (b ? kOz.b_block : kOz.a_block);
   };
   auto oz_exps = [&](int64_t R, int64_t K, bool b) {
-    return (int64_t)sizeof(int) * cdiv_i(R, b ? oz.tile_n : oz.tile_m) * cdiv_i(K, oz.kc) * (b ? oz.tile_n : oz.tile_m);
+    return (int64_t)sizeof(int) * cdiv_i(R, b ? kOz.tile_n : kOz.tile_m) * cdiv_i(K, kOz.kc) * (b ? kOz.tile_n : kOz.tile_m);
   };
   // bytes of an operand with its row exponents
   auto oz_size = [&](int64_t R, int64_t K, bool b) { return oz_bytes(R, K, b) + oz_exps(R, K, b); };
@@ -503,7 +502,7 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
     if (!oz_dims && !block_dims) return t;
     const int64_t allowed = std::max(limit, t.total), kx = pad16(s_), tail = oz_dims ? z : t.tail;
     auto elems = [&](int64_t bytes) { return pad16(cdiv_i(bytes, (int64_t)sizeof(T))); };
-    const int64_t A = oz.tile_m, B = oz.tile_n, K = std::min<int64_t>(s_, oz.kc), kb = kOzBlock;
+    const int64_t A = kOz.tile_m, B = kOz.tile_n, K = std::min<int64_t>(s_, kOz.kc), kb = kOzBlock;
     int64_t in_f_tl = 0, in_f_tl_min = 0, in_front = 0, in_front_min = 0;
     if (block_dims) {   // L D and L again, L and W's block row
       in_f_tl = elems(2 * oz_size(s_ - kb, kb, false) + oz_size(s_, kb, true));
@@ -523,7 +522,7 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
     t.total = std::min(full, allowed / 16 * 16);
     return t;
   };
-  auto use_oz = [&](int64_t s_, int64_t u_) { return oz_ok && front_temp(s_, u_).oz; };
+  std::vector<FrontTemp> temps(X->nfronts);   // by front id, filled by plan_memory
   int64_t arena[2] = {0, 0}, temp_level_max = 0, temp_front_max = 16;
   auto plan_memory = [&] {
     arena[0] = arena[1] = temp_level_max = 0;
@@ -533,11 +532,11 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
       for (auto [p, sn] : lev_fronts[lv]) {
         const Shape& sh = X->shapes[X->shape_of[p]];
         const int64_t s = sh.s[sn], u = sh.u[sn];
+        const FrontTemp& ft = temps[X->sn_base[p] + sn] = front_temp(s, u);
         if (u > 0) {
           uoff[X->sn_base[p] + sn] = slab;
-          slab += pad16(upd_packed_elems((int)u, use_tc(s, u) || use_oz(s, u) ? 128 : 64));
+          slab += pad16(upd_packed_elems((int)u, use_tc(s, u) || ft.oz ? 128 : 64));
         }
-        const FrontTemp ft = front_temp(s, u);
         const int64_t t = ft.total;
         use.digits = use.digits || ft.oz || ft.blocks;
         if (si != PSP_SI_NONE) use.front_max = std::max(use.front_max, use_tc(s, u) ? t : cuda_core_temp(s, u));
@@ -591,8 +590,7 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
     int64_t run = 0;
     bool fresh = true;   // every level starts a new group
     for (auto [p, sn] : lev_fronts[lv]) {
-      const Shape& sh = X->shapes[X->shape_of[p]];
-      const int64_t t = front_temp(sh.s[sn], sh.u[sn]).total;
+      const int64_t t = temps[X->sn_base[p] + sn].total;
       if (fresh || run + t > temp_budget) {
         groups.emplace_back();
         run = 0;
@@ -618,7 +616,7 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
   for (int p = 0; p < X->m; ++p) {
     const Shape& sh = X->shapes[X->shape_of[p]];
     for (int sn = 0; sn < sh.nsn; ++sn)
-      if (use_tc(sh.s[sn], sh.u[sn]) || use_oz(sh.s[sn], sh.u[sn])) upd_tile[X->sn_base[p] + sn] = 128;
+      if (use_tc(sh.s[sn], sh.u[sn]) || temps[X->sn_base[p] + sn].oz) upd_tile[X->sn_base[p] + sn] = 128;
   }
   DevBuf d_upd_ptr, d_upd_tile;
   upload(d_upd_ptr, upd_ptr);
@@ -804,7 +802,7 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
       blocks.push_back({});
       kx.push_back(nullptr);
       if (si != PSP_SI_NONE) {
-        const FrontTemp tp_ = front_temp(ft.s, ft.u);
+        const FrontTemp& tp_ = temps[ft.gfid];
         T* const base = tbase + toff;
         toff += tp_.total;
         T* const tail = base + tp_.total - tp_.kx - tp_.tail;
@@ -910,46 +908,46 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
       if (at.pass > more.size()) more.resize(at.pass);
       std::vector<OzPackTask>& op = at.pass == 0 ? optasks : more[at.pass - 1].packs;
       std::vector<OzGemmTask>& ot = at.pass == 0 ? otasks : more[at.pass - 1].tiles;
-      const int64_t nkb = cdiv_i(kb_ - ka, oz.k), nkc = cdiv_i(kb_ - ka, oz.kc);
+      const int64_t nkb = cdiv_i(kb_ - ka, kOz.k), nkc = cdiv_i(kb_ - ka, kOz.kc);
       unsigned char* const PA = at.rg.p + at.off;
       unsigned char* const PB = PA + oz_size(rb - ra, kb_ - ka, false);
       int* const EA = reinterpret_cast<int*>(PA + oz_bytes(rb - ra, kb_ - ka, false));
       int* const EB = reinterpret_cast<int*>(PB + oz_bytes(cb - ca, kb_ - ka, true));
       const size_t first = ot.size();
-      for (int64_t tj = ca; tj < cb; tj += oz.tile_n)
-        for (int64_t ti = ra; ti < rb; ti += oz.tile_m) {
+      for (int64_t tj = ca; tj < cb; tj += kOz.tile_n)
+        for (int64_t ti = ra; ti < rb; ti += kOz.tile_m) {
           OzTile w{};
           if (!tile(ti, tj, w)) continue;
           const int64_t k0 = std::max(w.k0, ka), k1 = std::min(w.k1, kb_);
           if (k0 >= k1) continue;
           OzGemmTask t{};
-          t.A = PA + (ti - ra) / oz.tile_m * nkb * oz.a_block;
-          t.B = PB + (tj - ca) / oz.tile_n * nkb * oz.b_block;
-          t.ea = EA + (ti - ra) / oz.tile_m * nkc * oz.tile_m;
-          t.eb = EB + (tj - ca) / oz.tile_n * nkc * oz.tile_n;
+          t.A = PA + (ti - ra) / kOz.tile_m * nkb * kOz.a_block;
+          t.B = PB + (tj - ca) / kOz.tile_n * nkb * kOz.b_block;
+          t.ea = EA + (ti - ra) / kOz.tile_m * nkc * kOz.tile_m;
+          t.eb = EB + (tj - ca) / kOz.tile_n * nkc * kOz.tile_n;
           t.C = reinterpret_cast<double2*>(w.C);
           t.ldc = (int)w.ldc;
-          t.m = (int)std::min<int64_t>(oz.tile_m, A.R - ti);
-          t.n = (int)std::min<int64_t>(oz.tile_n, B.R - tj);
-          t.kb0 = (int)((k0 - ka) / oz.k);
-          t.nkb = (int)(cdiv_i(k1 - ka, oz.k) - t.kb0);
+          t.m = (int)std::min<int64_t>(kOz.tile_m, A.R - ti);
+          t.n = (int)std::min<int64_t>(kOz.tile_n, B.R - tj);
+          t.kb0 = (int)((k0 - ka) / kOz.k);
+          t.nkb = (int)(cdiv_i(k1 - ka, kOz.k) - t.kb0);
           t.doff = w.doff;
           t.flags = k0 > w.k0 ? w.flags & ~GF_BETA0 : w.flags;   // a later piece adds to the ones before it
           ot.push_back(t);
         }
       if (ot.size() == first) return false;
       auto pack = [&](const OzOperand& X_, bool b, unsigned char* dst, int* exps, int64_t r_first, int64_t r_end) {
-        const int64_t rows = b ? oz.tile_n : oz.tile_m, block = b ? oz.b_block : oz.a_block;
-        for (int64_t r0 = r_first; r0 < r_end; r0 += oz.tile_m)
-          for (int64_t k0 = ka; k0 < kb_; k0 += oz.kc) {
+        const int64_t rows = b ? kOz.tile_n : kOz.tile_m, block = b ? kOz.b_block : kOz.a_block;
+        for (int64_t r0 = r_first; r0 < r_end; r0 += kOz.tile_m)
+          for (int64_t k0 = ka; k0 < kb_; k0 += kOz.kc) {
             OzPackTask t{};
             t.src = reinterpret_cast<const double2*>(X_.src);
             t.scale = reinterpret_cast<const double2*>(X_.scale);
             t.lds = (int)X_.lds;
-            t.dst = dst + ((r0 - r_first) / rows * nkb + (k0 - ka) / oz.k) * block;
-            t.exps = exps + ((r0 - r_first) / rows * nkc + (k0 - ka) / oz.kc) * rows;
-            t.sub_stride = nkb * oz.b_block;
-            t.exp_stride = nkc * oz.tile_n;
+            t.dst = dst + ((r0 - r_first) / rows * nkb + (k0 - ka) / kOz.k) * block;
+            t.exps = exps + ((r0 - r_first) / rows * nkc + (k0 - ka) / kOz.kc) * rows;
+            t.sub_stride = nkb * kOz.b_block;
+            t.exp_stride = nkc * kOz.tile_n;
             t.ld = (int)X_.ld;
             t.r0 = (int)r0;
             t.k0 = (int)k0;
@@ -981,8 +979,8 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
         oz_piece(A, B, K, bal, tile, at, 0, A.R, 0, B.R, 0, K);
         at.off += need;
       } else {
-        const int64_t k1 = std::min<int64_t>(K, oz.kc), rowA = oz_size(oz.tile_m, k1, false), rowB = oz_size(oz.tile_n, k1, true);
-        const int64_t nA = cdiv_i(A.R, oz.tile_m), nB = cdiv_i(B.R, oz.tile_n), room = at.rg.bytes;
+        const int64_t k1 = std::min<int64_t>(K, kOz.kc), rowA = oz_size(kOz.tile_m, k1, false), rowB = oz_size(kOz.tile_n, k1, true);
+        const int64_t nA = cdiv_i(A.R, kOz.tile_m), nB = cdiv_i(B.R, kOz.tile_n), room = at.rg.bytes;
         int64_t q = 1, a = nA, b = nB;   // 128s of columns, 128s of A's rows and 32s of B's per piece
         if (nA * rowA + nB * rowB <= room) {
           q = room / (nA * rowA + nB * rowB);
@@ -990,14 +988,14 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
           a = std::min(nA, std::max<int64_t>(1, (room - std::min(nB * rowB, room / 2)) / rowA));
           b = std::min(nB, std::max<int64_t>(1, (room - a * rowA) / rowB));
         }
-        for (int64_t ka = 0; ka < K; ka += q * oz.kc)
-          for (int64_t ra = 0; ra < A.R; ra += a * oz.tile_m)
-            for (int64_t ca = 0; ca < B.R; ca += b * oz.tile_n)
-              if (oz_piece(A, B, K, bal, tile, at, ra, std::min(A.R, ra + a * oz.tile_m), ca, std::min(B.R, ca + b * oz.tile_n), ka,
-                           std::min(K, ka + q * oz.kc)))
+        for (int64_t ka = 0; ka < K; ka += q * kOz.kc)
+          for (int64_t ra = 0; ra < A.R; ra += a * kOz.tile_m)
+            for (int64_t ca = 0; ca < B.R; ca += b * kOz.tile_n)
+              if (oz_piece(A, B, K, bal, tile, at, ra, std::min(A.R, ra + a * kOz.tile_m), ca, std::min(B.R, ca + b * kOz.tile_n), ka,
+                           std::min(K, ka + q * kOz.kc)))
                 ++at.pass;
       }
-      return (double)K * (A.R * (16.0 + oz.a_block / (oz.tile_m * oz.k)) + B.R * (16.0 + oz.b_block / (oz.tile_n * oz.k)));
+      return (double)K * (A.R * (16.0 + kOz.a_block / (kOz.tile_m * kOz.k)) + B.R * (16.0 + kOz.b_block / (kOz.tile_n * kOz.k)));
     };
     // the launches of a step: its columns' exponents, then operands and tiles pass by pass
     auto oz_launches = [&](Launch lx, Launch lp, Launch lt) {
@@ -1007,7 +1005,7 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
       if (lt.count == 0) return;
       auto tile_bytes = [&](Launch& l) {
         for (int64_t i = l.off; i < l.off + l.count; ++i)
-          l.bytes += (double)otasks[i].nkb * (oz.a_block + oz.b_block) + 32.0 * otasks[i].m * otasks[i].n;
+          l.bytes += (double)otasks[i].nkb * (kOz.a_block + kOz.b_block) + 32.0 * otasks[i].m * otasks[i].n;
       };
       if (stall_next) {
         otasks[lt.off].flags |= GF_TEST_STALL;
@@ -1165,7 +1163,7 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
               Balance{nullptr, nullptr, blk + b0, ld + 1},
               [&](int64_t ti, int64_t tj, OzTile& t) {
                 t = {ft.G + (b1 + tj) * ld + b1 + ti, ld, 0, kOzBlock, ti > tj ? kAll : (int)(ti - tj), GF_NEG};
-                return ti >= tj / oz.tile_m * oz.tile_m;
+                return ti >= tj / kOz.tile_m * kOz.tile_m;
               },
               at);
           lp.bytes += oz_product(
@@ -1463,7 +1461,7 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
                   OzOperand{ft.G + s_, ld, u_, TC_PACK_PLAIN}, OzOperand{ft.G, ld, s_, TC_PACK_UNIT_LOWER}, s_,
                   Balance{kx0, kx0 + s_, nullptr, 0},
                   [&](int64_t ti, int64_t tj, OzTile& t) {
-                    t = {ft.Z + tj * u_ + ti, u_, 0, std::min<int64_t>(tj + oz.tile_n, s_), kAll, GF_BETA0};
+                    t = {ft.Z + tj * u_ + ti, u_, 0, std::min<int64_t>(tj + kOz.tile_n, s_), kAll, GF_BETA0};
                     return true;
                   },
                   at);
@@ -1473,7 +1471,7 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
                   OzOperand{ft.Z, u_, u_, TC_PACK_PLAIN, ft.dinv, 1}, OzOperand{ft.Z, u_, u_, TC_PACK_PLAIN}, s_,
                   Balance{nullptr, nullptr, ft.dinv, 1},
                   [&](int64_t ti, int64_t tj, OzTile& t) {
-                    if (ti < tj / oz.tile_m * oz.tile_m) return false;
+                    if (ti < tj / kOz.tile_m * kOz.tile_m) return false;
                     t = {ft.U + upd_index((int)std::max(ti, tj), (int)tj, ft.u, 128) - std::max<int64_t>(0, tj - ti), 128, 0, s_,
                          ti > tj ? kAll : (int)(ti - tj), GF_NEG};
                     return true;

@@ -221,7 +221,7 @@ void launch_tc_pack(const TcPackTask* tasks, int ntasks, cudaStream_t st);
 void launch_tc_gemm(const TcGemmTask* tasks, int ntasks, int* status, cudaStream_t st);
 // tensor-core path of complex128 fronts: operands written once as eight base-256 digits, then 128 x 32 tiles
 struct OzShape { int tile_m, tile_n, k, kc; int64_t a_block, b_block; };   // tile, k per block and per row scale, bytes per block
-OzShape oz_shape();
+constexpr OzShape kOz{128, 32, 16, 128, 65536, 24576};
 struct OzPackTask {        // 128 rows x 128 k of an operand
   const double2* src;      // column-major source, ld
   const double2* scale;    // PLAIN only: column k times scale[k * lds] (nullptr: no scaling)
