@@ -24,9 +24,8 @@
 // each (48 by their shared-memory reads of 6 KB; 70 before their descriptors were unrolled to constants), and the
 // blocks' way from L2 (88 KB per 16 k) is next: with a sixth of the MMAs the time falls to 0.57.  One CTA per SM over
 // many tiles, so copies and MMAs of the next tile overlap this one's additions (one tile per CTA: 107 against 92 ms
-// then).  The front products of an 80^3 lens setup: 860 ms with FP64 FMAs, 76 ms here plus 29 ms to write the digits
-// and 3 ms for the columns' balance (the wide fronts' F_TL and inverse among them, psp_api.cu kOzBlock).  Without the
-// balance, which gives Z D^-1 different digits in the Schur update and in M_BL, the digits took 24 ms.
+// then).  The front products of an 80^3 lens setup: 860 ms with FP64 FMAs, 76 ms here plus 24 ms to write the digits
+// and 3 ms for the columns' balance (the wide fronts' F_TL and inverse among them, psp_api.cu kOzBlock).
 #include <cstdint>
 
 #include "cplx.cuh"
@@ -55,6 +54,7 @@ constexpr int EPI_THREADS = 256, THREADS = EPI_THREADS + 64;   // + the copying 
 constexpr int kEmptyRow = -(1 << 16);          // exponent of a row of zeros
 constexpr int kBadRow = 1 << 20;               // exponent of a row with an infinity or a NaN
 constexpr int kFar = 1 << 12;                  // balance of a column whose partner is zero: past every exponent
+constexpr int kNear = 4;                       // spread of two balances, in bits, over which one serves for the other
 
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
   uint64_t d = 0;
@@ -173,21 +173,41 @@ __global__ void __launch_bounds__(256) k_oz_colmax(const OzColTask* __restrict__
 // them from shared memory (K-major, 8-row x 16-byte core matrices).  Thread (row, half): k in [8 half, 8 half + 8) of
 // every 16.  Two passes over the source (the second from L2): row exponents, then digits.  The balance 2^s(k) of a
 // column is added to its entries' exponents.  HBM-bound: 16 bytes read and 32 (A) or 48 (B) written per entry.
+//
+// Z D^-1 is an operand of the Schur update, balanced by its scale D^-1 alone, and of M_BL, balanced by that and the columns
+// of Z and inv(L)^T.  Over 128 k the two balances differ by a constant, which the row exponents absorb, and by what the
+// columns' sizes vary besides; where that stays within kNear bits M_BL takes the Schur update's balance and digits (four
+// fifths of a 48^3 lens' front entries).  It costs up to those bits of the thirteen that the digits have beyond 64-bit
+// sums (2^-59 against 2^-46 for 128 terms; measured, M_BL's error stays at 1.4e-16 where FP64 products have 2e-15).  80^3
+// lens, k_oz_pack: 29.0 ms with Z D^-1 packed twice everywhere, 24.5 so (24.2 before products were balanced).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_oz_pack(const OzPackTask* __restrict__ tasks) {
-  __shared__ int emax_s[2][OM], bal[OKC];
+  __shared__ int emax_s[2][OM], bal[OKC], least, most;
   const OzPackTask tk = tasks[blockIdx.x];
   const int row = threadIdx.x & (OM - 1), half = threadIdx.x >> 7;
   const int rg = tk.r0 + row;
+  if (threadIdx.x == 0) {
+    least = kFar;
+    most = -kFar;
+  }
+  __syncthreads();
+  int s = 0, scale_s = 0;   // balance of column threadIdx.x, and by the scale alone
   if (threadIdx.x < OKC) {
     const int k = tk.k0 + threadIdx.x;
-    int s = 0;
     if (k < tk.K && (tk.ka || tk.kd)) {
       const int ea = tk.ka ? tk.ka[k] : 1, eb = tk.ka ? tk.kb[k] : 1, ed = tk.kd ? exponent(tk.kd[(int64_t)k * tk.ldk]) - 1023 : 0;
       s = ea == 0 ? kFar : eb == 0 ? -kFar : (eb - ea - ed) >> 1;
+      scale_s = -ed >> 1;
+      if (tk.near) {
+        atomicMin(&least, s - scale_s);
+        atomicMax(&most, s - scale_s);
+      }
     }
-    bal[threadIdx.x] = tk.rows_b ? -s : s;
   }
+  __syncthreads();
+  const bool near = tk.near && most - least <= kNear && most < kFar / 2 && least > -kFar / 2;
+  if (near && (tk.near & OZ_KEEP)) return;
+  if (threadIdx.x < OKC) bal[threadIdx.x] = (tk.rows_b ? -1 : 1) * (near ? scale_s : s);
   __syncthreads();
   auto load = [&](int k) {
     double2 v = make_double2(0.0, 0.0);

@@ -875,6 +875,7 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
       const int *ka = nullptr, *kb = nullptr;
       const T* kd = nullptr;
       int64_t ldk = 0;
+      int near = 0;     // OzNear, of the first operand
     };
     // The complex128 tensor-core products of one step: C = +-A B^T, A of RA rows (src, ld, its columns k times
     // scale[k lds]) and B of RB rows, over K columns.  tile(ti, tj, t) says whether a tile exists and gives its place
@@ -959,6 +960,7 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
             t.kb = bal.kb;
             t.kd = reinterpret_cast<const double2*>(bal.kd);
             t.ldk = (int)bal.ldk;
+            t.near = b ? bal.near & OZ_NEAR : bal.near;
             op.push_back(t);
           }
       };
@@ -1443,8 +1445,8 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
       }
       if constexpr (std::is_same<T, double2>::value) {
         // complex128 fronts on the tensor cores.  Phase 0: Z = F_BL inv(L)^T.  Phase 1: the Schur update (Z D^-1) Z^T; then
-        // (extended form) M_BL = (Z D^-1) inv(L), for which Z D^-1 is packed again, balanced against inv(L).  The
-        // Schur update's operands are balanced by their pivots alone.
+        // (extended form) M_BL = (Z D^-1) inv(L), for which Z D^-1 is packed again where it has to be balanced against
+        // inv(L).  The Schur update's operands are balanced by their pivots alone.
         for (int step = 0; step < (phase == 0 ? 1 : si == PSP_SI_EXTENDED ? 2 : 1); ++step) {
           Launch lx{OZCOL, f0, (int64_t)octasks.size(), 0, -1}, lp{OZPACK, f0, (int64_t)optasks.size(), 0, -1},
               lt{OZGEMM, f0, (int64_t)otasks.size(), 0, -1};
@@ -1479,11 +1481,13 @@ static void factor_attempt(psp_ctx_s* X, cudaStream_t st, const std::function<vo
                   at);
               lt.flops += 8.0 * s_ * u_ * (u_ + 1.0) / 2;
             } else {
+              // the Schur update's Z D^-1 is where this product packs it, unless either runs in pieces
+              const bool kept = oz_size(u_, s_, false) + std::max(oz_size(u_, s_, true), oz_size(s_, s_, true)) <= packs[f0 + f].bytes;
               lx.bytes += oz_colmax(ft.Z, u_, u_, s_, TC_PACK_PLAIN, kx0 + 2 * s_);
               lx.bytes += oz_colmax(ft.G, ld, s_, s_, TC_PACK_UNIT_LOWER_T, kx0 + 3 * s_);
               lp.bytes += oz_product(
                   OzOperand{ft.Z, u_, u_, TC_PACK_PLAIN, ft.dinv, 1}, OzOperand{ft.G, ld, s_, TC_PACK_UNIT_LOWER_T}, s_,
-                  Balance{kx0 + 2 * s_, kx0 + 3 * s_, ft.dinv, 1},
+                  Balance{kx0 + 2 * s_, kx0 + 3 * s_, ft.dinv, 1, kept ? OZ_NEAR | OZ_KEEP : OZ_NEAR},
                   [&](int64_t ti, int64_t tj, OzTile& t) {
                     t = {ft.G + tj * ld + s_ + ti, ld, tj, s_, kAll, GF_BETA0};
                     return true;

@@ -235,8 +235,11 @@ struct OzPackTask {        // 128 rows x 128 k of an operand
   const int* ka;           // balance of the product's columns k (k_oz_pack): exponents of A's columns before its scale ...
   const int* kb;           // ... and of B's (both nullptr: taken as equal)
   const double2* kd;       // A's scale, stride ldk (nullptr: none)
-  int ldk, pad_;
+  int ldk;
+  int near;                // OZ_NEAR: the scale's balance alone serves 128 k where it is close to the whole one; OZ_KEEP: and
+                           // then this operand's digits in that balance are in place already
 };
+enum OzNear { OZ_NEAR = 1, OZ_KEEP = 2 };
 struct OzColTask {         // 32 columns k of an operand: exponents of their largest entries
   const double2* src;
   int* out;                // out[k]
