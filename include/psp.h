@@ -112,7 +112,8 @@ typedef struct {
   int tc_min_dim;     /* complex64 path: fronts with s >= tc_min_dim and u >= tc_min_dim take the tensor
                          cores, the others CUDA cores; <= 0 selects the default (64) */
   int sweep_level_tasks; /* sweep schedule: tasks a tree level is split into at least (row / column
-                            blocks of sweep_min_rows to sweep_max_rows); <= 0 selects the default (304) */
+                            blocks of sweep_min_rows to sweep_max_rows); <= 0 selects the default: 304, and
+                            608 for one right-hand side on boxes with 0.8 GB of complex64 factors and more */
   int sweep_ctas_per_sm; /* sweep schedule: resident CTAs per SM of the persistent sweep (capped by
                             occupancy: the kernel is built for two); <= 0 selects the default (as many as fit) */
   int setup_temp_mb;   /* cap, in MiB, on the per-front temporaries of one batch of fronts during setup

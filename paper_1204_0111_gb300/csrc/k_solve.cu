@@ -635,8 +635,10 @@ __device__ __forceinline__ bool wait_count(const unsigned* p, unsigned target, i
 // Warm L2 with the factor lines a task will stream, while its dependencies are still being
 // waited for (the lines do not depend on them): up the tree rows [r0, r1) of the columns
 // j < min(r1, s), down the tree columns [c0, c1) from below their diagonal to the end.  One warp, at most
-// kPrefetchLines lines (the product reads the rest itself).
-constexpr int kPrefetchLines = 2048;
+// kPrefetchLines lines (the product reads the rest itself).  1024 lines: 40 MB over 304 CTAs; with 2048 those of large tasks
+// push each other out of L2 before they are read (one complex64 column, layered models: 176^3 85.4 / 83.3 ms, 200^3 134.4 /
+// 128.1; salt body 128^3 x 8 45.3 / 44.7; no difference up to 160^3), with 512 smaller ones arrive late (100^3 14.5 / 14.9)
+constexpr int kPrefetchLines = 1024;
 
 template <typename T>
 __device__ __forceinline__ void prefetch_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const int lane) {

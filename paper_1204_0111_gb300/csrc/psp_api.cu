@@ -293,19 +293,6 @@ struct psp_ctx_s {
   int64_t factor_elems = 0;
   size_t elem_bytes = 16;
   std::vector<int64_t> panel_fbase;
-  // solve plan
-  struct LevelPlan {
-    int64_t fwd_off = 0;
-    int nfwd = 0, smax = 0;
-    int64_t bwd_off = 0;
-    int nbwd = 0, ldmax = 0;
-    // second phases of the fronts (factors that keep L_BL): up rows r >= s, down columns
-    int64_t fwdB_off = 0, bwdB_off = 0;
-    int nfwdB = 0, nbwdB = 0;
-    double entries = 0;   // factor entries read by one direction of this level
-    double vec = 0;       // vector entries gathered / written by one direction
-  };
-  std::vector<std::vector<LevelPlan>> splan;
   // persistent sweep plan
   struct SweepPlan {
     DevBuf steps, queue;
@@ -313,7 +300,10 @@ struct psp_ctx_s {
     int64_t nfront_steps = 0;                 // fronts summed over the steps
     double entries = 0, vec = 0;              // algorithmic factor entries / vector words per sweep
   };
-  SweepPlan plans[3];              // 0: Alg. 1.5 over the handle's panels; 1: its forward part; 2: its backward part
+  // 0: Alg. 1.5 over the handle's panels; 1: its forward part; 2: its backward part.  plans[1]: the same in finer tasks, for
+  // one right-hand side (fine_plans)
+  SweepPlan plans[2][3];
+  bool fine_plans = false;
   DevBuf d_sweep_sync, d_front_recs;
   std::vector<DevBuf> d_rows;      // per shape: index words of the fronts' rows
   std::vector<int> front_base;     // per shape: its first record in d_front_recs
@@ -345,6 +335,7 @@ struct psp_ctx_s {
   bool use_tc = true;
   bool diag_fp64 = false;   // complex64: diagonal blocks factored and applied in complex128
   int tc_min_dim = 64;
+  bool sweep_tasks_given = false;   // sweep_level_tasks was asked for or tuned, not the default
   int sweep_level_tasks = 304, sweep_ctas_per_sm = 8, sweep_rhs_group = 0, solve_rhs_group = 0, sweep_min_rows = 4;
   int sweep_max_rows = 256;
   int sweep_claim_ahead = 1;   // tasks a sweep CTA holds besides the one it runs
@@ -1613,15 +1604,29 @@ static void factor_all(psp_ctx_s* X, cudaStream_t st, const std::function<void()
 // ---------------------------------------------------------------------------
 // Solve plan: per shape and level, forward row tasks and backward column tasks.
 // ---------------------------------------------------------------------------
-static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
-  SideStream side;   // the tables go up while the device still factors
+struct LevelPlan {
+  int64_t fwd_off = 0;
+  int nfwd = 0, smax = 0;
+  int64_t bwd_off = 0;
+  int nbwd = 0, ldmax = 0;
+  // second phases of the fronts (factors that keep L_BL): up rows r >= s, down columns
+  int64_t fwdB_off = 0, bwdB_off = 0;
+  int nfwdB = 0, nbwdB = 0;
+  double entries = 0;   // factor entries read by one direction of this level
+  double vec = 0;       // vector entries gathered / written by one direction
+};
+
+// One schedule: the three plans, a level split into at least level_tasks(shape) tasks.  Returns the counters its largest plan
+// needs.
+template <typename F>
+static size_t plan_schedule(psp_ctx_s* X, const SideStream& side, const F& level_tasks, psp_ctx_s::SweepPlan (&plans)[3]) {
   std::vector<SolveTask> tasks;
-  X->splan.assign(X->shapes.size(), {});
+  std::vector<std::vector<LevelPlan>> splan(X->shapes.size());
   for (size_t si = 0; si < X->shapes.size(); ++si) {
     const Shape& sh = X->shapes[si];
-    X->splan[si].resize(sh.nlevels);
+    splan[si].resize(sh.nlevels);
     for (int lv = 0; lv < sh.nlevels; ++lv) {
-      auto& P = X->splan[si][lv];
+      auto& P = splan[si][lv];
       int64_t rows = 0, cols = 0;
       for (int sn : sh.level_sns[lv]) {
         rows += sh.s[sn] + sh.u[sn];
@@ -1641,9 +1646,9 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
       // front gathers once)
       const int rmin = std::max(2, std::min(64, X->sweep_min_rows));
       int R = X->sweep_max_rows;
-      while (R > rmin && rows / R < X->sweep_level_tasks) R >>= 1;
+      while (R > rmin && rows / R < level_tasks(sh)) R >>= 1;
       int Cc = X->sweep_max_rows;
-      while (Cc > rmin && cols / Cc < X->sweep_level_tasks) Cc >>= 1;
+      while (Cc > rmin && cols / Cc < level_tasks(sh)) Cc >>= 1;
       const bool two = X->si_mode != PSP_SI_EXTENDED, tri = X->si_mode == PSP_SI_NONE;
       // extended factors: one pass per front and direction over all s + u rows; factors keeping L_BL:
       // up, rows r < s (one whole-front substitution task without inversion) then rows r >= s; down,
@@ -1686,7 +1691,7 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
     ntask_down.resize(ntask_down.size() + sh.nsn, 0);
     ntask_upA.resize(ntask_upA.size() + sh.nsn, 0);
     ntask_downA.resize(ntask_downA.size() + sh.nsn, 0);
-    for (const auto& P : X->splan[si]) {
+    for (const auto& P : splan[si]) {
       for (int t = 0; t < P.nfwd; ++t) ntask_upA[front_base[si] + tasks[P.fwd_off + t].sn]++;
       for (int t = 0; t < P.nbwd; ++t) ntask_downA[front_base[si] + tasks[P.bwd_off + t].sn]++;
       for (int t = 0; t < P.nfwdB; ++t) ntask_up[front_base[si] + tasks[P.fwdB_off + t].sn]++;
@@ -1702,7 +1707,7 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
   }
   X->sweep_smax = 0;
   X->sweep_ldmax = 0;
-  for (const auto& sp : X->splan)
+  for (const auto& sp : splan)
     for (const auto& P : sp) {
       X->sweep_smax = std::max(X->sweep_smax, P.smax);
       X->sweep_ldmax = std::max(X->sweep_ldmax, P.ldmax);
@@ -1715,7 +1720,7 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
   // step of its own problem.
   size_t sync_words = 0;
   for (int pi = 0; pi < 3; ++pi) {
-    psp_ctx_s::SweepPlan& SP = X->plans[pi];
+    psp_ctx_s::SweepPlan& SP = plans[pi];
     struct Step {
       int panel, mode, prob;   // mode 0: forward sweep (assign), 1: backward sweep (subtract)
     };
@@ -1816,7 +1821,7 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
         }
         queue.push_back(e);
       };
-      const auto& plan = X->splan[si];
+      const auto& plan = splan[si];
       for (size_t lv = 0; lv < plan.size(); ++lv) {
         for (int t = 0; t < plan[lv].nfwd; ++t) entry(tasks[plan[lv].fwd_off + t], 0);
         for (int t = 0; t < plan[lv].nfwdB; ++t) entry(tasks[plan[lv].fwdB_off + t], kDirUpB);
@@ -1858,6 +1863,30 @@ static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
     SP.nfront_steps = nfs;
     sync_words = std::max(sync_words, (size_t)words);
   }
+  return sync_words;
+}
+
+// complex64: bytes of a box's factors from which one right-hand side takes twice the tasks per level.  A panel solve then
+// streams its factors longer than its chain of levels waits, and shorter tasks shorten the end of each level; with several
+// columns the vectors that every task gathers cost more than that gives.  One column, layered models, 304 / 608 tasks:
+// 112^3 (0.6 GB a box) 20.7 / 22.8 ms, 120^3 26.1 / 26.0, 128^3 (0.86 GB) 33.0 / 31.1, 144^3 48.0 / 42.9, 160^3 67.0 / 59.7,
+// 176^3 90.4 / 85.1, 200^3 134.9 / 134.1 (then with k_sweep's shorter prefetch 83.3 and 128.1); eight columns: 128^3 74.0 /
+// 76.4, 160^3 140.6 / 148.7
+constexpr double kFineBoxBytes = 0.8e9;
+
+static void plan_solve(psp_ctx_s* X, cudaStream_t st) {
+  SideStream side;   // the tables go up while the device still factors
+  size_t sync_words = plan_schedule(X, side, [&](const Shape&) { return X->sweep_level_tasks; }, X->plans[0]);
+  auto fine = [&](const Shape& sh) { return sh.g_total * 8.0 >= kFineBoxBytes; };
+  X->fine_plans = X->prec == PSP_PREC_C64 && !X->sweep_tasks_given && std::any_of(X->shapes.begin(), X->shapes.end(), fine);
+  if (X->fine_plans)
+    sync_words = std::max(sync_words, plan_schedule(X, side, [&](const Shape& sh) { return X->sweep_level_tasks * (fine(sh) ? 2 : 1); },
+                                                    X->plans[1]));
+  else
+    for (auto& sp : X->plans[1]) {
+      sp.steps.release();
+      sp.queue.release();
+    }
   X->sweep_sync_words = sync_words;
   X->d_sweep_sync.alloc(X->sweep_sync_words * 4);
   side.join(st);
@@ -1882,7 +1911,7 @@ static void ensure_apply_ws(psp_ctx_s* X, int nrhs) {
 template <typename T>
 static void apply_core(psp_ctx_s* X, double2* u, int nrhs, T* xf, T* xb, T* upd, bool timed, cudaStream_t st,
                        int plan_index = 0) {
-  const psp_ctx_s::SweepPlan& SP = X->plans[plan_index];
+  const psp_ctx_s::SweepPlan& SP = X->plans[nrhs == 1 && X->fine_plans ? 1 : 0][plan_index];
   if (SP.nsteps == 0) return;   // an empty part (the backward part of a block holding the last panel alone)
   SweepArgs<T> sa{};
   sa.xf = xf;
@@ -2682,6 +2711,7 @@ static void init_options(psp_ctx_s* X, const psp_options& o) {
   // 304 = two CTAs on each of 152 SMs.  152 / 228 / 304 / 456 / 608 tasks per level: lens100 complex128 41.1 / 37.0 / 33.9 /
   // 34.3 / 36.4 ms, complex64 13.1 / 12.1 / 11.6 / 13.3 / 15.0; 88^3 x 8 complex64 19.8 / 18.9 / 18.2 / 20.4 / 22.6; salt body
   // 128^3 x 8 51.0 / 45.8 / 45.3 / 45.5 / 46.5; on 32^3 and 48^3 fewer gain up to 5 % (1.72 / 1.72 / 1.76 / 1.80 / 2.06)
+  X->sweep_tasks_given = o.sweep_level_tasks > 0;
   X->sweep_level_tasks = o.sweep_level_tasks > 0 ? o.sweep_level_tasks : 304;
   X->sweep_ctas_per_sm = o.sweep_ctas_per_sm > 0 ? o.sweep_ctas_per_sm : 8;
   X->sweep_rhs_group = o.sweep_rhs_group > 0 ? o.sweep_rhs_group : 0;
@@ -3098,11 +3128,12 @@ psp_status psp_tune_sweep(psp_handle X, int nrhs, int reps, void* stream, psp_sw
   cudaEvent_t e0, e1;
   PSP_CK(cudaEventCreate(&e0));
   PSP_CK(cudaEventCreate(&e1));
-  struct Sched { int lt, cps, rg, mr, xr, ca; };
+  struct Sched { int lt, cps, rg, mr, xr, ca; bool given; };   // given: lt is not the handle's default
   int timed = 0;
   auto time_one = [&](const Sched& c) {
-    if (c.lt != X->sweep_level_tasks || c.mr != X->sweep_min_rows || c.xr != X->sweep_max_rows) {
+    if (c.lt != X->sweep_level_tasks || c.given != X->sweep_tasks_given || c.mr != X->sweep_min_rows || c.xr != X->sweep_max_rows) {
       X->sweep_level_tasks = c.lt;
+      X->sweep_tasks_given = c.given;
       X->sweep_min_rows = c.mr;
       X->sweep_max_rows = c.xr;
       plan_solve(X, st);
@@ -3123,15 +3154,16 @@ psp_status psp_tune_sweep(psp_handle X, int nrhs, int reps, void* stream, psp_sw
   const bool was_timing = X->stats.timing;
   X->stats.timing = false;
   Sched best{X->sweep_level_tasks, X->sweep_ctas_per_sm, X->sweep_rhs_group, X->sweep_min_rows, X->sweep_max_rows,
-             X->sweep_claim_ahead};
+             X->sweep_claim_ahead, X->sweep_tasks_given};
+  const bool fine_plans = nrhs == 1 && X->fine_plans;   // the default splits some levels otherwise than 304 tasks asked for
   double best_ms = 0, initial_ms = 0;
   // schedules that come to the same tasks and the same launch are timed once
-  std::set<std::tuple<int, int, int, int, int, int>> seen;
+  std::set<std::tuple<int, int, int, int, int, int, bool>> seen;
   auto fresh = [&](const Sched& c) {
     const SweepFit f = X->prec == PSP_PREC_C64
                            ? sweep_fit<float2>(nrhs, X->si_mode, X->sweep_smax, X->sweep_ldmax, c.cps, c.rg)
                            : sweep_fit<double2>(nrhs, X->si_mode, X->sweep_smax, X->sweep_ldmax, c.cps, c.rg);
-    return seen.insert({c.lt, f.per_sm, f.rg, c.mr, c.xr, c.ca}).second;
+    return seen.insert({c.lt, f.per_sm, f.rg, c.mr, c.xr, c.ca, c.given && fine_plans}).second;
   };
   try {
     fresh(best);
@@ -3145,18 +3177,18 @@ psp_status psp_tune_sweep(psp_handle X, int nrhs, int reps, void* stream, psp_sw
       }
     };
     for (int xr : {64, 128, 256})
-      consider({best.lt, best.cps, best.rg, best.mr, xr, best.ca});
+      consider({best.lt, best.cps, best.rg, best.mr, xr, best.ca, best.given});
     for (int lt : {152, 304, 608, 1216, 2432})
-      consider({lt, best.cps, best.rg, best.mr, best.xr, best.ca});
+      consider({lt, best.cps, best.rg, best.mr, best.xr, best.ca, true});
     for (int cps : {2, 3, 4, 6, 8})
-      consider({best.lt, cps, best.rg, best.mr, best.xr, best.ca});
+      consider({best.lt, cps, best.rg, best.mr, best.xr, best.ca, best.given});
     if (nrhs > 1)
       for (int rg : {1, 2, 4, 8})
-        consider({best.lt, best.cps, rg, best.mr, best.xr, best.ca});
+        consider({best.lt, best.cps, rg, best.mr, best.xr, best.ca, best.given});
     for (int mr : {4, 8, 16, 32, 64})
-      consider({best.lt, best.cps, best.rg, mr, best.xr, best.ca});
+      consider({best.lt, best.cps, best.rg, mr, best.xr, best.ca, best.given});
     for (int ca : {1, 2})
-      consider({best.lt, best.cps, best.rg, best.mr, best.xr, ca});
+      consider({best.lt, best.cps, best.rg, best.mr, best.xr, ca, best.given});
   } catch (...) {
     X->stats.timing = was_timing;
     cudaEventDestroy(e0);
@@ -3166,8 +3198,10 @@ psp_status psp_tune_sweep(psp_handle X, int nrhs, int reps, void* stream, psp_sw
   X->stats.timing = was_timing;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (best.lt != X->sweep_level_tasks || best.mr != X->sweep_min_rows || best.xr != X->sweep_max_rows) {
+  if (best.lt != X->sweep_level_tasks || best.given != X->sweep_tasks_given || best.mr != X->sweep_min_rows ||
+      best.xr != X->sweep_max_rows) {
     X->sweep_level_tasks = best.lt;
+    X->sweep_tasks_given = best.given;
     X->sweep_min_rows = best.mr;
     X->sweep_max_rows = best.xr;
     plan_solve(X, st);
@@ -3177,7 +3211,7 @@ psp_status psp_tune_sweep(psp_handle X, int nrhs, int reps, void* stream, psp_sw
   X->sweep_claim_ahead = best.ca;
   if (out) {
     std::memset(out, 0, sizeof(*out));
-    out->sweep_level_tasks = best.lt;
+    out->sweep_level_tasks = fine_plans && !best.given ? 2 * best.lt : best.lt;   // what asks for the schedule kept
     out->sweep_ctas_per_sm = best.cps;
     out->sweep_rhs_group = best.rg;
     out->sweep_min_rows = best.mr;
