@@ -295,13 +295,30 @@ __device__ __forceinline__ void fwd_task(const TaskSlot<T>& sl, const SweepArgs<
   }
 }
 
+__device__ __forceinline__ float2 from_lane(const float2 v, const int l) {
+  return make_float2(__shfl_sync(0xffffffffu, v.x, l), __shfl_sync(0xffffffffu, v.y, l));
+}
+__device__ __forceinline__ double2 from_lane(const double2 v, const int l) {
+  return make_double2(__shfl_sync(0xffffffffu, v.x, l), __shfl_sync(0xffffffffu, v.y, l));
+}
+
+// Substitution through a 32 x 32 diagonal block by one warp, lane k holding row (up) or column (down) b + k of the vector in
+// registers.  The block's entries are read tri_cols columns at a time before they are used: read one by one, each is a trip
+// to L2 in the chain of 32, and with two CTAs per SM too few other fronts hide it.  One application without inversion, lens
+// models, read one by one -> so (before the warps had roles, with four CTAs per SM): 48^3 complex64 28.1 -> 14.6 ms (22.6),
+// 100^3 complex64 179.6 -> 97.9 (128.5), 100^3 complex128 364.6 -> 283.7 (339.0).
+template <typename T>
+constexpr int tri_cols() { return sizeof(T) == 8 ? 16 : 8; }
+
 // Without inversion (G keeps L_TL): the first phase up the tree of front sn by one CTA: w_S gathered
 // as above, then forward substitution y_S = L_TL^{-1} w_S in blocks of 32 columns (one warp solves
 // the diagonal block, all threads update the rows below it), x_S = D^{-1} y_S into xf, y_S into xb.
-// w: room for RG x s entries (right-hand side major), in shared memory or, for a front too wide for it, the front's
-// own entries of xb, which no other task reads or writes before this one is done.
-template <typename T, int RG>
-__device__ __noinline__ void fwd_tri_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr, T* w) {
+// The vector, RG x s entries (right-hand side major), is in shared memory or, for a front too wide for it (WIDE), in the
+// front's own entries of xb, which no other task reads or writes before this one is done.
+template <typename T, int RG, bool WIDE>
+__device__ __noinline__ void fwd_tri_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  T* const w = WIDE ? entry_ptr<T, RG>(sl.xb, a.n_loc, sl.fr.first, gr) : reinterpret_cast<T*>(smem);
   const int s = sl.fr.s, ld = s + sl.fr.u;
   const T* G = sl.G;
   const int tid = threadIdx.x;
@@ -319,15 +336,27 @@ __device__ __noinline__ void fwd_tri_task(const TaskSlot<T>& sl, const SweepArgs
     const int be = min(b + 32, s);
     if (warp == 0) {
       // diagonal block: y_j final, then w_k -= L[k, j] y_j for b <= j < k < be
-      for (int j = b; j < be; ++j) {
-        const int k = b + lane;
-        const T l = (k > j && k < be) ? __ldg(G + (int64_t)j * ld + k) : CplxTraits<T>::zero();
-        __syncwarp();
-        if (k > j && k < be)
+      constexpr int JB = tri_cols<T>();
+      const int k = b + lane;
+      T v[RG];
 #pragma unroll
-          for (int q = 0; q < RG; ++q) cfms(w[q * s + k], l, w[q * s + j]);
-        __syncwarp();
+      for (int q = 0; q < RG; ++q) v[q] = k < be ? w[q * s + k] : CplxTraits<T>::zero();
+      for (int j0 = b; j0 < be; j0 += JB) {
+        T l[JB];
+#pragma unroll
+        for (int t = 0; t < JB; ++t)
+          l[t] = (k > j0 + t && k < be) ? __ldg(G + (int64_t)(j0 + t) * ld + k) : CplxTraits<T>::zero();
+#pragma unroll
+        for (int t = 0; t < JB; ++t)
+#pragma unroll
+          for (int q = 0; q < RG; ++q) {
+            const T y = from_lane(v[q], j0 + t - b);
+            if (k > j0 + t && k < be) cfms(v[q], l[t], y);
+          }
       }
+      if (k < be)
+#pragma unroll
+        for (int q = 0; q < RG; ++q) w[q * s + k] = v[q];
     }
     compute_sync();
     // rows below the block: w_i -= sum_{j in block} L[i, j] y_j
@@ -335,6 +364,7 @@ __device__ __noinline__ void fwd_tri_task(const TaskSlot<T>& sl, const SweepArgs
       T acc[RG];
 #pragma unroll
       for (int q = 0; q < RG; ++q) acc[q] = CplxTraits<T>::zero();
+#pragma unroll 8
       for (int j = b; j < be; ++j) {
         const T l = __ldg(G + (int64_t)j * ld + i);
 #pragma unroll
@@ -515,9 +545,11 @@ __device__ __forceinline__ void bwd_task(const TaskSlot<T>& sl, const SweepArgs<
 // Without inversion: the second phase down the tree of front sn by one CTA: back substitution
 // L_TL^T x_S = t (t in xf) in blocks of 32 columns from the last, each block first takes the
 // products with the solved rows below it (one warp per column), then one warp solves the block.
-// x: RG x s entries (right-hand side major) as fwd_tri_task's w: t, overwritten by x block by block.
-template <typename T, int RG>
-__device__ __noinline__ void bwd_tri_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr, T* x) {
+template <typename T, int RG, bool WIDE>
+__device__ __noinline__ void bwd_tri_task(const TaskSlot<T>& sl, const SweepArgs<T>& a, const Group gr) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  // RG x s entries (right-hand side major) as in fwd_tri_task: t, overwritten by x block by block
+  T* const x = WIDE ? entry_ptr<T, RG>(sl.xb, a.n_loc, sl.fr.first, gr) : reinterpret_cast<T*>(smem);
   const int s = sl.fr.s, ld = s + sl.fr.u;
   const T* G = sl.G;
   const int tid = threadIdx.x;
@@ -554,15 +586,27 @@ __device__ __noinline__ void bwd_tri_task(const TaskSlot<T>& sl, const SweepArgs
     compute_sync();
     if (warp == 0) {
       // the block, from its last column: x_c final, then x_k -= L[c, k] x_c for b <= k < c
-      for (int c = be - 1; c >= b; --c) {
-        const int k = b + lane;
-        const T l = (k < c) ? __ldg(G + (int64_t)k * ld + c) : CplxTraits<T>::zero();
-        __syncwarp();
-        if (k < c)
+      constexpr int JB = tri_cols<T>();
+      const int k = b + lane;
+      T v[RG];
 #pragma unroll
-          for (int q = 0; q < RG; ++q) cfms(x[q * s + k], l, x[q * s + c]);
-        __syncwarp();
+      for (int q = 0; q < RG; ++q) v[q] = k < be ? x[q * s + k] : CplxTraits<T>::zero();
+      for (int c0 = b + 32 - JB; c0 >= b; c0 -= JB) {
+        T l[JB];
+#pragma unroll
+        for (int t = 0; t < JB; ++t)
+          l[t] = (k < c0 + t && c0 + t < be) ? __ldg(G + (int64_t)k * ld + c0 + t) : CplxTraits<T>::zero();
+#pragma unroll
+        for (int t = JB - 1; t >= 0; --t)
+#pragma unroll
+          for (int q = 0; q < RG; ++q) {
+            const T y = from_lane(v[q], c0 + t - b);
+            if (k < c0 + t && c0 + t < be) cfms(v[q], l[t], y);
+          }
       }
+      if (k < be)
+#pragma unroll
+        for (int q = 0; q < RG; ++q) x[q * s + k] = v[q];
     }
     compute_sync();
   }
@@ -775,12 +819,15 @@ __device__ __forceinline__ void signal_done(TaskSlot<T>* slots, const SweepArgs<
   }
 }
 
-// EXT: extended selective inversion (one task per front and direction); otherwise the forms that keep L_BL.
+// FORM: extended selective inversion (one task per front and direction), the forms that keep L_BL and inverses of L_TL, or no
+// inversion.  A kernel for each, so that none holds registers for another's tasks.
 // The registers are held to sweep_ctas CTAs per SM (65,536 / (320 threads x CTAs)).
 template <typename T, int RG>
 constexpr int sweep_ctas() { return 2; }
 
-template <typename T, int RG, bool EXT>
+enum SweepForm { kFormExtended, kFormInverse, kFormNone };
+
+template <typename T, int RG, int FORM>
 __global__ void __launch_bounds__(kSweepThreads, (sweep_ctas<T, RG>())) k_sweep(const __grid_constant__ SweepArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(16) TaskSlot<T> slots[2];
@@ -807,22 +854,22 @@ __global__ void __launch_bounds__(kSweepThreads, (sweep_ctas<T, RG>())) k_sweep(
                                    reinterpret_cast<uintptr_t>(sl.upd + g * RG * a.upd_ld)) & 15) == 0;
         if (g > 0) compute_sync();
         const int dir = sl.e.dir;
-        if constexpr (EXT) {
+        if constexpr (FORM == kFormExtended) {
           if (dir == 0) fwd_task<T, RG, 0, true>(sl, a, gr, smem);
           else bwd_task<T, RG, 0, true>(sl, a, gr, smem);
         } else {
-          const bool tri = a.si == PSP_SI_NONE;
-          T* const whole = a.tri_global ? entry_ptr<T, RG>(sl.xb, a.n_loc, sl.fr.first, gr) : reinterpret_cast<T*>(smem);
           if (dir == 0) {
-            if (tri) fwd_tri_task<T, RG>(sl, a, gr, whole);
-            else fwd_task<T, RG, 0, false>(sl, a, gr, smem);
+            if constexpr (FORM == kFormInverse) fwd_task<T, RG, 0, false>(sl, a, gr, smem);
+            else if (RG == 1 && a.tri_global) fwd_tri_task<T, 1, true>(sl, a, gr);
+            else fwd_tri_task<T, RG, false>(sl, a, gr);
           } else if (dir == kDirUpB) {
             fwd_task<T, RG, 1, false>(sl, a, gr, smem);
           } else if (dir == 1) {
             bwd_task<T, RG, 0, false>(sl, a, gr, smem);
           } else {
-            if (tri) bwd_tri_task<T, RG>(sl, a, gr, whole);
-            else bwd_task<T, RG, 1, false>(sl, a, gr, smem);
+            if constexpr (FORM == kFormInverse) bwd_task<T, RG, 1, false>(sl, a, gr, smem);
+            else if (RG == 1 && a.tri_global) bwd_tri_task<T, 1, true>(sl, a, gr);
+            else bwd_tri_task<T, RG, false>(sl, a, gr);
           }
         }
       }
@@ -832,9 +879,9 @@ __global__ void __launch_bounds__(kSweepThreads, (sweep_ctas<T, RG>())) k_sweep(
   }
 }
 
-template <typename T, int RG, bool EXT>
+template <typename T, int RG, int FORM>
 static int sweep_rg(const SweepArgs<T>& args, size_t smem, int max_per_sm, SweepFit* fit, cudaStream_t st) {
-  if (cudaFuncSetAttribute(k_sweep<T, RG, EXT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+  if (cudaFuncSetAttribute(k_sweep<T, RG, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
     cudaGetLastError();
     return -1;
   }
@@ -842,7 +889,7 @@ static int sweep_rg(const SweepArgs<T>& args, size_t smem, int max_per_sm, Sweep
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<T, RG, EXT>, kSweepThreads, smem) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<T, RG, FORM>, kSweepThreads, smem) != cudaSuccess ||
       per_sm < 1) {
     cudaGetLastError();
     return -1;
@@ -856,9 +903,9 @@ static int sweep_rg(const SweepArgs<T>& args, size_t smem, int max_per_sm, Sweep
   void* kargs[] = {&a};
   cudaError_t e;
   if (coop) {
-    e = cudaLaunchCooperativeKernel((const void*)k_sweep<T, RG, EXT>, dim3(sms * per_sm), dim3(kSweepThreads), kargs, smem, st);
+    e = cudaLaunchCooperativeKernel((const void*)k_sweep<T, RG, FORM>, dim3(sms * per_sm), dim3(kSweepThreads), kargs, smem, st);
   } else {   // one CTA alone takes the queue in order and never waits
-    k_sweep<T, RG, EXT><<<1, kSweepThreads, smem, st>>>(a);
+    k_sweep<T, RG, FORM><<<1, kSweepThreads, smem, st>>>(a);
     e = cudaGetLastError();
   }
   return e == cudaSuccess ? 0 : (int)e;
@@ -887,8 +934,9 @@ static int sweep_sized(const SweepArgs<T>& args, int smax, int ldmax, int max_pe
     a.tri_global = RG == 1 && whole + 2 * sizeof(TaskSlot<T>) > 226 * 1024;
     if (!a.tri_global && smem < whole) smem = whole;
   }
-  return a.si == PSP_SI_EXTENDED ? sweep_rg<T, RG, true>(a, smem, max_per_sm, fit, st)
-                                 : sweep_rg<T, RG, false>(a, smem, max_per_sm, fit, st);
+  if (a.si == PSP_SI_EXTENDED) return sweep_rg<T, RG, kFormExtended>(a, smem, max_per_sm, fit, st);
+  if (a.si == PSP_SI_NONE) return sweep_rg<T, RG, kFormNone>(a, smem, max_per_sm, fit, st);
+  return sweep_rg<T, RG, kFormInverse>(a, smem, max_per_sm, fit, st);
 }
 
 template <typename T>
