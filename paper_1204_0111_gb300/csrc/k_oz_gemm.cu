@@ -172,7 +172,8 @@ __global__ void __launch_bounds__(256) k_oz_colmax(const OzColTask* __restrict__
 // k_oz_pack: digits of 128 rows x 128 k of an operand (rows r0.., k from k0) per CTA, laid out as the MMAs read
 // them from shared memory (K-major, 8-row x 16-byte core matrices).  Thread (row, half): k in [8 half, 8 half + 8) of
 // every 16.  Two passes over the source (the second from L2): row exponents, then digits.  The balance 2^s(k) of a
-// column is added to its entries' exponents.  HBM-bound: 16 bytes read and 32 (A) or 48 (B) written per entry.
+// column is added to its entries' exponents.  16 bytes read and 32 (A) or 48 (B) written per entry, at 0.4 of DRAM's rate: the
+// passes' latency and the digits' integer instructions bound it.
 //
 // Z D^-1 is an operand of the Schur update, balanced by its scale D^-1 alone, and of M_BL, balanced by that and the columns
 // of Z and inv(L)^T.  Over 128 k the two balances differ by a constant, which the row exponents absorb, and by what the

@@ -2715,8 +2715,8 @@ static void init_options(psp_ctx_s* X, const psp_options& o) {
   X->sweep_level_tasks = o.sweep_level_tasks > 0 ? o.sweep_level_tasks : 304;
   X->sweep_ctas_per_sm = o.sweep_ctas_per_sm > 0 ? o.sweep_ctas_per_sm : 8;
   X->sweep_rhs_group = o.sweep_rhs_group > 0 ? o.sweep_rhs_group : 0;
-  // 4 against 8 rows: top levels of one or two fronts still have a task for every SM (100^3 lens complex128 33.9 / 35.7 ms,
-  // complex64 11.5 / 11.7 ms, the waveguide's 48^3 solve with four columns 193 / 213 ms; 2 rows: 35.0, 12.0, 185)
+  // 4 against 8 rows: top levels of one or two fronts still have a task for every SM (100^3 lens complex128 33.9 / 35.8 ms,
+  // complex64 11.6 / 11.8 ms, a 48^3 waveguide solve with four columns 193 / 213 ms; 2 rows: 35.0, 12.1, 185)
   X->sweep_min_rows = o.sweep_min_rows > 0 ? o.sweep_min_rows : 4;
   X->sweep_max_rows = o.sweep_max_rows > 0 ? std::min(256, std::max(64, o.sweep_max_rows)) : 256;
   X->sweep_claim_ahead = o.sweep_claim_ahead > 0 ? o.sweep_claim_ahead : 1;
