@@ -306,7 +306,9 @@ __device__ __forceinline__ double2 from_lane(const double2 v, const int l) {
 // registers.  The block's entries are read tri_cols columns at a time before they are used: read one by one, each is a trip
 // to L2 in the chain of 32, and with two CTAs per SM too few other fronts hide it.  One application without inversion, lens
 // models, read one by one -> so (before the warps had roles, with four CTAs per SM): 48^3 complex64 28.1 -> 14.6 ms (22.6),
-// 100^3 complex64 179.6 -> 97.9 (128.5), 100^3 complex128 364.6 -> 283.7 (339.0).
+// 100^3 complex64 179.6 -> 97.9 (128.5), 100^3 complex128 364.6 -> 268.5 (339.0).  Complex128 leaves out columns that no lane
+// needs, whose operations the FP64 pipe would run all the same (14^3 x 8 8.57 -> 7.62 ms, 72^3 x 8 772 -> 742); in
+// complex64 the branches cost more than they save (72^3 x 8 74.1 -> 79.2).
 template <typename T>
 constexpr int tri_cols() { return sizeof(T) == 8 ? 16 : 8; }
 
@@ -347,12 +349,14 @@ __device__ __noinline__ void fwd_tri_task(const TaskSlot<T>& sl, const SweepArgs
         for (int t = 0; t < JB; ++t)
           l[t] = (k > j0 + t && k < be) ? __ldg(G + (int64_t)(j0 + t) * ld + k) : CplxTraits<T>::zero();
 #pragma unroll
-        for (int t = 0; t < JB; ++t)
+        for (int t = 0; t < JB; ++t) {
+          if (sizeof(T) == 16 && j0 + t >= be - 1) break;   // no row below it
 #pragma unroll
           for (int q = 0; q < RG; ++q) {
             const T y = from_lane(v[q], j0 + t - b);
             if (k > j0 + t && k < be) cfms(v[q], l[t], y);
           }
+        }
       }
       if (k < be)
 #pragma unroll
@@ -597,12 +601,14 @@ __device__ __noinline__ void bwd_tri_task(const TaskSlot<T>& sl, const SweepArgs
         for (int t = 0; t < JB; ++t)
           l[t] = (k < c0 + t && c0 + t < be) ? __ldg(G + (int64_t)k * ld + c0 + t) : CplxTraits<T>::zero();
 #pragma unroll
-        for (int t = JB - 1; t >= 0; --t)
+        for (int t = JB - 1; t >= 0; --t) {
+          if (sizeof(T) == 16 && (c0 + t >= be || c0 + t == b)) continue;   // beyond the block, or no column before it
 #pragma unroll
           for (int q = 0; q < RG; ++q) {
             const T y = from_lane(v[q], c0 + t - b);
             if (k < c0 + t && c0 + t < be) cfms(v[q], l[t], y);
           }
+        }
       }
       if (k < be)
 #pragma unroll
